@@ -2,8 +2,8 @@
 //
 // Each CTA walks the query-major tile list the planner gave it.  A tile is 256 query rows
 // (two 128-row sub-tiles, "slots") of one head shard; for every head of the shard the CTA
-// streams the key/value blocks the rows can see, from the block that holds the start of the
-// first row's sample up to the diagonal block.  Blocks are cut at multiples of 128 on the
+// streams the key/value blocks the rows can see, from the diagonal block down to the block that
+// holds the start of the first row's sample.  Blocks are cut at multiples of 128 on the
 // pool's token axis, so the diagonal block of a sub-tile is aligned with it and every other
 // visible block is either dense or needs the per-row sample-start mask.
 //
@@ -11,9 +11,17 @@
 // thread, S read from TMEM, P written back to TMEM as bf16 over S), warp 8 issues TMA loads,
 // warp 9 issues tcgen05.mma, warps 10-11 only hand their registers to the softmax groups.
 // TMEM: S0 | S1 | O0 | O1, 128 fp32 columns each.
-// Pipeline per key block j:   PV0(j) S0(j+1) PV1(j) S1(j+1)   on the tensor pipe, while the
-// softmax group of one slot works during the other slot's MMAs.  P is handed over in two halves
-// (keys 0-63, then 64-127), so the first four key steps of PV run under the second half's exponentials.
+// Pipeline per key block j:   PV0(j) S0(j-1) PV1(j) S1(j-1)   on the tensor pipe, while the
+// softmax group of one slot works during the other slot's MMAs.  Slot 1 sees one block more than slot 0; walking
+// the blocks downwards puts its solitary block at the start of a tile, where slot 0 is still storing its last O.
+// P is handed over in two parts (keys 0-95, then 96-127), so that only a quarter of PV(j) is left to run when the
+// last exponential is done (two 65536-token samples, Hq 32: 60.9 ms, with halves 62.6).
+//
+// What bounds it: per key block and slot a chain S -> maximum -> exponentials -> PV -> S of about 3100 clk for 2048 clk
+// of MMA, and between tiles the drain and refill of that chain.  Masks as bit words and the O tile through a staging
+// tile and a bulk tensor store took most off the latter (a masked block cost 1000-3400 clk more than a dense one, the
+// row-per-thread stores 3500 clk per slot): 4096 tokens, 4 heads of 64: 39.0 -> 31.3 us; 10007 tokens in samples of up to
+// 400, 8 heads of 128: 45.1 -> 32.3 us; 131072 tokens, 32 / 8 heads of 128: 6.63 -> 6.25 ms (945 -> 1000 TFLOP/s).
 #include <math.h>
 
 #include "common.h"
@@ -29,6 +37,7 @@ namespace libra {
 constexpr int kBM = 128;            // rows per slot
 constexpr int kBN = 128;            // keys per block
 constexpr int kFwdThreads = 384;  // warps 10-11 only donate registers
+constexpr int kPFirst = 96;       // keys of P handed to the MMA role in the first part
 constexpr float kRescaleThreshold = 8.0f;  // log2 units: O is rescaled only when the max grows by more
 constexpr uint64_t kFwdDrainNs = 2000000;  // teardown after a give-up: budget for work already in flight to land
 
@@ -36,11 +45,12 @@ template <int D>
 struct FwdSmem {
     static constexpr int kHalfBytes = 128 * 128;              // 128 rows x 64 bf16 (one swizzle column)
     static constexpr int kTileBytes = kHalfBytes * (D / 64);  // one 128 x D operand tile
-    static constexpr int kStages = (D == 128) ? 5 : 8;
+    static constexpr int kStages = (D == 128) ? 4 : 8;
     static constexpr int kQOff = 0;
     static constexpr int kRingOff = 2 * kTileBytes;
-    static constexpr int kBarOff = kRingOff + kStages * kTileBytes;
-    // barriers: full[kStages], empty[kStages], q_full, q_empty, s_full[2], p_ready[2], o_done[2], p_half[2], drain
+    static constexpr int kStageOff = kRingOff + kStages * kTileBytes;  // O staging: per softmax warp 32 rows x 64 bf16
+    static constexpr int kBarOff = kStageOff + 8 * 4096;
+    // barriers: full[kStages], empty[kStages], q_full, q_empty, s_full[2], p_ready[2], o_done[2], p_part[2], drain
     static constexpr int kNumBars = 2 * kStages + 11;
     static constexpr int kMiscOff = kBarOff + kNumBars * 8;
     static constexpr int kBytes = kMiscOff + 16;
@@ -48,7 +58,6 @@ struct FwdSmem {
 };
 
 struct FwdParams {
-    __nv_bfloat16* out;
     float* lse;
     const int32_t* cta_offsets;
     const int32_t* cta_tiles;
@@ -64,24 +73,50 @@ struct FwdParams {
     uint32_t* tile_ns; // [tiles] time spent on each tile (slot 0's first softmax thread), ns
 };
 
-// Range of key blocks slot g of a tile sees; empty (lo > hi) if the slot lies past T.
-struct SlotRange {
-    int lo, hi;
+// One tile of the CTA's list: id, first row, key blocks lo[g] .. hi[g] of slot g (lo > hi: the slot lies past T).
+struct FwdTile {
+    int t;
+    int64_t q0;
+    int lo[2], hi[2];
 };
-__device__ __forceinline__ SlotRange slot_range(const int32_t* tok_start, int64_t T, int64_t qs) {
-    SlotRange r;
-    if (qs >= T) { r.lo = 1; r.hi = 0; return r; }
-    r.lo = tok_start[qs] / kBN;
-    r.hi = (int)(qs / kBN);
-    return r;
-}
-
-
+// Walks the list.  Ids are fetched two tiles and sample starts one tile ahead: a chain of two dependent global
+// loads between tiles would leave the tensor pipe idle for about 2000 clk.
+struct FwdTiles {
+    const FwdParams& p;
+    int idx, end;
+    int t1, t2, a1, b1;   // next tile: id, tok_start of the first row of each slot; id of the one after
+    __device__ __forceinline__ FwdTiles(const FwdParams& p_, int begin, int end_) : p(p_), idx(begin), end(end_), a1(0), b1(0) {
+        t1 = idx < end ? p.cta_tiles[idx] : -1;
+        t2 = idx + 1 < end ? p.cta_tiles[idx + 1] : -1;
+        fetch();
+    }
+    __device__ __forceinline__ void fetch() {
+        if (t1 < 0) return;
+        const int64_t q0 = (int64_t)(t1 / p.H) * (2 * kBM);
+        a1 = p.tok_start[q0];
+        b1 = q0 + kBM < p.T ? p.tok_start[q0 + kBM] : 0;
+    }
+    __device__ __forceinline__ bool next(FwdTile& x) {
+        if (t1 < 0) return false;
+        x.t = t1;
+        x.q0 = (int64_t)(t1 / p.H) * (2 * kBM);
+        x.hi[0] = (int)(x.q0 / kBN);
+        x.lo[0] = a1 / kBN;
+        const bool two = x.q0 + kBM < p.T;
+        x.hi[1] = two ? x.hi[0] + 1 : -1;
+        x.lo[1] = two ? b1 / kBN : 0;
+        ++idx;
+        t1 = t2;
+        t2 = idx + 1 < end ? p.cta_tiles[idx + 1] : -1;
+        fetch();
+        return true;
+    }
+};
 
 template <int D>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-           const __grid_constant__ CUtensorMap tm_v, const FwdParams p) {
+           const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_out, const FwdParams p) {
     using L = FwdSmem<D>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -93,7 +128,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     uint64_t* bar_sfull = bar_qfull + 2;   // [2]
     uint64_t* bar_pready = bar_qfull + 4;  // [2]
     uint64_t* bar_odone = bar_qfull + 6;   // [2]
-    uint64_t* bar_phalf = bar_qfull + 8;   // [2] P of the first 64 keys is in TMEM
+    uint64_t* bar_ppart = bar_qfull + 8;   // [2] P of the first kPFirst keys is in TMEM
     uint64_t* bar_drain = bar_qfull + 10;  // teardown after a give-up: every MMA issued so far has completed
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kMiscOff);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMiscOff + 4);
@@ -115,7 +150,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             mbar_init(&bar_sfull[g], 1);
             mbar_init(&bar_pready[g], kBM);
             mbar_init(&bar_odone[g], 1);
-            mbar_init(&bar_phalf[g], kBM);
+            mbar_init(&bar_ppart[g], kBM);
         }
         mbar_init(bar_drain, 1);
         abort_flag[0] = 0;
@@ -131,6 +166,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         prefetch_tmap(&tm_q);
         prefetch_tmap(&tm_k);
         prefetch_tmap(&tm_v);
+        prefetch_tmap(&tm_out);
     }
     tc_fence_before();
     __syncthreads();
@@ -149,150 +185,139 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     } else if (warp == 8) {
         // ---------------- TMA producer ----------------
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(LIBRA_FWD_REG_DEC));
-        const bool leader = elect_one();
-        uint32_t ring = 0, qcnt = 0;
-        bool ok = true;
-        for (int idx = tile_begin; idx < tile_end && ok && !p.inject_stall; ++idx) {
-            const int t = p.cta_tiles[idx];
-            const int64_t q0 = (int64_t)(t / p.H) * (2 * kBM);
-            const SlotRange r0 = slot_range(p.tok_start, p.T, q0);
-            const SlotRange r1 = slot_range(p.tok_start, p.T, q0 + kBM);
-            const bool act1 = r1.lo <= r1.hi;
-            const int lo = r0.lo, hi = act1 ? r1.hi : r0.hi;
-            for (int hh = 0; hh < heads_per_shard && ok; ++hh) {
-                const int h = (t % p.H) * heads_per_shard + hh;
-                const int kvh = h / G;
-                ok = warp_wait(bar_qempty, (qcnt & 1) ^ 1, abort_flag);
-                if (!ok) break;
-                if (leader) {
-                    mbar_arrive_expect_tx(bar_qfull, (act1 ? 2 : 1) * L::kTileBytes);
-                    for (int g = 0; g < (act1 ? 2 : 1); ++g)
-                        for (int half = 0; half < D / 64; ++half)
-                            tma_load_3d(smem + L::kQOff + g * L::kTileBytes + half * L::kHalfBytes, &tm_q, bar_qfull,
-                                        half * 64, h, (int)(q0 + g * kBM));
-                }
-                ++qcnt;
-                for (int j = lo; j <= hi && ok; ++j) {
-                    for (int kv = 0; kv < 2 && ok; ++kv) {  // K_j then V_j
-                        const uint32_t st = ring % L::kStages;
-                        ok = warp_wait(&bar_empty[st], ((ring / L::kStages) & 1) ^ 1, abort_flag);
-                        if (!ok) break;
-                        if (leader) {
+        if (elect_one()) {  // one elected thread runs the whole role
+            uint32_t ring = 0, qcnt = 0;
+            bool ok = true;
+            FwdTiles tiles(p, tile_begin, tile_end);
+            FwdTile x;
+            while (ok && !p.inject_stall && tiles.next(x)) {
+                const bool act1 = x.hi[1] >= 0;
+                const int top = act1 ? x.hi[1] : x.hi[0];
+                for (int hh = 0; hh < heads_per_shard && ok; ++hh) {
+                    const int h = (x.t % p.H) * heads_per_shard + hh;
+                    const int kvh = h / G;
+                    for (int j = top; j >= x.lo[0] && ok; --j) {
+                        for (int kv = 0; kv < 2; ++kv) {  // K_j then V_j
+                            const uint32_t st = ring % L::kStages;
+                            ok = mbar_wait(&bar_empty[st], ((ring / L::kStages) & 1) ^ 1, abort_flag);
+                            if (!ok) break;
                             mbar_arrive_expect_tx(&bar_full[st], L::kTileBytes);
                             for (int half = 0; half < D / 64; ++half)
                                 tma_load_3d(smem + L::kRingOff + st * L::kTileBytes + half * L::kHalfBytes,
                                             kv == 0 ? &tm_k : &tm_v, &bar_full[st], half * 64, kvh, j * kBN);
+                            ++ring;
+                            if (j == top && kv == 0) {   // Q behind the first K: the wait for its tile holds nothing else up
+                                ok = mbar_wait(bar_qempty, (qcnt & 1) ^ 1, abort_flag);
+                                if (!ok) break;
+                                mbar_arrive_expect_tx(bar_qfull, (act1 ? 2 : 1) * L::kTileBytes);
+                                for (int g = 1; g >= 0; --g)
+                                    for (int half = 0; half < D / 64; ++half)
+                                        if (g == 0 || act1)
+                                            tma_load_3d(smem + L::kQOff + g * L::kTileBytes + half * L::kHalfBytes, &tm_q,
+                                                        bar_qfull, half * 64, h, (int)(x.q0 + g * kBM));
+                                ++qcnt;
+                            }
                         }
-                        ++ring;
                     }
                 }
             }
-        }
-        if (leader && (!ok || abort_flag[0])) {
-            // Give-up path: nothing new is issued; the copies already issued land before shared memory is released.
-            if (qcnt > 0) mbar_wait_drain(bar_qfull, (qcnt - 1) & 1, kFwdDrainNs);
-            for (uint32_t b = 1; b <= (uint32_t)L::kStages && b <= ring; ++b)
-                mbar_wait_drain(&bar_full[(ring - b) % L::kStages], ((ring - b) / L::kStages) & 1, kFwdDrainNs);
+            if (!ok || abort_flag[0]) {
+                // Give-up path: nothing new is issued; the copies already issued land before shared memory is released.
+                if (qcnt > 0) mbar_wait_drain(bar_qfull, (qcnt - 1) & 1, kFwdDrainNs);
+                for (uint32_t b = 1; b <= (uint32_t)L::kStages && b <= ring; ++b)
+                    mbar_wait_drain(&bar_full[(ring - b) % L::kStages], ((ring - b) / L::kStages) & 1, kFwdDrainNs);
+            }
         }
         __syncwarp();
     } else if (warp == 9) {
         // ---------------- MMA issuer ----------------
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(LIBRA_FWD_REG_DEC));
-        const bool leader = elect_one();
-        constexpr uint32_t idesc_s = make_idesc(kBM, kBN, 0, 0);
-        constexpr uint32_t idesc_pv = make_idesc(kBM, D, 0, 1);
-        const uint32_t smem_base = smem_u32(smem);
-        uint32_t ring = 0, qcnt = 0;
-        uint32_t pcnt[2] = {0, 0};
-        bool ok = true;
-        // Base descriptors are built once; every MMA only adds a constant to them.
-        const uint64_t desc_q = make_sdesc(smem_base + L::kQOff, 16, 1024);                  // K-major Q slot 0
-        const uint64_t desc_k = make_sdesc(smem_base + L::kRingOff, 16, 1024);               // K-major ring stage 0
-        const uint64_t desc_v = make_sdesc(smem_base + L::kRingOff, L::kHalfBytes, 1024);    // MN-major ring stage 0
-        auto issue_s = [&](int g, uint32_t stage) {
-            const uint64_t qa = sdesc_advance(desc_q, g * L::kTileBytes);
-            const uint64_t ka = sdesc_advance(desc_k, stage * L::kTileBytes);
+        if (elect_one()) {  // one elected thread runs the whole role
+            constexpr uint32_t idesc_s = make_idesc(kBM, kBN, 0, 0);
+            constexpr uint32_t idesc_pv = make_idesc(kBM, D, 0, 1);
+            const uint32_t smem_base = smem_u32(smem);
+            uint32_t ring = 0, qcnt = 0;
+            uint32_t pcnt[2] = {0, 0};
+            bool ok = true;
+            // Base descriptors are built once; every MMA only adds a constant to them.
+            const uint64_t desc_q = make_sdesc(smem_base + L::kQOff, 16, 1024);                  // K-major Q slot 0
+            const uint64_t desc_k = make_sdesc(smem_base + L::kRingOff, 16, 1024);               // K-major ring stage 0
+            const uint64_t desc_v = make_sdesc(smem_base + L::kRingOff, L::kHalfBytes, 1024);    // MN-major ring stage 0
+            auto issue_s = [&](int g, uint32_t stage) {
+                const uint64_t qa = sdesc_advance(desc_q, g * L::kTileBytes);
+                const uint64_t ka = sdesc_advance(desc_k, stage * L::kTileBytes);
 #pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-                const uint32_t off = (kk / 4) * L::kHalfBytes + (kk % 4) * 32;
-                mma_ss(tmem_base + g * kBN, sdesc_advance(qa, off), sdesc_advance(ka, off), idesc_s, kk > 0);
-            }
-            tc_commit(&bar_sfull[g]);
-        };
-        // O[g] (+)= P[g] V over the key steps [kk0, kk1) of 16 keys; the softmax group hands P over in two halves
-        auto issue_pv = [&](int g, uint32_t stage, bool accumulate, int kk0, int kk1) {
-            const uint64_t va = sdesc_advance(desc_v, stage * L::kTileBytes);
+                for (int kk = 0; kk < D / 16; ++kk) {
+                    const uint32_t off = (kk / 4) * L::kHalfBytes + (kk % 4) * 32;
+                    mma_ss(tmem_base + g * kBN, sdesc_advance(qa, off), sdesc_advance(ka, off), idesc_s, kk > 0);
+                }
+                tc_commit(&bar_sfull[g]);
+            };
+            // O[g] (+)= P[g] V over the key steps [kk0, kk1) of 16 keys; the softmax group hands P over in two parts
+            auto issue_pv = [&](int g, uint32_t stage, bool accumulate, int kk0, int kk1) {
+                const uint64_t va = sdesc_advance(desc_v, stage * L::kTileBytes);
 #pragma unroll
-            for (int kk = kk0; kk < kk1; ++kk) {
-                mma_ts(tmem_base + 2 * kBN + g * D, tmem_base + g * kBN + kk * 8, sdesc_advance(va, kk * 2048), idesc_pv,
-                       (accumulate || kk > 0) ? 1u : 0u);
-            }
-            if (kk1 == kBN / 16) tc_commit(&bar_odone[g]);
-        };
-        for (int idx = tile_begin; idx < tile_end && ok; ++idx) {
-            const int t = p.cta_tiles[idx];
-            const int64_t q0 = (int64_t)(t / p.H) * (2 * kBM);
-            const SlotRange r[2] = {slot_range(p.tok_start, p.T, q0), slot_range(p.tok_start, p.T, q0 + kBM)};
-            const bool act1 = r[1].lo <= r[1].hi;
-            const int lo = r[0].lo, hi = act1 ? r[1].hi : r[0].hi;
-            for (int hh = 0; hh < heads_per_shard && ok; ++hh) {
-                ok = warp_wait(bar_qfull, qcnt & 1, abort_flag);
-                if (!ok) break;
-                ++qcnt;
-                // prologue: S(lo)
-                uint32_t st = ring % L::kStages;
-                ok = warp_wait(&bar_full[st], (ring / L::kStages) & 1, abort_flag);
-                if (!ok) break;
-                tc_fence_after();
-                if (leader) {
-                    for (int g = 0; g < 2; ++g)
-                        if (lo >= r[g].lo && lo <= r[g].hi) issue_s(g, st);
+                for (int kk = kk0; kk < kk1; ++kk) {
+                    mma_ts(tmem_base + 2 * kBN + g * D, tmem_base + g * kBN + kk * 8, sdesc_advance(va, kk * 2048), idesc_pv,
+                           (accumulate || kk > 0) ? 1u : 0u);
+                }
+                if (kk1 == kBN / 16) tc_commit(&bar_odone[g]);
+            };
+            FwdTiles tiles(p, tile_begin, tile_end);
+            FwdTile x;
+            while (ok && tiles.next(x)) {
+                const bool act1 = x.hi[1] >= 0;
+                const int top = act1 ? x.hi[1] : x.hi[0], lo = x.lo[0];
+                for (int hh = 0; hh < heads_per_shard && ok; ++hh) {
+                    // prologue: S of the top block (slot 1's diagonal block; slot 0's when the tile has no slot 1)
+                    uint32_t st = ring % L::kStages;
+                    ok = mbar_wait(&bar_full[st], (ring / L::kStages) & 1, abort_flag);
+                    if (ok) ok = mbar_wait(bar_qfull, qcnt & 1, abort_flag);
+                    if (!ok) break;
+                    ++qcnt;
+                    tc_fence_after();
+                    issue_s(act1 ? 1 : 0, st);
                     tc_commit(&bar_empty[st]);
-                    if (lo == hi) tc_commit(bar_qempty);  // no later MMA of this tile reads Q
-                }
-                ++ring;
-                for (int j = lo; j <= hi && ok; ++j) {
-                    const uint32_t st_v = ring % L::kStages;
-                    ok = warp_wait(&bar_full[st_v], (ring / L::kStages) & 1, abort_flag);
-                    if (!ok) break;
+                    if (lo == top) tc_commit(bar_qempty);  // no later MMA of this tile reads Q
                     ++ring;
-                    uint32_t st_k = 0;
-                    if (j + 1 <= hi) {
-                        st_k = ring % L::kStages;
-                        ok = warp_wait(&bar_full[st_k], (ring / L::kStages) & 1, abort_flag);
-                        if (!ok) break;
+                    for (int j = top; j >= lo && ok; --j) {
+                        const uint32_t st_v = ring % L::kStages;
+                        const uint32_t ph_v = (ring / L::kStages) & 1;
                         ++ring;
-                    }
-                    for (int g = 0; g < 2 && ok; ++g) {
-                        if (j >= r[g].lo && j <= r[g].hi) {
-                            ok = warp_wait(&bar_phalf[g], pcnt[g] & 1, abort_flag);   // P of keys 0..63
-                            if (!ok) break;
-                            tc_fence_after();
-                            if (leader) issue_pv(g, st_v, j != r[g].lo, 0, kBN / 32);
-                            ok = warp_wait(&bar_pready[g], pcnt[g] & 1, abort_flag);  // the rest, while those MMAs run
-                            if (!ok) break;
-                            ++pcnt[g];
-                            tc_fence_after();
-                            if (leader) issue_pv(g, st_v, j != r[g].lo, kBN / 32, kBN / 16);
+                        const bool more = j - 1 >= lo;
+                        const uint32_t st_k = ring % L::kStages;
+                        bool have_k = false, have_v = false;
+#pragma unroll
+                        for (int g = 0; g < 2; ++g) {
+                            if (j >= x.lo[g] && j <= x.hi[g]) {
+                                if (!have_v) { ok = mbar_wait(&bar_full[st_v], ph_v, abort_flag); have_v = true; }
+                                if (ok) ok = mbar_wait(&bar_ppart[g], pcnt[g] & 1, abort_flag);   // P of the first kPFirst keys
+                                if (!ok) break;
+                                tc_fence_after();
+                                issue_pv(g, st_v, j != x.hi[g], 0, kPFirst / 16);
+                                ok = mbar_wait(&bar_pready[g], pcnt[g] & 1, abort_flag);  // the rest, while those MMAs run
+                                if (!ok) break;
+                                ++pcnt[g];
+                                tc_fence_after();
+                                issue_pv(g, st_v, j != x.hi[g], kPFirst / 16, kBN / 16);
+                            }
+                            if (more && j - 1 >= x.lo[g] && j - 1 <= x.hi[g]) {
+                                if (!have_k) { ok = mbar_wait(&bar_full[st_k], (ring / L::kStages) & 1, abort_flag); have_k = true; }
+                                if (!ok) break;
+                                issue_s(g, st_k);
+                            }
                         }
-                        if (j + 1 <= hi && j + 1 >= r[g].lo && j + 1 <= r[g].hi) {
-                            if (leader) issue_s(g, st_k);
-                        }
-                    }
-                    if (!ok) break;
-                    if (leader) {
+                        if (!ok) break;
                         tc_commit(&bar_empty[st_v]);
-                        if (j + 1 <= hi) tc_commit(&bar_empty[st_k]);
-                        if (j + 1 == hi) tc_commit(bar_qempty);  // S(hi) was the last reader of Q: the next
+                        if (more) { tc_commit(&bar_empty[st_k]); ++ring; }
+                        if (j - 1 == lo) tc_commit(bar_qempty);  // S(lo) was the last reader of Q: the next
                     }                                            // tile's Q load overlaps the last block
-                    __syncwarp();
                 }
-                __syncwarp();
             }
-        }
-        if (leader && (!ok || abort_flag[0])) {   // give-up path: the MMAs already issued finish before TMEM is freed
-            tc_commit(bar_drain);
-            mbar_wait_drain(bar_drain, 0, kFwdDrainNs);
+            if (!ok || abort_flag[0]) {   // give-up path: the MMAs already issued finish before TMEM is freed
+                tc_commit(bar_drain);
+                mbar_wait_drain(bar_drain, 0, kFwdDrainNs);
+            }
         }
         __syncwarp();
     } else {
@@ -303,13 +328,32 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t t_s = tmem_base + lane_addr + g * kBN;
         const uint32_t t_o = tmem_base + lane_addr + 2 * kBN + g * D;
+        uint8_t* stage = smem + L::kStageOff + warp * 4096;
+        const uint64_t scale2 = f2_pack(p.scale_log2, p.scale_log2);
         uint32_t scnt = 0, ocnt = 0;
         bool ok = true;
-        for (int idx = tile_begin; idx < tile_end && ok; ++idx) {
-            const int t = p.cta_tiles[idx];
-            const int64_t qs = (int64_t)(t / p.H) * (2 * kBM) + g * kBM;
-            const SlotRange rg = slot_range(p.tok_start, p.T, qs);
-            if (rg.lo > rg.hi) continue;  // slot past the end of the pool
+        // O *= factor, once the PV of the previous block has landed in it
+        auto rescale_o = [&](float factor) -> bool {
+            if (!warp_wait(&bar_odone[g], (ocnt - 1) & 1, abort_flag)) return false;
+            tc_fence_after();
+#pragma unroll
+            for (int c = 0; c < D; c += 32) {
+                uint32_t orow[32];
+                tmem_ld32(t_o + c, orow);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) orow[i] = __float_as_uint(__uint_as_float(orow[i]) * factor);
+                tmem_st32(t_o + c, orow);
+            }
+            tmem_st_wait();
+            return true;
+        };
+        FwdTiles tiles(p, tile_begin, tile_end);
+        FwdTile x;
+        while (ok && tiles.next(x)) {
+            const int64_t qs = x.q0 + g * kBM;
+            const int lo = x.lo[g], hi = x.hi[g];
+            if (lo > hi) continue;  // slot past the end of the pool
             const uint64_t tile_t0 = threadIdx.x == 0 ? globaltimer_ns() : 0;
             const int64_t row = qs + row_in_tile;
             const bool row_ok = row < p.T;
@@ -318,9 +362,9 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             const int64_t last_row = (qs + kBM <= p.T ? qs + kBM : p.T) - 1;
             const int max_kstart = p.tok_start[last_row];
             for (int hh = 0; hh < heads_per_shard && ok; ++hh) {
-                const int h = (t % p.H) * heads_per_shard + hh;
+                const int h = (x.t % p.H) * heads_per_shard + hh;
                 float m_ref = -INFINITY, l_sum = 0.f;
-                for (int j = rg.lo; j <= rg.hi && ok; ++j) {
+                for (int j = hi; j >= lo && ok; --j) {
                     ok = warp_wait(&bar_sfull[g], scnt & 1, abort_flag);
                     if (!ok) break;
                     ++scnt;
@@ -332,13 +376,15 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                     tmem_ld32(t_s + 96, sr + 96);
                     tmem_ld_wait();
                     const int k0 = j * kBN;
-                    const bool need_mask = (k0 + kBN - 1 > qs) || (k0 < max_kstart) || !row_ok;
-                    if (need_mask) {
+                    if (j == hi || k0 < max_kstart || !row_ok) {
                         const int c_lo = row_ok ? kstart - k0 : kBN;        // first visible column
                         const int c_hi = row_ok ? (int)(row - k0) : -1;      // last visible column
 #pragma unroll
-                        for (int i = 0; i < kBN; ++i)
-                            if (i < c_lo || i > c_hi) sr[i] = 0xff800000u;  // -inf
+                        for (int w = 0; w < kBN / 32; ++w) {
+                            const uint32_t vis = range_bits(c_lo - 32 * w, c_hi - 32 * w);
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) sr[32 * w + i] = (vis >> i) & 1u ? sr[32 * w + i] : 0xff800000u;  // -inf
+                        }
                     }
                     float mx;
                     {   // eight independent chains keep the 3-input max off the latency-bound path
@@ -355,33 +401,17 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                     }
                     mx *= p.scale_log2;  // scale > 0, so the max commutes with it
                     // lazy rescale: keep the old reference unless the max grew by > threshold
-                    float m_new = m_ref;
-                    bool grow = false;
-                    if (mx > m_ref + kRescaleThreshold || (m_ref == -INFINITY && mx > -INFINITY)) {
-                        m_new = mx;
-                        grow = true;
+                    float factor = 1.0f;
+                    if (mx > m_ref + kRescaleThreshold) {
+                        factor = ex2_approx(m_ref - mx);   // m_ref = -inf gives 0
+                        m_ref = mx;
                     }
-                    const float factor = grow ? ex2_approx(m_ref - m_new) : 1.0f;  // m_ref=-inf gives 0
-                    const bool first = (j == rg.lo);
-                    if (!first && __any_sync(0xffffffffu, grow)) {
-                        // PV(j-1) must have landed in O before it is rescaled
-                        ok = warp_wait(&bar_odone[g], (ocnt - 1) & 1, abort_flag);
+                    if (j != hi && __any_sync(0xffffffffu, factor != 1.0f)) {
+                        ok = rescale_o(factor);
                         if (!ok) break;
-                        tc_fence_after();
-#pragma unroll
-                        for (int c = 0; c < D; c += 32) {
-                            uint32_t orow[32];
-                            tmem_ld32(t_o + c, orow);
-                            tmem_ld_wait();
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) orow[i] = __float_as_uint(__uint_as_float(orow[i]) * factor);
-                            tmem_st32(t_o + c, orow);
-                        }
                     }
                     l_sum *= factor;
-                    m_ref = m_new;
                     const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
-                    const uint64_t scale2 = f2_pack(p.scale_log2, p.scale_log2);
                     const uint64_t negm2 = f2_pack(-m_use, -m_use);
                     uint64_t psum2[4] = {f2_pack(0.f, 0.f), f2_pack(0.f, 0.f), f2_pack(0.f, 0.f), f2_pack(0.f, 0.f)};
 #pragma unroll
@@ -397,10 +427,10 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                             pk[i >> 1] = pack_bf16x2(p0, p1);
                         }
                         tmem_st16(t_s + (c >> 1), pk);
-                        if (c == kBN / 2 - 32) {  // P of the first 64 keys is complete: its PV steps can start
+                        if (c == kPFirst - 32) {  // P of the first kPFirst keys is complete: its PV steps can start
                             tmem_st_wait();
                             tc_fence_before();
-                            mbar_arrive(&bar_phalf[g]);
+                            mbar_arrive(&bar_ppart[g]);
                         }
                     }
                     {
@@ -419,32 +449,43 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 if (!ok) break;
                 tc_fence_after();
                 const float inv_l = (l_sum > 0.f) ? 1.0f / l_sum : 0.f;
-                __nv_bfloat16* orow_ptr = p.out + ((size_t)row * p.hq + h) * D;
+                // Through the warp's staging tile (32 rows x 128 bytes, 128-byte swizzle) and a bulk tensor store: one row
+                // per thread stored straight from registers touches 32 cache lines per instruction.  Rows past the end
+                // of the pool are dropped by the hardware.
 #pragma unroll
-                for (int c = 0; c < D; c += 32) {
-                    uint32_t orow[32];
+                for (int c = 0; c < D; c += 64) {
+                    uint32_t orow[64];
                     tmem_ld32(t_o + c, orow);
+                    tmem_ld32(t_o + c + 32, orow + 32);
                     tmem_ld_wait();
-                    if (row_ok) {
-                        uint4* dst = reinterpret_cast<uint4*>(orow_ptr + c);
+                    if (lane == 0) tma_store_wait_read();   // the store that last used the tile has read it
+                    __syncwarp();
 #pragma unroll
-                        for (int i = 0; i < 32; i += 8) {
-                            uint4 v;
-                            v.x = pack_bf16x2(__uint_as_float(orow[i]) * inv_l, __uint_as_float(orow[i + 1]) * inv_l);
-                            v.y = pack_bf16x2(__uint_as_float(orow[i + 2]) * inv_l, __uint_as_float(orow[i + 3]) * inv_l);
-                            v.z = pack_bf16x2(__uint_as_float(orow[i + 4]) * inv_l, __uint_as_float(orow[i + 5]) * inv_l);
-                            v.w = pack_bf16x2(__uint_as_float(orow[i + 6]) * inv_l, __uint_as_float(orow[i + 7]) * inv_l);
-                            dst[i >> 3] = v;
-                        }
+                    for (int ch = 0; ch < 8; ++ch) {
+                        uint4 v;
+                        const uint32_t* o = orow + 8 * ch;
+                        v.x = pack_bf16x2(__uint_as_float(o[0]) * inv_l, __uint_as_float(o[1]) * inv_l);
+                        v.y = pack_bf16x2(__uint_as_float(o[2]) * inv_l, __uint_as_float(o[3]) * inv_l);
+                        v.z = pack_bf16x2(__uint_as_float(o[4]) * inv_l, __uint_as_float(o[5]) * inv_l);
+                        v.w = pack_bf16x2(__uint_as_float(o[6]) * inv_l, __uint_as_float(o[7]) * inv_l);
+                        *reinterpret_cast<uint4*>(stage + lane * 128 + ((ch ^ (lane & 7)) << 4)) = v;
+                    }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        tma_store_3d(&tm_out, stage, c, h, (int)(qs + (warp & 3) * 32));
+                        tma_store_commit();
                     }
                 }
                 if (row_ok) p.lse[(size_t)h * p.T + row] = (m_ref + log2f(l_sum)) * 0.6931471805599453f;
                 // the next PV into this slot's O may only start after these reads: it is issued
-                // after this group's next p_ready arrival, which follows in program order
+                // after this group's next P arrival, which follows in program order
                 tc_fence_before();
             }
-            if (threadIdx.x == 0 && ok) p.tile_ns[t] = (uint32_t)(globaltimer_ns() - tile_t0);
+            if (threadIdx.x == 0 && ok) p.tile_ns[x.t] = (uint32_t)(globaltimer_ns() - tile_t0);
         }
+        // every bulk store this warp issued has completed before the CTA leaves
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
 
     // ---------------- teardown ----------------
@@ -516,8 +557,8 @@ int make_f32_3d_map(CUtensorMap* m, const void* base, int64_t T, int H, int d, i
 }
 
 template <int D>
-static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const FwdParams& prm, int W,
-                      cudaStream_t s) {
+static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tout,
+                      const FwdParams& prm, int W, cudaStream_t s) {
     using L = FwdSmem<D>;
     constexpr int kSlot = D == 128 ? 0 : 1;
     if (!cfg_done(kSlot)) {   // per device: the attribute belongs to the device's copy of the kernel
@@ -526,7 +567,7 @@ static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtens
         if (!regs_pool_ok(k_attn_fwd<D>, 256, LIBRA_FWD_REG_INC, 128, LIBRA_FWD_REG_DEC)) return LIBRA_ERR_UNSUPPORTED;
         cfg_mark(kSlot);
     }
-    k_attn_fwd<D><<<W, kFwdThreads, L::kAlloc, s>>>(tq, tk, tv, prm);
+    k_attn_fwd<D><<<W, kFwdThreads, L::kAlloc, s>>>(tq, tk, tv, tout, prm);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
@@ -561,14 +602,14 @@ extern "C" int libra_attn_pool_fwd(const void* q_dev, const void* k_dev, const v
         time_end(mp, 0, s);
         return rc256;
     }
-    CUtensorMap tq, tk, tv;
+    CUtensorMap tq, tk, tv, tout;
     int rc = make_thd_map(&tq, q_dev, plan->T, dims->hq, dims->head_dim, kBM);
     if (rc == LIBRA_OK) rc = make_thd_map(&tk, k_dev, plan->T, dims->hkv, dims->head_dim, kBN);
     if (rc == LIBRA_OK) rc = make_thd_map(&tv, v_dev, plan->T, dims->hkv, dims->head_dim, kBN);
+    if (rc == LIBRA_OK) rc = make_thd_map(&tout, out_dev, plan->T, dims->hq, dims->head_dim, 32);
     if (rc != LIBRA_OK) return rc;
 
     FwdParams prm;
-    prm.out = reinterpret_cast<__nv_bfloat16*>(out_dev);
     prm.lse = lse_dev;
     prm.cta_offsets = d.d_cta_offsets;
     prm.cta_tiles = d.d_cta_exec;
@@ -586,7 +627,8 @@ extern "C" int libra_attn_pool_fwd(const void* q_dev, const void* k_dev, const v
     prm.tile_ns = d.d_tile_ns;
     cudaMemsetAsync(plan->d_status + 1, 0, sizeof(int), s);   // the word reports the most recent launch
     time_begin(mp, 0, s);
-    rc = dims->head_dim == 128 ? launch_fwd<128>(tq, tk, tv, prm, d.W, s) : launch_fwd<64>(tq, tk, tv, prm, d.W, s);
+    rc = dims->head_dim == 128 ? launch_fwd<128>(tq, tk, tv, tout, prm, d.W, s)
+                               : launch_fwd<64>(tq, tk, tv, tout, prm, d.W, s);
     time_end(mp, 0, s);
     return rc;
 }
