@@ -476,9 +476,9 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         pf[j + 3] = ex2_sel(x3, jj + 3);
                     }
                     if (need_mask) {   // one uniform branch per half: the exponentials above stay one straight run
+                        const uint32_t vis = range_bits(j_lo - half * 32, j_hi - half * 32);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (half * 32 + j < j_lo || half * 32 + j > j_hi) pf[j] = 0.f;
+                        for (int j = 0; j < 32; ++j) pf[j] = (vis >> j) & 1u ? pf[j] : 0.f;
                     }
                     uint32_t pk[16];
 #pragma unroll

@@ -519,8 +519,11 @@ k_attn_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 }
                 if (need_mask) {
 #pragma unroll
-                    for (int i = 0; i < CW; ++i)
-                        if (i < c_lo || i > c_hi) pf[i] = 0.f;
+                    for (int w = 0; w < CW / 32; ++w) {
+                        const uint32_t vis = range_bits(c_lo - 32 * w, c_hi - 32 * w);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) pf[32 * w + i] = (vis >> i) & 1u ? pf[32 * w + i] : 0.f;
+                    }
                 }
                 // ---- dS = P o (dP - D), packed over this half's own dP columns ----
                 ok = warp_wait(bar_dpfull, blk & 1, abort_flag);

@@ -502,10 +502,11 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                             pf[j + 2] = ex2_approx(x2);
                             pf[j + 3] = ex2_approx(x3);
                         }
-                        if (need_mask) {
+                        if (need_mask) {   // as bits: compares per element became branches (10007 tokens in samples of up to
+                            // 400, 8 heads: this kernel 112.9 us with them, 102.6 without)
+                            const uint32_t vis = range_bits(j_lo - half * 32, j_hi - half * 32);
 #pragma unroll
-                            for (int j = 0; j < 32; ++j)
-                                if (half * 32 + j < j_lo || half * 32 + j > j_hi) pf[j] = 0.f;
+                            for (int j = 0; j < 32; ++j) pf[j] = (vis >> j) & 1u ? pf[j] : 0.f;
                         }
 #pragma unroll
                         for (int j = 0; j < 32; j += 2) pk[half * 16 + (j >> 1)] = pack_bf16x2(pf[j], pf[j + 1]);

@@ -381,6 +381,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                 // first and last visible column, counted from this thread's first column
                 const int c_lo = (int)(lo_abs - b0 > kBlk ? kBlk : lo_abs - b0) - col0;
                 const int c_hi = (int)(hi_abs - b0 < -1 ? -1 : hi_abs - b0) - col0;
+                const bool need_mask = __any_sync(0xffffffffu, c_lo > 0 || c_hi < NC - 1);   // most blocks are dense
                 const uint32_t s1 = L::slot1(itc);
                 const float* st = reinterpret_cast<const float*>(smem + L::kStatOff + s1 * 512) + col0;
                 if (L::kStatBytes > 0) {   // the streamed rows' statistics arrive with their first tile
@@ -396,9 +397,14 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                 tmem_ld_wait();
                 uint32_t pk[NC / 2];
                 if constexpr (MODE == FWD) {
+                    if (need_mask) {
 #pragma unroll
-                    for (int i = 0; i < kBlk; ++i)
-                        if (i < c_lo || i > c_hi) sr[i] = 0xff800000u;  // -inf
+                        for (int w = 0; w < kBlk / 32; ++w) {
+                            const uint32_t vis = range_bits(c_lo - 32 * w, c_hi - 32 * w);
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) sr[32 * w + i] = (vis >> i) & 1u ? sr[32 * w + i] : 0xff800000u;  // -inf
+                        }
+                    }
                     float mx = -INFINITY;
                     {
                         float pm[8];
@@ -452,8 +458,13 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
 #pragma unroll
                     for (int i = 0; i < NC; ++i) {
                         const float l2 = L::kKeyStationary ? st[i] : lse2r;
-                        const float e = ex2_approx(fmaf(__uint_as_float(sr[i]), p.scale_log2, -l2));
-                        pf[i] = (i < c_lo || i > c_hi) ? 0.f : e;
+                        pf[i] = ex2_approx(fmaf(__uint_as_float(sr[i]), p.scale_log2, -l2));
+                    }
+                    if (need_mask) {
+                        static_assert(MODE == FWD || NC == 32, "one mask word per compute thread");
+                        const uint32_t vis = range_bits(c_lo, c_hi);
+#pragma unroll
+                        for (int i = 0; i < NC; ++i) pf[i] = (vis >> i) & 1u ? pf[i] : 0.f;
                     }
                     if (MODE == DV) {
 #pragma unroll
