@@ -31,6 +31,15 @@ def test_random_windows(seed):
     _compare(rng.integers(0, hi, size=P * K).astype(np.int64), P)
 
 
+@pytest.mark.parametrize("P,K", [(1, 40), (2, 1), (3, 33), (64, 31), (2, 1024)])
+@pytest.mark.parametrize("hi", [1, 2, 2**40, 2**56])
+def test_waves_and_the_one_by_one_rule(P, K, hi):
+    """Equal works (long waves, pools that fill up inside one), works that differ little, and works whose sums pass the
+    53 bits of the wave keys (one sequence at a time)."""
+    rng = np.random.default_rng(P * K + hi % 97)
+    _compare((hi - 1 - rng.integers(0, max(1, hi // 4), size=P * K)).astype(np.int64), P)
+
+
 @pytest.mark.parametrize("P", [1, 4, 8, 32, 128])
 def test_long_tailed_window(P):
     spec = pools.config(3, 0.0, 7)
