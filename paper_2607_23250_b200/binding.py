@@ -305,7 +305,8 @@ def libra_tap_plan(cu_seqlens: torch.Tensor, seq_offsets, cp: int, block: int, n
 def libra_tap_schedule(cu_seqlens: torch.Tensor, seq_offsets, sigma: torch.Tensor, cp: int, block: int, n_shards: int,
                        hq: int, hkv: int, head_dim: int, capacity: int = 0, stream=None) -> torch.Tensor:
     """Transfer records [n, 6] (kind, src, dst, tok0, ntok, shard) implied by assignment `sigma` (device int32).
-    Two calls when `capacity` is 0: the first only counts."""
+    When `capacity` is 0 the records are taken in one call with room for as many as most assignments imply, and in a
+    second one when that was not enough."""
     assert cu_seqlens.is_cuda and cu_seqlens.dtype == torch.int32 and sigma.is_cuda and sigma.dtype == torch.int32
     so = (ctypes.c_int32 * len(seq_offsets))(*[int(x) for x in seq_offsets])
     P = len(seq_offsets) - 1
@@ -320,8 +321,12 @@ def libra_tap_schedule(cu_seqlens: torch.Tensor, seq_offsets, sigma: torch.Tenso
                                        _stream(stream)), "libra_tap_schedule")
         return rec
 
-    if capacity <= 0:
-        call(0)
-        capacity = int(n.item())
-    rec = call(capacity)
-    return rec[:min(capacity, int(n.item()))]
+    if capacity > 0:
+        rec = call(capacity)
+        return rec[:min(capacity, int(n.item()))]
+    room = sigma.numel() + 65536
+    rec = call(room)
+    count = int(n.item())
+    if count > room:
+        rec = call(count)
+    return rec[:count]

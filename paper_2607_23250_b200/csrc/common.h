@@ -73,6 +73,13 @@ inline void time_begin(libra_plan* p, int k, cudaStream_t s) {
 inline void time_end(libra_plan* p, int k, cudaStream_t s) {
     if (p->timing) { cudaEventRecord(p->ev[k][p->ev_count[k] % libra_plan::kTimeRing][1], s); ++p->ev_count[k]; }
 }
+// Stream-ordered device scratch from a memory pool of the library's own (one per device, made on first use, destroyed
+// with the library).  The driver's default pool hands everything back at every synchronisation, after which an
+// allocation costs from a hundred microseconds to tens of milliseconds; this one keeps at most kPoolKeep bytes across
+// synchronisations and gives back what is above that.
+constexpr size_t kPoolKeep = size_t(32) << 20;
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);
+inline void scratch_free(void* p, cudaStream_t s) { if (p) cudaFreeAsync(p, s); }
 extern std::atomic<int64_t> g_launches;
 inline void count_launch(int n = 1) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 }  // namespace libra

@@ -4,6 +4,7 @@
 // Integer work only; every result must equal the step-by-step definition bit for bit.
 #include <stdio.h>
 
+#include <mutex>
 #include <new>
 
 #include "common.h"
@@ -27,6 +28,43 @@ int check_plan_device(const libra_plan* plan) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return LIBRA_ERR_NO_DEVICE;
     return dev == plan->device ? LIBRA_OK : LIBRA_ERR_PLAN_MISMATCH;
+}
+
+namespace {
+struct ScratchPools {
+    std::mutex mu;
+    cudaMemPool_t pool[kMaxDevices] = {};
+    ~ScratchPools() {
+        for (cudaMemPool_t q : pool)
+            if (q) cudaMemPoolDestroy(q);
+    }
+};
+}  // namespace
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
+    static ScratchPools pools;
+    int dev = 0;
+    if (const cudaError_t e = cudaGetDevice(&dev); e != cudaSuccess) return e;
+    cudaMemPool_t pool = nullptr;
+    if (dev >= 0 && dev < kMaxDevices) {
+        std::lock_guard<std::mutex> lock(pools.mu);
+        if (!pools.pool[dev]) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t made;
+            if (cudaMemPoolCreate(&made, &props) == cudaSuccess) {
+                uint64_t keep = kPoolKeep;
+                cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
+                pools.pool[dev] = made;
+            } else {
+                cudaGetLastError();   // no pool of our own: the driver's default one below
+            }
+        }
+        pool = pools.pool[dev];
+    }
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
 }
 
 // ---- kernels --------------------------------------------------------------------------------

@@ -63,6 +63,16 @@ def test_long_tailed_pools(P, CP, B, H):
     assert loads.max() <= 1.03 * loads.mean() + max(1, oracle.tap_layout(cu, seq_off, CP, B, H, spec.hq, spec.hkv, spec.head_dim)["f"].max())
 
 
+@pytest.mark.parametrize("P,CP,max_len", [(3, 11, 90), (4, 17, 300), (8, 16, 200), (8, 17, 200), (8, 16, 5)])
+def test_worker_counts_around_the_one_warp_placement(P, CP, max_len):
+    """33, 68 and 128 workers (two to four per lane), 136 (a thread each) and samples so short that the residency rows
+    do not fit shared memory."""
+    rng = np.random.default_rng(P * CP + max_len)
+    seqs = [pools.random_layout(rng, 1500, max_len) for _ in range(P)]
+    cu = pools.cu_seqlens([x for s in seqs for x in s])
+    _compare(cu, np.arange(P + 1, dtype=np.int32) * 1500, CP, 100, 2, 8, 4, 64)
+
+
 def test_zero_length_samples_and_short_tail():
     _compare([0, 0, 3, 3, 3, 40, 40, 41], [0, 41], 2, 16, 2, 4, 2, 8)
     _compare([0, 7, 7, 30, 30], [0, 7, 30], 1, 4, 1, 2, 2, 8)
