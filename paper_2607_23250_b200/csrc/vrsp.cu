@@ -11,6 +11,7 @@
 
 #include "../../include/libra.h"
 #include "common.h"
+#include "waves.cuh"
 
 namespace libra {
 
@@ -53,86 +54,61 @@ __global__ void __launch_bounds__(256) k_vrsp_rank(const int64_t* __restrict__ w
     if (i < D && sub == 0) sorted[rank] = i;
 }
 
-// Placement in waves by one warp.  The pools with room form one sorted array of keys (load << 10 | pool) in shared
-// memory.  Sequence s of the coming batch goes to key[s] as long as key[s] lies below every key put back by the
-// sequences before it: nothing put back can then be the minimum earlier.  The longest such prefix (at most 32) is
-// placed at once, one sequence per pool; the keys put back by pools that still have room are ranked among themselves
-// and merged with the rest of the array, every key finding its place by a binary search in the other sequence; a full
-// pool leaves the array.  Sequence for sequence this is the one-by-one rule.  Needs 0 <= work and loads below 2^53
-// (the caller checks).  The serial chain is what bounds it: 1024 sequences into 128 pools, all three kernels: 76 us,
-// with an arg-min over all pools per sequence 502 us.
+// Placement in waves by one block (waves.cuh): the bins are the pools with room; a full pool leaves the array.  Needs
+// 0 <= work and loads below 2^53 (the caller checks).  1024 sequences into 128 pools, all three kernels: 31 us; 502 us
+// with an arg-min over all pools per sequence, 75 us in waves of up to 32 by one warp.
 __device__ void vrsp_place_waves(const int64_t* __restrict__ work, const int32_t* __restrict__ sorted, int D, int P, int K,
                                  int32_t* __restrict__ order, int32_t* __restrict__ pool_of_seq,
-                                 int64_t* __restrict__ pool_load, uint64_t* cur, uint64_t* nxt, int32_t* cnt) {
-    __shared__ uint64_t put_raw[32], back[32];
-    const int lane = threadIdx.x;
-    for (int k = lane; k < K; k += 32) { cur[k] = (uint64_t)k; cnt[k] = 0; }
-    __syncwarp();
-    int W = K;                                   // pools with room
-    int32_t s_l = lane < D ? sorted[lane] : 0;   // the coming 32 sequences, and the 32 after them
-    int64_t w_l = lane < D ? work[s_l] : 0;
-    for (int x0 = 0; x0 < D; x0 += 32) {
-        const int lim = D - x0 < 32 ? D - x0 : 32;
-        const int xn = x0 + 32 + lane;
-        const int32_t s_n = xn < D ? sorted[xn] : 0;
-        const int64_t w_n = xn < D ? work[s_n] : 0;
-        for (int i = 0; i < lim;) {
-            const int64_t w_s = __shfl_sync(0xffffffffu, w_l, (i + lane) & 31);
-            const int32_t sq = __shfl_sync(0xffffffffu, s_l, (i + lane) & 31);
-            const bool live = i + lane < lim && lane < W;
-            const uint64_t mine = lane < W ? cur[lane] : ~0ull;
-            const int pool = (int)(mine & 1023u);
+                                 int64_t* __restrict__ pool_load) {
+    __shared__ WaveSmem sm;
+    __shared__ int32_t cnt[kWaveMaxBins];
+    constexpr int kBatch = 512;
+    __shared__ int64_t wbuf[kBatch];
+    __shared__ int32_t sbuf[kBatch];
+    const int i = threadIdx.x, nthr = blockDim.x;
+    if (i < K) { sm.key[0][i] = (uint64_t)i; cnt[i] = 0; }
+    const int batch = 4 * nthr < kBatch ? 4 * nthr : kBatch;
+    int64_t w_n[4];
+    int32_t s_n[4];
+    auto fetch = [&](int x0) {                   // this thread's sequences of the batch at position x0 of the order
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int x = x0 + i + k * nthr;
+            const bool in = i + k * nthr < batch && x < D;
+            s_n[k] = in ? sorted[x] : 0;
+            w_n[k] = in ? work[s_n[k]] : 0;
+        }
+    };
+    fetch(0);
+    int W = K, cur = 0;                          // pools with room
+    for (int x0 = 0; x0 < D; x0 += batch) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i + k * nthr < batch) { wbuf[i + k * nthr] = w_n[k]; sbuf[i + k * nthr] = s_n[k]; }
+        __syncthreads();
+        if (x0 + batch < D) fetch(x0 + batch);
+        const int lim = D - x0 < batch ? D - x0 : batch;
+        for (int b = 0; b < lim;) {
+            const bool live = i < W && b + i < lim;
+            const int64_t w = live ? wbuf[b + i] : 0;
+            const uint64_t key = i < W ? sm.key[cur][i] : ~0ull;
+            const int pool = (int)(key & 1023u);
             const int had = live ? cnt[pool] : 0;
             const bool full = had + 1 >= P;
-            const uint64_t put = live && !full ? mine + ((uint64_t)w_s << 10) : ~0ull;
-            uint64_t before = put;               // smallest key put back by the lanes below this one
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint64_t other = __shfl_up_sync(0xffffffffu, before, o);
-                if (lane >= o && other < before) before = other;
-            }
-            before = __shfl_up_sync(0xffffffffu, before, 1);
-            if (lane == 0) before = ~0ull;
-            const unsigned fits = __ballot_sync(0xffffffffu, live && mine < before);
-            const int take = (~fits == 0u) ? 32 : __ffs(~fits) - 1;   // >= 1: the first key always fits
-            const bool placed = lane < take;
+            const uint64_t put = live && !full ? key + ((uint64_t)w << 10) : ~0ull;
+            const int take = wave_take(sm, key, put, live);   // >= 1: the first key always fits
+            const bool placed = i < take;
             if (placed) {
+                const int32_t sq = sbuf[b + i];
                 order[(int64_t)pool * P + had] = sq;   // pools are laid end to end in pool order
                 pool_of_seq[sq] = pool;
                 cnt[pool] = had + 1;
-                if (full) pool_load[pool] = (int64_t)(mine >> 10) + w_s;
+                if (full) pool_load[pool] = (int64_t)(key >> 10) + w;
             }
-            const unsigned keep = __ballot_sync(0xffffffffu, placed && !full);
-            const int nput = __popc(keep);
-            if (placed && !full) put_raw[__popc(keep & ((1u << lane) - 1u))] = put;
-            __syncwarp();
-            if (lane < nput) {
-                const uint64_t k = put_raw[lane];
-                int rank = 0;
-                for (int j = 0; j < nput; ++j) rank += put_raw[j] < k ? 1 : 0;   // all keys differ
-                back[rank] = k;
-            }
-            __syncwarp();
-            const int na = W - take;
-            for (int idx = lane; idx < na; idx += 32) {
-                const uint64_t k = cur[take + idx];
-                int lo = 0, hi = nput;
-                while (lo < hi) { const int mid = (lo + hi) >> 1; if (back[mid] < k) lo = mid + 1; else hi = mid; }
-                nxt[idx + lo] = k;
-            }
-            if (lane < nput) {
-                const uint64_t k = back[lane];
-                int lo = 0, hi = na;
-                while (lo < hi) { const int mid = (lo + hi) >> 1; if (cur[take + mid] < k) lo = mid + 1; else hi = mid; }
-                nxt[lane + lo] = k;
-            }
-            __syncwarp();
-            uint64_t* tmp = cur; cur = nxt; nxt = tmp;
-            W = na + nput;
-            i += take;
+            W = wave_merge(sm, cur, W, take, key, put, placed && !full);
+            cur ^= 1;
+            b += take;
         }
-        s_l = s_n;
-        w_l = w_n;
     }
 }
 
@@ -142,19 +118,18 @@ __device__ void vrsp_place_waves(const int64_t* __restrict__ work, const int32_t
 // what removing it from the algorithm's heap does.  Popping the heap's minimum (load, k) is the
 // lexicographic arg-min taken here.
 template <int PER>
-__global__ void __launch_bounds__(32) k_vrsp_place(const int64_t* __restrict__ work, const int32_t* __restrict__ sorted,
+__global__ void __launch_bounds__(1024) k_vrsp_place(const int64_t* __restrict__ work, const int32_t* __restrict__ sorted,
                                                    int D, int P, int K, int32_t* __restrict__ order,
                                                    int32_t* __restrict__ pool_of_seq, int64_t* __restrict__ pool_load) {
     const int lane = threadIdx.x;
     {   // sorted descending: the first work bounds every load, the last one tells whether any is negative
-        extern __shared__ __align__(16) uint64_t keys[];   // two key arrays and the fill counts, K entries each
         const int64_t most = work[sorted[0]], least = work[sorted[D - 1]];
         if (least >= 0 && most < (int64_t(1) << 52) / P) {
-            vrsp_place_waves(work, sorted, D, P, K, order, pool_of_seq, pool_load, keys, keys + K,
-                             reinterpret_cast<int32_t*>(keys + 2 * K));
+            vrsp_place_waves(work, sorted, D, P, K, order, pool_of_seq, pool_load);
             return;
         }
     }
+    if (threadIdx.x >= 32) return;
     int64_t load[PER];
     int32_t cnt[PER];
 #pragma unroll
@@ -224,14 +199,14 @@ extern "C" int libra_vrsp_place(const int64_t* work_dev, int n_sequences, int po
     const int D = n_sequences, P = pool_size, K = D / P;
     if (K > 1024 || D > (1 << 20)) return LIBRA_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t smem = (size_t)K * (2 * sizeof(uint64_t) + sizeof(int32_t));   // at most 20 KB
+    const int threads = (K + 31) / 32 * 32;
     k_vrsp_rank<<<(D + 15) / 16, 256, 0, s>>>(work_dev, D, scratch_dev);
     if (K <= 32)
-        k_vrsp_place<1><<<1, 32, smem, s>>>(work_dev, scratch_dev, D, P, K, order_dev, pool_of_seq_dev, pool_load_dev);
+        k_vrsp_place<1><<<1, threads, 0, s>>>(work_dev, scratch_dev, D, P, K, order_dev, pool_of_seq_dev, pool_load_dev);
     else if (K <= 128)
-        k_vrsp_place<4><<<1, 32, smem, s>>>(work_dev, scratch_dev, D, P, K, order_dev, pool_of_seq_dev, pool_load_dev);
+        k_vrsp_place<4><<<1, threads, 0, s>>>(work_dev, scratch_dev, D, P, K, order_dev, pool_of_seq_dev, pool_load_dev);
     else
-        k_vrsp_place<32><<<1, 32, smem, s>>>(work_dev, scratch_dev, D, P, K, order_dev, pool_of_seq_dev, pool_load_dev);
+        k_vrsp_place<32><<<1, threads, 0, s>>>(work_dev, scratch_dev, D, P, K, order_dev, pool_of_seq_dev, pool_load_dev);
     count_launch(2);
     return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
