@@ -161,7 +161,8 @@ int libra_plan_export(const libra_plan_t* plan, int direction, int64_t* weight_h
 int libra_plan_export_pairs(const libra_plan_t* plan, int32_t* key_block_host, int32_t* query_chunk_host,
                             int* chunk_tokens_host);
 
-/* Frees the plan's device and host memory (synchronises the device first). NULL is OK. */
+/* Frees the plan's device and host memory.  Synchronises the device first, unless the plan was built and used on the
+ * legacy default stream only: the memory is then released in that stream's order. NULL is OK. */
 int libra_plan_destroy(libra_plan_t* plan);
 
 /* ---- attention -----------------------------------------------------------------------

@@ -763,6 +763,7 @@ extern "C" int libra_attn_pool_bwd(const void* q_dev, const void* k_dev, const v
     float* dvec = reinterpret_cast<float*>(workspace_dev);
     float* lse2 = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace_dev) + ws.stat_bytes);
     cudaStream_t s = (cudaStream_t)stream;
+    if (s) const_cast<libra_plan_t*>(plan)->other_stream = 1;
     cudaMemsetAsync(plan->d_status + 2, 0, sizeof(int), s);   // the word reports the most recent launch
 
     const float scale = dims->softmax_scale > 0.f ? dims->softmax_scale : 1.0f / sqrtf((float)D);

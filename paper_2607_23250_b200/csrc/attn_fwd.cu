@@ -595,6 +595,7 @@ extern "C" int libra_attn_pool_fwd(const void* q_dev, const void* k_dev, const v
     const float scale = dims->softmax_scale > 0.f ? dims->softmax_scale : 1.0f / sqrtf((float)dims->head_dim);
     cudaStream_t s = (cudaStream_t)stream;
     libra_plan_t* mp = const_cast<libra_plan_t*>(plan);
+    if (s) mp->other_stream = 1;
     if (dims->head_dim == 256) {
         cudaMemsetAsync(plan->d_status + 1, 0, sizeof(int), s);
         time_begin(mp, 0, s);

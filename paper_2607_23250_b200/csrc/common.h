@@ -43,6 +43,10 @@ struct libra_plan {
     int device = 0;
     int sm_count = 0;
     cudaStream_t stream = nullptr;
+    static constexpr int kMaxBlocks = 2;
+    void* blocks[kMaxBlocks] = {};   // the device memory all pointers below lead into
+    int n_blocks = 0;
+    int other_stream = 0;            // built or used on a stream other than the legacy one
     int32_t* d_tok_start = nullptr;  // [T] first token of the sample that holds token t
     int32_t* d_tok_end = nullptr;    // [T] one past the last token of that sample
     int* d_status = nullptr;         // [4] word 0: plan status; word 1: fwd; word 2: bwd

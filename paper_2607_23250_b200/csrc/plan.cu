@@ -8,6 +8,7 @@
 #include <new>
 
 #include "common.h"
+#include "waves.cuh"
 
 namespace libra {
 
@@ -69,24 +70,20 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
 
 // ---- kernels --------------------------------------------------------------------------------
 
-// cu_seqlens checks: starts at 0, non-decreasing, ends at T.
-__global__ void k_validate(const int32_t* __restrict__ cu, int n, int64_t T, int* status) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j > n) return;
-    bool bad = false;
-    if (j == 0 && cu[0] != 0) bad = true;
-    if (j == n && cu[n] != T) bad = true;
-    if (j < n && cu[j + 1] < cu[j]) bad = true;
-    if (bad) atomicExch(status, LIBRA_ERR_BAD_SEQLENS);
-}
-
-// For every token: the bounds [start, end) of the sample that holds it.
-// The search keeps every index inside [0, n] whatever cu contains, and the bounds are clamped to
-// start <= t < end <= T, so that a malformed cu_seqlens (flagged by k_validate) can never make a
+// cu_seqlens checks (starts at 0, non-decreasing, ends at T) and, for every token, the bounds [start, end) of the sample
+// that holds it.  The search keeps every index inside [0, n] whatever cu contains, and the bounds are clamped to
+// start <= t < end <= T, so that a malformed cu_seqlens (flagged in *status) can never make a
 // later kernel form an address outside its tensors.
 __global__ void k_token_bounds(const int32_t* __restrict__ cu, int n, int64_t T, int32_t* __restrict__ tok_start,
-                               int32_t* __restrict__ tok_end) {
+                               int32_t* __restrict__ tok_end, int* status) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t <= n) {
+        bool bad = false;
+        if (t == 0 && cu[0] != 0) bad = true;
+        if (t == n && cu[n] != T) bad = true;
+        if (t < n && cu[t + 1] < cu[t]) bad = true;
+        if (bad) atomicExch(status, LIBRA_ERR_BAD_SEQLENS);
+    }
     if (t >= T) return;
     int lo = 0, hi = n;  // find the last j in [0, n) with cu[j] <= t
     while (hi - lo > 1) {
@@ -98,269 +95,189 @@ __global__ void k_token_bounds(const int32_t* __restrict__ cu, int n, int64_t T,
     tok_end[t] = (int32_t)(e < t + 1 ? t + 1 : (e > T ? T : e));
 }
 
+// What the kernels below need of one direction; the directions of a plan share launches.
+struct DirView {
+    int64_t NB, NT;
+    int tile, H, W, key_major, g, unit_cost;   // g: cost_block of LIBRA_WEIGHT_BLOCKS, 0 = pair counts
+    int64_t* weight_blk;
+    int32_t* blk_order;     // null: pair tiles (id = head * NB + block, placed in id order)
+    int32_t* cta_of_tile;
+    int32_t* pos;
+    int32_t* cta_offsets;
+    int32_t* cta_tiles;
+    int32_t* cta_exec;
+    int64_t* loads;
+};
+struct DirViews {
+    DirView v[3];
+};
+
 // Weight of block b (Eq. 6): a token at position p of a sample of length len contributes
 // p + 1 pairs as a query (keys 0..p) and len - p pairs as a key (queries p..len-1).
-__global__ void k_block_weights(const int32_t* __restrict__ tok_start, const int32_t* __restrict__ tok_end,
-                                int64_t T, int tile, int64_t NB, int key_major, int64_t* __restrict__ weight_blk) {
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= NB) return;
-    const int64_t t0 = b * tile;
-    const int64_t t1 = (t0 + tile < T) ? t0 + tile : T;
-    int64_t w = 0;
-    for (int64_t t = t0; t < t1; ++t) w += key_major ? (int64_t)tok_end[t] - t : t - (int64_t)tok_start[t] + 1;
-    weight_blk[b] = w;
-}
-
 // Block-count weight (LIBRA_WEIGHT_BLOCKS): the token axis is cut into chunks at multiples of g.  For a
 // chunk of query rows [r0, r1] the visible keys span the chunks from the one holding the first key of r0's
 // sample to the one holding r1 (row r0 sees a key in every chunk of that range, later rows see no chunk
 // outside it); for a chunk of keys [c0, c1] the attending queries span the chunks from the one holding c0
 // to the one holding the last token of c1's sample.
-__global__ void k_block_weights_blocks(const int32_t* __restrict__ tok_start, const int32_t* __restrict__ tok_end,
-                                       int64_t T, int tile, int64_t NB, int key_major, int g, int unit_cost,
-                                       int64_t* __restrict__ weight_blk) {
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= NB) return;
-    const int64_t t0 = b * tile;
-    const int64_t t1 = (t0 + tile < T) ? t0 + tile : T;
+// One warp per block (a thread per block read its tokens one after the other: 20 us at 32768 tokens, 4 now).
+__global__ void k_block_weights(const int32_t* __restrict__ tok_start, const int32_t* __restrict__ tok_end,
+                                int64_t T, const DirViews views) {
+    const DirView& d = views.v[blockIdx.y];
+    const int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (b >= d.NB) return;
+    const int64_t t0 = b * d.tile;
+    const int64_t t1 = (t0 + d.tile < T) ? t0 + d.tile : T;
     int64_t w = 0;
-    for (int64_t c = t0 / g; c * g < t1; ++c) {
-        const int64_t first = c * g > t0 ? c * g : t0;
-        const int64_t last = ((c + 1) * g < t1 ? (c + 1) * g : t1) - 1;
-        const int64_t n = key_major ? ((int64_t)tok_end[last] - 1) / g - first / g + 1
-                                    : last / g - (int64_t)tok_start[first] / g + 1;
-        w += 8 * n + unit_cost;
+    if (d.g == 0) {
+        for (int64_t t = t0 + lane; t < t1; t += 32)
+            w += d.key_major ? (int64_t)tok_end[t] - t : t - (int64_t)tok_start[t] + 1;
+    } else {
+        for (int64_t c = t0 / d.g + lane; c * d.g < t1; c += 32) {
+            const int64_t first = c * d.g > t0 ? c * d.g : t0;
+            const int64_t last = ((c + 1) * d.g < t1 ? (c + 1) * d.g : t1) - 1;
+            const int64_t n = d.key_major ? ((int64_t)tok_end[last] - 1) / d.g - first / d.g + 1
+                                          : last / d.g - (int64_t)tok_start[first] / d.g + 1;
+            w += 8 * n + d.unit_cost;
+        }
     }
-    weight_blk[b] = w;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    if (lane == 0) d.weight_blk[b] = w;
 }
 
 // Order of Algorithm 2: decreasing weight, then increasing id.  All H shards of a block weigh
 // the same and their ids b*H+h are consecutive, so ordering the blocks orders the tiles.
-// rank(b) = number of blocks that precede b; one thread per block, O(NB) each.
-__global__ void k_rank_blocks(const int64_t* __restrict__ weight_blk, int64_t NB, int32_t* __restrict__ blk_order) {
-    __shared__ int64_t sw[256];
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t wb = b < NB ? weight_blk[b] : 0;
-    int64_t rank = 0;
-    for (int64_t base = 0; base < NB; base += 256) {
-        const int64_t o = base + threadIdx.x;
-        sw[threadIdx.x] = o < NB ? weight_blk[o] : -1;
+// rank(b) = number of blocks that precede b; sixteen lanes share a block's comparisons.
+__global__ void __launch_bounds__(256) k_rank_blocks(const DirViews views) {
+    const DirView& d = views.v[blockIdx.y];
+    __shared__ int64_t sw[1024];
+    if (blockIdx.x * (int64_t)16 >= d.NB) return;
+    const int64_t b = blockIdx.x * (int64_t)16 + (threadIdx.x >> 4);
+    const int sub = threadIdx.x & 15;
+    const int64_t wb = b < d.NB ? d.weight_blk[b] : 0;
+    int rank = 0;
+    for (int64_t base = 0; base < d.NB; base += 1024) {
+        const int lim = (int)(d.NB - base < 1024 ? d.NB - base : 1024);
+        for (int o = threadIdx.x; o < lim; o += 256) sw[o] = d.weight_blk[base + o];
         __syncthreads();
-        const int lim = (int)((NB - base < 256) ? NB - base : 256);
-        for (int i = 0; i < lim; ++i) {
-            const int64_t w = sw[i];
-            rank += (w > wb) || (w == wb && base + i < b);
+        for (int k = sub; k < lim; k += 16) {
+            const int64_t w = sw[k];
+            rank += (w > wb) || (w == wb && base + k < b);
         }
         __syncthreads();
     }
-    if (b < NB) blk_order[rank] = (int32_t)b;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (b < d.NB && sub == 0) d.blk_order[rank] = (int32_t)b;
 }
 
-// Sequential placement by one warp (Algorithm 2's greedy rule: the next tile goes to the least-loaded worker, lowest
-// index among equals).  The workers are kept as ONE sorted array of keys (load << 10 | worker) in shared memory; loads
-// stay below 2^53 (checked on the host from the weight total) and there are at most 1024 workers, so a key fits 64 bits.
-//   * Consecutive tiles are placed in waves.  Tile s of a batch goes to key[s], the s-th worker of the array, as long
-//     as key[s] lies below every key put back by the tiles before it (key[s'] + w[s'], s' < s): nothing put back can
-//     then overtake it.  The longest such prefix (at most 32 tiles) is placed at once, one tile per worker; the keys
-//     put back are ranked among themselves and merged with the rest of the array (every key finds its place by a
-//     binary search in the other sequence).  With equal weights (the H head shards of a block) the condition is
-//     key[s] < key[0] + w.  The result is tile for tile what the one-by-one rule gives.
-//   * When fewer than kWaveMin tiles can go at once, one tile takes the first key and re-inserts it: the warp counts
-//     the keys below the new one and shifts that part of the array down by one.
-constexpr int kPlaceMaxW = 1024;
-constexpr int kWaveMin = 4;
+// Placement (Algorithm 2's greedy rule: the next tile goes to the least-loaded worker, lowest index among equals) in
+// waves, one block per direction (waves.cuh).  Loads stay below 2^53 (checked on the host from the weight total) and
+// there are at most 1024 workers, so a key fits 64 bits.  Tiles come in batches held in shared memory, the next batch in
+// registers.  Both directions of 131072 tokens with 32 / 8 heads (16384 and 13464 tiles): 0.6 ms, by a warp per direction
+// 1.4 ms; of two 65536-token samples (69632 pair tiles): 1.5 and 5.3 ms.
+constexpr int kPlaceBatch = 512;
 
-struct PlaceJob {
-    const int64_t* weight_blk;
-    const int32_t* blk_order;   // null: tiles in id order, id = head * NB + block
-    int64_t NB, NT;
-    int H, W;
-    int32_t* cta_of_tile;
-    int32_t* pos;
-    int32_t* cta_offsets;
-    int64_t* loads;
-};
-struct PlaceJobs {
-    PlaceJob job[3];            // the directions of a plan are independent: one block (one warp) each
-};
-
-template <int PER>   // PER * 32 >= W
-__global__ void __launch_bounds__(32) k_place(const PlaceJobs jobs) {
-    const PlaceJob& jb = jobs.job[blockIdx.x];
-    const int64_t* __restrict__ weight_blk = jb.weight_blk;
-    const int32_t* __restrict__ blk_order = jb.blk_order;
-    const int64_t NB = jb.NB, NT = jb.NT;
+__global__ void __launch_bounds__(kWaveMaxBins) k_place(const DirViews views) {
+    const DirView& jb = views.v[blockIdx.x];
+    __shared__ WaveSmem sm;
+    __shared__ int32_t cnt[kWaveMaxBins];        // tiles per worker so far
+    __shared__ int64_t wbuf[kPlaceBatch];
+    __shared__ int32_t tbuf[kPlaceBatch];
+    __shared__ int32_t warp_sum[32];
+    const int i = threadIdx.x, nthr = blockDim.x, lane = i & 31, warp = i >> 5;
+    const int64_t NT = jb.NT, NB = jb.NB;
     const int H = jb.H, W = jb.W;
-    int32_t* __restrict__ cta_of_tile = jb.cta_of_tile;
-    int32_t* __restrict__ pos = jb.pos;
-    int32_t* __restrict__ cta_offsets = jb.cta_offsets;
-    int64_t* __restrict__ loads = jb.loads;
-    __shared__ uint64_t key_a[kPlaceMaxW], key_b[kPlaceMaxW];   // the sorted array and its next version
-    __shared__ uint64_t back[32];                               // keys put back by a wave, in order
-    __shared__ uint64_t put_raw[32];                            // the same in tile order
-    __shared__ int32_t cnt[kPlaceMaxW];                         // tiles per worker so far
-    const int lane = threadIdx.x;
-    uint64_t* cur = key_a;
-    uint64_t* nxt = key_b;
-    for (int r = lane; r < W; r += 32) { cur[r] = (uint64_t)r; cnt[r] = 0; }
-    __syncwarp();
-    for (int64_t x0 = 0; x0 < NT; x0 += 32) {
-        // each lane fetches one upcoming tile
-        const int64_t xl = x0 + lane;
-        int64_t w_l = -1;
-        int32_t t_l = 0;
-        if (xl < NT) {
-            if (blk_order) {
-                const int32_t blk = blk_order[xl / H];
-                w_l = weight_blk[blk];
-                t_l = (int32_t)((int64_t)blk * H + xl % H);
-            } else {
-                w_l = weight_blk[xl % NB];
-                t_l = (int32_t)xl;
+    if (i < W) sm.key[0][i] = (uint64_t)i;
+    cnt[i] = 0;
+    const int batch = 4 * nthr < kPlaceBatch ? 4 * nthr : kPlaceBatch;
+    int64_t w_n[4];
+    int32_t t_n[4];
+    auto fetch = [&](int64_t x0) {               // this thread's tiles of the batch at position x0 of the order
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t x = x0 + i + (int64_t)k * nthr;
+            w_n[k] = 0;
+            t_n[k] = 0;
+            if (i + k * nthr < batch && x < NT) {
+                const int64_t blk = jb.blk_order ? jb.blk_order[x / H] : x % NB;
+                w_n[k] = jb.weight_blk[blk];
+                t_n[k] = jb.blk_order ? (int32_t)(blk * H + x % H) : (int32_t)x;   // pair tiles: in id order
             }
         }
-        const int lim = (int)((NT - x0 < 32) ? NT - x0 : 32);
-        int i = 0;
-        while (i < lim) {
-            const int64_t w = __shfl_sync(0xffffffffu, w_l, i);
-            if (w == 0) {
-                // weightless tiles all go to the first worker and change nothing else
-                const unsigned same = __ballot_sync(0xffffffffu, w_l == 0) >> i;
-                int n = (~same == 0u) ? 32 : __ffs(~same) - 1;
-                if (n > lim - i) n = lim - i;
-                const int r0 = (int)(cur[0] & 1023u);
-                const int base = cnt[r0];
-                __syncwarp();
-                if (lane >= i && lane < i + n) { cta_of_tile[t_l] = r0; pos[t_l] = base + (lane - i); }
-                if (lane == 0) cnt[r0] = base + n;
-                __syncwarp();
-                i += n;
-                continue;
-            }
-            // lane s looks at tile i + s of the batch and at key[s]
-            const int64_t w_s = __shfl_sync(0xffffffffu, w_l, (i + lane) & 31);
-            const bool live = i + lane < lim && lane < W && w_s > 0;
-            const uint64_t first = cur[0];
-            const uint64_t add = (uint64_t)w << 10;
-            const uint64_t mine_k = lane < W ? cur[lane] : ~0ull;
-            const uint64_t put = live ? mine_k + ((uint64_t)w_s << 10) : ~0ull;
-            uint64_t before = put;                                // min of the keys put back by the lanes below this one
+    };
+    fetch(0);
+    int cur = 0;
+    for (int64_t x0 = 0; x0 < NT; x0 += batch) {
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint64_t other = __shfl_up_sync(0xffffffffu, before, o);
-                if (lane >= o && other < before) before = other;
+        for (int k = 0; k < 4; ++k)
+            if (i + k * nthr < batch) { wbuf[i + k * nthr] = w_n[k] > 0 ? w_n[k] : 0; tbuf[i + k * nthr] = t_n[k]; }
+        __syncthreads();
+        fetch(x0 + batch);
+        const int lim = (int)(NT - x0 < batch ? NT - x0 : batch);
+        for (int b = 0; b < lim;) {
+            const bool live = i < W && b + i < lim;
+            const uint64_t key = i < W ? sm.key[cur][i] : ~0ull;
+            const uint64_t put = live ? key + ((uint64_t)wbuf[b + i] << 10) : ~0ull;
+            const int take = wave_take(sm, key, put, live);   // >= 1: the first key always fits
+            if (i < take) {
+                const int32_t t = tbuf[b + i];
+                const int r = (int)(key & 1023u), had = cnt[r];
+                jb.cta_of_tile[t] = r;
+                jb.pos[t] = had;
+                cnt[r] = had + 1;
             }
-            before = __shfl_up_sync(0xffffffffu, before, 1);
-            if (lane == 0) before = ~0ull;
-            const unsigned fits = __ballot_sync(0xffffffffu, live && mine_k < before);
-            const int take = (~fits == 0u) ? 32 : __ffs(~fits) - 1;
-            if (take < kWaveMin) {
-                // one tile: the first key, put back w heavier at its new place
-                const uint64_t k1 = first + add;
-                const int r0 = (int)(first & 1023u);
-                int below = 0;                                    // keys of cur[1..W) below the new key
-                uint64_t mine[PER];
-#pragma unroll
-                for (int u = 0; u < PER; ++u) {
-                    const int idx = 1 + lane + 32 * u;
-                    mine[u] = idx < W ? cur[idx] : ~0ull;
-                    below += (idx < W && mine[u] < k1) ? 1 : 0;
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
-                __syncwarp();
-#pragma unroll
-                for (int u = 0; u < PER; ++u) {
-                    const int idx = 1 + lane + 32 * u;
-                    if (idx <= below) cur[idx - 1] = mine[u];     // the keys below the new one move down by one
-                }
-                if (lane == 0) cur[below] = k1;
-                const int32_t t = __shfl_sync(0xffffffffu, t_l, i);
-                if (lane == 0) { cta_of_tile[t] = r0; pos[t] = cnt[r0]; cnt[r0] += 1; }
-                __syncwarp();
-                i += 1;
-                continue;
-            }
-            // ---- a wave: tile i + s goes to the worker of key[s], s < take; the workers are distinct ----
-            {
-                const int32_t t = __shfl_sync(0xffffffffu, t_l, (i + lane) & 31);
-                if (lane < take) {
-                    const int r = (int)(mine_k & 1023u);
-                    cta_of_tile[t] = r;
-                    pos[t] = cnt[r];
-                    cnt[r] += 1;
-                    put_raw[lane] = put;
-                }
-                __syncwarp();
-                if (lane < take) {   // the keys put back, ranked among themselves (all keys differ)
-                    int rank = 0;
-                    for (int j = 0; j < take; ++j) rank += put_raw[j] < put ? 1 : 0;
-                    back[rank] = put;
-                }
-                __syncwarp();
-                // the rest of the array and the keys put back, merged into the new sorted array
-                const int na = W - take;
-                for (int idx = lane; idx < na; idx += 32) {       // a key of the array: keys put back that are below it
-                    const uint64_t k = cur[take + idx];
-                    int lo = 0, hi = take;
-                    while (lo < hi) { const int mid = (lo + hi) >> 1; if (back[mid] < k) lo = mid + 1; else hi = mid; }
-                    nxt[idx + lo] = k;
-                }
-                if (lane < take) {                                 // a key put back: keys of the array below it
-                    const uint64_t k = back[lane];
-                    int lo = 0, hi = na;
-                    while (lo < hi) { const int mid = (lo + hi) >> 1; if (cur[take + mid] < k) lo = mid + 1; else hi = mid; }
-                    nxt[lane + lo] = k;
-                }
-                __syncwarp();
-                uint64_t* tmp = cur; cur = nxt; nxt = tmp;
-            }
-            i += take;
+            wave_merge(sm, cur, W, take, key, put, i < take);
+            cur ^= 1;
+            b += take;
         }
     }
-    __syncwarp();
-    for (int idx = lane; idx < W; idx += 32) {
-        const uint64_t k = cur[idx];
-        loads[k & 1023u] = (int64_t)(k >> 10);
+    __syncthreads();
+    if (i < W) {
+        const uint64_t k = sm.key[cur][i];
+        jb.loads[k & 1023u] = (int64_t)(k >> 10);
     }
-    for (int r = lane; r < W; r += 32) cta_offsets[r + 1] = cnt[r];
-    __syncwarp();
-    if (lane == 0) {  // counts -> offsets
-        cta_offsets[0] = 0;
-        int32_t run = 0;
-        for (int r = 0; r < W; ++r) { run += cta_offsets[r + 1]; cta_offsets[r + 1] = run; }
-    }
+    int incl = i < W ? cnt[i] : 0;               // counts -> offsets
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+    if (lane == 31) warp_sum[warp] = incl;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) incl += warp_sum[w];
+    if (i < W) jb.cta_offsets[i + 1] = incl;
+    if (i == 0) jb.cta_offsets[0] = 0;
 }
 
-__global__ void k_scatter_lists(const int32_t* __restrict__ cta_of_tile, const int32_t* __restrict__ pos,
-                                const int32_t* __restrict__ cta_offsets, int64_t NT, int32_t* __restrict__ cta_tiles) {
+__global__ void k_scatter_lists(const DirViews views) {
+    const DirView& d = views.v[blockIdx.y];
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= NT) return;
-    cta_tiles[cta_offsets[cta_of_tile[t]] + pos[t]] = (int32_t)t;
+    if (t >= d.NT) return;
+    d.cta_tiles[d.cta_offsets[d.cta_of_tile[t]] + d.pos[t]] = (int32_t)t;
 }
 
 // Execution order inside a worker's list.  The placement fixes WHICH tiles a worker runs; the order
 // it runs them in is free.  Sorting every list by (head shard, block) makes all workers sweep
 // the same head and neighbouring blocks at about the same time, so that the tiles several workers
 // read (K/V in the forward and the dQ kernel, Q/dO in the dK/dV kernel) are more often found in L2.
-// One thread block per worker, rank sort.
-__global__ void k_exec_order(const int32_t* __restrict__ cta_offsets, const int32_t* __restrict__ cta_tiles, int H,
-                             int64_t NB, int32_t* __restrict__ cta_exec) {
+// One thread block per worker, rank sort.  (Pair tiles are placed in id order: their lists are in execution order.)
+__global__ void k_exec_order(const DirViews views) {
+    const DirView& d = views.v[blockIdx.y];
     const int r = blockIdx.x;
-    const int beg = cta_offsets[r], n = cta_offsets[r + 1] - beg;
+    if (!d.blk_order || r >= d.W) return;
+    const int beg = d.cta_offsets[r], n = d.cta_offsets[r + 1] - beg;
     if (n > 16384) {  // quadratic sort too slow: keep placement order
-        for (int i = threadIdx.x; i < n; i += blockDim.x) cta_exec[beg + i] = cta_tiles[beg + i];
+        for (int i = threadIdx.x; i < n; i += blockDim.x) d.cta_exec[beg + i] = d.cta_tiles[beg + i];
         return;
     }
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int32_t t = cta_tiles[beg + i];
-        const int64_t key = (int64_t)(t % H) * NB + t / H;
+        const int32_t t = d.cta_tiles[beg + i];
+        const int64_t key = (int64_t)(t % d.H) * d.NB + t / d.H;
         int rank = 0;
         for (int j = 0; j < n; ++j) {
-            const int32_t u = cta_tiles[beg + j];
-            rank += ((int64_t)(u % H) * NB + u / H) < key;
+            const int32_t u = d.cta_tiles[beg + j];
+            rank += ((int64_t)(u % d.H) * d.NB + u / d.H) < key;
         }
-        cta_exec[beg + rank] = t;
+        d.cta_exec[beg + rank] = t;
     }
 }
 
@@ -374,37 +291,39 @@ __device__ __forceinline__ int64_t pair_last_row_block(const int32_t* tok_end, i
     const int64_t last_key = ((j + 1) * tile < T ? (j + 1) * tile : T) - 1;
     return ((int64_t)tok_end[last_key] - 1) / tile;
 }
-__global__ void k_pair_chunks(const int32_t* __restrict__ tok_end, int64_t T, int tile, int R, int64_t NKB, int64_t NC,
-                              int32_t* __restrict__ first_j, int32_t* __restrict__ count) {
-    const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (c >= NC) return;
-    int64_t lo = 0, hi = NKB;   // first j with last(j) / R >= c
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (pair_last_row_block(tok_end, T, tile, mid) / R >= c) hi = mid; else lo = mid + 1;
+// One block: the key-block range of every query chunk, the exclusive prefix sum of the counts, their total in base[NC].
+__global__ void __launch_bounds__(1024) k_pair_chunks(const int32_t* __restrict__ tok_end, int64_t T, int tile, int R, int64_t NKB,
+                                                      int64_t NC, int32_t* __restrict__ first_j, int32_t* __restrict__ count,
+                                                      int64_t* __restrict__ base) {
+    __shared__ int64_t part[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int64_t run = 0;
+    for (int64_t c0 = 0; c0 < NC; c0 += 1024) {
+        const int64_t c = c0 + threadIdx.x;
+        int64_t n = 0;
+        if (c < NC) {
+            int64_t lo = 0, hi = NKB;   // first j with last(j) / R >= c
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (pair_last_row_block(tok_end, T, tile, mid) / R >= c) hi = mid; else lo = mid + 1;
+            }
+            const int64_t last = (c + 1) * R - 1 < NKB - 1 ? (c + 1) * R - 1 : NKB - 1;
+            n = last >= lo ? last - lo + 1 : 0;
+            first_j[c] = (int32_t)lo;
+            count[c] = (int32_t)n;
+        }
+        int64_t incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int64_t v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+        if (lane == 31) part[warp] = incl;
+        __syncthreads();
+        int64_t before = 0, all = 0;
+        for (int w = 0; w < 32; ++w) { if (w < warp) before += part[w]; all += part[w]; }
+        if (c < NC) base[c] = run + before + incl - n;
+        run += all;
+        __syncthreads();
     }
-    const int64_t last = (c + 1) * R - 1 < NKB - 1 ? (c + 1) * R - 1 : NKB - 1;
-    first_j[c] = (int32_t)lo;
-    count[c] = (int32_t)(last >= lo ? last - lo + 1 : 0);
-}
-// One block: exclusive prefix sum of count[0..n) into base, total into *total.
-__global__ void __launch_bounds__(1024) k_scan_i32(const int32_t* __restrict__ count, int64_t n, int64_t* __restrict__ base,
-                                                   int64_t* __restrict__ total) {
-    __shared__ int64_t part[1024];
-    const int64_t per = (n + blockDim.x - 1) / blockDim.x;
-    const int64_t x0 = threadIdx.x * per, x1 = x0 + per < n ? x0 + per : n;
-    int64_t sum = 0;
-    for (int64_t x = x0; x < x1; ++x) sum += count[x];
-    part[threadIdx.x] = sum;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int64_t run = 0;
-        for (int i = 0; i < (int)blockDim.x; ++i) { const int64_t v = part[i]; part[i] = run; run += v; }
-        *total = run;
-    }
-    __syncthreads();
-    int64_t run = part[threadIdx.x];
-    for (int64_t x = x0; x < x1; ++x) { base[x] = run; run += count[x]; }
+    if (threadIdx.x == 0) base[NC] = run;
 }
 // Weight of pair-block (c, j): its live cells, min(last(j), c R + R - 1) - max(j, c R) + 1.
 __global__ void k_pair_fill(const int32_t* __restrict__ tok_end, int64_t T, int tile, int R, int64_t NC,
@@ -438,126 +357,179 @@ __global__ void k_expand_order(const int32_t* __restrict__ blk_order, int64_t NT
 
 static inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 1) / block); }
 
-static void free_dir(PlanDir& d) {
-    cudaFree(d.d_weight_blk); cudaFree(d.d_blk_order); cudaFree(d.d_cta_of_tile); cudaFree(d.d_pos);
-    cudaFree(d.d_cta_offsets); cudaFree(d.d_cta_tiles); cudaFree(d.d_cta_exec); cudaFree(d.d_loads); cudaFree(d.d_busy); cudaFree(d.d_busy2); cudaFree(d.d_tile_ns);
-    cudaFree(d.d_u_blk); cudaFree(d.d_u_chunk);
-    d = PlanDir();
+// The plan's device memory: two stream-ordered blocks, carved into arrays.  (A cudaMalloc and a cudaFree per
+// array cost 0.5 + 0.4 ms a plan, and now and then ten times that.)
+static int plan_block(libra_plan* p, size_t bytes, uint8_t** out) {
+    if (p->n_blocks == libra_plan::kMaxBlocks) return LIBRA_ERR_CUDA;
+    void* q = nullptr;
+    if (scratch_alloc(&q, bytes ? bytes : 1, p->stream) != cudaSuccess) return LIBRA_ERR_CUDA;
+    p->blocks[p->n_blocks++] = q;
+    *out = reinterpret_cast<uint8_t*>(q);
+    return LIBRA_OK;
+}
+struct Carver {
+    uint8_t* at = nullptr;   // null: only sizes are added up
+    size_t used = 0;
+    template <typename X>
+    void take(X** p, int64_t n) {
+        if (at) *p = reinterpret_cast<X*>(at + used);
+        used += (sizeof(X) * (size_t)(n ? n : 1) + 255) & ~size_t(255);
+    }
+};
+// Arrays that start out as zeros (`zeros`), then the rest.
+static void carve_dir(PlanDir& d, Carver& c, bool zeros, bool pairs) {
+    if (zeros) {
+        c.take(&d.d_busy, 2 * d.W);
+        c.take(&d.d_busy2, 2 * d.W);
+        c.take(&d.d_tile_ns, d.NT);
+        return;
+    }
+    c.take(&d.d_weight_blk, d.NB);
+    if (!pairs) c.take(&d.d_blk_order, d.NB);
+    c.take(&d.d_cta_of_tile, d.NT);
+    c.take(&d.d_pos, d.NT);
+    c.take(&d.d_cta_offsets, d.W + 1);
+    c.take(&d.d_cta_tiles, d.NT);
+    if (!pairs) c.take(&d.d_cta_exec, d.NT);
+    c.take(&d.d_loads, d.W);
+    if (pairs) {
+        c.take(&d.d_u_blk, d.NB);
+        c.take(&d.d_u_chunk, d.NB);
+        d.d_cta_exec = d.d_cta_tiles;   // placed in id order: the lists already are in execution order
+    }
+}
+
+// Sizes a direction's kernels and tables can take; NB is known.
+static int check_dir(const libra_plan* p, PlanDir& d, bool pairs) {
+    const int64_t T = p->T;
+    if (d.NB * (int64_t)d.H >= (int64_t)INT32_MAX) return LIBRA_ERR_OVERFLOW;
+    // a worker's load is at most the weight total <= H * T^2 / 2 + ...; the placement packs load * 1024 + index
+    if ((long double)d.H * (long double)T * (long double)T >= 9.0e15L) return LIBRA_ERR_OVERFLOW;
+    if (!pairs && d.NB > 65536) return LIBRA_ERR_UNSUPPORTED;  // the rank sort is quadratic in blocks
+    if (d.W > kWaveMaxBins) return LIBRA_ERR_UNSUPPORTED;
+    d.NT = d.NB * d.H;
+    return LIBRA_OK;
+}
+
+static DirView view_of(const PlanDir& d, int key_major, const libra_plan_opts& o) {
+    DirView v = {};
+    v.NB = d.NB; v.NT = d.NT; v.tile = d.tile; v.H = d.H; v.W = d.W; v.key_major = key_major;
+    v.g = o.weight_model == LIBRA_WEIGHT_BLOCKS ? (o.cost_block ? o.cost_block : 128) : 0;
+    v.unit_cost = key_major ? o.unit_cost_kv : o.unit_cost_q;
+    v.weight_blk = d.d_weight_blk; v.blk_order = d.d_blk_order; v.cta_of_tile = d.d_cta_of_tile; v.pos = d.d_pos;
+    v.cta_offsets = d.d_cta_offsets; v.cta_tiles = d.d_cta_tiles; v.cta_exec = d.d_cta_exec; v.loads = d.d_loads;
+    return v;
 }
 
 // The pair-blocks of a plan: counts per query chunk, their prefix sums, and the total read back (one synchronous
-// 8-byte copy).  The query chunk is doubled while there are more than 262144 pair-blocks (the placement is
-// sequential, about a third of a microsecond per tile).
+// 8-byte copy).  The query chunk is doubled while there are more than 262144 pair-blocks.
 struct PairTables { int32_t* first_j = nullptr; int32_t* count = nullptr; int64_t* base = nullptr; int64_t NC = 0; };
-static void free_pair_tables(PairTables& t) { cudaFree(t.first_j); cudaFree(t.count); cudaFree(t.base); t = PairTables(); }
+static int64_t pair_chunks_of(int64_t T, const PlanDir& d) {
+    const int64_t NKB = (T + d.tile - 1) / d.tile, R = d.chunk / d.tile;
+    return (NKB + R - 1) / R;
+}
 static int count_pair_blocks(libra_plan* p, PlanDir& d, PairTables& tb) {
     const int64_t T = p->T, NKB = (T + d.tile - 1) / d.tile;
     for (;;) {
-        const int R = d.chunk / d.tile;
-        tb.NC = (NKB + R - 1) / R;
-        if (cudaMalloc((void**)&tb.first_j, sizeof(int32_t) * tb.NC) != cudaSuccess ||
-            cudaMalloc((void**)&tb.count, sizeof(int32_t) * tb.NC) != cudaSuccess ||
-            cudaMalloc((void**)&tb.base, sizeof(int64_t) * (tb.NC + 1)) != cudaSuccess)
-            { free_pair_tables(tb); return LIBRA_ERR_CUDA; }
-        k_pair_chunks<<<(unsigned)((tb.NC + 127) / 128), 128, 0, p->stream>>>(p->d_tok_end, T, d.tile, R, NKB, tb.NC,
-                                                                             tb.first_j, tb.count);
-        k_scan_i32<<<1, 1024, 0, p->stream>>>(tb.count, tb.NC, tb.base, tb.base + tb.NC);
-        count_launch(2);
+        tb.NC = pair_chunks_of(T, d);   // never more than the tables were carved for
+        k_pair_chunks<<<1, 1024, 0, p->stream>>>(p->d_tok_end, T, d.tile, d.chunk / d.tile, NKB, tb.NC, tb.first_j, tb.count,
+                                                tb.base);
+        count_launch();
         int64_t nu = 0;
         if (cudaMemcpyAsync(&nu, tb.base + tb.NC, sizeof(int64_t), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess ||
-            cudaStreamSynchronize(p->stream) != cudaSuccess) { free_pair_tables(tb); return LIBRA_ERR_CUDA; }
+            cudaStreamSynchronize(p->stream) != cudaSuccess)
+            return LIBRA_ERR_CUDA;
         d.NB = nu;
         if (nu <= 262144) return LIBRA_OK;
-        free_pair_tables(tb);
         if ((int64_t)d.chunk * 2 > (int64_t)1 << 30) return LIBRA_ERR_UNSUPPORTED;
         d.chunk *= 2;
     }
 }
 
-// First half of a direction: sizes, allocations, weights and block order; fills the placement job.
-static int build_dir(libra_plan* p, PlanDir& d, int key_major, const libra_plan_opts& o, bool pairs, PlaceJob* job) {
+// Builds the directions asked for; p->dir[k].tile / H / W / chunk are set.
+static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o, const bool (&want)[3]) {
     const int64_t T = p->T;
-    PairTables tb;
-    if (pairs) {
-        const int rcp = count_pair_blocks(p, d, tb);
-        if (rcp != LIBRA_OK) return rcp;
-    } else {
-        d.NB = (T + d.tile - 1) / d.tile;
-    }
-    if (d.NB * (int64_t)d.H >= (int64_t)INT32_MAX) { free_pair_tables(tb); return LIBRA_ERR_OVERFLOW; }
-    // a worker's load is at most the weight total <= H * T^2 / 2 + ...; the placement packs load * 1024 + index
-    if ((long double)d.H * (long double)T * (long double)T >= 9.0e15L) return LIBRA_ERR_OVERFLOW;
-    if (!pairs && d.NB > 65536) return LIBRA_ERR_UNSUPPORTED;  // the rank sort is quadratic in blocks
-    if (d.W > 1024) return LIBRA_ERR_UNSUPPORTED;
-    d.NT = d.NB * d.H;
-    cudaError_t e = cudaSuccess;
-    auto A = [&](void** ptr, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(ptr, bytes ? bytes : 1); };
-    A((void**)&d.d_weight_blk, sizeof(int64_t) * d.NB);
-    A((void**)&d.d_blk_order, sizeof(int32_t) * d.NB);
-    A((void**)&d.d_cta_of_tile, sizeof(int32_t) * d.NT);
-    A((void**)&d.d_pos, sizeof(int32_t) * d.NT);
-    A((void**)&d.d_cta_offsets, sizeof(int32_t) * (d.W + 1));
-    A((void**)&d.d_cta_tiles, sizeof(int32_t) * d.NT);
-    A((void**)&d.d_cta_exec, sizeof(int32_t) * d.NT);
-    A((void**)&d.d_loads, sizeof(int64_t) * d.W);
-    A((void**)&d.d_busy, sizeof(uint64_t) * 2 * d.W);
-    A((void**)&d.d_busy2, sizeof(uint64_t) * 2 * d.W);
-    A((void**)&d.d_tile_ns, sizeof(uint32_t) * d.NT);
-    if (pairs) {
-        A((void**)&d.d_u_blk, sizeof(int32_t) * d.NB);
-        A((void**)&d.d_u_chunk, sizeof(int32_t) * d.NB);
-    }
-    if (e != cudaSuccess) { free_pair_tables(tb); return LIBRA_ERR_CUDA; }
     cudaStream_t s = p->stream;
-    cudaMemsetAsync(d.d_busy, 0, sizeof(uint64_t) * 2 * d.W, s);
-    cudaMemsetAsync(d.d_busy2, 0, sizeof(uint64_t) * 2 * d.W, s);
-    cudaMemsetAsync(d.d_tile_ns, 0, sizeof(uint32_t) * d.NT, s);
-    if (pairs) {
+    for (int k = 0; k < 2; ++k) {
+        if (!want[k]) continue;
+        p->dir[k].NB = (T + p->dir[k].tile - 1) / p->dir[k].tile;
+        if (const int rc = check_dir(p, p->dir[k], false); rc != LIBRA_OK) return rc;
+    }
+    PairTables tb;
+    if (want[2] && p->dir[2].chunk % p->dir[2].tile) return LIBRA_ERR_INVALID_ARG;
+    // ---- token bounds, the directions whose sizes are known, the pair tables; zeros first
+    size_t zero_bytes = 0;
+    auto carve = [&](Carver& c) {
+        c.take(&p->d_status, 4);
+        for (int k = 0; k < 2; ++k)
+            if (want[k]) carve_dir(p->dir[k], c, true, false);
+        zero_bytes = c.used;
+        c.take(&p->d_tok_start, T);
+        c.take(&p->d_tok_end, T);
+        for (int k = 0; k < 2; ++k)
+            if (want[k]) carve_dir(p->dir[k], c, false, false);
+        if (want[2]) {
+            const int64_t NC = pair_chunks_of(T, p->dir[2]);
+            c.take(&tb.first_j, NC);
+            c.take(&tb.count, NC);
+            c.take(&tb.base, NC + 1);
+        }
+    };
+    Carver sizes, mem;
+    carve(sizes);
+    if (const int rc = plan_block(p, sizes.used, &mem.at); rc != LIBRA_OK) return rc;
+    carve(mem);
+    cudaMemsetAsync(mem.at, 0, zero_bytes, s);
+    const int64_t span = T > p->n + 1 ? T : p->n + 1;
+    k_token_bounds<<<grid_for(span, 256), 256, 0, s>>>(cu, p->n, T, p->d_tok_start, p->d_tok_end, p->d_status);
+    count_launch();
+    // ---- pair tiles: their number comes back, then their arrays
+    if (want[2]) {
+        PlanDir& d = p->dir[2];
+        if (const int rc = count_pair_blocks(p, d, tb); rc != LIBRA_OK) return rc;
+        if (const int rc = check_dir(p, d, true); rc != LIBRA_OK) return rc;
+        Carver ps, pm;
+        carve_dir(d, ps, true, true);
+        const size_t pair_zero = ps.used;
+        carve_dir(d, ps, false, true);
+        if (const int rc = plan_block(p, ps.used, &pm.at); rc != LIBRA_OK) return rc;
+        carve_dir(d, pm, true, true);
+        carve_dir(d, pm, false, true);
+        cudaMemsetAsync(pm.at, 0, pair_zero, s);
         k_pair_fill<<<(unsigned)tb.NC, 128, 0, s>>>(p->d_tok_end, T, d.tile, d.chunk / d.tile, tb.NC, tb.first_j, tb.count,
                                                     tb.base, d.d_u_blk, d.d_u_chunk, d.d_weight_blk);
-        cudaStreamSynchronize(s);   // the tables are read by the kernel above
-        free_pair_tables(tb);
-    } else if (o.weight_model == LIBRA_WEIGHT_BLOCKS)
-        k_block_weights_blocks<<<grid_for(d.NB, 128), 128, 0, s>>>(p->d_tok_start, p->d_tok_end, T, d.tile, d.NB,
-                                                                   key_major, o.cost_block ? o.cost_block : 128,
-                                                                   key_major ? o.unit_cost_kv : o.unit_cost_q,
-                                                                   d.d_weight_blk);
-    else
-        k_block_weights<<<grid_for(d.NB, 128), 128, 0, s>>>(p->d_tok_start, p->d_tok_end, T, d.tile, d.NB, key_major,
-                                                            d.d_weight_blk);
-    if (!pairs) k_rank_blocks<<<grid_for(d.NB, 256), 256, 0, s>>>(d.d_weight_blk, d.NB, d.d_blk_order);
-    job->weight_blk = d.d_weight_blk;
-    job->blk_order = pairs ? nullptr : d.d_blk_order;   // pair tiles are placed in id order
-    job->NB = d.NB; job->NT = d.NT; job->H = d.H; job->W = d.W;
-    job->cta_of_tile = d.d_cta_of_tile; job->pos = d.d_pos; job->cta_offsets = d.d_cta_offsets; job->loads = d.d_loads;
-    count_launch(2);
-    return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
-}
-
-// The placements of all directions in one launch (a block of one warp per direction).
-static int place_all(const PlaceJobs& jobs, int n, int max_w, cudaStream_t s) {
+        count_launch();
+    }
+    // ---- weights, order, placement and lists of all directions together
+    DirViews views = {};
+    int n = 0, max_w = 0;
+    int64_t max_nb = 0, max_nt = 0;
+    for (int k = 0; k < 2; ++k)
+        if (want[k]) {
+            views.v[n++] = view_of(p->dir[k], k == 1, o);
+            max_nb = p->dir[k].NB > max_nb ? p->dir[k].NB : max_nb;
+        }
+    if (n > 0) {
+        k_block_weights<<<dim3(grid_for(max_nb * 32, 256), n), 256, 0, s>>>(p->d_tok_start, p->d_tok_end, T, views);
+        k_rank_blocks<<<dim3(grid_for(max_nb, 16), n), 256, 0, s>>>(views);
+        count_launch(2);
+    }
+    const int n_sorted = n;
+    if (want[2]) views.v[n++] = view_of(p->dir[2], 1, o);
     if (n == 0) return LIBRA_OK;
-    if (max_w <= 160)
-        k_place<5><<<n, 32, 0, s>>>(jobs);
-    else if (max_w <= 320)
-        k_place<10><<<n, 32, 0, s>>>(jobs);
-    else
-        k_place<32><<<n, 32, 0, s>>>(jobs);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
-}
-
-// Second half of a direction: the per-worker lists from the placement.
-static int finish_dir(libra_plan* p, PlanDir& d, bool pairs) {
-    cudaStream_t s = p->stream;
-    k_scatter_lists<<<grid_for(d.NT, 256), 256, 0, s>>>(d.d_cta_of_tile, d.d_pos, d.d_cta_offsets, d.NT,
-                                                        d.d_cta_tiles);
-    if (pairs)   // placed in id order: the lists already are in execution order
-        cudaMemcpyAsync(d.d_cta_exec, d.d_cta_tiles, sizeof(int32_t) * d.NT, cudaMemcpyDeviceToDevice, s);
-    else
-        k_exec_order<<<d.W, 256, 0, s>>>(d.d_cta_offsets, d.d_cta_tiles, d.H, d.NB, d.d_cta_exec);
+    for (int k = 0; k < 3; ++k)
+        if (want[k]) {
+            max_nt = p->dir[k].NT > max_nt ? p->dir[k].NT : max_nt;
+            max_w = p->dir[k].W > max_w ? p->dir[k].W : max_w;
+        }
+    k_place<<<n, (max_w + 31) / 32 * 32, 0, s>>>(views);   // the directions' placements side by side
+    k_scatter_lists<<<dim3(grid_for(max_nt > 0 ? max_nt : 1, 256), n), 256, 0, s>>>(views);
     count_launch(2);
-    d.enabled = 1;
+    if (n_sorted > 0) {
+        k_exec_order<<<dim3(max_w, n_sorted), 256, 0, s>>>(views);
+        count_launch();
+    }
+    for (int k = 0; k < 3; ++k) p->dir[k].enabled = want[k] ? 1 : 0;
     return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
 
@@ -595,45 +567,17 @@ extern "C" int libra_plan_tiles(const int32_t* cu_seqlens_dev, int n_samples, in
     libra_plan* p = new (std::nothrow) libra_plan();
     if (!p) return LIBRA_ERR_CUDA;
     p->T = T; p->n = n_samples; p->device = dev; p->sm_count = sms; p->stream = s;
-    int rc = LIBRA_OK;
-    if (cudaMalloc((void**)&p->d_tok_start, sizeof(int32_t) * T) != cudaSuccess ||
-        cudaMalloc((void**)&p->d_tok_end, sizeof(int32_t) * T) != cudaSuccess ||
-        cudaMalloc((void**)&p->d_status, sizeof(int) * 4) != cudaSuccess)
-        rc = LIBRA_ERR_CUDA;
-    if (rc == LIBRA_OK) {
-        cudaMemsetAsync(p->d_status, 0, sizeof(int) * 4, s);
-        k_validate<<<grid_for(n_samples + 1, 128), 128, 0, s>>>(cu_seqlens_dev, n_samples, T, p->d_status);
-        k_token_bounds<<<grid_for(T, 256), 256, 0, s>>>(cu_seqlens_dev, n_samples, T, p->d_tok_start, p->d_tok_end);
-        count_launch(2);
-        const int dirs = o.directions ? o.directions : (LIBRA_DIR_Q | LIBRA_DIR_KV);
-        const int W = o.n_workers ? o.n_workers : sms;
-        PlaceJobs jobs = {};
-        int n_jobs = 0;
-        bool built[3] = {false, false, false};
-        if (dirs & LIBRA_DIR_Q) {
-            PlanDir& d = p->dir[0];
-            d.tile = tile_q; d.H = n_heads; d.W = W;
-            rc = build_dir(p, d, 0, o, false, &jobs.job[n_jobs]);
-            if (rc == LIBRA_OK) { built[0] = true; ++n_jobs; }
-        }
-        if (rc == LIBRA_OK && (dirs & LIBRA_DIR_KV)) {
-            PlanDir& d = p->dir[1];
-            d.tile = o.tile_kv ? o.tile_kv : 128; d.H = o.n_heads_kv ? o.n_heads_kv : n_heads; d.W = W;
-            rc = build_dir(p, d, 1, o, false, &jobs.job[n_jobs]);
-            if (rc == LIBRA_OK) { built[1] = true; ++n_jobs; }
-        }
-        if (rc == LIBRA_OK && (dirs & LIBRA_DIR_PAIR)) {
-            PlanDir& d = p->dir[2];
-            d.tile = o.tile_kv ? o.tile_kv : 128; d.H = o.n_heads_kv ? o.n_heads_kv : n_heads; d.W = W;
-            d.chunk = o.pair_chunk ? o.pair_chunk : 4096;
-            rc = d.chunk % d.tile ? LIBRA_ERR_INVALID_ARG : build_dir(p, d, 1, o, true, &jobs.job[n_jobs]);
-            if (rc == LIBRA_OK) { built[2] = true; ++n_jobs; }
-        }
-        // the directions are independent: their placements run side by side, one warp each
-        if (rc == LIBRA_OK) rc = place_all(jobs, n_jobs, W, s);
-        for (int k = 0; k < 3 && rc == LIBRA_OK; ++k)
-            if (built[k]) rc = finish_dir(p, p->dir[k], k == 2);
+    if (s) p->other_stream = 1;
+    const int dirs = o.directions ? o.directions : (LIBRA_DIR_Q | LIBRA_DIR_KV);
+    const bool want[3] = {(dirs & LIBRA_DIR_Q) != 0, (dirs & LIBRA_DIR_KV) != 0, (dirs & LIBRA_DIR_PAIR) != 0};
+    for (int k = 0; k < 3; ++k) {
+        PlanDir& d = p->dir[k];
+        d.tile = k == 0 ? tile_q : (o.tile_kv ? o.tile_kv : 128);
+        d.H = k == 0 ? n_heads : (o.n_heads_kv ? o.n_heads_kv : n_heads);
+        d.W = o.n_workers ? o.n_workers : sms;
+        d.chunk = k == 2 ? (o.pair_chunk ? o.pair_chunk : 4096) : 0;
     }
+    const int rc = build_plan(p, cu_seqlens_dev, o, want);
     if (rc != LIBRA_OK) {
         libra_plan_destroy(p);
         return rc;
@@ -725,13 +669,14 @@ extern "C" int libra_plan_export_pairs(const libra_plan_t* plan, int32_t* key_bl
 
 extern "C" int libra_plan_destroy(libra_plan_t* plan) {
     if (!plan) return LIBRA_OK;
-    cudaDeviceSynchronize();
-    free_dir(plan->dir[0]);
-    free_dir(plan->dir[1]);
-    free_dir(plan->dir[2]);
-    cudaFree(plan->d_tok_start);
-    cudaFree(plan->d_tok_end);
-    cudaFree(plan->d_status);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev != plan->device) cudaSetDevice(plan->device);
+    // Used on the legacy stream only (which outlives every plan): its order keeps the memory until the last kernel that
+    // reads it is done, and the caller's next launches need not wait for an idle GPU.
+    if (plan->other_stream) cudaDeviceSynchronize();
+    for (int k = 0; k < plan->n_blocks; ++k) scratch_free(plan->blocks[k], nullptr);
+    if (dev != plan->device) cudaSetDevice(dev);
     for (int a = 0; a < libra_plan::kTimedKernels; ++a)
         for (int r = 0; r < libra_plan::kTimeRing; ++r)
             for (int b = 0; b < 2; ++b)
