@@ -78,7 +78,7 @@ struct DkvParams {
     int64_t T, Tpad;
     int hq, hkv;
     float scale, scale_log2;
-    int* status;
+    int* outcome;            // [gridDim.x] 0 or what kept this CTA from doing its work
     const int* plan_status;  // the planner's verdict on cu_seqlens: non-zero = do not run
     uint32_t wait_limit_ns;
     int inject_stall;        // test aid: the producer issues no loads, so the consumers' waits run out
@@ -132,11 +132,7 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const int cta = blockIdx.x;
 
     if ((smem_u32(smem) & 1023u) != 0) {  // the swizzled tiles need a 1024-byte aligned base
-        if (threadIdx.x == 0) atomicExch(p.status, LIBRA_ERR_CUDA);
-        return;
-    }
-    if (const int ps = *p.plan_status; ps != 0) {  // malformed cu_seqlens: report and leave
-        if (threadIdx.x == 0) { atomicExch(p.status, ps); p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
+        if (threadIdx.x == 0) p.outcome[cta] = LIBRA_ERR_CUDA;
         return;
     }
     if (threadIdx.x == 0) {
@@ -158,17 +154,23 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         abort_flag[0] = 0;
         abort_flag[1] = (int)p.wait_limit_ns;
         fence_mbar_init();
-        p.busy[2 * cta] = globaltimer_ns();
-    }
-    if (warp == kDkvMmaWarp) {
-        tmem_alloc(tmem_slot, 512);
-        tmem_relinquish();
     }
     if (warp == kDkvTmaWarp && lane == 0) {
         prefetch_tmap(&tm_q);
         prefetch_tmap(&tm_k);
         prefetch_tmap(&tm_v);
         prefetch_tmap(&tm_do);
+    }
+    grid_dep_wait();
+    grid_dep_launch();   // the dQ kernel needs nothing that this one writes: it takes the SMs that fall free
+    if (const int ps = *p.plan_status; ps != 0) {  // malformed cu_seqlens: report and leave
+        if (threadIdx.x == 0) { p.outcome[cta] = ps; p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
+        return;
+    }
+    if (threadIdx.x == 0) p.busy[2 * cta] = globaltimer_ns();
+    if (warp == kDkvMmaWarp) {
+        tmem_alloc(tmem_slot, 512);
+        tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
@@ -531,7 +533,7 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     __syncthreads();
     if (warp == kDkvMmaWarp) tmem_dealloc(tmem_base, 512);
     if (threadIdx.x == 0) {
-        if (abort_flag[0]) atomicExch(p.status, LIBRA_ERR_TIMEOUT);
+        p.outcome[cta] = abort_flag[0] ? LIBRA_ERR_TIMEOUT : LIBRA_OK;
         p.busy[2 * cta + 1] = globaltimer_ns();
     }
 }
@@ -551,7 +553,12 @@ namespace libra {
 template <int D>
 __global__ void k_bwd_prep(const __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ dout,
                            const float* __restrict__ lse, int64_t T, int64_t Tpad, int hq, float* __restrict__ dvec,
-                           float* __restrict__ lse2) {
+                           float* __restrict__ lse2, float4* __restrict__ clear, int64_t n_clear) {
+    // the accumulators that the coming kernels add to (none: n_clear = 0)
+    grid_dep_wait();
+    grid_dep_launch();
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_clear; i += (int64_t)gridDim.x * blockDim.x)
+        clear[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const int64_t groups = Tpad / 32;  // Tpad is a multiple of 128
@@ -640,13 +647,24 @@ static int launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtens
         cfg_mark(kSlot);
     }
     time_begin(mp, 1, s);
-    k_attn_bwd_dkdv<D><<<Wa, kBwdThreads, DkvSmem<D>::kBytes, s>>>(tq, tk, tv, tdo, pa);
+    cudaError_t e = launch_dependent(k_attn_bwd_dkdv<D>, Wa, kBwdThreads, DkvSmem<D>::kBytes, s, tq, tk, tv, tdo, pa);
     time_end(mp, 1, s);
     time_begin(mp, 2, s);
-    k_attn_bwd_dq<D><<<Wb, kDqThreads, DqSmem<D>::kBytes, s>>>(tq, tk, tv, tdo, tdq, pb);
+    if (e == cudaSuccess)
+        e = launch_dependent(k_attn_bwd_dq<D>, Wb, kDqThreads, DqSmem<D>::kBytes, s, tq, tk, tv, tdo, tdq, pb);
     time_end(mp, 2, s);
     count_launch(2);
-    return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
+    return e == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
+}
+
+// Row statistics; `clear` (16-byte words) is zeroed on the way: one pass over memory less to launch.
+template <int D>
+static cudaError_t launch_prep(const void* out, const void* dout, const float* lse, int64_t T, int64_t Tpad, int hq, float* dvec,
+                               float* lse2, float* clear, size_t clear_bytes, cudaStream_t s) {
+    const int64_t warps = Tpad / 32 * hq;
+    count_launch();
+    return launch_dependent(k_bwd_prep<D>, (unsigned)((warps * 32 + 255) / 256), 256u, 0, s, (const __nv_bfloat16*)out,
+                            (const __nv_bfloat16*)dout, lse, T, Tpad, hq, dvec, lse2, (float4*)clear, (int64_t)(clear_bytes / 16));
 }
 
 }  // namespace libra
@@ -707,22 +725,22 @@ static int launch_fused(const void* q_dev, const void* k_dev, const void* v_dev,
     fp.T = T; fp.Tpad = ws.Tpad; fp.NU = d.NB;
     fp.hq = dims->hq; fp.hkv = dims->hkv; fp.R = d.chunk / d.tile;
     fp.scale_log2 = scale * 1.4426950408889634f;
-    fp.status = plan->d_status + 2; fp.plan_status = plan->d_status;
+    fp.outcome = plan->d_outcome[1]; fp.plan_status = plan->d_status;
     fp.wait_limit_ns = plan->wait_limit_ns; fp.inject_stall = plan->inject_stall;
     fp.busy = d.d_busy;
     fp.tile_ns = d.d_tile_ns;
     time_begin(mp, 4, s);
-    cudaMemsetAsync(dq_acc, 0, ws.dq_acc_bytes + 2 * ws.dkv_acc_bytes, s);   // the three accumulators are contiguous
-    k_attn_bwd_fused<<<d.W, kFusedThreads, FusedSmem::kBytes, s>>>(tq, tk, tv, tdo, tacc, tdkacc, tdvacc, fp);
+    cudaError_t e = launch_dependent(k_attn_bwd_fused, d.W, kFusedThreads, FusedSmem::kBytes, s, tq, tk, tv, tdo, tacc, tdkacc,
+                                     tdvacc, fp);
     time_end(mp, 4, s);
     time_begin(mp, 5, s);
-    const int64_t nq8 = T * dims->hq * 128 / 8, nk8 = T * dims->hkv * 128 / 8;
-    k_bwd_fused_finish<<<(unsigned)((nq8 + 255) / 256), 256, 0, s>>>(dq_acc, (__nv_bfloat16*)dq_dev, nq8, scale);
-    k_bwd_fused_finish<<<(unsigned)((nk8 + 255) / 256), 256, 0, s>>>(dk_acc, (__nv_bfloat16*)dk_dev, nk8, scale);
-    k_bwd_fused_finish<<<(unsigned)((nk8 + 255) / 256), 256, 0, s>>>(dv_acc, (__nv_bfloat16*)dv_dev, nk8, 1.0f);
+    if (e == cudaSuccess) {
+        const int64_t nq8 = T * dims->hq * 128 / 8, nk8 = T * dims->hkv * 128 / 8;
+        e = launch_finish({{dq_acc, dk_acc, dv_acc}, {dq_dev, dk_dev, dv_dev}, {nq8, nk8, nk8}, {scale, scale, 1.0f}}, s);
+    }
     time_end(mp, 5, s);
-    count_launch(4);
-    return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
+    count_launch();
+    return e == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
 
 extern "C" int libra_attn_pool_bwd(const void* q_dev, const void* k_dev, const void* v_dev, const void* out_dev,
@@ -764,34 +782,30 @@ extern "C" int libra_attn_pool_bwd(const void* q_dev, const void* k_dev, const v
     float* lse2 = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace_dev) + ws.stat_bytes);
     cudaStream_t s = (cudaStream_t)stream;
     if (s) const_cast<libra_plan_t*>(plan)->other_stream = 1;
-    cudaMemsetAsync(plan->d_status + 2, 0, sizeof(int), s);   // the word reports the most recent launch
 
     const float scale = dims->softmax_scale > 0.f ? dims->softmax_scale : 1.0f / sqrtf((float)D);
     if (D == 256) {   // row statistics, then the three passes of the 256-wide kernel
         libra_plan_t* mp256 = const_cast<libra_plan_t*>(plan);
         time_begin(mp256, 3, s);
-        const int64_t warps = ws.Tpad / 32 * dims->hq;
-        k_bwd_prep<256><<<(unsigned)((warps * 32 + 255) / 256), 256, 0, s>>>(
-            (const __nv_bfloat16*)out_dev, (const __nv_bfloat16*)dout_dev, lse_dev, T, ws.Tpad, dims->hq, dvec, lse2);
-        count_launch();
-        time_end(mp256, 3, s);
         float* dk_acc = nullptr;
         float* dv_acc = nullptr;
         if (fused) {
             dk_acc = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace_dev) + 2 * ws.stat_bytes);
             dv_acc = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace_dev) + 2 * ws.stat_bytes + ws.dkv_acc_bytes);
-            cudaMemsetAsync(dk_acc, 0, 2 * ws.dkv_acc_bytes, s);
         }
+        const cudaError_t e256 = launch_prep<256>(out_dev, dout_dev, lse_dev, T, ws.Tpad, dims->hq, dvec, lse2, dk_acc,
+                                                  fused ? 2 * ws.dkv_acc_bytes : 0, s);
+        time_end(mp256, 3, s);
+        if (e256 != cudaSuccess) return LIBRA_ERR_CUDA;
+        mp256->bwd_mask = 2 | 4 | 8;
         int rc256 = launch_bwd_d256(q_dev, k_dev, v_dev, dout_dev, dq_dev, dk_dev, dv_dev, lse2, dvec, ws.Tpad, dk_acc,
                                     dv_acc, plan, dims, scale, s);
         if (rc256 == LIBRA_OK && fused) {
             time_begin(mp256, 5, s);
             const int64_t nk8 = T * dims->hkv * 256 / 8;
-            k_bwd_fused_finish<<<(unsigned)((nk8 + 255) / 256), 256, 0, s>>>(dk_acc, (__nv_bfloat16*)dk_dev, nk8, scale);
-            k_bwd_fused_finish<<<(unsigned)((nk8 + 255) / 256), 256, 0, s>>>(dv_acc, (__nv_bfloat16*)dv_dev, nk8, 1.0f);
+            if (launch_finish({{dk_acc, dv_acc, nullptr}, {dk_dev, dv_dev, nullptr}, {nk8, nk8, 0}, {scale, 1.0f, 0.f}}, s) != cudaSuccess)
+                rc256 = LIBRA_ERR_CUDA;
             time_end(mp256, 5, s);
-            count_launch(2);
-            if (cudaGetLastError() != cudaSuccess) rc256 = LIBRA_ERR_CUDA;
         }
         return rc256;
     }
@@ -806,17 +820,14 @@ extern "C" int libra_attn_pool_bwd(const void* q_dev, const void* k_dev, const v
     libra_plan_t* mp0 = const_cast<libra_plan_t*>(plan);
     time_begin(mp0, 3, s);
     {
-        const int64_t warps = ws.Tpad / 32 * dims->hq;
-        const unsigned grid = (unsigned)((warps * 32 + 255) / 256);
-        if (D == 128)
-            k_bwd_prep<128><<<grid, 256, 0, s>>>((const __nv_bfloat16*)out_dev, (const __nv_bfloat16*)dout_dev, lse_dev,
-                                                 T, ws.Tpad, dims->hq, dvec, lse2);
-        else
-            k_bwd_prep<64><<<grid, 256, 0, s>>>((const __nv_bfloat16*)out_dev, (const __nv_bfloat16*)dout_dev, lse_dev,
-                                                T, ws.Tpad, dims->hq, dvec, lse2);
-        count_launch();
+        float* acc = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace_dev) + 2 * ws.stat_bytes);
+        const size_t acc_bytes = fused ? ws.dq_acc_bytes + 2 * ws.dkv_acc_bytes : 0;   // the three accumulators are contiguous
+        const cudaError_t e = D == 128 ? launch_prep<128>(out_dev, dout_dev, lse_dev, T, ws.Tpad, dims->hq, dvec, lse2, acc, acc_bytes, s)
+                                       : launch_prep<64>(out_dev, dout_dev, lse_dev, T, ws.Tpad, dims->hq, dvec, lse2, acc, acc_bytes, s);
+        if (e != cudaSuccess) return LIBRA_ERR_CUDA;
     }
     time_end(mp0, 3, s);
+    mp0->bwd_mask = fused ? 2 : 2 | 8;
     if (fused)
         return launch_fused(q_dev, k_dev, v_dev, dout_dev, dq_dev, dk_dev, dv_dev, reinterpret_cast<uint8_t*>(workspace_dev),
                             ws, plan, dims, scale, s);
@@ -834,7 +845,7 @@ extern "C" int libra_attn_pool_bwd(const void* q_dev, const void* k_dev, const v
     pa.hkv = dims->hkv;
     pa.scale = scale;
     pa.scale_log2 = scale * 1.4426950408889634f;
-    pa.status = plan->d_status + 2;
+    pa.outcome = plan->d_outcome[1];
     pa.plan_status = plan->d_status;
     pa.wait_limit_ns = plan->wait_limit_ns;
     pa.inject_stall = plan->inject_stall;
@@ -853,7 +864,8 @@ extern "C" int libra_attn_pool_bwd(const void* q_dev, const void* k_dev, const v
     pb.H = dq_dir.H;
     pb.scale = scale;
     pb.scale_log2 = scale * 1.4426950408889634f;
-    pb.status = plan->d_status + 2;
+    pb.outcome = plan->d_outcome[3];
+    pb.side_by_side = side_by_side(dkv_dir.NT, dkv_dir.W);
     pb.plan_status = plan->d_status;
     pb.wait_limit_ns = plan->wait_limit_ns;
     pb.inject_stall = plan->inject_stall;

@@ -58,7 +58,8 @@ struct DqParams {
     int64_t T, Tpad;
     int hq, hkv, H;
     float scale, scale_log2;
-    int* status;
+    int* outcome;
+    int side_by_side;        // start without waiting for the dK/dV kernel
     const int* plan_status;
     uint32_t wait_limit_ns;
     int inject_stall;
@@ -141,11 +142,16 @@ k_attn_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     const int cta = blockIdx.x;
 
     if ((smem_u32(smem) & 1023u) != 0) {
-        if (threadIdx.x == 0) atomicExch(p.status, LIBRA_ERR_CUDA);
+        if (threadIdx.x == 0) p.outcome[cta] = LIBRA_ERR_CUDA;
+        grid_dep_wait();
         return;
     }
+    // The row statistics are complete: the dK/dV kernel ahead waited for them before it let this one start.  Nothing else
+    // is needed from it, so the wait for its end may come last (a stream's later work waits for this kernel only).
+    if (!p.side_by_side) grid_dep_wait();
     if (const int ps = *p.plan_status; ps != 0) {  // malformed cu_seqlens: report and leave
-        if (threadIdx.x == 0) { atomicExch(p.status, ps); p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
+        if (threadIdx.x == 0) { p.outcome[cta] = ps; p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
+        grid_dep_wait();
         return;
     }
     if (threadIdx.x == 0) {
@@ -591,9 +597,10 @@ k_attn_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     __syncthreads();
     if (warp == kDqMmaWarp) tmem_dealloc(tmem_base, 512);
     if (threadIdx.x == 0) {
-        if (*abort_flag) atomicExch(p.status, LIBRA_ERR_TIMEOUT);
+        p.outcome[cta] = *abort_flag ? LIBRA_ERR_TIMEOUT : LIBRA_OK;
         p.busy[2 * cta + 1] = globaltimer_ns();
     }
+    grid_dep_wait();
 }
 
 }  // namespace libra

@@ -67,7 +67,7 @@ struct FusedParams {
     int64_t T, Tpad, NU;
     int hq, hkv, R;           // R = row blocks per query chunk
     float scale_log2;
-    int* status;
+    int* outcome;
     const int* plan_status;
     uint32_t wait_limit_ns;
     int inject_stall;
@@ -171,11 +171,7 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     const int cta = blockIdx.x;
 
     if ((smem_u32(smem) & 1023u) != 0) {
-        if (threadIdx.x == 0) atomicExch(p.status, LIBRA_ERR_CUDA);
-        return;
-    }
-    if (const int ps = *p.plan_status; ps != 0) {  // malformed cu_seqlens: report and leave
-        if (threadIdx.x == 0) { atomicExch(p.status, ps); p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
+        if (threadIdx.x == 0) p.outcome[cta] = LIBRA_ERR_CUDA;
         return;
     }
     if (threadIdx.x == 0) {
@@ -199,11 +195,6 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         abort_flag[0] = 0;
         abort_flag[1] = (int)p.wait_limit_ns;
         fence_mbar_init();
-        p.busy[2 * cta] = globaltimer_ns();
-    }
-    if (warp == kFuMmaWarp) {
-        tmem_alloc(tmem_slot, 512);
-        tmem_relinquish();
     }
     if (warp == kFuTmaWarp && lane == 0) {
         prefetch_tmap(&tm_q);
@@ -213,6 +204,16 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         prefetch_tmap(&tm_dqacc);
         prefetch_tmap(&tm_dkacc);
         prefetch_tmap(&tm_dvacc);
+    }
+    grid_dep_wait();
+    if (const int ps = *p.plan_status; ps != 0) {  // malformed cu_seqlens: report and leave
+        if (threadIdx.x == 0) { p.outcome[cta] = ps; p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
+        return;
+    }
+    if (threadIdx.x == 0) p.busy[2 * cta] = globaltimer_ns();
+    if (warp == kFuMmaWarp) {
+        tmem_alloc(tmem_slot, 512);
+        tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
@@ -578,15 +579,30 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     __syncthreads();
     if (warp == kFuMmaWarp) tmem_dealloc(tmem_base, 512);
     if (threadIdx.x == 0) {
-        if (abort_flag[0]) atomicExch(p.status, LIBRA_ERR_TIMEOUT);
+        p.outcome[cta] = abort_flag[0] ? LIBRA_ERR_TIMEOUT : LIBRA_OK;
         p.busy[2 * cta + 1] = globaltimer_ns();
     }
 }
 
-// dq = scale * dq_acc, dk = scale * dk_acc, dv = dv_acc, rounded to bf16 (8 elements per thread).
-__global__ void k_bwd_fused_finish(const float* __restrict__ acc, __nv_bfloat16* __restrict__ out, int64_t n8, float mul) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n8) return;
+// dq = scale * dq_acc, dk = scale * dk_acc, dv = dv_acc, rounded to bf16 (8 elements per thread), in one launch.
+struct FinishArgs {
+    const float* acc[3];
+    void* out[3];
+    int64_t n8[3];
+    float mul[3];
+};
+__global__ void k_bwd_fused_finish(const FinishArgs f) {
+    grid_dep_wait();
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    // (selected, not indexed: an index into the arguments would copy them to local memory, twice the time)
+    const float* acc = f.acc[0];
+    void* out = f.out[0];
+    float mul = f.mul[0];
+    int64_t n = f.n8[0];
+    if (i >= n) { i -= n; acc = f.acc[1]; out = f.out[1]; mul = f.mul[1]; n = f.n8[1];
+        if (i >= n) { i -= n; acc = f.acc[2]; out = f.out[2]; mul = f.mul[2]; n = f.n8[2]; }
+    }
+    if (i >= n) return;
     const float4 a = reinterpret_cast<const float4*>(acc)[2 * i], b = reinterpret_cast<const float4*>(acc)[2 * i + 1];
     uint4 w;
     w.x = pack_bf16x2(a.x * mul, a.y * mul);
@@ -594,6 +610,11 @@ __global__ void k_bwd_fused_finish(const float* __restrict__ acc, __nv_bfloat16*
     w.z = pack_bf16x2(b.x * mul, b.y * mul);
     w.w = pack_bf16x2(b.z * mul, b.w * mul);
     reinterpret_cast<uint4*>(out)[i] = w;
+}
+static cudaError_t launch_finish(const FinishArgs& f, cudaStream_t s) {
+    const int64_t n = f.n8[0] + f.n8[1] + f.n8[2];
+    count_launch();
+    return launch_dependent(k_bwd_fused_finish, (unsigned)((n + 255) / 256), 256u, 0, s, f);
 }
 
 }  // namespace libra

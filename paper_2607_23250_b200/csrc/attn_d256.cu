@@ -87,7 +87,8 @@ struct Params {
     int64_t NU;
     int R;                  // 128-row blocks per query chunk
     float scale, scale_log2;
-    int* status;
+    int* outcome;
+    int side_by_side;       // DK, DQ: start without waiting for the pass ahead
     const int* plan_status;
     uint32_t wait_limit_ns;
     int inject_stall;
@@ -189,11 +190,17 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
     const int cta = blockIdx.x;
 
     if ((smem_u32(smem) & 1023u) != 0) {
-        if (threadIdx.x == 0) atomicExch(p.status, LIBRA_ERR_CUDA);
+        if (threadIdx.x == 0) p.outcome[cta] = LIBRA_ERR_CUDA;
+        grid_dep_wait();
         return;
     }
+    // The dK and dQ passes need what the dV pass had waited for and nothing of the pass ahead: they take the SMs that
+    // fall free and wait for the pass ahead before they end.
+    if (MODE == FWD || MODE == DV || !p.side_by_side) grid_dep_wait();
+    if (MODE == DV || MODE == DK) grid_dep_launch();
     if (const int ps = *p.plan_status; ps != 0) {  // malformed cu_seqlens: report and leave
-        if (threadIdx.x == 0) { atomicExch(p.status, ps); p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
+        if (threadIdx.x == 0) { p.outcome[cta] = ps; p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
+        if (MODE == DK || MODE == DQ) grid_dep_wait();
         return;
     }
     if (threadIdx.x == 0) {
@@ -548,9 +555,10 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
     __syncthreads();
     if (warp == kMmaWarp) tmem_dealloc(tmem_base, 512);
     if (threadIdx.x == 0) {
-        if (abort_flag[0]) atomicExch(p.status, LIBRA_ERR_TIMEOUT);
+        p.outcome[cta] = abort_flag[0] ? LIBRA_ERR_TIMEOUT : LIBRA_OK;
         p.busy[2 * cta + 1] = globaltimer_ns();
     }
+    if (MODE == DK || MODE == DQ) grid_dep_wait();
 }
 
 template <int MODE>
@@ -562,9 +570,9 @@ static int launch(const CUtensorMap& sa, const CUtensorMap& sb, const CUtensorMa
             return LIBRA_ERR_CUDA;
         cfg_mark(8 + MODE);
     }
-    k_attn_d256<MODE><<<W, kThreads, L::kBytes, s>>>(sa, sb, t1, t2, prm);
     count_launch();
-    return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
+    return launch_dependent(k_attn_d256<MODE>, W, kThreads, L::kBytes, s, sa, sb, t1, t2, prm) == cudaSuccess ? LIBRA_OK
+                                                                                                          : LIBRA_ERR_CUDA;
 }
 
 }  // namespace d256
@@ -590,7 +598,7 @@ int launch_fwd_d256(const void* q, const void* k, const void* v, void* out, floa
     prm.Tpad = (plan->T + 127) / 128 * 128;
     prm.hq = dims->hq; prm.hkv = dims->hkv; prm.H = d.H;
     prm.scale = scale; prm.scale_log2 = scale * 1.4426950408889634f;
-    prm.status = plan->d_status + 1; prm.plan_status = plan->d_status;
+    prm.outcome = plan->d_outcome[0]; prm.plan_status = plan->d_status;
     prm.wait_limit_ns = plan->wait_limit_ns; prm.inject_stall = plan->inject_stall;
     prm.busy = d.d_busy;
     return launch<FWD>(tq, tq, tk, tv, prm, d.W, s);
@@ -623,11 +631,11 @@ int launch_bwd_d256(const void* q, const void* k, const void* v, const void* dou
     prm.Tpad = Tpad;
     prm.hq = dims->hq; prm.hkv = dims->hkv; prm.H = dq_dir.H;
     prm.scale = scale; prm.scale_log2 = scale * 1.4426950408889634f;
-    prm.status = plan->d_status + 2; prm.plan_status = plan->d_status;
+    prm.outcome = plan->d_outcome[1]; prm.plan_status = plan->d_status;
     prm.wait_limit_ns = plan->wait_limit_ns; prm.inject_stall = plan->inject_stall;
     libra_plan* mp = const_cast<libra_plan*>(plan);
     // dV and dK: key-major lists
-    prm.cta_offsets = kv_dir.d_cta_offsets; prm.cta_tiles = kv_dir.d_cta_exec; prm.busy = kv_dir.d_busy;
+    prm.cta_offsets = kv_dir.d_cta_offsets; prm.cta_tiles = kv_dir.d_cta_exec; prm.busy = kv_dir.d_busy2;   // the dK pass runs beside the dV pass and is the one reported
     if (pairs) { prm.u_blk = kv_dir.d_u_blk; prm.u_chunk = kv_dir.d_u_chunk; prm.NU = kv_dir.NB; prm.R = kv_dir.chunk / kv_dir.tile; }
     time_begin(mp, 1, s);
     prm.out = reinterpret_cast<__nv_bfloat16*>(dv);
@@ -635,6 +643,9 @@ int launch_bwd_d256(const void* q, const void* k, const void* v, const void* dou
     rc = launch<DV>(k128, k128, q64, do64, prm, kv_dir.W, s);
     prm.out = reinterpret_cast<__nv_bfloat16*>(dk);
     prm.acc32 = dk_acc;
+    prm.outcome = plan->d_outcome[2];
+    prm.side_by_side = side_by_side(kv_dir.NT, kv_dir.W);
+    prm.busy = kv_dir.d_busy;
     if (rc == LIBRA_OK) rc = launch<DK>(k128, v128, q64, do64, prm, kv_dir.W, s);
     time_end(mp, 1, s);
     prm.acc32 = nullptr;
@@ -642,6 +653,7 @@ int launch_bwd_d256(const void* q, const void* k, const void* v, const void* dou
     // dQ: query-major lists
     prm.cta_offsets = dq_dir.d_cta_offsets; prm.cta_tiles = dq_dir.d_cta_exec; prm.busy = dq_dir.d_busy2;
     prm.out = reinterpret_cast<__nv_bfloat16*>(dq);
+    prm.outcome = plan->d_outcome[3];
     time_begin(mp, 2, s);
     rc = launch<DQ>(q128, do128, k64, v64, prm, dq_dir.W, s);
     time_end(mp, 2, s);

@@ -65,7 +65,7 @@ struct FwdParams {
     int64_t T;
     int hq, hkv, H;
     float scale_log2;  // softmax scale * log2(e)
-    int* status;       // word to flag LIBRA_ERR_TIMEOUT in
+    int* outcome;      // [gridDim.x] 0 or what kept this CTA from doing its work
     const int* plan_status;  // the planner's verdict on cu_seqlens: non-zero = do not run
     uint32_t wait_limit_ns;  // budget of one device-side wait
     int inject_stall;        // test aid: the producer issues no loads, so the consumers' waits run out
@@ -137,11 +137,6 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const int lane = threadIdx.x & 31;
     const int cta = blockIdx.x;
 
-    // A plan whose cu_seqlens failed the planner's check is never executed: report and leave.
-    if (const int ps = *p.plan_status; ps != 0) {
-        if (threadIdx.x == 0) { atomicExch(p.status, ps); p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
-        return;
-    }
     if (threadIdx.x == 0) {
         for (int i = 0; i < L::kStages; ++i) { mbar_init(&bar_full[i], 1); mbar_init(&bar_empty[i], 1); }
         mbar_init(bar_qfull, 1);
@@ -156,17 +151,23 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         abort_flag[0] = 0;
         abort_flag[1] = (int)p.wait_limit_ns;
         fence_mbar_init();
-        p.busy[2 * cta] = globaltimer_ns();
-    }
-    if (warp == 9) {
-        tmem_alloc(tmem_slot, 512);
-        tmem_relinquish();
     }
     if (warp == 8 && lane == 0) {
         prefetch_tmap(&tm_q);
         prefetch_tmap(&tm_k);
         prefetch_tmap(&tm_v);
         prefetch_tmap(&tm_out);
+    }
+    grid_dep_wait();
+    // A plan whose cu_seqlens failed the planner's check is never executed: report and leave.
+    if (const int ps = *p.plan_status; ps != 0) {
+        if (threadIdx.x == 0) { p.outcome[cta] = ps; p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
+        return;
+    }
+    if (threadIdx.x == 0) p.busy[2 * cta] = globaltimer_ns();
+    if (warp == 9) {
+        tmem_alloc(tmem_slot, 512);
+        tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
@@ -493,7 +494,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     __syncthreads();
     if (warp == 9) tmem_dealloc(tmem_base, 512);
     if (threadIdx.x == 0) {
-        if (*abort_flag) atomicExch(p.status, LIBRA_ERR_TIMEOUT);
+        p.outcome[cta] = *abort_flag ? LIBRA_ERR_TIMEOUT : LIBRA_OK;
         p.busy[2 * cta + 1] = globaltimer_ns();
     }
 }
@@ -567,9 +568,9 @@ static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtens
         if (!regs_pool_ok(k_attn_fwd<D>, 256, LIBRA_FWD_REG_INC, 128, LIBRA_FWD_REG_DEC)) return LIBRA_ERR_UNSUPPORTED;
         cfg_mark(kSlot);
     }
-    k_attn_fwd<D><<<W, kFwdThreads, L::kAlloc, s>>>(tq, tk, tv, tout, prm);
     count_launch();
-    return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
+    return launch_dependent(k_attn_fwd<D>, W, kFwdThreads, L::kAlloc, s, tq, tk, tv, tout, prm) == cudaSuccess ? LIBRA_OK
+                                                                                                           : LIBRA_ERR_CUDA;
 }
 
 }  // namespace libra
@@ -597,7 +598,6 @@ extern "C" int libra_attn_pool_fwd(const void* q_dev, const void* k_dev, const v
     libra_plan_t* mp = const_cast<libra_plan_t*>(plan);
     if (s) mp->other_stream = 1;
     if (dims->head_dim == 256) {
-        cudaMemsetAsync(plan->d_status + 1, 0, sizeof(int), s);
         time_begin(mp, 0, s);
         const int rc256 = launch_fwd_d256(q_dev, k_dev, v_dev, out_dev, lse_dev, plan, dims, scale, s);
         time_end(mp, 0, s);
@@ -620,13 +620,12 @@ extern "C" int libra_attn_pool_fwd(const void* q_dev, const void* k_dev, const v
     prm.hkv = dims->hkv;
     prm.H = d.H;
     prm.scale_log2 = scale * 1.4426950408889634f;
-    prm.status = plan->d_status + 1;
+    prm.outcome = plan->d_outcome[0];
     prm.plan_status = plan->d_status;
     prm.wait_limit_ns = plan->wait_limit_ns;
     prm.inject_stall = plan->inject_stall;
     prm.busy = d.d_busy;
     prm.tile_ns = d.d_tile_ns;
-    cudaMemsetAsync(plan->d_status + 1, 0, sizeof(int), s);   // the word reports the most recent launch
     time_begin(mp, 0, s);
     rc = dims->head_dim == 128 ? launch_fwd<128>(tq, tk, tv, tout, prm, d.W, s)
                                : launch_fwd<64>(tq, tk, tv, tout, prm, d.W, s);

@@ -49,7 +49,12 @@ struct libra_plan {
     int other_stream = 0;            // built or used on a stream other than the legacy one
     int32_t* d_tok_start = nullptr;  // [T] first token of the sample that holds token t
     int32_t* d_tok_end = nullptr;    // [T] one past the last token of that sample
-    int* d_status = nullptr;         // [4] word 0: plan status; word 1: fwd; word 2: bwd
+    int* d_status = nullptr;         // the planner's verdict on cu_seqlens
+    // Outcome of each CTA of the last launch of a kernel (0 or LIBRA_ERR_*), written by every CTA when it leaves, so
+    // that nothing has to be cleared before a launch: forward; dK/dV, fused or dV pass; dK pass; dQ kernel or pass.
+    int* d_outcome[4] = {};          // [W] each
+    int W = 0;                       // workers of every direction
+    int bwd_mask = 0;                // which of d_outcome[1..3] the last backward wrote
     libra::PlanDir dir[3];           // 0 = query-major, 1 = key-major, 2 = pair tiles (key block x query chunk)
     uint32_t wait_limit_ns = 2000000000u;  // budget of one device-side wait (libra_plan_set_wait_limit_ns)
     int inject_stall = 0;            // test aid: the producer role issues no loads (libra_plan_inject_stall)
@@ -106,6 +111,35 @@ int launch_bwd_d256(const void* q, const void* k, const void* v, const void* dou
                     const float* lse2, const float* dvec, int64_t Tpad, float* dk_acc, float* dv_acc,
                     const libra_plan* plan, const libra_dims* dims, float scale, cudaStream_t s);
 }  // namespace libra
+
+// Launch whose blocks may start before the kernel ahead of it on the stream is done (programmatic dependent launch):
+// launch latency and prologues then overlap that kernel's last blocks.  Every kernel launched so executes
+// grid_dep_wait() (ptx.cuh) before it touches anything another kernel writes, or, where it only needs what the kernel
+// ahead had itself waited for, before it ends.  A step on 10007 tokens (forward, statistics, fused backward,
+// conversion): 175 -> 153 us with the clearing of accumulators and status words moved into those kernels.
+template <typename... KArgs, typename... Args>
+static inline cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                                           const Args&... args) {
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
+// Whether two backward kernels over the same pool that do not depend on one another run side by side: while the first has
+// few tiles for the SMs (`tiles` on `workers`) the second takes the idle ones; beyond that they only push one another's
+// tiles out of L2.  Forward and backward, 4 heads of 64 on 4096 / 16384 / 65536 tokens (1, 3.5 and 14 tiles per worker): 67
+// -> 55, 471 -> 392, 3147 -> 3140 us; 32 / 1 heads of 256 on 1500 / 32768 / 65536 tokens (0.1, 1.7, 3.5): 1431 -> 774 us,
+// 21.9 -> 19.2, 130 -> 115 ms; 128 / 4 heads of 256 on 32768 tokens, pair tiles (11.6): 99.9 -> 103.4 ms.
+constexpr int64_t kOverlapTiles = 8;   // per worker
+inline bool side_by_side(int64_t tiles, int workers) { return tiles <= kOverlapTiles * workers; }
 
 // setmaxnreg moves registers inside the pool the CTA got at launch (registers per thread as compiled x
 // threads): what the shrinking warps release must cover what the growing warps ask for, or the last

@@ -460,7 +460,8 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
     // ---- token bounds, the directions whose sizes are known, the pair tables; zeros first
     size_t zero_bytes = 0;
     auto carve = [&](Carver& c) {
-        c.take(&p->d_status, 4);
+        c.take(&p->d_status, 1);
+        for (int k = 0; k < 4; ++k) c.take(&p->d_outcome[k], p->W);
         for (int k = 0; k < 2; ++k)
             if (want[k]) carve_dir(p->dir[k], c, true, false);
         zero_bytes = c.used;
@@ -568,13 +569,14 @@ extern "C" int libra_plan_tiles(const int32_t* cu_seqlens_dev, int n_samples, in
     if (!p) return LIBRA_ERR_CUDA;
     p->T = T; p->n = n_samples; p->device = dev; p->sm_count = sms; p->stream = s;
     if (s) p->other_stream = 1;
+    p->W = o.n_workers ? o.n_workers : sms;
     const int dirs = o.directions ? o.directions : (LIBRA_DIR_Q | LIBRA_DIR_KV);
     const bool want[3] = {(dirs & LIBRA_DIR_Q) != 0, (dirs & LIBRA_DIR_KV) != 0, (dirs & LIBRA_DIR_PAIR) != 0};
     for (int k = 0; k < 3; ++k) {
         PlanDir& d = p->dir[k];
         d.tile = k == 0 ? tile_q : (o.tile_kv ? o.tile_kv : 128);
         d.H = k == 0 ? n_heads : (o.n_heads_kv ? o.n_heads_kv : n_heads);
-        d.W = o.n_workers ? o.n_workers : sms;
+        d.W = p->W;
         d.chunk = k == 2 ? (o.pair_chunk ? o.pair_chunk : 4096) : 0;
     }
     const int rc = build_plan(p, cu_seqlens_dev, o, want);
@@ -609,10 +611,10 @@ extern "C" int libra_plan_info(const libra_plan_t* plan, int direction, int64_t*
 
 extern "C" int libra_plan_status(const libra_plan_t* plan) {
     if (!plan) return LIBRA_ERR_INVALID_ARG;
-    int st[4] = {0, 0, 0, 0};
+    int st = 0;
     if (cudaStreamSynchronize(plan->stream) != cudaSuccess) return LIBRA_ERR_CUDA;
-    if (cudaMemcpy(st, plan->d_status, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess) return LIBRA_ERR_CUDA;
-    return st[0];
+    if (cudaMemcpy(&st, plan->d_status, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess) return LIBRA_ERR_CUDA;
+    return st;
 }
 
 extern "C" int libra_plan_export(const libra_plan_t* plan, int direction, int64_t* weight_host, int32_t* order_host,
@@ -694,16 +696,23 @@ extern "C" int libra_busy_times(const libra_plan_t* plan, int which, uint64_t* n
                                                               : (which == LIBRA_KERNEL_BWD_DKDV ? LIBRA_DIR_KV : LIBRA_DIR_Q));
     if (!d) return LIBRA_ERR_PLAN_MISMATCH;
     if (cudaDeviceSynchronize() != cudaSuccess) return LIBRA_ERR_CUDA;
-    uint64_t* tmp = new (std::nothrow) uint64_t[2 * (size_t)d->W];
+    uint64_t* tmp = new (std::nothrow) uint64_t[3 * (size_t)d->W];   // the stamps, then one kernel's outcomes
     if (!tmp) return LIBRA_ERR_CUDA;
-    int st[4] = {0, 0, 0, 0};
+    int* outcome = reinterpret_cast<int*>(tmp + 2 * (size_t)d->W);
+    int st = 0;
     const uint64_t* src = which == LIBRA_KERNEL_BWD_DQ ? d->d_busy2 : d->d_busy;
     cudaError_t e = cudaMemcpy(tmp, src, sizeof(uint64_t) * 2 * d->W, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) e = cudaMemcpy(st, plan->d_status, sizeof(st), cudaMemcpyDeviceToHost);
+    const int mask = which == LIBRA_KERNEL_FWD ? 1 : plan->bwd_mask;
+    for (int k = 0; k < 4 && e == cudaSuccess; ++k) {
+        if (!((mask >> k) & 1)) continue;
+        e = cudaMemcpy(outcome, plan->d_outcome[k], sizeof(int) * d->W, cudaMemcpyDeviceToHost);
+        for (int r = 0; r < d->W && e == cudaSuccess; ++r)
+            if (outcome[r] != 0) st = outcome[r];
+    }
     for (int r = 0; r < d->W; ++r) ns_host[r] = tmp[2 * r + 1] >= tmp[2 * r] ? tmp[2 * r + 1] - tmp[2 * r] : 0;
     delete[] tmp;
     if (e != cudaSuccess) return LIBRA_ERR_CUDA;
-    return st[which == LIBRA_KERNEL_FWD ? 1 : 2];
+    return st;
 }
 
 extern "C" int libra_tile_times(const libra_plan_t* plan, int which, uint32_t* ns_host) {

@@ -1,0 +1,50 @@
+"""Passes that follow one another on a stream without a wait in between: the library's kernels start before the one ahead
+has finished and some run side by side, so every pass must still see its own inputs and statistics only.  The two-kernel
+forms are bit-reproducible and are compared bit for bit with passes that were waited for; the accumulating forms by the
+rounding bound 2^-7 of their fp32 sums in another order (bf16 results)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_23250_b200 import pools
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d,hq,hkv,pairs", [(64, 4, 2, False), (128, 4, 2, False), (128, 4, 2, True), (256, 2, 1, False),
+                                            (256, 2, 1, True)])
+@pytest.mark.parametrize("T", [130, 3000, 50000])     # one tile, tiles on a part of the SMs, more tiles than run side by side
+def test_back_to_back_passes(d, hq, hkv, pairs, T):
+    from paper_2607_23250_b200 import binding as lb
+    if T == 50000 and d == 256:
+        T = 20000
+    rng = np.random.default_rng(T + d)
+    cu = torch.from_numpy(pools.cu_seqlens(pools.random_layout(rng, T, 700))).cuda()
+    directions = lb.LIBRA_DIR_Q | (lb.LIBRA_DIR_PAIR if pairs else lb.LIBRA_DIR_KV)
+    plan = lb.libra_plan_tiles(cu, hq, 256, directions=directions, tile_kv=128, n_heads_kv=hkv, pair_chunk=256 if T < 50000 else 0)
+    ins = [pools.make_tensors(T, hq, hkv, d, seed=s, device="cuda") for s in (1, 2)]
+    out, lse = torch.empty_like(ins[0]["q"]), torch.empty((hq, T), dtype=torch.float32, device="cuda")
+    grads = [torch.empty_like(ins[0][n]) for n in ("q", "k", "v")]
+    ws = torch.empty(lb.libra_attn_pool_bwd_workspace_bytes(plan, ins[0]["q"], ins[0]["k"]), dtype=torch.uint8, device="cuda")
+
+    def step(i):
+        x = ins[i]
+        lb.libra_attn_pool_fwd(x["q"], x["k"], x["v"], plan, out=out, lse=lse)
+        lb.libra_attn_pool_bwd(x["q"], x["k"], x["v"], out, lse, x["dout"], plan, dq=grads[0], dk=grads[1], dv=grads[2], workspace=ws)
+        return [t.clone() for t in (out, lse, *grads)]
+
+    want = []
+    for i in (0, 1):
+        want.append(step(i))
+        torch.cuda.synchronize()
+    got = [(i, step(i)) for i in (0, 1, 0, 1, 1, 0)]
+    torch.cuda.synchronize()
+    plan.busy_times(lb.KERNEL_FWD)
+    plan.busy_times(lb.KERNEL_BWD_FUSED if pairs else lb.KERNEL_BWD_DKDV)     # raises on a kernel timeout status
+    for i, res in got:
+        for k, (a, b) in enumerate(zip(res, want[i])):
+            if pairs and k >= 2:
+                assert (a.float() - b.float()).abs().max() <= 2.0 ** -7 * b.float().abs().max()
+            else:
+                assert torch.equal(a, b), k
+    plan.destroy()
