@@ -2,8 +2,8 @@
 //
 // A 128 x 256 bf16 operand tile is 64 KB and an accumulator of 128 rows x 256 head-dim columns takes half of
 // TMEM, so the 128-wide kernels do not stretch to this width.  One kernel template covers the four passes; every
-// pass keeps one side of the score matrix stationary (128 rows: its operand tile(s) stay in shared memory, its
-// accumulator in TMEM) and streams the other side in blocks of 64 rows (32 KB tiles):
+// pass keeps one side of the score matrix stationary (its operand tile(s) stay in shared memory, its
+// accumulator in TMEM) and streams the other side in blocks of 64 rows:
 //
 //   FWD  queries stationary   S  = Q K^T          P = softmax (online, lazy rescale)      O  += P V
 //   DV   keys stationary      S^T = K Q^T         P^T = exp2(S^T c - LSE)                 dV += P^T dO
@@ -12,6 +12,15 @@
 //
 // dK and dV cannot share TMEM with S^T and dP^T at this width (2 x 256 accumulator columns), so the gradient takes
 // three passes and recomputes S (eight GEMMs per cell for the five of the definition).
+//
+// Two CTAs work on 256 stationary rows (128 each) with cta_group::2 MMAs, so that each loads only half of every streamed
+// tile: with 128 rows per CTA a pass read 64 KB from L2 for 128 x 64 x 512 MACs per GEMM pair, 5 to 7 TB/s, and each of its
+// N = 64 MMAs took 48 cycles for the 32 of its products (forward / dV + dK / dQ of one 32768-token sample at Hq 128, Hkv 4:
+// 21.3 / 52.8 / 22.7 ms, now 16.0 / 39.0 / 22.4).  Of a streamed tile that is the B operand of an X GEMM (N = its 64 rows) a CTA holds 32 rows;
+// of one that the accumulating GEMM multiplies with (N = 256 head-dim columns) it holds 128 columns; the tile that is
+// both (Q in DK, K in DQ) is loaded in both halves.  The leader (even rank) issues all MMAs; its barriers count the
+// copies and the compute warps of both CTAs; commits arrive in both.
+//
 // TMEM: X1 (2 x 64, double-buffered) | X2 (64) | W (32: the bf16 result of the element-wise step, A operand of the
 // last GEMM) | acc (256).
 // Roles (320 threads): warps 0-7 compute, warp 8 one TMA thread, warp 9 one MMA thread.  In the gradient passes two
@@ -19,7 +28,7 @@
 // forward keeps one thread per row, because the running maximum and sum of a row live in its registers (warps 4-7
 // idle there).  Per streamed block: X1 (and X2) are issued, the compute warps turn them into W, the accumulating GEMM
 // is issued; X1 of the next block is issued ahead, so it runs under the element-wise step of the current one.
-// Tiles are prefetched through a ring of 32 KB slots.  Masks follow the sample bounds per element.
+// Masks follow the sample bounds per element, in blocks that a bound crosses.
 #include <math.h>
 
 #include "common.h"
@@ -44,28 +53,28 @@ struct Cfg {
     static constexpr bool kHasX2 = (MODE == DK || MODE == DQ);
     static constexpr int kGroups = MODE == FWD ? 1 : 2;      // compute threads per stationary row
     static constexpr int kCols = 64 / kGroups;               // columns of a streamed block per compute thread
-    static constexpr int kStationary = kHasX2 ? 2 : 1;       // resident 64 KB tiles
-    static constexpr int kSlots = kHasX2 ? 3 : 4;            // ring of 32 KB tiles
+    static constexpr int kStationary = kHasX2 ? 2 : 1;       // resident 64 KB tiles per CTA
+    static constexpr int kStreams = kHasX2 ? 3 : 2;          // streamed halves per block: X1's, [X2's,] the accumulating GEMM's
+    static constexpr int kAcc = kStreams - 1;                // the last one
+    static constexpr int kStages = kHasX2 ? 2 : 4;           // blocks in flight
     static constexpr int kBig = 65536, kBigHalf = 16384;     // 128 x 256 bf16: four column halves of 128 rows x 128 B
-    static constexpr int kSmall = 32768, kSmallHalf = 8192;  // 64 x 256 bf16: four column halves of 64 rows x 128 B
+    static constexpr int kHalfTile = 16384;                  // 32 x 256: four columns of 32 rows x 128 B, or 64 x 128: two of 64
+    static constexpr int kRowHalf = 4096, kColHalf = 8192;   // one such column of 64 elements
     static constexpr int kStatBytes = MODE == DV ? 256 : (MODE == DK ? 512 : 0);   // per streamed block: lse2[64], dvec[64]
     static constexpr int kSaOff = 0;
     static constexpr int kSbOff = kBig;
     static constexpr int kRingOff = kStationary * kBig;
-    static constexpr int kStatOff = kRingOff + kSlots * kSmall;
-    static constexpr int kBarOff = kStatOff + kSlots * 512;
-    // full[kSlots], empty[kSlots], st_full, st_empty, x1_full[2], x2_full, w_ready, acc_done, acc_free, drain, acc_step
-    static constexpr int kNumBars = 2 * kSlots + 10;
+    static constexpr int kStatOff = kRingOff + kStreams * kStages * kHalfTile;
+    static constexpr int kBarOff = kStatOff + kStages * 512;
+    // full, empty [kStreams][kStages], stat[kStages], st_full, st_empty, x1_full[2], x2_full, w_ready, acc_done, acc_free,
+    // drain, acc_step
+    static constexpr int kNumBars = 2 * kStreams * kStages + kStages + 10;
     static constexpr int kMiscOff = kBarOff + kNumBars * 8;
     static constexpr int kBytes = kMiscOff + 16;
     static_assert(kBytes <= kSmemMax, "exceeds the shared memory of an sm_100 CTA");
-    // Ring slots by stream and iteration i (counted over the whole kernel): the first streamed tile alternates
-    // between slots 0 and 1; the second has slot 2 to itself when it only feeds X2 (it is free again as soon as X2 has
-    // run, so its successor loads early), else it alternates between slots 2 and 3.
-    __host__ __device__ static constexpr uint32_t slot1(uint32_t i) { return i & 1; }
-    __host__ __device__ static constexpr uint32_t phase1(uint32_t i) { return (i >> 1) & 1; }
-    __host__ __device__ static constexpr uint32_t slot2(uint32_t i) { return kHasX2 ? 2 : 2 + (i & 1); }
-    __host__ __device__ static constexpr uint32_t phase2(uint32_t i) { return kHasX2 ? (i & 1) : ((i >> 1) & 1); }
+    __host__ __device__ static constexpr int tile_off(int stream, uint32_t stage) {
+        return kRingOff + (stream * kStages + (int)stage) * kHalfTile;
+    }
 };
 
 struct Params {
@@ -79,7 +88,8 @@ struct Params {
     const int32_t* tok_end;
     int64_t T, Tpad;
     int hq, hkv, H;         // H: head shards of the query-major lists (FWD, DQ)
-    // key-stationary passes over pair tiles (key block x query chunk x kv head) instead of key-major tiles: the
+    int W;                  // FWD, DQ: workers of the lists; a pair of CTAs runs the lists of two
+    // key-stationary passes over pair tiles (256 keys x query chunk x kv head) instead of key-major tiles: the
     // accumulator of a unit is added to acc32 [T, Hkv, 256] (fp32) and rounded by a later kernel
     float* acc32;           // null: key-major tiles, results stored as bf16 by the pass itself
     const int32_t* u_blk;   // [NU] key block of pair-block u
@@ -95,67 +105,60 @@ struct Params {
     uint64_t* busy;
 };
 
-// Walks the units of a CTA's tile list in the order every role uses.
-//   key-stationary passes: one unit per key-major tile (128 keys x one kv head); its iterations are the query heads of
-//   the group times the 64-row query blocks from the diagonal to the end of the last key's sample;
-//   query-stationary passes: a query-major tile (256 rows x head shard) gives one unit per head and 128-row half; its
-//   iterations are the 64-key blocks from the start of the first row's sample to the diagonal.
+// Walks the units of a CTA pair in the order every role of both CTAs uses.
+//   key-stationary passes: one unit per tile of the pair's list (256 keys x one kv head); its iterations are the query
+//   heads of the group times the 64-row query blocks from the diagonal to the end of the last key's sample (of the chunk);
+//   query-stationary passes: a query-major tile (256 rows x head shard) of the lists of two workers gives one unit per
+//   head; its iterations are the 64-key blocks from the start of the first row's sample to the diagonal.
+// r0 is the first of this CTA's 128 stationary rows.
 template <int MODE>
 struct Units {
     const Params& p;
-    int idx, end, hh, g, hps, G;
-    int64_t r0;                  // first stationary row
+    int idx, end, hh, hps, G;
+    int64_t r0;
     int h, kvh, b_lo, n_blk, n_it;
     __device__ Units(const Params& p_, int cta) : p(p_) {
-        idx = p.cta_offsets[cta];
-        end = p.cta_offsets[cta + 1];
+        const int c = cta >> 1;
+        if (Cfg<MODE>::kKeyStationary) {
+            idx = p.cta_offsets[c];
+            end = p.cta_offsets[c + 1];
+        } else {   // neighbouring lists are contiguous
+            idx = p.cta_offsets[2 * c];
+            end = p.cta_offsets[2 * c + 2 < p.W ? 2 * c + 2 : p.W];
+        }
         G = p.hq / p.hkv;
         hps = Cfg<MODE>::kKeyStationary ? 1 : p.hq / p.H;
-        hh = 0;
-        g = -1;
-        if (Cfg<MODE>::kKeyStationary) --idx;
+        hh = hps - 1;
+        --idx;
     }
-    __device__ bool next() {
+    __device__ bool next(uint32_t rank) {
+        if (++hh == hps) { hh = 0; if (++idx >= end) return false; }
+        const int t = p.cta_tiles[idx];
         if constexpr (Cfg<MODE>::kKeyStationary) {
-            if (++idx >= end) return false;
-            const int t = p.cta_tiles[idx];
+            const int j = p.acc32 ? p.u_blk[(int)(t % p.NU)] : t / p.hkv;
+            kvh = p.acc32 ? (int)(t / p.NU) : t % p.hkv;
+            const int64_t k0 = (int64_t)j * (2 * kRows), last_key = k0 + 2 * kRows - 1 < p.T ? k0 + 2 * kRows - 1 : p.T - 1;
+            int last64 = (p.tok_end[last_key] - 1) / kBlk;
+            b_lo = (int)(k0 / kBlk);
             if (p.acc32) {   // pair tile: the query blocks of one chunk only
-                const int pb = (int)(t % p.NU);
-                kvh = (int)(t / p.NU);
-                const int j = p.u_blk[pb], c = p.u_chunk[pb];
-                r0 = (int64_t)j * kRows;
-                const int64_t last_key = r0 + kRows - 1 < p.T ? r0 + kRows - 1 : p.T - 1;
-                const int last64 = (p.tok_end[last_key] - 1) / kBlk;
-                const int lo128 = c * p.R > j ? c * p.R : j;
-                const int hi64 = 2 * (c * p.R + p.R - 1) + 1;
-                b_lo = 2 * lo128;
-                n_blk = (hi64 < last64 ? hi64 : last64) - b_lo + 1;
-            } else {
-                kvh = t % p.hkv;
-                r0 = (int64_t)(t / p.hkv) * kRows;
-                const int64_t last_key = r0 + kRows - 1 < p.T ? r0 + kRows - 1 : p.T - 1;
-                b_lo = (int)(r0 / kBlk);
-                n_blk = (p.tok_end[last_key] - 1) / kBlk - b_lo + 1;
+                const int c = p.u_chunk[(int)(t % p.NU)], lo64 = 2 * c * p.R, hi64 = 2 * (c * p.R + p.R) - 1;
+                b_lo = lo64 > b_lo ? lo64 : b_lo;
+                last64 = hi64 < last64 ? hi64 : last64;
             }
+            n_blk = last64 - b_lo + 1;
             h = kvh * G;
             n_it = G * n_blk;
-            return true;
+            r0 = k0 + rank * kRows;
         } else {
-        for (;;) {
-            if (++g == 2) { g = 0; if (++hh == hps) { hh = 0; ++idx; } }
-            if (idx >= end) return false;
-            const int t = p.cta_tiles[idx];
-            r0 = (int64_t)(t / p.H) * (2 * kRows) + g * kRows;
-            if (r0 >= p.T) continue;   // the second half of the pool's last tile may lie past its end
+            const int64_t q0 = (int64_t)(t / p.H) * (2 * kRows), last_row = q0 + 2 * kRows - 1 < p.T ? q0 + 2 * kRows - 1 : p.T - 1;
             h = (t % p.H) * hps + hh;
             kvh = h / G;
-            const int64_t last_row = r0 + kRows - 1 < p.T ? r0 + kRows - 1 : p.T - 1;
-            b_lo = p.tok_start[r0] / kBlk;
+            b_lo = p.tok_start[q0] / kBlk;
             n_blk = (int)(last_row / kBlk) - b_lo + 1;
             n_it = n_blk;
-            return true;
+            r0 = q0 + rank * kRows;
         }
-        }
+        return true;
     }
     // head and first row of the streamed block of iteration it
     __device__ int stream_head(int it) const { return Cfg<MODE>::kKeyStationary ? h + it / n_blk : kvh; }
@@ -163,33 +166,36 @@ struct Units {
 };
 
 template <int MODE>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ CUtensorMap tm_sb,
-            const __grid_constant__ CUtensorMap tm_t1, const __grid_constant__ CUtensorMap tm_t2, const Params p) {
+            const __grid_constant__ CUtensorMap tm_t0, const __grid_constant__ CUtensorMap tm_t1,
+            const __grid_constant__ CUtensorMap tm_t2, const Params p) {
     using L = Cfg<MODE>;
-    constexpr int S = L::kSlots;
+    constexpr int S = L::kStages, N = L::kStreams;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::kBarOff);
-    uint64_t* bar_full = bars;
-    uint64_t* bar_empty = bars + S;
-    uint64_t* b2 = bars + 2 * S;
-    uint64_t* bar_stfull = b2 + 0;
+    uint64_t* bar_full = bars;                 // [N][S] leader: both CTAs' halves have landed
+    uint64_t* bar_empty = bars + N * S;        // [N][S] the MMA that read it has run
+    uint64_t* bar_stat = bars + 2 * N * S;     // [S] statistics of a streamed block (each CTA its own copy)
+    uint64_t* b2 = bar_stat + S;
+    uint64_t* bar_stfull = b2 + 0;             // leader
     uint64_t* bar_stempty = b2 + 1;
-    uint64_t* bar_x2full = b2 + 3;
-    uint64_t* bar_wready = b2 + 4;
-    uint64_t* bar_accdone = b2 + 5;
-    uint64_t* bar_accfree = b2 + 6;
-    uint64_t* bar_drain = b2 + 7;
-    uint64_t* bar_accstep = b2 + 8;    // the accumulating GEMM of an iteration has run: W may be rewritten, acc rescaled
-    uint64_t* bar_x1full = b2 + 9;     // [2] one per X1 buffer: X1 of the next block is committed a block ahead
+    uint64_t* bar_x2full = b2 + 2;
+    uint64_t* bar_wready = b2 + 3;             // leader: W is in both CTAs' TMEM
+    uint64_t* bar_accdone = b2 + 4;
+    uint64_t* bar_accfree = b2 + 5;            // leader
+    uint64_t* bar_drain = b2 + 6;
+    uint64_t* bar_accstep = b2 + 7;    // the accumulating GEMM of an iteration has run: W may be rewritten, acc rescaled
+    uint64_t* bar_x1full = b2 + 8;     // [2] one per X1 buffer: X1 of the next block is committed a block ahead
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kMiscOff);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMiscOff + 4);
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int cta = blockIdx.x;
+    const uint32_t rank = cluster_rank();
 
-    if ((smem_u32(smem) & 1023u) != 0) {
+    if ((smem_u32(smem) & 1023u) != 0) {   // (the same in both CTAs)
         if (threadIdx.x == 0) p.outcome[cta] = LIBRA_ERR_CUDA;
         grid_dep_wait();
         return;
@@ -204,15 +210,16 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
         return;
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&bar_empty[s], 1); }
+        for (int s = 0; s < N * S; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&bar_empty[s], 1); }
+        for (int s = 0; s < S; ++s) mbar_init(&bar_stat[s], 1);
         mbar_init(bar_stfull, 1);
         mbar_init(bar_stempty, 1);
         mbar_init(&bar_x1full[0], 1);
         mbar_init(&bar_x1full[1], 1);
         mbar_init(bar_x2full, 1);
-        mbar_init(bar_wready, kRows * L::kGroups);
+        mbar_init(bar_wready, 2 * 4 * L::kGroups);    // a compute warp's lanes arrive as one
         mbar_init(bar_accdone, 1);
-        mbar_init(bar_accfree, kRows * L::kGroups);
+        mbar_init(bar_accfree, 2 * 4 * L::kGroups);
         mbar_init(bar_drain, 1);
         mbar_init(bar_accstep, 1);
         abort_flag[0] = 0;
@@ -221,129 +228,135 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
         p.busy[2 * cta] = globaltimer_ns();
     }
     if (warp == kMmaWarp) {
-        tmem_alloc(tmem_slot, 512);
-        tmem_relinquish();
+        tmem_alloc_pair(tmem_slot, 512);
+        tmem_relinquish_pair();
     }
     if (warp == kTmaWarp && lane == 0) {
         prefetch_tmap(&tm_sa);
         if (L::kStationary == 2) prefetch_tmap(&tm_sb);
+        prefetch_tmap(&tm_t0);
         prefetch_tmap(&tm_t1);
-        prefetch_tmap(&tm_t2);
+        if (N == 3) prefetch_tmap(&tm_t2);
     }
     tc_fence_before();
     __syncthreads();
+    cluster_sync();      // both CTAs' barriers are initialised and their TMEM is allocated
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == kTmaWarp) {
-        // ---------------- TMA producer ----------------
+        // ---------------- TMA producer (each CTA loads its own halves; the leader's barriers count both) ----------------
         if (elect_one()) {
             Units<MODE> u(p, cta);
             uint32_t n = 0, uc = 0;          // n: iterations so far (over all units)
-            uint32_t armed[S] = {};          // per slot: 1 + parity of the phase last armed (0: never)
             bool ok = true;
-            while (ok && !p.inject_stall && u.next()) {
+            const uint32_t stfull0 = map_to_rank(bar_stfull, 0);
+            while (ok && !p.inject_stall && u.next(rank)) {
                 ok = mbar_wait(bar_stempty, (uc & 1) ^ 1, abort_flag);
                 if (!ok) break;
-                mbar_arrive_expect_tx(bar_stfull, L::kStationary * L::kBig);
+                if (rank == 0) mbar_arrive_expect_tx(bar_stfull, 2 * L::kStationary * L::kBig);
                 const int st_head = L::kKeyStationary ? u.kvh : u.h;
                 for (int half = 0; half < 4; ++half) {
-                    tma_load_3d(smem + L::kSaOff + half * L::kBigHalf, &tm_sa, bar_stfull, half * 64, st_head, (int)u.r0);
+                    tma_load_3d_pair(smem + L::kSaOff + half * L::kBigHalf, &tm_sa, stfull0, half * 64, st_head, (int)u.r0);
                     if (L::kStationary == 2)
-                        tma_load_3d(smem + L::kSbOff + half * L::kBigHalf, &tm_sb, bar_stfull, half * 64, st_head, (int)u.r0);
+                        tma_load_3d_pair(smem + L::kSbOff + half * L::kBigHalf, &tm_sb, stfull0, half * 64, st_head, (int)u.r0);
                 }
                 ++uc;
                 for (int it = 0; it < u.n_it && ok; ++it, ++n) {
                     const int sh = u.stream_head(it), row = u.stream_row(it);
-                    for (int which = 0; which < 2 && ok; ++which) {
-                        const uint32_t s = which == 0 ? L::slot1(n) : L::slot2(n);
-                        const uint32_t ph = which == 0 ? L::phase1(n) : L::phase2(n);
-                        ok = mbar_wait(&bar_empty[s], ph ^ 1, abort_flag);
+                    const uint32_t s = n % S, ph = (n / S) & 1;
+                    for (int k = 0; k < N && ok; ++k) {
+                        ok = mbar_wait(&bar_empty[k * S + s], ph ^ 1, abort_flag);
                         if (!ok) break;
-                        mbar_arrive_expect_tx(&bar_full[s], L::kSmall + (which == 0 ? L::kStatBytes : 0));
-                        armed[s] = 1 + ph;
-                        for (int half = 0; half < 4; ++half)
-                            tma_load_3d(smem + L::kRingOff + s * L::kSmall + half * L::kSmallHalf, which == 0 ? &tm_t1 : &tm_t2,
-                                        &bar_full[s], half * 64, sh, row);
-                        if (which == 0 && L::kStatBytes >= 256)
-                            bulk_load_1d(smem + L::kStatOff + s * 512, p.lse2 + (size_t)sh * p.Tpad + row, 256, &bar_full[s]);
-                        if (which == 0 && L::kStatBytes == 512)
-                            bulk_load_1d(smem + L::kStatOff + s * 512 + 256, p.dvec + (size_t)sh * p.Tpad + row, 256, &bar_full[s]);
+                        if (rank == 0) mbar_arrive_expect_tx(&bar_full[k * S + s], 2 * L::kHalfTile);
+                        const uint32_t full0 = map_to_rank(&bar_full[k * S + s], 0);
+                        uint8_t* dst = smem + L::tile_off(k, s);
+                        if (k == L::kAcc) {
+                            for (int c = 0; c < 2; ++c)   // this CTA's 128 of the 256 columns
+                                tma_load_3d_pair(dst + c * L::kColHalf, N == 3 ? &tm_t2 : &tm_t1, full0, 128 * (int)rank + 64 * c, sh, row);
+                        } else {
+                            for (int c = 0; c < 4; ++c)   // this CTA's 32 of the 64 rows
+                                tma_load_3d_pair(dst + c * L::kRowHalf, k == 0 ? &tm_t0 : &tm_t1, full0, 64 * c, sh, row + 32 * (int)rank);
+                        }
+                        if (k == L::kAcc && L::kStatBytes > 0) {   // the slot's last reader was ahead of this stream's MMA
+                            mbar_arrive_expect_tx(&bar_stat[s], L::kStatBytes);
+                            bulk_load_1d(smem + L::kStatOff + s * 512, p.lse2 + (size_t)sh * p.Tpad + row, 256, &bar_stat[s]);
+                            if (L::kStatBytes == 512)
+                                bulk_load_1d(smem + L::kStatOff + s * 512 + 256, p.dvec + (size_t)sh * p.Tpad + row, 256, &bar_stat[s]);
+                        }
                     }
                 }
             }
             if (!ok || abort_flag[0]) {   // give-up path: the copies already issued land before shared memory is released
-                if (uc > 0) mbar_wait_drain(bar_stfull, (uc - 1) & 1, kDrainNs);
-                for (int b = 0; b < S; ++b)
-                    if (armed[b]) mbar_wait_drain(&bar_full[b], armed[b] - 1, kDrainNs);
+                const uint64_t t0 = globaltimer_ns();
+                while (globaltimer_ns() - t0 < kDrainNs) {}
             }
         }
         __syncwarp();
     } else if (warp == kMmaWarp) {
-        // ---------------- MMA issuer ----------------
-        if (elect_one()) {
-            constexpr uint32_t idesc_x = make_idesc(kRows, kBlk, 0, 0);    // X = stationary x streamed^T, both K-major
-            constexpr uint32_t idesc_acc = make_idesc(kRows, kD, 0, 1);    // acc += W (TMEM) x streamed tile, MN-major
+        // ---------------- MMA issuer (the leader's, for both) ----------------
+        if (rank == 0 && elect_one()) {
+            constexpr uint32_t idesc_x = make_idesc(2 * kRows, kBlk, 0, 0);    // X = stationary x streamed^T, both K-major
+            constexpr uint32_t idesc_acc = make_idesc(2 * kRows, kD, 0, 1);    // acc += W (TMEM) x streamed tile, MN-major
             const uint32_t sb = smem_u32(smem);
-            const uint64_t kdesc0 = make_sdesc(sb, 16, 1024);              // K-major view at offset 0
-            const uint64_t mdesc0 = make_sdesc(sb, L::kSmallHalf, 1024);   // MN-major view of a 64-row tile
+            const uint64_t kdesc0 = make_sdesc(sb, 16, 1024);               // K-major view at offset 0
+            const uint64_t mdesc0 = make_sdesc(sb, L::kColHalf, 1024);      // MN-major view of a 64-row tile
             auto issue_x = [&](uint32_t d_col, uint32_t a_off, uint32_t b_off) {
                 const uint64_t da = sdesc_advance(kdesc0, a_off), db = sdesc_advance(kdesc0, b_off);
 #pragma unroll
                 for (int kk = 0; kk < kD / 16; ++kk)
-                    mma_ss(tmem_base + d_col, sdesc_advance(da, (kk / 4) * L::kBigHalf + (kk % 4) * 32),
-                           sdesc_advance(db, (kk / 4) * L::kSmallHalf + (kk % 4) * 32), idesc_x, kk > 0);
+                    mma_ss_pair(tmem_base + d_col, sdesc_advance(da, (kk / 4) * L::kBigHalf + (kk % 4) * 32),
+                                sdesc_advance(db, (kk / 4) * L::kRowHalf + (kk % 4) * 32), idesc_x, kk > 0);
             };
             Units<MODE> u(p, cta);
             uint32_t uc = 0, itc = 0;
             bool ok = true;
-            while (ok && u.next()) {
-                ok = mbar_wait(bar_stfull, uc & 1, abort_flag);
-                if (ok) ok = mbar_wait(&bar_full[L::slot1(itc)], L::phase1(itc), abort_flag);
-                if (!ok) break;
+            // X1 of iteration i into its buffer; its streamed half is free again as soon as it has run
+            auto do_x1 = [&](uint32_t i) -> bool {
+                if (!mbar_wait(&bar_full[i % S], (i / S) & 1, abort_flag)) return false;
                 tc_fence_after();
-                issue_x(kColX1 + (itc & 1) * 64, L::kSaOff, L::kRingOff + L::slot1(itc) * L::kSmall);
-                tc_commit(&bar_x1full[itc & 1]);
+                issue_x(kColX1 + (i & 1) * 64, L::kSaOff, L::tile_off(0, i % S));
+                tc_commit_pair(&bar_x1full[i & 1]);
+                tc_commit_pair(&bar_empty[i % S]);
+                return true;
+            };
+            while (ok && u.next(rank)) {
+                ok = mbar_wait(bar_stfull, uc & 1, abort_flag);
+                if (ok) ok = do_x1(itc);
+                if (!ok) break;
                 for (int it = 0; it < u.n_it && ok; ++it, ++itc) {
-                    const uint32_t s1 = L::slot1(itc), s2 = L::slot2(itc);
-                    ok = mbar_wait(&bar_full[s2], L::phase2(itc), abort_flag);
-                    if (!ok) break;
+                    const uint32_t s = itc % S, ph = (itc / S) & 1;
                     if (L::kHasX2) {
-                        tc_fence_after();
-                        issue_x(kColX2, L::kSbOff, L::kRingOff + s2 * L::kSmall);
-                        tc_commit(bar_x2full);
-                        tc_commit(&bar_empty[s2]);   // the second streamed tile only feeds X2
-                    }
-                    if (it + 1 < u.n_it) {
-                        // X1 of the next block into the other buffer (read out two iterations ago): it runs while the
-                        // compute warps work on this block
-                        ok = mbar_wait(&bar_full[L::slot1(itc + 1)], L::phase1(itc + 1), abort_flag);
+                        ok = mbar_wait(&bar_full[S + s], ph, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        issue_x(kColX1 + ((itc + 1) & 1) * 64, L::kSaOff, L::kRingOff + L::slot1(itc + 1) * L::kSmall);
-                        tc_commit(&bar_x1full[(itc + 1) & 1]);
+                        issue_x(kColX2, L::kSbOff, L::tile_off(1, s));
+                        tc_commit_pair(bar_x2full);
+                        tc_commit_pair(&bar_empty[S + s]);
                     }
-                    ok = mbar_wait(bar_wready, itc & 1, abort_flag);
+                    // X1 of the next block into the other buffer (read out two iterations ago): it runs while the
+                    // compute warps work on this block
+                    if (it + 1 < u.n_it) ok = do_x1(itc + 1);
+                    if (ok) ok = mbar_wait(&bar_full[L::kAcc * S + s], ph, abort_flag);
+                    if (ok) ok = mbar_wait(bar_wready, itc & 1, abort_flag);
                     if (ok && it == 0 && uc > 0) ok = mbar_wait(bar_accfree, (uc - 1) & 1, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                     {
-                        const uint32_t sbt = L::kHasX2 ? s1 : s2;   // FWD: V, DV: dO; DK: Q, DQ: K
-                        const uint64_t db = sdesc_advance(mdesc0, L::kRingOff + sbt * L::kSmall);
+                        const uint64_t db = sdesc_advance(mdesc0, L::tile_off(L::kAcc, s));
 #pragma unroll
                         for (int kk = 0; kk < kBlk / 16; ++kk)
-                            mma_ts(tmem_base + kColAcc, tmem_base + kColW + kk * 8, sdesc_advance(db, kk * 2048), idesc_acc,
-                                   (it > 0 || kk > 0) ? 1u : 0u);
+                            mma_ts_pair(tmem_base + kColAcc, tmem_base + kColW + kk * 8, sdesc_advance(db, kk * 2048), idesc_acc,
+                                        (it > 0 || kk > 0) ? 1u : 0u);
                     }
-                    tc_commit(bar_accstep);
-                    tc_commit(&bar_empty[s1]);
-                    if (!L::kHasX2) tc_commit(&bar_empty[s2]);
-                    if (it == u.n_it - 1) { tc_commit(bar_accdone); tc_commit(bar_stempty); }
+                    tc_commit_pair(bar_accstep);
+                    tc_commit_pair(&bar_empty[L::kAcc * S + s]);
+                    if (it == u.n_it - 1) { tc_commit_pair(bar_accdone); tc_commit_pair(bar_stempty); }
                 }
                 ++uc;
             }
             if (!ok || abort_flag[0]) {
-                tc_commit(bar_drain);
+                tc_commit_pair(bar_drain);
                 mbar_wait_drain(bar_drain, 0, kDrainNs);
             }
         }
@@ -360,10 +373,11 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
         const uint32_t t_x2 = tmem_base + lane_addr + kColX2 + col0;
         const uint32_t t_w = tmem_base + lane_addr + kColW + col0 / 2;
         const uint32_t t_acc = tmem_base + lane_addr + kColAcc + grp * (kD / L::kGroups);
+        const uint32_t wready0 = map_to_rank(bar_wready, 0), accfree0 = map_to_rank(bar_accfree, 0);
         Units<MODE> u(p, cta);
         uint32_t uc = 0, itc = 0;
         bool ok = true;
-        while (ok && u.next()) {
+        while (ok && u.next(rank)) {
             const int64_t row = u.r0 + r;            // this thread's query row (FWD, DQ) or key (DV, DK)
             const bool row_ok = row < p.T;
             // visible columns of streamed block starting at b0: [lo_abs - b0, hi_abs - b0]
@@ -380,8 +394,10 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
             float m_ref = -INFINITY, l_sum = 0.f;    // FWD
             float lse2r = 0.f, dvecr = 0.f;          // DQ
             if (MODE == DQ) {
-                lse2r = p.lse2[(size_t)u.h * p.Tpad + row];   // row < Tpad always
-                dvecr = p.dvec[(size_t)u.h * p.Tpad + row];
+                if (row_ok) {                                 // (this CTA's rows may lie past the end of the pool)
+                    lse2r = p.lse2[(size_t)u.h * p.Tpad + row];
+                    dvecr = p.dvec[(size_t)u.h * p.Tpad + row];
+                }
             }
             for (int it = 0; it < u.n_it && ok; ++it, ++itc) {
                 const int64_t b0 = u.stream_row(it);
@@ -389,10 +405,10 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                 const int c_lo = (int)(lo_abs - b0 > kBlk ? kBlk : lo_abs - b0) - col0;
                 const int c_hi = (int)(hi_abs - b0 < -1 ? -1 : hi_abs - b0) - col0;
                 const bool need_mask = __any_sync(0xffffffffu, c_lo > 0 || c_hi < NC - 1);   // most blocks are dense
-                const uint32_t s1 = L::slot1(itc);
+                const uint32_t s1 = itc % S;
                 const float* st = reinterpret_cast<const float*>(smem + L::kStatOff + s1 * 512) + col0;
-                if (L::kStatBytes > 0) {   // the streamed rows' statistics arrive with their first tile
-                    ok = warp_wait(&bar_full[s1], L::phase1(itc), abort_flag);
+                if (L::kStatBytes > 0) {   // the streamed rows' statistics
+                    ok = warp_wait(&bar_stat[s1], (itc / S) & 1, abort_flag);
                     if (!ok) break;
                 }
                 ok = warp_wait(&bar_x1full[itc & 1], (itc >> 1) & 1, abort_flag);
@@ -462,10 +478,23 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                 } else {
                     // P = exp2(S c - LSE) on the visible elements, 0 elsewhere
                     float pf[NC];
+                    const uint64_t scale2 = f2_pack(p.scale_log2, p.scale_log2), neg1 = f2_pack(-1.f, -1.f);
+                    const uint64_t nl2 = f2_pack(-lse2r, -lse2r);
 #pragma unroll
-                    for (int i = 0; i < NC; ++i) {
-                        const float l2 = L::kKeyStationary ? st[i] : lse2r;
-                        pf[i] = ex2_approx(fmaf(__uint_as_float(sr[i]), p.scale_log2, -l2));
+                    for (int i = 0; i < NC; i += 4) {   // 16-byte broadcast loads of the streamed rows' LSE
+                        uint64_t n01 = nl2, n23 = nl2;
+                        if (L::kKeyStationary) {
+                            const ulonglong2 l4 = *reinterpret_cast<const ulonglong2*>(st + i);
+                            n01 = f2_mul(l4.x, neg1);
+                            n23 = f2_mul(l4.y, neg1);
+                        }
+                        float x0, x1, x2, x3;
+                        f2_unpack(f2_fma(f2_pack(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), scale2, n01), x0, x1);
+                        f2_unpack(f2_fma(f2_pack(__uint_as_float(sr[i + 2]), __uint_as_float(sr[i + 3])), scale2, n23), x2, x3);
+                        pf[i] = ex2_approx(x0);
+                        pf[i + 1] = ex2_approx(x1);
+                        pf[i + 2] = ex2_approx(x2);
+                        pf[i + 3] = ex2_approx(x3);
                     }
                     if (need_mask) {
                         static_assert(MODE == FWD || NC == 32, "one mask word per compute thread");
@@ -484,14 +513,28 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
 #pragma unroll
                         for (int c = 0; c < NC; c += 32) tmem_ld32(t_x2 + c, dp + c);
                         tmem_ld_wait();
+                        const uint64_t nd2 = f2_pack(-dvecr, -dvecr);
 #pragma unroll
-                        for (int i = 0; i < NC; i += 2) {
-                            const float d0 = L::kKeyStationary ? st[64 + i] : dvecr;
-                            const float d1 = L::kKeyStationary ? st[64 + i + 1] : dvecr;
-                            pk[i >> 1] = pack_bf16x2(pf[i] * (__uint_as_float(dp[i]) - d0), pf[i + 1] * (__uint_as_float(dp[i + 1]) - d1));
+                        for (int i = 0; i < NC; i += 4) {
+                            uint64_t n01 = nd2, n23 = nd2;
+                            if (L::kKeyStationary) {
+                                const ulonglong2 d4 = *reinterpret_cast<const ulonglong2*>(st + 64 + i);
+                                n01 = f2_mul(d4.x, neg1);
+                                n23 = f2_mul(d4.y, neg1);
+                            }
+                            float y0, y1, y2, y3;
+                            f2_unpack(f2_mul(f2_pack(pf[i], pf[i + 1]),
+                                             f2_add(f2_pack(__uint_as_float(dp[i]), __uint_as_float(dp[i + 1])), n01)), y0, y1);
+                            f2_unpack(f2_mul(f2_pack(pf[i + 2], pf[i + 3]),
+                                             f2_add(f2_pack(__uint_as_float(dp[i + 2]), __uint_as_float(dp[i + 3])), n23)), y2, y3);
+                            pk[i >> 1] = pack_bf16x2(y0, y1);
+                            pk[(i >> 1) + 1] = pack_bf16x2(y2, y3);
                         }
                     }
                 }
+                // (the results exist before the wait: left to itself the compiler moves the exponentials behind it)
+#pragma unroll
+                for (int i = 0; i < NC / 2; ++i) asm volatile("" : "+r"(pk[i]));
                 if (itc > 0) {   // the previous accumulating GEMM has consumed W
                     ok = warp_wait(bar_accstep, (itc - 1) & 1, abort_flag);
                     if (!ok) break;
@@ -501,7 +544,8 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                 for (int c = 0; c < NC / 2; c += 16) tmem_st16(t_w + c, pk + c);
                 tmem_st_wait();
                 tc_fence_before();
-                mbar_arrive(bar_wready);
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(wready0);
             }
             if (!ok) break;
             // ---- unit epilogue: the accumulator leaves TMEM ----
@@ -545,7 +589,8 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
             }
             if (MODE == FWD && row_ok) p.lse[(size_t)u.h * p.T + row] = (m_ref + log2f(l_sum)) * 0.6931471805599453f;
             tc_fence_before();
-            mbar_arrive(bar_accfree);
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(accfree0);
             ++uc;
         }
     }
@@ -553,7 +598,9 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
     // ---------------- teardown ----------------
     tc_fence_before();
     __syncthreads();
-    if (warp == kMmaWarp) tmem_dealloc(tmem_base, 512);
+    cluster_sync();      // nothing of the other CTA is on its way here any more
+    tc_fence_after();
+    if (warp == kMmaWarp) tmem_dealloc_pair(tmem_base, 512);
     if (threadIdx.x == 0) {
         p.outcome[cta] = abort_flag[0] ? LIBRA_ERR_TIMEOUT : LIBRA_OK;
         p.busy[2 * cta + 1] = globaltimer_ns();
@@ -562,7 +609,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
 }
 
 template <int MODE>
-static int launch(const CUtensorMap& sa, const CUtensorMap& sb, const CUtensorMap& t1, const CUtensorMap& t2,
+static int launch(const CUtensorMap& sa, const CUtensorMap& sb, const CUtensorMap& t0, const CUtensorMap& t1, const CUtensorMap& t2,
                   const Params& prm, int W, cudaStream_t s) {
     using L = Cfg<MODE>;
     if (!cfg_done(8 + MODE)) {   // per device
@@ -571,8 +618,9 @@ static int launch(const CUtensorMap& sa, const CUtensorMap& sb, const CUtensorMa
         cfg_mark(8 + MODE);
     }
     count_launch();
-    return launch_dependent(k_attn_d256<MODE>, W, kThreads, L::kBytes, s, sa, sb, t1, t2, prm) == cudaSuccess ? LIBRA_OK
-                                                                                                          : LIBRA_ERR_CUDA;
+    const unsigned grid = 2 * ((W + 1) / 2);   // a pair of CTAs for every two workers
+    return launch_dependent(k_attn_d256<MODE>, grid, kThreads, L::kBytes, s, sa, sb, t0, t1, t2, prm) == cudaSuccess ? LIBRA_OK
+                                                                                                                : LIBRA_ERR_CUDA;
 }
 
 }  // namespace d256
@@ -582,9 +630,9 @@ int launch_fwd_d256(const void* q, const void* k, const void* v, void* out, floa
                     const libra_dims* dims, float scale, cudaStream_t s) {
     using namespace d256;
     const PlanDir& d = plan->dir[0];
-    CUtensorMap tq, tk, tv;
+    CUtensorMap tq, tk, tv;   // K by halves of a block's rows, V by halves of its columns
     int rc = make_thd_map(&tq, q, plan->T, dims->hq, kD, kRows);
-    if (rc == LIBRA_OK) rc = make_thd_map(&tk, k, plan->T, dims->hkv, kD, kBlk);
+    if (rc == LIBRA_OK) rc = make_thd_map(&tk, k, plan->T, dims->hkv, kD, kBlk / 2);
     if (rc == LIBRA_OK) rc = make_thd_map(&tv, v, plan->T, dims->hkv, kD, kBlk);
     if (rc != LIBRA_OK) return rc;
     Params prm = {};
@@ -596,12 +644,12 @@ int launch_fwd_d256(const void* q, const void* k, const void* v, void* out, floa
     prm.tok_end = plan->d_tok_end;
     prm.T = plan->T;
     prm.Tpad = (plan->T + 127) / 128 * 128;
-    prm.hq = dims->hq; prm.hkv = dims->hkv; prm.H = d.H;
+    prm.hq = dims->hq; prm.hkv = dims->hkv; prm.H = d.H; prm.W = d.W;
     prm.scale = scale; prm.scale_log2 = scale * 1.4426950408889634f;
     prm.outcome = plan->d_outcome[0]; prm.plan_status = plan->d_status;
     prm.wait_limit_ns = plan->wait_limit_ns; prm.inject_stall = plan->inject_stall;
     prm.busy = d.d_busy;
-    return launch<FWD>(tq, tq, tk, tv, prm, d.W, s);
+    return launch<FWD>(tq, tq, tk, tv, tv, prm, d.W, s);
 }
 
 // Backward at head_dim 256: the dV and dK passes over the key-major lists, the dQ pass over the query-major lists.
@@ -612,16 +660,21 @@ int launch_bwd_d256(const void* q, const void* k, const void* v, const void* dou
     using namespace d256;
     const PlanDir& dq_dir = plan->dir[0];
     const bool pairs = dk_acc != nullptr;            // key-stationary passes over pair tiles, fp32 accumulators
-    const PlanDir& kv_dir = plan->dir[pairs ? 2 : 1];
-    CUtensorMap q128, do128, k128, v128, q64, do64, k64, v64;
+    const PlanDir& kv_dir = plan->dir[3];            // 256 keys a tile, in pair tiles or key-major
+    if (!kv_dir.enabled || (kv_dir.d_u_blk != nullptr) != pairs) return LIBRA_ERR_PLAN_MISMATCH;
+    // whole 128-row tiles (stationary), halves of a streamed block's rows (32) and of its columns (64-row boxes)
+    CUtensorMap q128, do128, k128, v128, q32, do32, k32, v32, q64, do64, k64;
     int rc = make_thd_map(&q128, q, plan->T, dims->hq, kD, kRows);
     if (rc == LIBRA_OK) rc = make_thd_map(&do128, dout, plan->T, dims->hq, kD, kRows);
     if (rc == LIBRA_OK) rc = make_thd_map(&k128, k, plan->T, dims->hkv, kD, kRows);
     if (rc == LIBRA_OK) rc = make_thd_map(&v128, v, plan->T, dims->hkv, kD, kRows);
+    if (rc == LIBRA_OK) rc = make_thd_map(&q32, q, plan->T, dims->hq, kD, kBlk / 2);
+    if (rc == LIBRA_OK) rc = make_thd_map(&do32, dout, plan->T, dims->hq, kD, kBlk / 2);
+    if (rc == LIBRA_OK) rc = make_thd_map(&k32, k, plan->T, dims->hkv, kD, kBlk / 2);
+    if (rc == LIBRA_OK) rc = make_thd_map(&v32, v, plan->T, dims->hkv, kD, kBlk / 2);
     if (rc == LIBRA_OK) rc = make_thd_map(&q64, q, plan->T, dims->hq, kD, kBlk);
     if (rc == LIBRA_OK) rc = make_thd_map(&do64, dout, plan->T, dims->hq, kD, kBlk);
     if (rc == LIBRA_OK) rc = make_thd_map(&k64, k, plan->T, dims->hkv, kD, kBlk);
-    if (rc == LIBRA_OK) rc = make_thd_map(&v64, v, plan->T, dims->hkv, kD, kBlk);
     if (rc != LIBRA_OK) return rc;
     Params prm = {};
     prm.lse2 = lse2; prm.dvec = dvec;
@@ -629,24 +682,24 @@ int launch_bwd_d256(const void* q, const void* k, const void* v, const void* dou
     prm.tok_end = plan->d_tok_end;
     prm.T = plan->T;
     prm.Tpad = Tpad;
-    prm.hq = dims->hq; prm.hkv = dims->hkv; prm.H = dq_dir.H;
+    prm.hq = dims->hq; prm.hkv = dims->hkv; prm.H = dq_dir.H; prm.W = dq_dir.W;
     prm.scale = scale; prm.scale_log2 = scale * 1.4426950408889634f;
     prm.outcome = plan->d_outcome[1]; prm.plan_status = plan->d_status;
     prm.wait_limit_ns = plan->wait_limit_ns; prm.inject_stall = plan->inject_stall;
     libra_plan* mp = const_cast<libra_plan*>(plan);
     // dV and dK: key-major lists
-    prm.cta_offsets = kv_dir.d_cta_offsets; prm.cta_tiles = kv_dir.d_cta_exec; prm.busy = kv_dir.d_busy2;   // the dK pass runs beside the dV pass and is the one reported
-    if (pairs) { prm.u_blk = kv_dir.d_u_blk; prm.u_chunk = kv_dir.d_u_chunk; prm.NU = kv_dir.NB; prm.R = kv_dir.chunk / kv_dir.tile; }
+    prm.cta_offsets = kv_dir.d_cta_offsets; prm.cta_tiles = kv_dir.d_cta_exec; prm.busy = plan->dir[pairs ? 2 : 1].d_busy2;   // the dK pass runs beside the dV pass and is the one reported
+    if (pairs) { prm.u_blk = kv_dir.d_u_blk; prm.u_chunk = kv_dir.d_u_chunk; prm.NU = kv_dir.NB; prm.R = kv_dir.chunk / kRows; }
     time_begin(mp, 1, s);
     prm.out = reinterpret_cast<__nv_bfloat16*>(dv);
     prm.acc32 = dv_acc;
-    rc = launch<DV>(k128, k128, q64, do64, prm, kv_dir.W, s);
+    rc = launch<DV>(k128, k128, q32, do64, do64, prm, plan->W, s);
     prm.out = reinterpret_cast<__nv_bfloat16*>(dk);
     prm.acc32 = dk_acc;
     prm.outcome = plan->d_outcome[2];
     prm.side_by_side = side_by_side(kv_dir.NT, kv_dir.W);
-    prm.busy = kv_dir.d_busy;
-    if (rc == LIBRA_OK) rc = launch<DK>(k128, v128, q64, do64, prm, kv_dir.W, s);
+    prm.busy = plan->dir[pairs ? 2 : 1].d_busy;
+    if (rc == LIBRA_OK) rc = launch<DK>(k128, v128, q32, do32, q64, prm, plan->W, s);
     time_end(mp, 1, s);
     prm.acc32 = nullptr;
     if (rc != LIBRA_OK) return rc;
@@ -655,7 +708,7 @@ int launch_bwd_d256(const void* q, const void* k, const void* v, const void* dou
     prm.out = reinterpret_cast<__nv_bfloat16*>(dq);
     prm.outcome = plan->d_outcome[3];
     time_begin(mp, 2, s);
-    rc = launch<DQ>(q128, do128, k64, v64, prm, dq_dir.W, s);
+    rc = launch<DQ>(q128, do128, k32, v32, k64, prm, dq_dir.W, s);
     time_end(mp, 2, s);
     return rc;
 }

@@ -55,7 +55,9 @@ struct libra_plan {
     int* d_outcome[4] = {};          // [W] each
     int W = 0;                       // workers of every direction
     int bwd_mask = 0;                // which of d_outcome[1..3] the last backward wrote
-    libra::PlanDir dir[3];           // 0 = query-major, 1 = key-major, 2 = pair tiles (key block x query chunk)
+    // 0 = query-major, 1 = key-major, 2 = pair tiles (key block x query chunk), 3 = the key-stationary tiles of kernels that
+    // run on pairs of CTAs: as 2 when that is there, else as 1, with 256 keys a tile and a worker for every two
+    libra::PlanDir dir[4];
     uint32_t wait_limit_ns = 2000000000u;  // budget of one device-side wait (libra_plan_set_wait_limit_ns)
     int inject_stall = 0;            // test aid: the producer role issues no loads (libra_plan_inject_stall)
     int timing = 0;                  // record events around the main kernels

@@ -109,7 +109,7 @@ struct DirView {
     int64_t* loads;
 };
 struct DirViews {
-    DirView v[3];
+    DirView v[4];
 };
 
 // Weight of block b (Eq. 6): a token at position p of a sample of length len contributes
@@ -287,13 +287,14 @@ __global__ void k_exec_order(const DirViews views) {
 // of the sample that holds the key block's last key.  Pair-block (c, j) = key block j against the R = chunk / tile
 // row blocks of query chunk c, present when one of them is live; numbered chunk by chunk, key blocks ascending.
 // last(j) never decreases with j, so the key blocks of a chunk are the range first(c) .. min(NKB, (c+1) R) - 1.
-__device__ __forceinline__ int64_t pair_last_row_block(const int32_t* tok_end, int64_t T, int tile, int64_t j) {
-    const int64_t last_key = ((j + 1) * tile < T ? (j + 1) * tile : T) - 1;
-    return ((int64_t)tok_end[last_key] - 1) / tile;
+// Key blocks of kt tokens against row blocks of rt tokens (kt a multiple of rt; the pair tiles proper have kt = rt).
+__device__ __forceinline__ int64_t pair_last_row_block(const int32_t* tok_end, int64_t T, int kt, int rt, int64_t j) {
+    const int64_t last_key = ((j + 1) * kt < T ? (j + 1) * kt : T) - 1;
+    return ((int64_t)tok_end[last_key] - 1) / rt;
 }
 // One block: the key-block range of every query chunk, the exclusive prefix sum of the counts, their total in base[NC].
-__global__ void __launch_bounds__(1024) k_pair_chunks(const int32_t* __restrict__ tok_end, int64_t T, int tile, int R, int64_t NKB,
-                                                      int64_t NC, int32_t* __restrict__ first_j, int32_t* __restrict__ count,
+__global__ void __launch_bounds__(1024) k_pair_chunks(const int32_t* __restrict__ tok_end, int64_t T, int kt, int rt, int R,
+                                                      int64_t NKB, int64_t NC, int32_t* __restrict__ first_j, int32_t* __restrict__ count,
                                                       int64_t* __restrict__ base) {
     __shared__ int64_t part[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -305,9 +306,10 @@ __global__ void __launch_bounds__(1024) k_pair_chunks(const int32_t* __restrict_
             int64_t lo = 0, hi = NKB;   // first j with last(j) / R >= c
             while (lo < hi) {
                 const int64_t mid = (lo + hi) >> 1;
-                if (pair_last_row_block(tok_end, T, tile, mid) / R >= c) hi = mid; else lo = mid + 1;
+                if (pair_last_row_block(tok_end, T, kt, rt, mid) / R >= c) hi = mid; else lo = mid + 1;
             }
-            const int64_t last = (c + 1) * R - 1 < NKB - 1 ? (c + 1) * R - 1 : NKB - 1;
+            const int64_t end = ((c + 1) * R * rt - 1) / kt;   // the key block of the chunk's last row
+            const int64_t last = end < NKB - 1 ? end : NKB - 1;
             n = last >= lo ? last - lo + 1 : 0;
             first_j[c] = (int32_t)lo;
             count[c] = (int32_t)n;
@@ -326,7 +328,7 @@ __global__ void __launch_bounds__(1024) k_pair_chunks(const int32_t* __restrict_
     if (threadIdx.x == 0) base[NC] = run;
 }
 // Weight of pair-block (c, j): its live cells, min(last(j), c R + R - 1) - max(j, c R) + 1.
-__global__ void k_pair_fill(const int32_t* __restrict__ tok_end, int64_t T, int tile, int R, int64_t NC,
+__global__ void k_pair_fill(const int32_t* __restrict__ tok_end, int64_t T, int kt, int rt, int R, int64_t NC,
                             const int32_t* __restrict__ first_j, const int32_t* __restrict__ count,
                             const int64_t* __restrict__ base, int32_t* __restrict__ u_blk,
                             int32_t* __restrict__ u_chunk, int64_t* __restrict__ weight_blk) {
@@ -334,8 +336,8 @@ __global__ void k_pair_fill(const int32_t* __restrict__ tok_end, int64_t T, int 
     if (c >= NC) return;
     for (int x = threadIdx.x; x < count[c]; x += blockDim.x) {
         const int64_t j = first_j[c] + x, u = base[c] + x;
-        const int64_t last = pair_last_row_block(tok_end, T, tile, j);
-        const int64_t i0 = j > c * R ? j : c * R, i1 = last < c * R + R - 1 ? last : c * R + R - 1;
+        const int64_t last = pair_last_row_block(tok_end, T, kt, rt, j), first = j * kt / rt;
+        const int64_t i0 = first > c * R ? first : c * R, i1 = last < c * R + R - 1 ? last : c * R + R - 1;
         u_blk[u] = (int32_t)j;
         u_chunk[u] = (int32_t)c;
         weight_blk[u] = i1 - i0 + 1;
@@ -379,8 +381,8 @@ struct Carver {
 // Arrays that start out as zeros (`zeros`), then the rest.
 static void carve_dir(PlanDir& d, Carver& c, bool zeros, bool pairs) {
     if (zeros) {
-        c.take(&d.d_busy, 2 * d.W);
-        c.take(&d.d_busy2, 2 * d.W);
+        c.take(&d.d_busy, 2 * (d.W + 1));    // kernels on pairs of CTAs round the workers up to even
+        c.take(&d.d_busy2, 2 * (d.W + 1));
         c.take(&d.d_tile_ns, d.NT);
         return;
     }
@@ -424,56 +426,66 @@ static DirView view_of(const PlanDir& d, int key_major, const libra_plan_opts& o
 // The pair-blocks of a plan: counts per query chunk, their prefix sums, and the total read back (one synchronous
 // 8-byte copy).  The query chunk is doubled while there are more than 262144 pair-blocks.
 struct PairTables { int32_t* first_j = nullptr; int32_t* count = nullptr; int64_t* base = nullptr; int64_t NC = 0; };
-static int64_t pair_chunks_of(int64_t T, const PlanDir& d) {
-    const int64_t NKB = (T + d.tile - 1) / d.tile, R = d.chunk / d.tile;
-    return (NKB + R - 1) / R;
+static int64_t pair_chunks_of(int64_t T, const PlanDir& d, int rt) {
+    const int64_t NRB = (T + rt - 1) / rt, R = d.chunk / rt;
+    return (NRB + R - 1) / R;
 }
-static int count_pair_blocks(libra_plan* p, PlanDir& d, PairTables& tb) {
-    const int64_t T = p->T, NKB = (T + d.tile - 1) / d.tile;
+// d: the pair tiles, row blocks of d.tile tokens; wide: the same with wider key blocks, or null.
+static int count_pair_blocks(libra_plan* p, PlanDir& d, PairTables& tb, PlanDir* wide, PairTables& tbw) {
+    const int64_t T = p->T;
     for (;;) {
-        tb.NC = pair_chunks_of(T, d);   // never more than the tables were carved for
-        k_pair_chunks<<<1, 1024, 0, p->stream>>>(p->d_tok_end, T, d.tile, d.chunk / d.tile, NKB, tb.NC, tb.first_j, tb.count,
-                                                tb.base);
-        count_launch();
-        int64_t nu = 0;
-        if (cudaMemcpyAsync(&nu, tb.base + tb.NC, sizeof(int64_t), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess ||
-            cudaStreamSynchronize(p->stream) != cudaSuccess)
-            return LIBRA_ERR_CUDA;
-        d.NB = nu;
-        if (nu <= 262144) return LIBRA_OK;
+        int64_t nu[2] = {0, 0};
+        for (int k = 0; k < (wide ? 2 : 1); ++k) {
+            PlanDir& x = k == 0 ? d : *wide;
+            PairTables& t = k == 0 ? tb : tbw;
+            t.NC = pair_chunks_of(T, d, d.tile);   // never more than the tables were carved for
+            k_pair_chunks<<<1, 1024, 0, p->stream>>>(p->d_tok_end, T, x.tile, d.tile, d.chunk / d.tile, (T + x.tile - 1) / x.tile, t.NC,
+                                                    t.first_j, t.count, t.base);
+            count_launch();
+            if (cudaMemcpyAsync(&nu[k], t.base + t.NC, sizeof(int64_t), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess)
+                return LIBRA_ERR_CUDA;
+        }
+        if (cudaStreamSynchronize(p->stream) != cudaSuccess) return LIBRA_ERR_CUDA;
+        d.NB = nu[0];
+        if (wide) { wide->NB = nu[1]; wide->chunk = d.chunk; }
+        if (d.NB <= 262144) return LIBRA_OK;
         if ((int64_t)d.chunk * 2 > (int64_t)1 << 30) return LIBRA_ERR_UNSUPPORTED;
         d.chunk *= 2;
     }
 }
 
 // Builds the directions asked for; p->dir[k].tile / H / W / chunk are set.
-static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o, const bool (&want)[3]) {
+static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o, const bool (&want)[4]) {
     const int64_t T = p->T;
     cudaStream_t s = p->stream;
-    for (int k = 0; k < 2; ++k) {
-        if (!want[k]) continue;
+    const bool wide_pairs = want[3] && want[2];                   // the wide tiles are pair tiles
+    const bool sorted[4] = {want[0], want[1], false, want[3] && !want[2]};   // sizes known, placed heaviest first
+    for (int k = 0; k < 4; ++k) {
+        if (!sorted[k]) continue;
         p->dir[k].NB = (T + p->dir[k].tile - 1) / p->dir[k].tile;
         if (const int rc = check_dir(p, p->dir[k], false); rc != LIBRA_OK) return rc;
     }
-    PairTables tb;
+    PairTables tb, tbw;
     if (want[2] && p->dir[2].chunk % p->dir[2].tile) return LIBRA_ERR_INVALID_ARG;
     // ---- token bounds, the directions whose sizes are known, the pair tables; zeros first
     size_t zero_bytes = 0;
     auto carve = [&](Carver& c) {
         c.take(&p->d_status, 1);
-        for (int k = 0; k < 4; ++k) c.take(&p->d_outcome[k], p->W);
-        for (int k = 0; k < 2; ++k)
-            if (want[k]) carve_dir(p->dir[k], c, true, false);
+        for (int k = 0; k < 4; ++k) c.take(&p->d_outcome[k], p->W + 1);
+        for (int k = 0; k < 4; ++k)
+            if (sorted[k]) carve_dir(p->dir[k], c, true, false);
         zero_bytes = c.used;
         c.take(&p->d_tok_start, T);
         c.take(&p->d_tok_end, T);
-        for (int k = 0; k < 2; ++k)
-            if (want[k]) carve_dir(p->dir[k], c, false, false);
+        for (int k = 0; k < 4; ++k)
+            if (sorted[k]) carve_dir(p->dir[k], c, false, false);
         if (want[2]) {
-            const int64_t NC = pair_chunks_of(T, p->dir[2]);
-            c.take(&tb.first_j, NC);
-            c.take(&tb.count, NC);
-            c.take(&tb.base, NC + 1);
+            const int64_t NC = pair_chunks_of(T, p->dir[2], p->dir[2].tile);
+            for (PairTables* t : {&tb, &tbw}) {
+                c.take(&t->first_j, NC);
+                c.take(&t->count, NC);
+                c.take(&t->base, NC + 1);
+            }
         }
     };
     Carver sizes, mem;
@@ -486,28 +498,36 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
     count_launch();
     // ---- pair tiles: their number comes back, then their arrays
     if (want[2]) {
-        PlanDir& d = p->dir[2];
-        if (const int rc = count_pair_blocks(p, d, tb); rc != LIBRA_OK) return rc;
-        if (const int rc = check_dir(p, d, true); rc != LIBRA_OK) return rc;
+        if (const int rc = count_pair_blocks(p, p->dir[2], tb, wide_pairs ? &p->dir[3] : nullptr, tbw); rc != LIBRA_OK) return rc;
         Carver ps, pm;
-        carve_dir(d, ps, true, true);
-        const size_t pair_zero = ps.used;
-        carve_dir(d, ps, false, true);
+        size_t pair_zero = 0;
+        for (int k = 2; k < (wide_pairs ? 4 : 3); ++k)
+            if (const int rc = check_dir(p, p->dir[k], true); rc != LIBRA_OK) return rc;
+        auto carve_pairs = [&](Carver& c) {
+            for (int k = 2; k < (wide_pairs ? 4 : 3); ++k) carve_dir(p->dir[k], c, true, true);
+            pair_zero = c.used;
+            for (int k = 2; k < (wide_pairs ? 4 : 3); ++k) carve_dir(p->dir[k], c, false, true);
+        };
+        carve_pairs(ps);
         if (const int rc = plan_block(p, ps.used, &pm.at); rc != LIBRA_OK) return rc;
-        carve_dir(d, pm, true, true);
-        carve_dir(d, pm, false, true);
+        carve_pairs(pm);
         cudaMemsetAsync(pm.at, 0, pair_zero, s);
-        k_pair_fill<<<(unsigned)tb.NC, 128, 0, s>>>(p->d_tok_end, T, d.tile, d.chunk / d.tile, tb.NC, tb.first_j, tb.count,
-                                                    tb.base, d.d_u_blk, d.d_u_chunk, d.d_weight_blk);
-        count_launch();
+        for (int k = 2; k < (wide_pairs ? 4 : 3); ++k) {
+            PlanDir& d = p->dir[k];
+            const PairTables& t = k == 2 ? tb : tbw;
+            const int rt = p->dir[2].tile;
+            k_pair_fill<<<(unsigned)t.NC, 128, 0, s>>>(p->d_tok_end, T, d.tile, rt, d.chunk / rt, t.NC, t.first_j, t.count, t.base,
+                                                       d.d_u_blk, d.d_u_chunk, d.d_weight_blk);
+            count_launch();
+        }
     }
     // ---- weights, order, placement and lists of all directions together
     DirViews views = {};
     int n = 0, max_w = 0;
     int64_t max_nb = 0, max_nt = 0;
-    for (int k = 0; k < 2; ++k)
-        if (want[k]) {
-            views.v[n++] = view_of(p->dir[k], k == 1, o);
+    for (int k = 0; k < 4; ++k)
+        if (sorted[k]) {
+            views.v[n++] = view_of(p->dir[k], k != 0, o);
             max_nb = p->dir[k].NB > max_nb ? p->dir[k].NB : max_nb;
         }
     if (n > 0) {
@@ -516,9 +536,10 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
         count_launch(2);
     }
     const int n_sorted = n;
-    if (want[2]) views.v[n++] = view_of(p->dir[2], 1, o);
+    for (int k = 2; k < 4; ++k)
+        if (want[k] && !sorted[k]) views.v[n++] = view_of(p->dir[k], 1, o);
     if (n == 0) return LIBRA_OK;
-    for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < 4; ++k)
         if (want[k]) {
             max_nt = p->dir[k].NT > max_nt ? p->dir[k].NT : max_nt;
             max_w = p->dir[k].W > max_w ? p->dir[k].W : max_w;
@@ -530,7 +551,7 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
         k_exec_order<<<dim3(max_w, n_sorted), 256, 0, s>>>(views);
         count_launch();
     }
-    for (int k = 0; k < 3; ++k) p->dir[k].enabled = want[k] ? 1 : 0;
+    for (int k = 0; k < 4; ++k) p->dir[k].enabled = want[k] ? 1 : 0;
     return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
 
@@ -571,12 +592,15 @@ extern "C" int libra_plan_tiles(const int32_t* cu_seqlens_dev, int n_samples, in
     if (s) p->other_stream = 1;
     p->W = o.n_workers ? o.n_workers : sms;
     const int dirs = o.directions ? o.directions : (LIBRA_DIR_Q | LIBRA_DIR_KV);
-    const bool want[3] = {(dirs & LIBRA_DIR_Q) != 0, (dirs & LIBRA_DIR_KV) != 0, (dirs & LIBRA_DIR_PAIR) != 0};
-    for (int k = 0; k < 3; ++k) {
+    const int tile_kv = o.tile_kv ? o.tile_kv : 128;
+    const bool keys = (dirs & (LIBRA_DIR_KV | LIBRA_DIR_PAIR)) != 0;
+    const bool want[4] = {(dirs & LIBRA_DIR_Q) != 0, (dirs & LIBRA_DIR_KV) != 0, (dirs & LIBRA_DIR_PAIR) != 0,
+                          keys && tile_kv == 128};
+    for (int k = 0; k < 4; ++k) {
         PlanDir& d = p->dir[k];
-        d.tile = k == 0 ? tile_q : (o.tile_kv ? o.tile_kv : 128);
+        d.tile = k == 0 ? tile_q : (k == 3 ? 256 : tile_kv);
         d.H = k == 0 ? n_heads : (o.n_heads_kv ? o.n_heads_kv : n_heads);
-        d.W = p->W;
+        d.W = k == 3 ? (p->W + 1) / 2 : p->W;
         d.chunk = k == 2 ? (o.pair_chunk ? o.pair_chunk : 4096) : 0;
     }
     const int rc = build_plan(p, cu_seqlens_dev, o, want);

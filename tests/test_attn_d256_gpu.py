@@ -96,6 +96,13 @@ def test_head_shards_wider_than_one_head():
     _check(*_run([900, 256 * 2 + 100], 4, 2, seed=6, H=2, W=5))
 
 
+@pytest.mark.parametrize("pairs", [False, True])
+@pytest.mark.parametrize("T,W", [(1, 1), (127, 2), (128, 3), (129, 1), (255, 2), (257, 3), (384, 1), (641, 5)])
+def test_pairs_of_ctas(T, W, pairs):
+    """256 stationary rows on two CTAs: the second one's rows end at, before or inside the tile; odd numbers of workers."""
+    _check(*_run([T], 2, 1, seed=T, W=W, pairs=pairs, chunk=128))
+
+
 def test_peaked_softmax():
     _check(*_run([700, 900], 2, 2, seed=7, qscale=3.0))
 
