@@ -16,18 +16,21 @@
 // Two CTAs work on 256 stationary rows (128 each) with cta_group::2 MMAs, so that each loads only half of every streamed
 // tile: with 128 rows per CTA a pass read 64 KB from L2 for 128 x 64 x 512 MACs per GEMM pair, 5 to 7 TB/s, and each of its
 // N = 64 MMAs took 48 cycles for the 32 of its products (forward / dV + dK / dQ of one 32768-token sample at Hq 128, Hkv 4:
-// 21.3 / 52.8 / 22.7 ms, now 16.0 / 39.0 / 22.4).  Of a streamed tile that is the B operand of an X GEMM (N = its 64 rows) a CTA holds 32 rows;
+// 21.5 / 54.1 / 22.7 ms, now 15.3 / 33.9 / 20.9; the clock is at 1.35 GHz then, the power limit's).  Of a streamed tile that is the B operand of an X GEMM (N = its 64 rows) a CTA holds 32 rows;
 // of one that the accumulating GEMM multiplies with (N = 256 head-dim columns) it holds 128 columns; the tile that is
 // both (Q in DK, K in DQ) is loaded in both halves.  The leader (even rank) issues all MMAs; its barriers count the
 // copies and the compute warps of both CTAs; commits arrive in both.
 //
-// TMEM: X1 (2 x 64, double-buffered) | X2 (64) | W (32: the bf16 result of the element-wise step, A operand of the
-// last GEMM) | acc (256).
+// TMEM: X1, X2, W (32 columns a block: the bf16 result of the element-wise step, A operand of the last GEMM) in 256
+// columns, acc (256).  FWD, DV: X1 3 x 64 | W 2 x 32; X1 runs two blocks ahead.  DK, DQ: X1 2 x 64 | X2 2 x 64, one block
+// ahead; W lies over the first half of each thread group's columns of X1, which that group has read by then.
 // Roles (320 threads): warps 0-7 compute, warp 8 one TMA thread, warp 9 one MMA thread.  In the gradient passes two
 // threads share a stationary row (32 of the block's 64 columns each; warps w and w + 4 reach the same TMEM lanes); the
 // forward keeps one thread per row, because the running maximum and sum of a row live in its registers (warps 4-7
 // idle there).  Per streamed block: X1 (and X2) are issued, the compute warps turn them into W, the accumulating GEMM
-// is issued; X1 of the next block is issued ahead, so it runs under the element-wise step of the current one.
+// is issued; X1 and X2 of the next block are issued ahead, so they run under the element-wise step of the current one
+// (a dV / dK / dQ block: 1650 / 2330 / 2400 cycles with only X1 ahead and one W, 1220 / 1920 / 2020 now; of MMAs 1024 /
+// 1536 / 1536).
 // Masks follow the sample bounds per element, in blocks that a bound crosses.
 #include <math.h>
 
@@ -42,7 +45,7 @@ constexpr int kTmaWarp = 8, kMmaWarp = 9;
 constexpr int kRows = 128;       // stationary rows per unit
 constexpr int kBlk = 64;         // streamed rows per block
 constexpr int kD = 256;
-constexpr uint32_t kColX1 = 0 /* and 64 */, kColX2 = 128, kColW = 192, kColAcc = 256;
+constexpr uint32_t kColAcc = 256;
 constexpr uint64_t kDrainNs = 2000000;
 constexpr int kSmemMax = 232448;
 enum Mode { FWD = 0, DV = 1, DK = 2, DQ = 3 };
@@ -66,12 +69,20 @@ struct Cfg {
     static constexpr int kRingOff = kStationary * kBig;
     static constexpr int kStatOff = kRingOff + kStreams * kStages * kHalfTile;
     static constexpr int kBarOff = kStatOff + kStages * 512;
-    // full, empty [kStreams][kStages], stat[kStages], st_full, st_empty, x1_full[2], x2_full, w_ready, acc_done, acc_free,
-    // drain, acc_step
-    static constexpr int kNumBars = 2 * kStreams * kStages + kStages + 10;
+    // full, empty [kStreams][kStages], stat[kStages], st_full, st_empty, acc_done, acc_free, drain, x1_full[3], x2_full[2],
+    // w_ready[2], acc_step[2]
+    static constexpr int kNumBars = 2 * kStreams * kStages + kStages + 15;
     static constexpr int kMiscOff = kBarOff + kNumBars * 8;
     static constexpr int kBytes = kMiscOff + 16;
     static_assert(kBytes <= kSmemMax, "exceeds the shared memory of an sm_100 CTA");
+    // TMEM columns of a block's X1, X2 and W (see above)
+    static constexpr uint32_t kX1Bufs = kHasX2 ? 2 : 3;
+    __device__ static constexpr uint32_t col_x1(uint32_t b) { return 64 * b; }
+    __device__ static constexpr uint32_t col_x2(uint32_t b) { return 128 + 64 * b; }
+    // W columns of the block's streamed rows 16 kk .. 16 kk + 15; b is the block's parity
+    __device__ static constexpr uint32_t col_w(uint32_t b, uint32_t kk) {
+        return kHasX2 ? col_x1(b) + (kk >> 1) * 32 + (kk & 1) * 8 : 192 + 32 * b + 8 * kk;
+    }
     __host__ __device__ static constexpr int tile_off(int stream, uint32_t stage) {
         return kRingOff + (stream * kStages + (int)stage) * kHalfTile;
     }
@@ -160,9 +171,8 @@ struct Units {
         }
         return true;
     }
-    // head and first row of the streamed block of iteration it
-    __device__ int stream_head(int it) const { return Cfg<MODE>::kKeyStationary ? h + it / n_blk : kvh; }
-    __device__ int stream_row(int it) const { return (b_lo + (Cfg<MODE>::kKeyStationary ? it % n_blk : it)) * kBlk; }
+    // First row of the streamed block j of a head; the iterations of a unit take its heads in turn, blocks ascending.
+    __device__ int stream_row(int j) const { return (b_lo + j) * kBlk; }
 };
 
 template <int MODE>
@@ -180,13 +190,14 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
     uint64_t* b2 = bar_stat + S;
     uint64_t* bar_stfull = b2 + 0;             // leader
     uint64_t* bar_stempty = b2 + 1;
-    uint64_t* bar_x2full = b2 + 2;
-    uint64_t* bar_wready = b2 + 3;             // leader: W is in both CTAs' TMEM
-    uint64_t* bar_accdone = b2 + 4;
-    uint64_t* bar_accfree = b2 + 5;            // leader
-    uint64_t* bar_drain = b2 + 6;
-    uint64_t* bar_accstep = b2 + 7;    // the accumulating GEMM of an iteration has run: W may be rewritten, acc rescaled
-    uint64_t* bar_x1full = b2 + 8;     // [2] one per X1 buffer: X1 of the next block is committed a block ahead
+    uint64_t* bar_accdone = b2 + 2;
+    uint64_t* bar_accfree = b2 + 3;            // leader
+    uint64_t* bar_drain = b2 + 4;
+    uint64_t* bar_x1full = b2 + 5;     // [3] one per X1 buffer, [2] per X2 buffer: committed one or two blocks ahead
+    uint64_t* bar_x2full = b2 + 8;
+    // by the block's parity (the compute warps may be a block ahead of the issuer, the issuer of the accumulating GEMM):
+    uint64_t* bar_wready = b2 + 10;    // [2] leader: W is in both CTAs' TMEM
+    uint64_t* bar_accstep = b2 + 12;   // [2] the accumulating GEMM has run: W may be rewritten, acc rescaled
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kMiscOff);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMiscOff + 4);
 
@@ -214,14 +225,15 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
         for (int s = 0; s < S; ++s) mbar_init(&bar_stat[s], 1);
         mbar_init(bar_stfull, 1);
         mbar_init(bar_stempty, 1);
-        mbar_init(&bar_x1full[0], 1);
-        mbar_init(&bar_x1full[1], 1);
-        mbar_init(bar_x2full, 1);
-        mbar_init(bar_wready, 2 * 4 * L::kGroups);    // a compute warp's lanes arrive as one
+        for (int b = 0; b < 3; ++b) mbar_init(&bar_x1full[b], 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&bar_x2full[b], 1);
+            mbar_init(&bar_wready[b], 2 * 4 * L::kGroups);    // a compute warp's lanes arrive as one
+            mbar_init(&bar_accstep[b], 1);
+        }
         mbar_init(bar_accdone, 1);
         mbar_init(bar_accfree, 2 * 4 * L::kGroups);
         mbar_init(bar_drain, 1);
-        mbar_init(bar_accstep, 1);
         abort_flag[0] = 0;
         abort_flag[1] = (int)p.wait_limit_ns;
         fence_mbar_init();
@@ -262,8 +274,9 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                         tma_load_3d_pair(smem + L::kSbOff + half * L::kBigHalf, &tm_sb, stfull0, half * 64, st_head, (int)u.r0);
                 }
                 ++uc;
+                int sh = L::kKeyStationary ? u.h : u.kvh, j = 0;
                 for (int it = 0; it < u.n_it && ok; ++it, ++n) {
-                    const int sh = u.stream_head(it), row = u.stream_row(it);
+                    const int row = u.stream_row(j);
                     const uint32_t s = n % S, ph = (n / S) & 1;
                     for (int k = 0; k < N && ok; ++k) {
                         ok = mbar_wait(&bar_empty[k * S + s], ph ^ 1, abort_flag);
@@ -285,6 +298,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                                 bulk_load_1d(smem + L::kStatOff + s * 512 + 256, p.dvec + (size_t)sh * p.Tpad + row, 256, &bar_stat[s]);
                         }
                     }
+                    if (++j == u.n_blk) { j = 0; ++sh; }
                 }
             }
             if (!ok || abort_flag[0]) {   // give-up path: the copies already issued land before shared memory is released
@@ -310,35 +324,40 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
             };
             Units<MODE> u(p, cta);
             uint32_t uc = 0, itc = 0;
+            uint32_t xi = 0, xb = 0;   // next block to multiply, its X1 buffer
             bool ok = true;
-            // X1 of iteration i into its buffer; its streamed half is free again as soon as it has run
-            auto do_x1 = [&](uint32_t i) -> bool {
-                if (!mbar_wait(&bar_full[i % S], (i / S) & 1, abort_flag)) return false;
+            // X1 (and X2) of the next block; its streamed halves are free again as soon as they have run
+            auto do_x = [&]() -> bool {
+                const uint32_t s = xi % S, ph = (xi / S) & 1;
+                if (!mbar_wait(&bar_full[s], ph, abort_flag)) return false;
                 tc_fence_after();
-                issue_x(kColX1 + (i & 1) * 64, L::kSaOff, L::tile_off(0, i % S));
-                tc_commit_pair(&bar_x1full[i & 1]);
-                tc_commit_pair(&bar_empty[i % S]);
+                issue_x(L::col_x1(xb), L::kSaOff, L::tile_off(0, s));
+                tc_commit_pair(&bar_x1full[xb]);
+                tc_commit_pair(&bar_empty[s]);
+                if (L::kHasX2) {
+                    if (!mbar_wait(&bar_full[S + s], ph, abort_flag)) return false;
+                    tc_fence_after();
+                    issue_x(L::col_x2(xb), L::kSbOff, L::tile_off(1, s));
+                    tc_commit_pair(&bar_x2full[xb]);
+                    tc_commit_pair(&bar_empty[S + s]);
+                }
+                ++xi;
+                if (++xb == L::kX1Bufs) xb = 0;
                 return true;
             };
+            constexpr int kAhead = (int)L::kX1Bufs - 1;
             while (ok && u.next(rank)) {
                 ok = mbar_wait(bar_stfull, uc & 1, abort_flag);
-                if (ok) ok = do_x1(itc);
+                for (int it = 0; it < kAhead && it < u.n_it && ok; ++it) ok = do_x();
                 if (!ok) break;
                 for (int it = 0; it < u.n_it && ok; ++it, ++itc) {
-                    const uint32_t s = itc % S, ph = (itc / S) & 1;
-                    if (L::kHasX2) {
-                        ok = mbar_wait(&bar_full[S + s], ph, abort_flag);
-                        if (!ok) break;
-                        tc_fence_after();
-                        issue_x(kColX2, L::kSbOff, L::tile_off(1, s));
-                        tc_commit_pair(bar_x2full);
-                        tc_commit_pair(&bar_empty[S + s]);
-                    }
-                    // X1 of the next block into the other buffer (read out two iterations ago): it runs while the
-                    // compute warps work on this block
-                    if (it + 1 < u.n_it) ok = do_x1(itc + 1);
+                    const uint32_t s = itc % S, ph = (itc / S) & 1, b = itc & 1;
+                    // The X GEMMs of a block ahead run under the element-wise step of this one.  Their buffers were read out
+                    // before W of the previous block was ready, and its accumulating GEMM, which may read W there, is ahead
+                    // of them in the pipe.
+                    if (it + kAhead < u.n_it) ok = do_x();
                     if (ok) ok = mbar_wait(&bar_full[L::kAcc * S + s], ph, abort_flag);
-                    if (ok) ok = mbar_wait(bar_wready, itc & 1, abort_flag);
+                    if (ok) ok = mbar_wait(&bar_wready[b], (itc >> 1) & 1, abort_flag);
                     if (ok && it == 0 && uc > 0) ok = mbar_wait(bar_accfree, (uc - 1) & 1, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
@@ -346,10 +365,10 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                         const uint64_t db = sdesc_advance(mdesc0, L::tile_off(L::kAcc, s));
 #pragma unroll
                         for (int kk = 0; kk < kBlk / 16; ++kk)
-                            mma_ts_pair(tmem_base + kColAcc, tmem_base + kColW + kk * 8, sdesc_advance(db, kk * 2048), idesc_acc,
+                            mma_ts_pair(tmem_base + kColAcc, tmem_base + L::col_w(b, kk), sdesc_advance(db, kk * 2048), idesc_acc,
                                         (it > 0 || kk > 0) ? 1u : 0u);
                     }
-                    tc_commit_pair(bar_accstep);
+                    tc_commit_pair(&bar_accstep[b]);
                     tc_commit_pair(&bar_empty[L::kAcc * S + s]);
                     if (it == u.n_it - 1) { tc_commit_pair(bar_accdone); tc_commit_pair(bar_stempty); }
                 }
@@ -369,13 +388,12 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
         const int col0 = grp * NC;
         const int r = (warp & 3) * 32 + lane;
         const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t t_x1 = tmem_base + lane_addr + kColX1 + col0;
-        const uint32_t t_x2 = tmem_base + lane_addr + kColX2 + col0;
-        const uint32_t t_w = tmem_base + lane_addr + kColW + col0 / 2;
-        const uint32_t t_acc = tmem_base + lane_addr + kColAcc + grp * (kD / L::kGroups);
+        const uint32_t t_base = tmem_base + lane_addr;
+        const uint32_t t_acc = t_base + kColAcc + grp * (kD / L::kGroups);
         const uint32_t wready0 = map_to_rank(bar_wready, 0), accfree0 = map_to_rank(bar_accfree, 0);
         Units<MODE> u(p, cta);
         uint32_t uc = 0, itc = 0;
+        uint32_t xb = 0, xph = 0;                    // X1 buffer of the block and its phase
         bool ok = true;
         while (ok && u.next(rank)) {
             const int64_t row = u.r0 + r;            // this thread's query row (FWD, DQ) or key (DV, DK)
@@ -383,14 +401,16 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
             // visible columns of streamed block starting at b0: [lo_abs - b0, hi_abs - b0]
             //   query-stationary: keys from the start of the row's sample to the row itself
             //   key-stationary:   queries from the key itself to the end of its sample
-            int64_t lo_abs, hi_abs;
+            int lo_abs, hi_abs;
             if (L::kKeyStationary) {
-                lo_abs = row;
-                hi_abs = row_ok ? (int64_t)p.tok_end[row] - 1 : -1;
+                lo_abs = (int)row;
+                hi_abs = row_ok ? p.tok_end[row] - 1 : -1;
             } else {
-                lo_abs = row_ok ? (int64_t)p.tok_start[row] : 0;
-                hi_abs = row_ok ? row : -1;
+                lo_abs = row_ok ? p.tok_start[row] : 0;
+                hi_abs = row_ok ? (int)row : -1;
             }
+            lo_abs -= col0;                          // counted from this thread's first column
+            hi_abs -= col0;
             float m_ref = -INFINITY, l_sum = 0.f;    // FWD
             float lse2r = 0.f, dvecr = 0.f;          // DQ
             if (MODE == DQ) {
@@ -399,11 +419,13 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                     dvecr = p.dvec[(size_t)u.h * p.Tpad + row];
                 }
             }
+            int j = 0;
             for (int it = 0; it < u.n_it && ok; ++it, ++itc) {
-                const int64_t b0 = u.stream_row(it);
-                // first and last visible column, counted from this thread's first column
-                const int c_lo = (int)(lo_abs - b0 > kBlk ? kBlk : lo_abs - b0) - col0;
-                const int c_hi = (int)(hi_abs - b0 < -1 ? -1 : hi_abs - b0) - col0;
+                const int b0 = u.stream_row(j);
+                if (++j == u.n_blk) j = 0;
+                // first and last visible of this thread's columns
+                const int c_lo = lo_abs - b0, c_hi = hi_abs - b0;
+                const uint32_t wb = itc & 1;
                 const bool need_mask = __any_sync(0xffffffffu, c_lo > 0 || c_hi < NC - 1);   // most blocks are dense
                 const uint32_t s1 = itc % S;
                 const float* st = reinterpret_cast<const float*>(smem + L::kStatOff + s1 * 512) + col0;
@@ -411,13 +433,14 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                     ok = warp_wait(&bar_stat[s1], (itc / S) & 1, abort_flag);
                     if (!ok) break;
                 }
-                ok = warp_wait(&bar_x1full[itc & 1], (itc >> 1) & 1, abort_flag);
+                ok = warp_wait(&bar_x1full[xb], xph, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
                 uint32_t sr[NC];
 #pragma unroll
-                for (int c = 0; c < NC; c += 32) tmem_ld32(t_x1 + (itc & 1) * 64 + c, sr + c);
+                for (int c = 0; c < NC; c += 32) tmem_ld32(t_base + L::col_x1(xb) + col0 + c, sr + c);
                 tmem_ld_wait();
+                if (++xb == L::kX1Bufs) { xb = 0; xph ^= 1; }
                 uint32_t pk[NC / 2];
                 if constexpr (MODE == FWD) {
                     if (need_mask) {
@@ -460,8 +483,8 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                         pk[i >> 1] = pack_bf16x2(p0, p1);
                     }
                     if (it > 0 && __any_sync(0xffffffffu, grow)) {
-                        // O is rescaled once the previous block's accumulation has landed (its W is spent then, too)
-                        ok = warp_wait(bar_accstep, (itc - 1) & 1, abort_flag);
+                        // O is rescaled once the previous block's accumulation has landed
+                        ok = warp_wait(&bar_accstep[wb ^ 1], ((itc - 1) >> 1) & 1, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
 #pragma unroll
@@ -506,12 +529,12 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
 #pragma unroll
                         for (int i = 0; i < NC; i += 2) pk[i >> 1] = pack_bf16x2(pf[i], pf[i + 1]);
                     } else {
-                        ok = warp_wait(bar_x2full, itc & 1, abort_flag);
+                        ok = warp_wait(&bar_x2full[wb], (itc >> 1) & 1, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
                         uint32_t dp[NC];
 #pragma unroll
-                        for (int c = 0; c < NC; c += 32) tmem_ld32(t_x2 + c, dp + c);
+                        for (int c = 0; c < NC; c += 32) tmem_ld32(t_base + L::col_x2(wb) + col0 + c, dp + c);
                         tmem_ld_wait();
                         const uint64_t nd2 = f2_pack(-dvecr, -dvecr);
 #pragma unroll
@@ -535,17 +558,17 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                 // (the results exist before the wait: left to itself the compiler moves the exponentials behind it)
 #pragma unroll
                 for (int i = 0; i < NC / 2; ++i) asm volatile("" : "+r"(pk[i]));
-                if (itc > 0) {   // the previous accumulating GEMM has consumed W
-                    ok = warp_wait(bar_accstep, (itc - 1) & 1, abort_flag);
+                if (!L::kHasX2 && itc > 1) {   // the accumulating GEMM of two blocks ago has consumed W
+                    ok = warp_wait(&bar_accstep[wb], ((itc >> 1) - 1) & 1, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                 }
 #pragma unroll
-                for (int c = 0; c < NC / 2; c += 16) tmem_st16(t_w + c, pk + c);
+                for (int c = 0; c < NC / 2; c += 16) tmem_st16(t_base + L::col_w(wb, (uint32_t)(col0 + 2 * c) / 16), pk + c);
                 tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(wready0);
+                if (lane == 0) mbar_arrive_cluster(wready0 + 8 * wb);
             }
             if (!ok) break;
             // ---- unit epilogue: the accumulator leaves TMEM ----

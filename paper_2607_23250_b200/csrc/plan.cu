@@ -438,8 +438,8 @@ static int count_pair_blocks(libra_plan* p, PlanDir& d, PairTables& tb, PlanDir*
         for (int k = 0; k < (wide ? 2 : 1); ++k) {
             PlanDir& x = k == 0 ? d : *wide;
             PairTables& t = k == 0 ? tb : tbw;
-            t.NC = pair_chunks_of(T, d, d.tile);   // never more than the tables were carved for
-            k_pair_chunks<<<1, 1024, 0, p->stream>>>(p->d_tok_end, T, x.tile, d.tile, d.chunk / d.tile, (T + x.tile - 1) / x.tile, t.NC,
+            t.NC = pair_chunks_of(T, x, d.tile);   // never more than the tables were carved for
+            k_pair_chunks<<<1, 1024, 0, p->stream>>>(p->d_tok_end, T, x.tile, d.tile, x.chunk / d.tile, (T + x.tile - 1) / x.tile, t.NC,
                                                     t.first_j, t.count, t.base);
             count_launch();
             if (cudaMemcpyAsync(&nu[k], t.base + t.NC, sizeof(int64_t), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess)
@@ -447,10 +447,11 @@ static int count_pair_blocks(libra_plan* p, PlanDir& d, PairTables& tb, PlanDir*
         }
         if (cudaStreamSynchronize(p->stream) != cudaSuccess) return LIBRA_ERR_CUDA;
         d.NB = nu[0];
-        if (wide) { wide->NB = nu[1]; wide->chunk = d.chunk; }
-        if (d.NB <= 262144) return LIBRA_OK;
+        if (wide) wide->NB = nu[1];
+        if (nu[0] <= 262144 && nu[1] <= 262144) return LIBRA_OK;
         if ((int64_t)d.chunk * 2 > (int64_t)1 << 30) return LIBRA_ERR_UNSUPPORTED;
-        d.chunk *= 2;
+        if (nu[0] > 262144) d.chunk *= 2;
+        if (nu[1] > 262144) wide->chunk *= 2;
     }
 }
 
@@ -480,11 +481,12 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
         for (int k = 0; k < 4; ++k)
             if (sorted[k]) carve_dir(p->dir[k], c, false, false);
         if (want[2]) {
-            const int64_t NC = pair_chunks_of(T, p->dir[2], p->dir[2].tile);
-            for (PairTables* t : {&tb, &tbw}) {
-                c.take(&t->first_j, NC);
-                c.take(&t->count, NC);
-                c.take(&t->base, NC + 1);
+            for (int k = 2; k < (wide_pairs ? 4 : 3); ++k) {
+                const int64_t NC = pair_chunks_of(T, p->dir[k], p->dir[2].tile);
+                PairTables& t = k == 2 ? tb : tbw;
+                c.take(&t.first_j, NC);
+                c.take(&t.count, NC);
+                c.take(&t.base, NC + 1);
             }
         }
     };
@@ -601,7 +603,17 @@ extern "C" int libra_plan_tiles(const int32_t* cu_seqlens_dev, int n_samples, in
         d.tile = k == 0 ? tile_q : (k == 3 ? 256 : tile_kv);
         d.H = k == 0 ? n_heads : (o.n_heads_kv ? o.n_heads_kv : n_heads);
         d.W = k == 3 ? (p->W + 1) / 2 : p->W;
-        d.chunk = k == 2 ? (o.pair_chunk ? o.pair_chunk : 4096) : 0;
+        d.chunk = k >= 2 ? (o.pair_chunk ? o.pair_chunk : 4096) : 0;
+        if (k == 3) {
+            // The 256-wide kernels go through a tile's heads one after the other and their workers are out of step, so what
+            // the workers of a query chunk read lies anywhere in its Q and dO of a kv head's group: 1 KB a row and head,
+            // 134 MB at 4096 rows of 32 heads, more than L2 holds.  16384 rows x heads keep it at 16 MB and cut a short pool
+            // into enough tiles (dV + dK of 32768 / 16384 / 3000 tokens, 32 query heads per kv head: 37.0 / 8.86 / 0.88 ms with
+            // 4096 rows a chunk, 33.9 / 7.60 / 0.29 ms with 512); 256 rows a chunk gained nothing more on the long ones.
+            const int64_t rows = (int64_t)16384 * d.H / n_heads / 128 * 128;
+            const int64_t least = rows < 128 ? 128 : rows;
+            if (d.chunk > least) d.chunk = (int)least;
+        }
     }
     const int rc = build_plan(p, cu_seqlens_dev, o, want);
     if (rc != LIBRA_OK) {
