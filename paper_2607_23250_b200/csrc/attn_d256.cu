@@ -15,8 +15,8 @@
 //
 // Two CTAs work on 256 stationary rows (128 each) with cta_group::2 MMAs, so that each loads only half of every streamed
 // tile: with 128 rows per CTA a pass read 64 KB from L2 for 128 x 64 x 512 MACs per GEMM pair, 5 to 7 TB/s, and each of its
-// N = 64 MMAs took 48 cycles for the 32 of its products (forward / dV + dK / dQ of one 32768-token sample at Hq 128, Hkv 4:
-// 21.5 / 54.1 / 22.7 ms, now 15.3 / 33.9 / 20.9; the clock is at 1.35 GHz then, the power limit's).  Of a streamed tile that is the B operand of an X GEMM (N = its 64 rows) a CTA holds 32 rows;
+// N = 64 MMAs took 48 cycles for the 32 of its products (forward / dV + dK / dQ of one 32768-token sequence at Hq 128, Hkv 4:
+// 21.5 / 54.1 / 22.7 ms, now 14.3 / 33.9 / 20.7; the clock is at 1.35 GHz then, the power limit's).  Of a streamed tile that is the B operand of an X GEMM (N = its 64 rows) a CTA holds 32 rows;
 // of one that the accumulating GEMM multiplies with (N = 256 head-dim columns) it holds 128 columns; the tile that is
 // both (Q in DK, K in DQ) is loaded in both halves.  The leader (even rank) issues all MMAs; its barriers count the
 // copies and the compute warps of both CTAs; commits arrive in both.
@@ -26,8 +26,8 @@
 // ahead; W lies over the first half of each thread group's columns of X1, which that group has read by then.
 // Roles (320 threads): warps 0-7 compute, warp 8 one TMA thread, warp 9 one MMA thread.  In the gradient passes two
 // threads share a stationary row (32 of the block's 64 columns each; warps w and w + 4 reach the same TMEM lanes); the
-// forward keeps one thread per row, because the running maximum and sum of a row live in its registers (warps 4-7
-// idle there).  Per streamed block: X1 (and X2) are issued, the compute warps turn them into W, the accumulating GEMM
+// forward keeps one thread per row, because the running maximum and sum of a row live in its registers (warps 4-7 write
+// the output tiles there).  Per streamed block: X1 (and X2) are issued, the compute warps turn them into W, the accumulating GEMM
 // is issued; X1 and X2 of the next block are issued ahead, so they run under the element-wise step of the current one
 // (a dV / dK / dQ block: 1650 / 2330 / 2400 cycles with only X1 ahead and one W, 1220 / 1920 / 2020 now; of MMAs 1024 /
 // 1536 / 1536).
@@ -59,19 +59,24 @@ struct Cfg {
     static constexpr int kStationary = kHasX2 ? 2 : 1;       // resident 64 KB tiles per CTA
     static constexpr int kStreams = kHasX2 ? 3 : 2;          // streamed halves per block: X1's, [X2's,] the accumulating GEMM's
     static constexpr int kAcc = kStreams - 1;                // the last one
-    static constexpr int kStages = kHasX2 ? 2 : 4;           // blocks in flight
+    // FWD holds the tiles of this unit and the next: its units are a few blocks of a short sample.  A DV tile has all the
+    // heads of the group: three blocks in flight for that cost its launch 20 % (dV + dK 34.9 -> 37.7 ms).
+    static constexpr int kStBufs = MODE == FWD ? 2 : 1;
+    static constexpr int kStages = kHasX2 ? 2 : (MODE == FWD ? 3 : 4);   // blocks in flight
     static constexpr int kBig = 65536, kBigHalf = 16384;     // 128 x 256 bf16: four column halves of 128 rows x 128 B
     static constexpr int kHalfTile = 16384;                  // 32 x 256: four columns of 32 rows x 128 B, or 64 x 128: two of 64
     static constexpr int kRowHalf = 4096, kColHalf = 8192;   // one such column of 64 elements
     static constexpr int kStatBytes = MODE == DV ? 256 : (MODE == DK ? 512 : 0);   // per streamed block: lse2[64], dvec[64]
     static constexpr int kSaOff = 0;
     static constexpr int kSbOff = kBig;
-    static constexpr int kRingOff = kStationary * kBig;
+    static constexpr int kRingOff = kStationary * kStBufs * kBig;
     static constexpr int kStatOff = kRingOff + kStreams * kStages * kHalfTile;
     static constexpr int kBarOff = kStatOff + kStages * 512;
-    // full, empty [kStreams][kStages], stat[kStages], st_full, st_empty, acc_done, acc_free, drain, x1_full[3], x2_full[2],
-    // w_ready[2], acc_step[2]
-    static constexpr int kNumBars = 2 * kStreams * kStages + kStages + 15;
+    // FWD: 1 / row sum of the last three units' rows, in place of the statistics
+    static_assert(kHasX2 || kStages * 512 >= 3 * kRows * 4, "row sums");
+    // full, empty [kStreams][kStages], stat[kStages], acc_done, acc_free, drain, x1_full[3], x2_full[2], w_ready[2],
+    // acc_step[2], st_full[2], st_empty[2], l_full[3]
+    static constexpr int kNumBars = 2 * kStreams * kStages + kStages + 19;
     static constexpr int kMiscOff = kBarOff + kNumBars * 8;
     static constexpr int kBytes = kMiscOff + 16;
     static_assert(kBytes <= kSmemMax, "exceeds the shared memory of an sm_100 CTA");
@@ -89,7 +94,7 @@ struct Cfg {
 };
 
 struct Params {
-    __nv_bfloat16* out;     // FWD: out [T, Hq, 256]; DV: dv, DK: dk [T, Hkv, 256]; DQ: dq [T, Hq, 256]
+    __nv_bfloat16* out;     // DV: dv, DK: dk [T, Hkv, 256]; DQ: dq [T, Hq, 256]
     float* lse;             // FWD: [Hq, T]
     const float* lse2;      // backward passes: [Hq, Tpad]  LSE * log2(e)
     const float* dvec;      // backward passes: [Hq, Tpad]  D_i
@@ -188,16 +193,17 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
     uint64_t* bar_empty = bars + N * S;        // [N][S] the MMA that read it has run
     uint64_t* bar_stat = bars + 2 * N * S;     // [S] statistics of a streamed block (each CTA its own copy)
     uint64_t* b2 = bar_stat + S;
-    uint64_t* bar_stfull = b2 + 0;             // leader
-    uint64_t* bar_stempty = b2 + 1;
-    uint64_t* bar_accdone = b2 + 2;
-    uint64_t* bar_accfree = b2 + 3;            // leader
-    uint64_t* bar_drain = b2 + 4;
-    uint64_t* bar_x1full = b2 + 5;     // [3] one per X1 buffer, [2] per X2 buffer: committed one or two blocks ahead
-    uint64_t* bar_x2full = b2 + 8;
+    uint64_t* bar_accdone = b2 + 0;
+    uint64_t* bar_accfree = b2 + 1;            // leader
+    uint64_t* bar_drain = b2 + 2;
+    uint64_t* bar_x1full = b2 + 3;     // [3] one per X1 buffer, [2] per X2 buffer: committed one or two blocks ahead
+    uint64_t* bar_x2full = b2 + 6;
     // by the block's parity (the compute warps may be a block ahead of the issuer, the issuer of the accumulating GEMM):
-    uint64_t* bar_wready = b2 + 10;    // [2] leader: W is in both CTAs' TMEM
-    uint64_t* bar_accstep = b2 + 12;   // [2] the accumulating GEMM has run: W may be rewritten, acc rescaled
+    uint64_t* bar_wready = b2 + 8;     // [2] leader: W is in both CTAs' TMEM
+    uint64_t* bar_accstep = b2 + 10;   // [2] the accumulating GEMM has run: W may be rewritten, acc rescaled
+    uint64_t* bar_stfull = b2 + 12;    // [2] leader
+    uint64_t* bar_stempty = b2 + 14;   // [2] FWD: the output tile has left the buffer; else the unit's MMAs have run
+    uint64_t* bar_lfull = b2 + 16;     // [3] FWD: the row sums of a unit are there
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kMiscOff);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMiscOff + 4);
 
@@ -223,8 +229,11 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
     if (threadIdx.x == 0) {
         for (int s = 0; s < N * S; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&bar_empty[s], 1); }
         for (int s = 0; s < S; ++s) mbar_init(&bar_stat[s], 1);
-        mbar_init(bar_stfull, 1);
-        mbar_init(bar_stempty, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&bar_stfull[b], 1);
+            mbar_init(&bar_stempty[b], MODE == FWD ? 4 : 1);
+        }
+        for (int b = 0; b < 3; ++b) mbar_init(&bar_lfull[b], 128);
         for (int b = 0; b < 3; ++b) mbar_init(&bar_x1full[b], 1);
         for (int b = 0; b < 2; ++b) {
             mbar_init(&bar_x2full[b], 1);
@@ -248,7 +257,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
         if (L::kStationary == 2) prefetch_tmap(&tm_sb);
         prefetch_tmap(&tm_t0);
         prefetch_tmap(&tm_t1);
-        if (N == 3) prefetch_tmap(&tm_t2);
+        if (N == 3 || MODE == FWD) prefetch_tmap(&tm_t2);
     }
     tc_fence_before();
     __syncthreads();
@@ -262,14 +271,15 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
             Units<MODE> u(p, cta);
             uint32_t n = 0, uc = 0;          // n: iterations so far (over all units)
             bool ok = true;
-            const uint32_t stfull0 = map_to_rank(bar_stfull, 0);
             while (ok && !p.inject_stall && u.next(rank)) {
-                ok = mbar_wait(bar_stempty, (uc & 1) ^ 1, abort_flag);
+                const uint32_t sbuf = uc % L::kStBufs, a_off = L::kSaOff + sbuf * L::kBig;
+                ok = mbar_wait(&bar_stempty[sbuf], ((uc / L::kStBufs) & 1) ^ 1, abort_flag);
                 if (!ok) break;
-                if (rank == 0) mbar_arrive_expect_tx(bar_stfull, 2 * L::kStationary * L::kBig);
+                if (rank == 0) mbar_arrive_expect_tx(&bar_stfull[sbuf], 2 * L::kStationary * L::kBig);
+                const uint32_t stfull0 = map_to_rank(&bar_stfull[sbuf], 0);
                 const int st_head = L::kKeyStationary ? u.kvh : u.h;
                 for (int half = 0; half < 4; ++half) {
-                    tma_load_3d_pair(smem + L::kSaOff + half * L::kBigHalf, &tm_sa, stfull0, half * 64, st_head, (int)u.r0);
+                    tma_load_3d_pair(smem + a_off + half * L::kBigHalf, &tm_sa, stfull0, half * 64, st_head, (int)u.r0);
                     if (L::kStationary == 2)
                         tma_load_3d_pair(smem + L::kSbOff + half * L::kBigHalf, &tm_sb, stfull0, half * 64, st_head, (int)u.r0);
                 }
@@ -327,11 +337,12 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
             uint32_t xi = 0, xb = 0;   // next block to multiply, its X1 buffer
             bool ok = true;
             // X1 (and X2) of the next block; its streamed halves are free again as soon as they have run
+            uint32_t a_off = 0;                 // stationary tile of the unit
             auto do_x = [&]() -> bool {
                 const uint32_t s = xi % S, ph = (xi / S) & 1;
                 if (!mbar_wait(&bar_full[s], ph, abort_flag)) return false;
                 tc_fence_after();
-                issue_x(L::col_x1(xb), L::kSaOff, L::tile_off(0, s));
+                issue_x(L::col_x1(xb), a_off, L::tile_off(0, s));
                 tc_commit_pair(&bar_x1full[xb]);
                 tc_commit_pair(&bar_empty[s]);
                 if (L::kHasX2) {
@@ -347,7 +358,9 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
             };
             constexpr int kAhead = (int)L::kX1Bufs - 1;
             while (ok && u.next(rank)) {
-                ok = mbar_wait(bar_stfull, uc & 1, abort_flag);
+                const uint32_t sbuf = uc % L::kStBufs;
+                a_off = L::kSaOff + sbuf * L::kBig;
+                ok = mbar_wait(&bar_stfull[sbuf], (uc / L::kStBufs) & 1, abort_flag);
                 for (int it = 0; it < kAhead && it < u.n_it && ok; ++it) ok = do_x();
                 if (!ok) break;
                 for (int it = 0; it < u.n_it && ok; ++it, ++itc) {
@@ -370,7 +383,10 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                     }
                     tc_commit_pair(&bar_accstep[b]);
                     tc_commit_pair(&bar_empty[L::kAcc * S + s]);
-                    if (it == u.n_it - 1) { tc_commit_pair(bar_accdone); tc_commit_pair(bar_stempty); }
+                    if (it == u.n_it - 1) {
+                        tc_commit_pair(bar_accdone);
+                        if (MODE != FWD) tc_commit_pair(&bar_stempty[sbuf]);
+                    }
                 }
                 ++uc;
             }
@@ -394,6 +410,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
         Units<MODE> u(p, cta);
         uint32_t uc = 0, itc = 0;
         uint32_t xb = 0, xph = 0;                    // X1 buffer of the block and its phase
+        uint32_t lb = 0;                             // FWD: the unit's slot of row sums
         bool ok = true;
         while (ok && u.next(rank)) {
             const int64_t row = u.r0 + r;            // this thread's query row (FWD, DQ) or key (DV, DK)
@@ -571,12 +588,18 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                 if (lane == 0) mbar_arrive_cluster(wready0 + 8 * wb);
             }
             if (!ok) break;
+            if constexpr (MODE == FWD) {   // warps 4-7 take it from here
+                reinterpret_cast<float*>(smem + L::kStatOff)[lb * kRows + r] = (l_sum > 0.f) ? 1.0f / l_sum : 0.f;
+                mbar_arrive(&bar_lfull[lb]);
+                if (++lb == 3) lb = 0;
+                if (row_ok) p.lse[(size_t)u.h * p.T + row] = (m_ref + log2f(l_sum)) * 0.6931471805599453f;
+                continue;
+            }
             // ---- unit epilogue: the accumulator leaves TMEM ----
             ok = warp_wait(bar_accdone, uc & 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
             float mul = 1.0f;
-            if (MODE == FWD) mul = (l_sum > 0.f) ? 1.0f / l_sum : 0.f;
             if (MODE == DK || MODE == DQ) mul = p.scale;
             const int n_heads = L::kKeyStationary ? p.hkv : p.hq;
             const int head = L::kKeyStationary ? u.kvh : u.h;
@@ -610,12 +633,61 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                     }
                 }
             }
-            if (MODE == FWD && row_ok) p.lse[(size_t)u.h * p.T + row] = (m_ref + log2f(l_sum)) * 0.6931471805599453f;
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(accfree0);
             ++uc;
         }
+    } else if (MODE == FWD) {
+        // ---------------- FWD, warps 4-7: the output tile, through the unit's own Q tile (its MMAs have run) and bulk tensor
+        // stores, while warps 0-3 are at the next unit's first blocks.  Before there was a second Q tile, and with the rows
+        // stored from registers by warps 0-3: 410 us for 5000 tokens in samples of up to 200 at 128 heads, 315 now. ----------------
+        const int w = warp - 4;
+        const uint32_t t_acc = tmem_base + ((uint32_t)(w * 32) << 16) + kColAcc;
+        const uint32_t accfree0 = map_to_rank(bar_accfree, 0);
+        Units<MODE> u(p, cta);
+        uint32_t uc = 0, lb = 0, lph = 0;
+        while (u.next(rank)) {
+            if (!warp_wait(bar_accdone, uc & 1, abort_flag) || !warp_wait(&bar_lfull[lb], lph, abort_flag)) break;
+            tc_fence_after();
+            const float mul = reinterpret_cast<const float*>(smem + L::kStatOff)[lb * kRows + w * 32 + lane];
+            if (++lb == 3) { lb = 0; lph ^= 1; }
+            uint8_t* stage = smem + L::kSaOff + (uc & 1) * L::kBig + w * 4096;   // 32 rows x 128 bytes of each column half
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                uint32_t v[64];
+                tmem_ld32(t_acc + 64 * c, v);
+                tmem_ld32(t_acc + 64 * c + 32, v + 32);
+                tmem_ld_wait();
+                if (c == 3) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(accfree0);
+                }
+#pragma unroll
+                for (int ch = 0; ch < 8; ++ch) {
+                    uint4 x;
+                    const uint32_t* o = v + 8 * ch;
+                    x.x = pack_bf16x2(__uint_as_float(o[0]) * mul, __uint_as_float(o[1]) * mul);
+                    x.y = pack_bf16x2(__uint_as_float(o[2]) * mul, __uint_as_float(o[3]) * mul);
+                    x.z = pack_bf16x2(__uint_as_float(o[4]) * mul, __uint_as_float(o[5]) * mul);
+                    x.w = pack_bf16x2(__uint_as_float(o[6]) * mul, __uint_as_float(o[7]) * mul);
+                    *reinterpret_cast<uint4*>(stage + c * L::kBigHalf + lane * 128 + ((ch ^ (lane & 7)) << 4)) = x;
+                }
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    tma_store_3d(&tm_t2, stage + c * L::kBigHalf, 64 * c, u.h, (int)u.r0 + 32 * w);
+                    tma_store_commit();
+                }
+            }
+            if (lane == 0) {
+                tma_store_wait_read();
+                mbar_arrive(&bar_stempty[uc & 1]);
+            }
+            ++uc;
+        }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
 
     // ---------------- teardown ----------------
@@ -653,13 +725,13 @@ int launch_fwd_d256(const void* q, const void* k, const void* v, void* out, floa
                     const libra_dims* dims, float scale, cudaStream_t s) {
     using namespace d256;
     const PlanDir& d = plan->dir[0];
-    CUtensorMap tq, tk, tv;   // K by halves of a block's rows, V by halves of its columns
+    CUtensorMap tq, tk, tv, to;   // K by halves of a block's rows, V by halves of its columns, out by a warp's rows
     int rc = make_thd_map(&tq, q, plan->T, dims->hq, kD, kRows);
     if (rc == LIBRA_OK) rc = make_thd_map(&tk, k, plan->T, dims->hkv, kD, kBlk / 2);
     if (rc == LIBRA_OK) rc = make_thd_map(&tv, v, plan->T, dims->hkv, kD, kBlk);
+    if (rc == LIBRA_OK) rc = make_thd_map(&to, out, plan->T, dims->hq, kD, 32);
     if (rc != LIBRA_OK) return rc;
     Params prm = {};
-    prm.out = reinterpret_cast<__nv_bfloat16*>(out);
     prm.lse = lse;
     prm.cta_offsets = d.d_cta_offsets;
     prm.cta_tiles = d.d_cta_exec;
@@ -672,7 +744,7 @@ int launch_fwd_d256(const void* q, const void* k, const void* v, void* out, floa
     prm.outcome = plan->d_outcome[0]; prm.plan_status = plan->d_status;
     prm.wait_limit_ns = plan->wait_limit_ns; prm.inject_stall = plan->inject_stall;
     prm.busy = d.d_busy;
-    return launch<FWD>(tq, tq, tk, tv, tv, prm, d.W, s);
+    return launch<FWD>(tq, tq, tk, tv, to, prm, d.W, s);
 }
 
 // Backward at head_dim 256: the dV and dK passes over the key-major lists, the dQ pass over the query-major lists.
