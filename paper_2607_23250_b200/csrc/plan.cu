@@ -292,10 +292,35 @@ __device__ __forceinline__ int64_t pair_last_row_block(const int32_t* tok_end, i
     const int64_t last_key = ((j + 1) * kt < T ? (j + 1) * kt : T) - 1;
     return ((int64_t)tok_end[last_key] - 1) / rt;
 }
-// One block: the key-block range of every query chunk, the exclusive prefix sum of the counts, their total in base[NC].
-__global__ void __launch_bounds__(1024) k_pair_chunks(const int32_t* __restrict__ tok_end, int64_t T, int kt, int rt, int R,
-                                                      int64_t NKB, int64_t NC, int32_t* __restrict__ first_j, int32_t* __restrict__ count,
-                                                      int64_t* __restrict__ base) {
+// Chunk sizes under consideration, for the tiles proper and the wide ones: one block each finds the key-block range of
+// every query chunk, the exclusive prefix sum of the counts and their total (base[NC] and totals[block]); one more block
+// for either finds the most live cells of a key block (totals[kPairCands + k]).
+struct PairTables { int dir = 0, kt = 0, R = 0; int32_t* first_j = nullptr; int32_t* count = nullptr; int64_t* base = nullptr; int64_t NC = 0; };
+constexpr int kPairCands = 12;
+struct PairCands { PairTables c[kPairCands]; int n = 0; int rt = 0; int kt[2] = {}; };
+__global__ void __launch_bounds__(1024) k_pair_chunks(const int32_t* __restrict__ tok_end, int64_t T, const __grid_constant__ PairCands cands,
+                                                      int64_t* __restrict__ totals) {
+    const int rt = cands.rt;
+    if ((int)blockIdx.x >= cands.n) {
+        __shared__ int longest;
+        const int k = blockIdx.x - cands.n, kt = cands.kt[k];
+        if (threadIdx.x == 0) longest = 0;
+        __syncthreads();
+        int most = 0;
+        for (int64_t j = threadIdx.x; j * kt < T; j += 1024) {
+            const int64_t n = pair_last_row_block(tok_end, T, kt, rt, j) - j * kt / rt + 1;
+            most = n > most ? (int)n : most;
+        }
+        atomicMax(&longest, most);
+        __syncthreads();
+        if (threadIdx.x == 0) totals[kPairCands + k] = longest;
+        return;
+    }
+    const PairTables& t = cands.c[blockIdx.x];
+    const int kt = t.kt, R = t.R;
+    const int64_t NKB = (T + kt - 1) / kt, NC = t.NC;
+    int32_t *first_j = t.first_j, *count = t.count;
+    int64_t* base = t.base;
     __shared__ int64_t part[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t run = 0;
@@ -325,7 +350,7 @@ __global__ void __launch_bounds__(1024) k_pair_chunks(const int32_t* __restrict_
         run += all;
         __syncthreads();
     }
-    if (threadIdx.x == 0) base[NC] = run;
+    if (threadIdx.x == 0) { base[NC] = run; totals[blockIdx.x] = run; }
 }
 // Weight of pair-block (c, j): its live cells, min(last(j), c R + R - 1) - max(j, c R) + 1.
 __global__ void k_pair_fill(const int32_t* __restrict__ tok_end, int64_t T, int kt, int rt, int R, int64_t NC,
@@ -423,35 +448,69 @@ static DirView view_of(const PlanDir& d, int key_major, const libra_plan_opts& o
     return v;
 }
 
-// The pair-blocks of a plan: counts per query chunk, their prefix sums, and the total read back (one synchronous
-// 8-byte copy).  The query chunk is doubled while there are more than 262144 pair-blocks.
-struct PairTables { int32_t* first_j = nullptr; int32_t* count = nullptr; int64_t* base = nullptr; int64_t NC = 0; };
-static int64_t pair_chunks_of(int64_t T, const PlanDir& d, int rt) {
-    const int64_t NRB = (T + rt - 1) / rt, R = d.chunk / rt;
-    return (NRB + R - 1) / R;
+// ---- the pair-blocks of a plan: one table per chunk size under consideration; their totals are read back in one synchronous
+// copy and decide the size.
+static int64_t pair_chunks_of(int64_t T, int rt, int R) { return ((T + rt - 1) / rt + R - 1) / R; }
+// Chunk sizes for direction k, the largest first: the one asked for, or halves down to a row block.
+static void add_pair_cands(const libra_plan* p, PairCands& cands, int k, bool halves) {
+    const PlanDir& d = p->dir[k];
+    int R = d.chunk / cands.rt;
+    for (int x = 0; x < (halves ? kPairCands / 2 : 1) && R > 0; ++x, R /= 2) {
+        PairTables& t = cands.c[cands.n++];
+        t.dir = k;
+        t.kt = d.tile;
+        t.R = R;
+        t.NC = pair_chunks_of(p->T, cands.rt, R);
+    }
 }
-// d: the pair tiles, row blocks of d.tile tokens; wide: the same with wider key blocks, or null.
-static int count_pair_blocks(libra_plan* p, PlanDir& d, PairTables& tb, PlanDir* wide, PairTables& tbw) {
-    const int64_t T = p->T;
+// The chunk size of direction k.  In units of one cell of one query head (3.1 us), a worker's time over its mean is about
+// the tiles it starts, 3 each (operands in, accumulators out), and up to the length of one tile, R cells of G heads: idle
+// at the end.  Fused backward, best of 4096 ... 128 rows (4096): one sequence of 1500 tokens, 32 / 8 heads: 128, 60 us
+// (120); 12000 tokens, 4 / 1 heads: 1024, 159 us (345); 10007 tokens in samples of up to 400, 8 / 2 heads: 128, 64 us (91);
+// 16000 tokens, 32 / 4 heads: 1024, 0.98 ms (1.28); 32768 tokens, 32 / 8 heads: 2048, 5.88 ms (5.93), 128: 7.31; one sample of
+// 32768: 4096, 23.4 ms, 2048: 23.6, 128: 29.8.  The rule's choice is within 4 % of the best on each of ten such pools.
+static const PairTables* choose_pair_chunk(const libra_plan* p, const PairCands& cands, const int64_t* totals, int k, double G) {
+    const PairTables* best = nullptr;
+    double least = 0;
+    for (int x = 0; x < cands.n; ++x) {
+        const PairTables& t = cands.c[x];
+        if (t.dir != k || totals[x] > 262144) continue;
+        const double longest = (double)totals[kPairCands + k - 2];
+        const double cost = 3.0 * totals[x] * p->dir[k].H / p->dir[k].W + G * (t.R < longest ? t.R : longest);
+        if (!best || cost < least) { best = &t; least = cost; }
+    }
+    return best;
+}
+static double heads_per_kv(const libra_plan* p) { return p->dir[0].H > p->dir[2].H ? (double)p->dir[0].H / p->dir[2].H : 1.0; }
+// Counts, choice and, while every size has more than 262144 pair-blocks, twice the largest.
+static int count_pair_blocks(libra_plan* p, PairCands& cands, int64_t* d_totals, PairTables (&chosen)[4], double G) {
+    const int dirs = cands.c[cands.n - 1].dir == 3 ? 2 : 1;
     for (;;) {
-        int64_t nu[2] = {0, 0};
-        for (int k = 0; k < (wide ? 2 : 1); ++k) {
-            PlanDir& x = k == 0 ? d : *wide;
-            PairTables& t = k == 0 ? tb : tbw;
-            t.NC = pair_chunks_of(T, x, d.tile);   // never more than the tables were carved for
-            k_pair_chunks<<<1, 1024, 0, p->stream>>>(p->d_tok_end, T, x.tile, d.tile, x.chunk / d.tile, (T + x.tile - 1) / x.tile, t.NC,
-                                                    t.first_j, t.count, t.base);
-            count_launch();
-            if (cudaMemcpyAsync(&nu[k], t.base + t.NC, sizeof(int64_t), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess)
-                return LIBRA_ERR_CUDA;
+        int64_t totals[kPairCands + 2];
+        k_pair_chunks<<<cands.n + dirs, 1024, 0, p->stream>>>(p->d_tok_end, p->T, cands, d_totals);
+        count_launch();
+        if (cudaMemcpyAsync(totals, d_totals, sizeof(totals), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess ||
+            cudaStreamSynchronize(p->stream) != cudaSuccess)
+            return LIBRA_ERR_CUDA;
+        bool all = true;
+        for (int k = 2; k < 2 + dirs; ++k) {
+            const PairTables* t = choose_pair_chunk(p, cands, totals, k, G);
+            if (t) {
+                p->dir[k].NB = totals[t - cands.c];
+                p->dir[k].chunk = t->R * cands.rt;
+                chosen[k] = *t;
+                continue;
+            }
+            all = false;
+            for (int x = 0; x < cands.n; ++x) {
+                PairTables& c = cands.c[x];
+                if (c.dir != k) continue;
+                if ((int64_t)c.R * 2 * cands.rt > (int64_t)1 << 30) return LIBRA_ERR_UNSUPPORTED;
+                c.R *= 2;
+                c.NC = pair_chunks_of(p->T, cands.rt, c.R);   // never more than the tables were carved for
+            }
         }
-        if (cudaStreamSynchronize(p->stream) != cudaSuccess) return LIBRA_ERR_CUDA;
-        d.NB = nu[0];
-        if (wide) wide->NB = nu[1];
-        if (nu[0] <= 262144 && nu[1] <= 262144) return LIBRA_OK;
-        if ((int64_t)d.chunk * 2 > (int64_t)1 << 30) return LIBRA_ERR_UNSUPPORTED;
-        if (nu[0] > 262144) d.chunk *= 2;
-        if (nu[1] > 262144) wide->chunk *= 2;
+        if (all) return LIBRA_OK;
     }
 }
 
@@ -466,8 +525,17 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
         p->dir[k].NB = (T + p->dir[k].tile - 1) / p->dir[k].tile;
         if (const int rc = check_dir(p, p->dir[k], false); rc != LIBRA_OK) return rc;
     }
-    PairTables tb, tbw;
-    if (want[2] && p->dir[2].chunk % p->dir[2].tile) return LIBRA_ERR_INVALID_ARG;
+    PairCands cands;
+    PairTables chosen[4];
+    int64_t* d_totals = nullptr;
+    if (want[2]) {
+        if (p->dir[2].chunk % p->dir[2].tile) return LIBRA_ERR_INVALID_ARG;
+        cands.rt = p->dir[2].tile;
+        for (int k = 2; k < (wide_pairs ? 4 : 3); ++k) {
+            cands.kt[k - 2] = p->dir[k].tile;
+            add_pair_cands(p, cands, k, o.pair_chunk == 0);
+        }
+    }
     // ---- token bounds, the directions whose sizes are known, the pair tables; zeros first
     size_t zero_bytes = 0;
     auto carve = [&](Carver& c) {
@@ -481,12 +549,12 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
         for (int k = 0; k < 4; ++k)
             if (sorted[k]) carve_dir(p->dir[k], c, false, false);
         if (want[2]) {
-            for (int k = 2; k < (wide_pairs ? 4 : 3); ++k) {
-                const int64_t NC = pair_chunks_of(T, p->dir[k], p->dir[2].tile);
-                PairTables& t = k == 2 ? tb : tbw;
-                c.take(&t.first_j, NC);
-                c.take(&t.count, NC);
-                c.take(&t.base, NC + 1);
+            c.take(&d_totals, kPairCands + 2);
+            for (int x = 0; x < cands.n; ++x) {
+                PairTables& t = cands.c[x];
+                c.take(&t.first_j, t.NC);
+                c.take(&t.count, t.NC);
+                c.take(&t.base, t.NC + 1);
             }
         }
     };
@@ -500,7 +568,7 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
     count_launch();
     // ---- pair tiles: their number comes back, then their arrays
     if (want[2]) {
-        if (const int rc = count_pair_blocks(p, p->dir[2], tb, wide_pairs ? &p->dir[3] : nullptr, tbw); rc != LIBRA_OK) return rc;
+        if (const int rc = count_pair_blocks(p, cands, d_totals, chosen, heads_per_kv(p)); rc != LIBRA_OK) return rc;
         Carver ps, pm;
         size_t pair_zero = 0;
         for (int k = 2; k < (wide_pairs ? 4 : 3); ++k)
@@ -516,10 +584,9 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
         cudaMemsetAsync(pm.at, 0, pair_zero, s);
         for (int k = 2; k < (wide_pairs ? 4 : 3); ++k) {
             PlanDir& d = p->dir[k];
-            const PairTables& t = k == 2 ? tb : tbw;
-            const int rt = p->dir[2].tile;
-            k_pair_fill<<<(unsigned)t.NC, 128, 0, s>>>(p->d_tok_end, T, d.tile, rt, d.chunk / rt, t.NC, t.first_j, t.count, t.base,
-                                                       d.d_u_blk, d.d_u_chunk, d.d_weight_blk);
+            const PairTables& t = chosen[k];
+            k_pair_fill<<<(unsigned)t.NC, 128, 0, s>>>(p->d_tok_end, T, t.kt, cands.rt, t.R, t.NC, t.first_j, t.count, t.base, d.d_u_blk,
+                                                       d.d_u_chunk, d.d_weight_blk);
             count_launch();
         }
     }
@@ -607,9 +674,8 @@ extern "C" int libra_plan_tiles(const int32_t* cu_seqlens_dev, int n_samples, in
         if (k == 3) {
             // The 256-wide kernels go through a tile's heads one after the other and their workers are out of step, so what
             // the workers of a query chunk read lies anywhere in its Q and dO of a kv head's group: 1 KB a row and head,
-            // 134 MB at 4096 rows of 32 heads, more than L2 holds.  16384 rows x heads keep it at 16 MB and cut a short pool
-            // into enough tiles (dV + dK of 32768 / 16384 / 3000 tokens, 32 query heads per kv head: 37.0 / 8.86 / 0.88 ms with
-            // 4096 rows a chunk, 33.9 / 7.60 / 0.29 ms with 512); 256 rows a chunk gained nothing more on the long ones.
+            // 134 MB at 4096 rows of 32 heads, more than L2 holds.  At most 16384 rows x heads keep it at 16 MB (dV + dK of
+            // 32768 tokens, 32 query heads per kv head: 37.0 ms with 4096 rows a chunk, 33.9 with 512; 256 gained no more).
             const int64_t rows = (int64_t)16384 * d.H / n_heads / 128 * 128;
             const int64_t least = rows < 128 ? 128 : rows;
             if (d.chunk > least) d.chunk = (int)least;

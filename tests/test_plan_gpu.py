@@ -144,3 +144,16 @@ def test_pair_chunk_is_widened_until_the_pair_blocks_fit():
     # a 60000-token sample at 16-token blocks and chunks would have about 7 million pair-blocks
     cu = np.array([0, 60000], dtype=np.int32)
     assert _compare_pairs(cu, 1, 16, 16, 7) > 16
+
+
+@pytest.mark.parametrize("T,longest,H_kv,W", [(1, 1, 1, 148), (128, 128, 1, 148), (129, 129, 2, 3), (12000, 12000, 1, 148),
+                                              (4097, 4097, 1, 1), (40000, 40000, 8, 148), (262144, 100, 1, 148)])
+def test_pair_chunk_left_to_the_planner(T, longest, H_kv, W):
+    """Sizes at which it takes the smallest, a middle and the largest chunk: the tiles are the oracle's for that chunk."""
+    lengths = pools.random_layout(np.random.default_rng(T), T, longest) if longest < T else [T]
+    chunk = _compare_pairs(pools.cu_seqlens(lengths), H_kv, 128, 0, W)
+    assert chunk in (4096, 2048, 1024, 512, 256, 128)
+    if T in (1, 128, 40000, 262144):     # nothing to split; long enough for the largest; tiles that hardly depend on it
+        assert chunk == 4096
+    if T == 12000:
+        assert chunk < 4096
