@@ -41,6 +41,8 @@ constexpr int kPFirst = 96;       // keys of P handed to the MMA role in the fir
 constexpr float kRescaleThreshold = 8.0f;  // log2 units: O is rescaled only when the max grows by more
 constexpr uint64_t kFwdDrainNs = 2000000;  // teardown after a give-up: budget for work already in flight to land
 
+constexpr int kShareBlocks = 6;    // key blocks of a tile from which two CTAs share it; the hand-over costs two or three of them
+
 template <int D>
 struct FwdSmem {
     static constexpr int kHalfBytes = 128 * 128;              // 128 rows x 64 bf16 (one swizzle column)
@@ -50,8 +52,9 @@ struct FwdSmem {
     static constexpr int kRingOff = 2 * kTileBytes;
     static constexpr int kStageOff = kRingOff + kStages * kTileBytes;  // O staging: per softmax warp 32 rows x 64 bf16
     static constexpr int kBarOff = kStageOff + 8 * 4096;
-    // barriers: full[kStages], empty[kStages], q_full, q_empty, s_full[2], p_ready[2], o_done[2], p_part[2], drain
-    static constexpr int kNumBars = 2 * kStages + 11;
+    // barriers: full[kStages], empty[kStages], q_full, q_empty, s_full[2], p_ready[2], o_done[2], p_part[2], drain, spent,
+    // partial
+    static constexpr int kNumBars = 2 * kStages + 13;
     static constexpr int kMiscOff = kBarOff + kNumBars * 8;
     static constexpr int kBytes = kMiscOff + 16;
     static constexpr int kAlloc = kBytes + 1024;  // slack to align the base to 1024 B
@@ -78,6 +81,23 @@ struct FwdTile {
     int t;
     int64_t q0;
     int lo[2], hi[2];
+    // A tile that a pair of CTAs shares: `shared`, and part[g] when both have key blocks of slot g.
+    bool shared, part[2];
+    // Takes the CTA's part: rank 0 the upper half of the key blocks, rank 1 the lower; false when nothing is left for it.
+    __device__ __forceinline__ bool take_half(uint32_t rank) {
+        const int top = hi[1] >= 0 ? hi[1] : hi[0], n = top - lo[0] + 1;
+        shared = n >= kShareBlocks;
+        part[0] = part[1] = false;
+        if (!shared) return rank == 0;
+        const int mid = (lo[0] + top + 2) / 2;   // lo[0] < mid <= hi[0]
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            part[g] = lo[g] <= hi[g] && lo[g] < mid;
+            if (rank == 0) lo[g] = part[g] ? mid : lo[g];
+            else { hi[g] = part[g] ? mid - 1 : -1; lo[g] = part[g] ? lo[g] : 0; }   // slot 1's sample may start in the upper half
+        }
+        return true;
+    }
 };
 // Walks the list.  Ids are fetched two tiles and sample starts one tile ahead: a chain of two dependent global
 // loads between tiles would leave the tensor pipe idle for about 2000 clk.
@@ -113,7 +133,73 @@ struct FwdTiles {
     }
 };
 
+// What a thread of a shared tile does when its slot's MMAs are done.  take: 0 the other CTA has nothing of the slot; 1 it
+// takes the other's partial output over into its own, in TMEM; 2 it gives its own away.  Returns false on a timeout.  (A
+// function of its own: inlined, it cost the loop over key blocks 0.4 us each in spilled registers.)
 template <int D>
+__device__ __noinline__ bool exchange_partial(uint8_t* smem, uint64_t* bars, uint32_t tmem_base, int take, float& m_ref, float& l_sum) {
+    using L = FwdSmem<D>;
+    uint64_t* bar_spent = bars + 2 * L::kStages + 11;
+    uint64_t* bar_partial = bar_spent + 1;
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMiscOff + 4);
+    const int warp = threadIdx.x >> 5, g = warp >> 2, row_in_tile = threadIdx.x & 127;
+    const uint32_t peer = cluster_rank() ^ 1;
+    const uint32_t t_o = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + 2 * kBN + g * D;
+    float4* partial = reinterpret_cast<float4*>(smem + L::kRingOff) + row_in_tile;   // [D / 4][128]
+    float* sums = reinterpret_cast<float*>(smem + L::kQOff) + row_in_tile;           // [2][128]
+    // this CTA's ring and Q tiles are spent when the threads of both slots have arrived
+    fence_cluster();
+    mbar_arrive_cluster(map_to_rank(bar_spent, peer));
+    if (take == 0) return true;
+    if (take == 2) {
+        if (!warp_wait(bar_spent, 0, abort_flag)) return false;
+        fence_cluster();
+        const uint32_t dst = map_to_rank(partial, peer), dst_s = map_to_rank(sums, peer);
+#pragma unroll
+        for (int c = 0; c < D; c += 32) {
+            uint32_t o[32];
+            tmem_ld32(t_o + c, o);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 32; i += 4) st_cluster4(dst + (c + i) * (kBM * 4), o + i);
+        }
+        st_cluster(dst_s, m_ref);
+        st_cluster(dst_s + kBM * 4, l_sum);
+        fence_cluster();
+        mbar_arrive_cluster(map_to_rank(bar_partial, peer));
+        return true;
+    }
+    if (!warp_wait(bar_partial, 0, abort_flag)) return false;
+    fence_cluster();
+    const float m1 = sums[0], l1 = sums[kBM], m = fmaxf(m_ref, m1);
+    const float own = m > -INFINITY ? ex2_approx(m_ref - m) : 1.0f, other = m > -INFINITY ? ex2_approx(m1 - m) : 0.f;
+    m_ref = m;
+    l_sum = l_sum * own + l1 * other;
+#pragma unroll
+    for (int c = 0; c < D; c += 32) {
+        uint32_t o[32];
+        tmem_ld32(t_o + c, o);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) {
+            const float4 v = partial[(c + i) / 4 * kBM];
+            o[i] = __float_as_uint(__uint_as_float(o[i]) * own + v.x * other);
+            o[i + 1] = __float_as_uint(__uint_as_float(o[i + 1]) * own + v.y * other);
+            o[i + 2] = __float_as_uint(__uint_as_float(o[i + 2]) * own + v.z * other);
+            o[i + 3] = __float_as_uint(__uint_as_float(o[i + 3]) * own + v.w * other);
+        }
+        tmem_st32(t_o + c, o);
+    }
+    tmem_st_wait();
+    return true;
+}
+
+// PAIR: a cluster of two CTAs goes through the list of a worker of its own and shares its tiles by key blocks.  When there
+// is no more than a tile for every two SMs, the longest tile is the launch: 16 of its key blocks take 26 us (4096 tokens, 4
+// heads of 64), at the rate of one slot's chain for each, with 84 SMs idle.  Each rank takes
+// the other's maxima, sums and output of the slot of its own number through distributed shared memory and combines: 28.4 ->
+// 21.5 us there, one sample of 4096 tokens, 4 heads of 128: 55.3 -> 38.1.
+template <int D, bool PAIR>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
            const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_out, const FwdParams p) {
@@ -130,14 +216,20 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     uint64_t* bar_odone = bar_qfull + 6;   // [2]
     uint64_t* bar_ppart = bar_qfull + 8;   // [2] P of the first kPFirst keys is in TMEM
     uint64_t* bar_drain = bar_qfull + 10;  // teardown after a give-up: every MMA issued so far has completed
+    uint64_t* bar_spent = bar_qfull + 11;    // PAIR: the other CTA's ring is spent, a partial output may go there
+    uint64_t* bar_partial = bar_qfull + 12;  // PAIR: the other CTA's partial output is here
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kMiscOff);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMiscOff + 4);
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int cta = blockIdx.x;
+    const uint32_t rank = PAIR ? cluster_rank() : 0;
+    const int worker = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+    const int cta = PAIR ? worker + (int)(rank * (gridDim.x >> 1)) : worker;   // where the CTA reports
 
     if (threadIdx.x == 0) {
+        mbar_init(bar_spent, 2 * kBM);
+        mbar_init(bar_partial, kBM);
         for (int i = 0; i < L::kStages; ++i) { mbar_init(&bar_full[i], 1); mbar_init(&bar_empty[i], 1); }
         mbar_init(bar_qfull, 1);
         mbar_init(bar_qempty, 1);
@@ -158,10 +250,12 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         prefetch_tmap(&tm_v);
         prefetch_tmap(&tm_out);
     }
+    if (PAIR) cluster_arrive();
     grid_dep_wait();
     // A plan whose cu_seqlens failed the planner's check is never executed: report and leave.
     if (const int ps = *p.plan_status; ps != 0) {
         if (threadIdx.x == 0) { p.outcome[cta] = ps; p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
+        if (PAIR) cluster_wait();
         return;
     }
     if (threadIdx.x == 0) p.busy[2 * cta] = globaltimer_ns();
@@ -171,11 +265,12 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     }
     tc_fence_before();
     __syncthreads();
+    if (PAIR) cluster_wait();   // the other CTA's barriers are initialised
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    const int tile_begin = p.cta_offsets[cta];
-    const int tile_end = p.cta_offsets[cta + 1];
+    const int tile_begin = p.cta_offsets[worker];
+    const int tile_end = p.cta_offsets[worker + 1];
     const int heads_per_shard = p.hq / p.H;
     const int G = p.hq / p.hkv;
 
@@ -192,6 +287,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             FwdTiles tiles(p, tile_begin, tile_end);
             FwdTile x;
             while (ok && !p.inject_stall && tiles.next(x)) {
+                if (PAIR && !x.take_half(cluster_rank())) continue;
                 const bool act1 = x.hi[1] >= 0;
                 const int top = act1 ? x.hi[1] : x.hi[0];
                 for (int hh = 0; hh < heads_per_shard && ok; ++hh) {
@@ -267,6 +363,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             FwdTiles tiles(p, tile_begin, tile_end);
             FwdTile x;
             while (ok && tiles.next(x)) {
+                if (PAIR && !x.take_half(cluster_rank())) continue;
                 const bool act1 = x.hi[1] >= 0;
                 const int top = act1 ? x.hi[1] : x.hi[0], lo = x.lo[0];
                 for (int hh = 0; hh < heads_per_shard && ok; ++hh) {
@@ -278,6 +375,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                     ++qcnt;
                     tc_fence_after();
                     issue_s(act1 ? 1 : 0, st);
+                    if (PAIR && act1 && x.hi[0] == top) issue_s(0, st);   // the lower half of a shared tile
                     tc_commit(&bar_empty[st]);
                     if (lo == top) tc_commit(bar_qempty);  // no later MMA of this tile reads Q
                     ++ring;
@@ -352,9 +450,13 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         FwdTiles tiles(p, tile_begin, tile_end);
         FwdTile x;
         while (ok && tiles.next(x)) {
+            if (PAIR && !x.take_half(cluster_rank())) continue;
             const int64_t qs = x.q0 + g * kBM;
             const int lo = x.lo[g], hi = x.hi[g];
-            if (lo > hi) continue;  // slot past the end of the pool
+            if (lo > hi) {  // slot past the end of the pool, or all in the other CTA
+                if (PAIR && x.shared) mbar_arrive_cluster(map_to_rank(bar_spent, cluster_rank() ^ 1));
+                continue;
+            }
             const uint64_t tile_t0 = threadIdx.x == 0 ? globaltimer_ns() : 0;
             const int64_t row = qs + row_in_tile;
             const bool row_ok = row < p.T;
@@ -377,9 +479,9 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                     tmem_ld32(t_s + 96, sr + 96);
                     tmem_ld_wait();
                     const int k0 = j * kBN;
-                    if (j == hi || k0 < max_kstart || !row_ok) {
-                        const int c_lo = row_ok ? kstart - k0 : kBN;        // first visible column
-                        const int c_hi = row_ok ? (int)(row - k0) : -1;      // last visible column
+                    if (j == hi || k0 < max_kstart) {   // (rows past the pool: anything finite)
+                        const int c_lo = row_ok ? kstart - k0 : 0;           // first visible column
+                        const int c_hi = row_ok ? (int)(row - k0) : kBN;     // last visible column
 #pragma unroll
                         for (int w = 0; w < kBN / 32; ++w) {
                             const uint32_t vis = range_bits(c_lo - 32 * w, c_hi - 32 * w);
@@ -449,6 +551,14 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 ok = warp_wait(&bar_odone[g], (ocnt - 1) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
+                if (PAIR && x.shared) {
+                    const int take = x.part[g] ? ((int)cluster_rank() == g ? 1 : 2) : 0;
+                    float m = m_ref, l = l_sum;
+                    ok = __all_sync(0xffffffffu, exchange_partial<D>(smem, bars, tmem_base, take, m, l));
+                    m_ref = m;
+                    l_sum = l;
+                    if (!ok || take == 2) break;
+                }
                 const float inv_l = (l_sum > 0.f) ? 1.0f / l_sum : 0.f;
                 // Through the warp's staging tile (32 rows x 128 bytes, 128-byte swizzle) and a bulk tensor store: one row
                 // per thread stored straight from registers touches 32 cache lines per instruction.  Rows past the end
@@ -483,7 +593,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                 // after this group's next P arrival, which follows in program order
                 tc_fence_before();
             }
-            if (threadIdx.x == 0 && ok) p.tile_ns[x.t] = (uint32_t)(globaltimer_ns() - tile_t0);
+            if (threadIdx.x == 0 && ok && (!PAIR || cluster_rank() == 0)) p.tile_ns[x.t] = (uint32_t)(globaltimer_ns() - tile_t0);
         }
         // every bulk store this warp issued has completed before the CTA leaves
         if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
@@ -492,6 +602,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     // ---------------- teardown ----------------
     tc_fence_before();
     __syncthreads();
+    if (PAIR) cluster_sync();   // nothing of the other CTA is on its way here any more
     if (warp == 9) tmem_dealloc(tmem_base, 512);
     if (threadIdx.x == 0) {
         p.outcome[cta] = *abort_flag ? LIBRA_ERR_TIMEOUT : LIBRA_OK;
@@ -557,20 +668,21 @@ int make_f32_3d_map(CUtensorMap* m, const void* base, int64_t T, int H, int d, i
     return r == CUDA_SUCCESS ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
 
-template <int D>
+template <int D, bool PAIR>
 static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tout,
                       const FwdParams& prm, int W, cudaStream_t s) {
     using L = FwdSmem<D>;
-    constexpr int kSlot = D == 128 ? 0 : 1;
+    constexpr int kSlot = (D == 128 ? 0 : 1) + (PAIR ? 5 : 0);
     if (!cfg_done(kSlot)) {   // per device: the attribute belongs to the device's copy of the kernel
-        if (cudaFuncSetAttribute(k_attn_fwd<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kAlloc) != cudaSuccess)
+        if (cudaFuncSetAttribute(k_attn_fwd<D, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kAlloc) != cudaSuccess)
             return LIBRA_ERR_CUDA;
-        if (!regs_pool_ok(k_attn_fwd<D>, 256, LIBRA_FWD_REG_INC, 128, LIBRA_FWD_REG_DEC)) return LIBRA_ERR_UNSUPPORTED;
+        if (!regs_pool_ok(k_attn_fwd<D, PAIR>, 256, LIBRA_FWD_REG_INC, 128, LIBRA_FWD_REG_DEC)) return LIBRA_ERR_UNSUPPORTED;
         cfg_mark(kSlot);
     }
     count_launch();
-    return launch_dependent(k_attn_fwd<D>, W, kFwdThreads, L::kAlloc, s, tq, tk, tv, tout, prm) == cudaSuccess ? LIBRA_OK
-                                                                                                           : LIBRA_ERR_CUDA;
+    const cudaError_t e = launch_dependent<PAIR ? 2 : 1>(k_attn_fwd<D, PAIR>, PAIR ? W / 2 * 2 : W, kFwdThreads, L::kAlloc, s, tq, tk, tv,
+                                                         tout, prm);
+    return e == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
 
 }  // namespace libra
@@ -627,8 +739,14 @@ extern "C" int libra_attn_pool_fwd(const void* q_dev, const void* k_dev, const v
     prm.busy = d.d_busy;
     prm.tile_ns = d.d_tile_ns;
     time_begin(mp, 0, s);
-    rc = dims->head_dim == 128 ? launch_fwd<128>(tq, tk, tv, tout, prm, d.W, s)
-                               : launch_fwd<64>(tq, tk, tv, tout, prm, d.W, s);
+    // Two CTAs a tile when there are two for each (the first NT workers then have one tile each), a tile is one head (the
+    // exchange goes through the spent ring) and samples average four key blocks: 4000 tokens, 4 heads of 128, in samples of
+    // up to 300 / 800 / 4000 tokens took 12.0 / 18.0 / 55.3 us with one CTA a tile and 14.0 / 18.4 / 38.1 with two.
+    const bool pair = d.NT <= d.W / 2 && d.H == dims->hq && plan->T >= 4 * kBN * (int64_t)plan->n;
+    if (dims->head_dim == 128)
+        rc = pair ? launch_fwd<128, true>(tq, tk, tv, tout, prm, d.W, s) : launch_fwd<128, false>(tq, tk, tv, tout, prm, d.W, s);
+    else
+        rc = pair ? launch_fwd<64, true>(tq, tk, tv, tout, prm, d.W, s) : launch_fwd<64, false>(tq, tk, tv, tout, prm, d.W, s);
     time_end(mp, 0, s);
     return rc;
 }

@@ -119,10 +119,11 @@ int launch_bwd_d256(const void* q, const void* k, const void* v, const void* dou
 // grid_dep_wait() (ptx.cuh) before it touches anything another kernel writes, or, where it only needs what the kernel
 // ahead had itself waited for, before it ends.  A step on 10007 tokens (forward, statistics, fused backward,
 // conversion): 175 -> 153 us with the clearing of accumulators and status words moved into those kernels.
-template <typename... KArgs, typename... Args>
+template <unsigned CLUSTER = 1, typename... KArgs, typename... Args>
 static inline cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
                                            const Args&... args) {
-    cudaLaunchAttribute attr = {};
+    cudaLaunchAttribute attrs[2] = {};
+    cudaLaunchAttribute& attr = attrs[0];
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
@@ -130,8 +131,11 @@ static inline cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned gr
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    attrs[1].id = cudaLaunchAttributeClusterDimension;
+    attrs[1].val.clusterDim.x = CLUSTER;
+    attrs[1].val.clusterDim.y = attrs[1].val.clusterDim.z = 1;
+    cfg.attrs = attrs;
+    cfg.numAttrs = CLUSTER > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 

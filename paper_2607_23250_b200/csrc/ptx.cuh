@@ -67,9 +67,11 @@ __device__ __forceinline__ uint32_t cluster_rank() {
     return r;
 }
 // Barrier of all threads of the cluster, with release / acquire of shared memory at cluster scope.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 // Address (shared::cluster window) of this CTA's shared-memory location in the cluster's CTA of the given rank.
 __device__ __forceinline__ uint32_t map_to_rank(const void* p, uint32_t rank) {
@@ -82,6 +84,15 @@ __device__ __forceinline__ uint32_t map_to_rank(const void* p, uint32_t rank) {
 // 64-row block of the 256-wide kernels up by about 1100 cycles (a training step of 99 ms took 76 ms without).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// Before an arrival that hands shared memory over to, and after a wait that takes it over from, the other CTA.
+__device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
+__device__ __forceinline__ void st_cluster(uint32_t cluster_addr, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster4(uint32_t cluster_addr, const uint32_t* v) {
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3])
+                 : "memory");
 }
 // Returns true when the phase with the given parity has completed, false on timeout or when
 // another thread has already flagged an abort in ctl[0] (shared memory).

@@ -72,6 +72,16 @@ def test_boundary_lengths_and_three_samples_in_one_tile():
     _check(o, l, o_ref, l_ref, cu)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("lengths", [[513], [640], [641], [769], [896, 30], [70, 1500, 600], [30, 1000, 1100], [1300, 900], [2049], [3000]])
+def test_tiles_shared_by_two_ctas(lengths, d):
+    """Few tiles: from six key blocks on, two CTAs share one.  Odd and even block counts, tiles without a second slot, samples
+    that end in the first or the second slot of a tile or start in the upper half of its key blocks; the scores are peaked
+    so that either half may hold a row's maximum."""
+    o, l, o_ref, l_ref, cu = _run(lengths, 2, 1, d, seed=sum(lengths), qscale=2.0)
+    _check(o, l, o_ref, l_ref, cu)
+
+
 def test_peaked_softmax_and_score_offset():
     # Q scaled x8 makes the running max move a lot (exercises the O rescale path)
     o, l, o_ref, l_ref, cu = _run([700, 900], 2, 2, 64, seed=4, qscale=8.0)
