@@ -112,7 +112,7 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     uint64_t* bar_qfull = bars + 2;               // [QS]
     uint64_t* bar_qempty = bar_qfull + QS;        // [QS] dK(it) has run: Q stage free, dS^T columns free
     uint64_t* bar_dofull = bar_qempty + QS;       // [DS]
-    uint64_t* bar_doempty = bar_dofull + DS;      // [DS] dV(it) has run: dO stage free
+    uint64_t* bar_doempty = bar_dofull + DS;      // [DS] dV(it) has run and the dS group has read D(it): dO stage free
     uint64_t* bar_sfull = bar_doempty + DS;
     uint64_t* bar_xfree1 = bar_sfull + 1;   // S^T(it) has been read out of region X: dP^T(it) may overwrite it
     uint64_t* bar_dpfull = bar_sfull + 2;
@@ -139,7 +139,7 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         mbar_init(bar_kvfull, 1);
         mbar_init(bar_kvempty, 1);
         for (int s = 0; s < QS; ++s) { mbar_init(&bar_qfull[s], 1); mbar_init(&bar_qempty[s], 1); }
-        for (int s = 0; s < DS; ++s) { mbar_init(&bar_dofull[s], 1); mbar_init(&bar_doempty[s], 1); }
+        for (int s = 0; s < DS; ++s) { mbar_init(&bar_dofull[s], 1); mbar_init(&bar_doempty[s], 5); }   // the commit behind dV(it) + 4 warps
         mbar_init(bar_sfull, 1);
         mbar_init(bar_xfree1, 256);
         mbar_init(bar_dpfull, 1);
@@ -378,6 +378,9 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         xs[j >> 1] = pack_bf16x2(a0, a1);
                         xs[(j >> 1) + 1] = pack_bf16x2(b0, b1);
                     }
+                    // (dV(it) alone does not free D: a warp held up here, by instruction fetches say, read the next block's)
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bar_doempty[ds]);
                 }
                 // dS^T(it-1) must have been consumed by dK(it-1) before its columns are rewritten
                 if (it_all > 0) {
