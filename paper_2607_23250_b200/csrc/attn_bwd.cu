@@ -60,8 +60,8 @@ struct DkvSmem {
     static constexpr int kDvecOff = kLseOff + kQStages * 512;        // per dO stage: dvec[128]
     static constexpr int kBarOff = kDvecOff + kDoStages * 512;
     // kv_full, kv_empty, q_full[3], q_empty[3], do_full[2], do_empty[2], s_full, x_free1, dp_full, x_free2,
-    // p_half, p_ready, p_free, ds_ready, dkv_full, dkv_empty, drain
-    static constexpr int kNumBars = 2 + 2 * kQStages + 2 * kDoStages + 11;
+    // p_half, p_ready, p_free, ds_ready, dkv_full, dkv_empty, drain, spent, partial
+    static constexpr int kNumBars = 2 + 2 * kQStages + 2 * kDoStages + 13;
     static constexpr int kMiscOff = kBarOff + kNumBars * 8;
     static constexpr int kBytes = kMiscOff + 16;
     static_assert(kBytes <= kSmemMax, "exceeds the shared memory of an sm_100 CTA");
@@ -98,7 +98,82 @@ __device__ __forceinline__ void tmem_ld128(uint32_t taddr, uint32_t* r) {
     tmem_ld32(taddr + 96, r + 96);
 }
 
+// The iterations (query heads of the group times query blocks) of a tile that the CTA of a cluster takes.
+__device__ __forceinline__ int share_begin(int n_it, uint32_t rank, uint32_t size) { return (int)((int64_t)n_it * rank / size); }
+
+// End of a tile that a cluster shares, for a thread of an exp group: group 0 finishes dK, group 1 dV.  Every CTA gives the
+// others the columns that they finish, D / size each, and adds up the partial sums of its own in the order of the ranks
+// (the result does not depend on which is ready first).  t_acc: the group's accumulator, gdst: the key's row or null.
+// Returns false on a timeout.
 template <int D>
+__device__ __noinline__ bool finish_shared(uint8_t* smem, uint64_t* bar_spent, uint32_t t_acc, int n_it, float mul,
+                                           __nv_bfloat16* gdst, volatile int* abort_flag) {
+    const uint32_t size = cluster_size(), rank = cluster_rank();
+    uint64_t* bar_partial = bar_spent + 1;
+    const int grp = threadIdx.x >> 7, row = threadIdx.x & 127, lane = threadIdx.x & 31, n = D / (int)size;
+    auto has = [&](uint32_t q) { return share_begin(n_it, q, size) < share_begin(n_it, q + 1, size); };
+    auto part = [&](uint32_t q, int c) {   // columns c .. c + 3 of rank q's partial sums
+        return reinterpret_cast<float4*>(smem) + (((int)q * 2 + grp) * n + c) / 4 * 128 + row;
+    };
+    auto tell = [&](uint64_t* bar) {
+        fence_cluster();
+        __syncwarp();
+        if (lane == 0) {
+            fence_cluster();
+            for (uint32_t q = 0; q < size; ++q)
+                if (q != rank) mbar_arrive_cluster(map_to_rank(bar, q));
+        }
+        __syncwarp();
+    };
+    tell(bar_spent);                       // the operand tiles of this CTA may be overwritten
+    if (!warp_wait(bar_spent, 0, abort_flag)) return false;
+    fence_cluster();
+    if (has(rank))
+        for (uint32_t q = 0; q < size; ++q) {
+            if (q == rank) continue;
+            for (int c = 0; c < n; c += 8) {
+                uint32_t v[8];
+                tmem_ld8(t_acc + q * n + c, v);
+                tmem_ld_wait();
+                st_cluster4(map_to_rank(part(rank, c), q), v);
+                st_cluster4(map_to_rank(part(rank, c + 4), q), v + 4);
+            }
+        }
+    tell(bar_partial);
+    if (!warp_wait(bar_partial, 0, abort_flag)) return false;
+    fence_cluster();
+    for (int c = 0; c < n; c += 8) {
+        float sum[8] = {};
+        for (uint32_t q = 0; q < size; ++q) {
+            if (!has(q)) continue;
+            uint32_t v[8];
+            if (q == rank) {
+                tmem_ld8(t_acc + q * n + c, v);
+                tmem_ld_wait();
+            } else {
+                *reinterpret_cast<float4*>(v) = *part(q, c);
+                *reinterpret_cast<float4*>(v + 4) = *part(q, c + 4);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) sum[i] += __uint_as_float(v[i]);
+        }
+        if (gdst) {
+            uint4 w;
+            w.x = pack_bf16x2(sum[0] * mul, sum[1] * mul);
+            w.y = pack_bf16x2(sum[2] * mul, sum[3] * mul);
+            w.z = pack_bf16x2(sum[4] * mul, sum[5] * mul);
+            w.w = pack_bf16x2(sum[6] * mul, sum[7] * mul);
+            *reinterpret_cast<uint4*>(gdst + rank * n + c) = w;
+        }
+    }
+    return true;
+}
+
+// SHARE: a cluster of CTAs goes through the list of a worker of its own, a tile at most, and shares its iterations.  With
+// fewer tiles than SMs the longest, G heads times the blocks of its sample, is the launch.  Step with one CTA a tile and with several: 2000 tokens, 8 /
+// 2 heads of 64: 104.6 -> 65.8 us (4 CTAs); 4000 tokens in one sample, 4 / 1 heads of 128: 237.9 -> 146.4 (4); 1500 tokens, 4 /
+// 1 heads: 96.8 -> 60.4 (8); 9000 tokens: 236.9 -> 162.3 (2).
+template <int D, bool SHARE>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
@@ -124,12 +199,15 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     uint64_t* bar_dkvfull = bar_sfull + 8;
     uint64_t* bar_dkvempty = bar_sfull + 9;
     uint64_t* bar_drain = bar_sfull + 10;   // teardown after a give-up: every MMA issued so far has completed
+    uint64_t* bar_spent = bar_sfull + 11;   // SHARE: the other CTAs' operand tiles may be overwritten; then partial sums are here
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kMiscOff);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMiscOff + 4);
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int cta = blockIdx.x;
+    const uint32_t size = SHARE ? cluster_size() : 1, rank = SHARE ? cluster_rank() : 0;
+    const int worker = SHARE ? (int)(blockIdx.x / size) : (int)blockIdx.x;
+    const int cta = SHARE ? worker + (int)(rank * (gridDim.x / size)) : worker;   // where the CTA reports
 
     if ((smem_u32(smem) & 1023u) != 0) {  // the swizzled tiles need a 1024-byte aligned base
         if (threadIdx.x == 0) p.outcome[cta] = LIBRA_ERR_CUDA;
@@ -151,6 +229,8 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         mbar_init(bar_dkvfull, 1);
         mbar_init(bar_dkvempty, 256);
         mbar_init(bar_drain, 1);
+        mbar_init(bar_spent, 8 * (size - 1) + !SHARE);   // a warp of the exp groups arrives as one
+        mbar_init(bar_spent + 1, 8 * (size - 1) + !SHARE);
         abort_flag[0] = 0;
         abort_flag[1] = (int)p.wait_limit_ns;
         fence_mbar_init();
@@ -174,12 +254,13 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     }
     tc_fence_before();
     __syncthreads();
+    if (SHARE) cluster_sync();   // the other CTAs' barriers are initialised
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     constexpr uint32_t kColX = 0, kColP = 128, kColDS = 192, kColDK = 256, kColDV = 256 + D;
 
-    const int unit_begin = p.cta_offsets[cta];
-    const int unit_end = p.cta_offsets[cta + 1];
+    const int unit_begin = p.cta_offsets[worker];
+    const int unit_end = p.cta_offsets[worker + 1];
     const int G = p.hq / p.hkv;
 
     if (warp > kDkvMmaWarp) {
@@ -196,6 +277,9 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 const int64_t k0 = (int64_t)(t / p.hkv) * kBlk;
                 const int i_lo = (int)(k0 / kBlk);
                 const int nblk = last_q_block(p.tok_end, p.T, k0) - i_lo + 1;
+                const int it0 = SHARE ? share_begin(G * nblk, rank, size) : 0;
+                const int n_it = (SHARE ? share_begin(G * nblk, rank + 1, size) : G * nblk) - it0;
+                if (SHARE && n_it == 0) break;
                 ok = mbar_wait(bar_kvempty, (ucnt & 1) ^ 1, abort_flag);
                 if (!ok) break;
                 mbar_arrive_expect_tx(bar_kvfull, 2 * L::kTileBytes);
@@ -204,10 +288,9 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     tma_load_3d(smem + L::kVOff + half * L::kHalfBytes, &tm_v, bar_kvfull, half * 64, kvh, (int)k0);
                 }
                 ++ucnt;
-                const int n_it = G * nblk;
                 for (int it = 0; it < n_it && ok; ++it, ++it_all) {
-                    const int h = kvh * G + it / nblk;
-                    const int qb = (i_lo + it % nblk) * kBlk;
+                    const int h = kvh * G + (it0 + it) / nblk;
+                    const int qb = (i_lo + (it0 + it) % nblk) * kBlk;
                     const uint32_t qs = it_all % QS, ds = it_all % DS;
                     ok = mbar_wait(&bar_qempty[qs], ((it_all / QS) & 1) ^ 1, abort_flag);
                     if (!ok) break;
@@ -281,7 +364,8 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 const int64_t k0 = (int64_t)(t / p.hkv) * kBlk;
                 const int i_lo = (int)(k0 / kBlk);
                 const int nblk = last_q_block(p.tok_end, p.T, k0) - i_lo + 1;
-                const int n_it = G * nblk;
+                const int n_it = SHARE ? share_begin(G * nblk, rank + 1, size) - share_begin(G * nblk, rank, size) : G * nblk;
+                if (SHARE && n_it == 0) break;
                 ok = mbar_wait(bar_kvfull, ucnt & 1, abort_flag);
                 if (!ok) break;
                 // S(0): region X is free once dP of the previous unit's last iteration has been read
@@ -352,7 +436,7 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             const int64_t k0 = (int64_t)(t / p.hkv) * kBlk;
             const int i_lo = (int)(k0 / kBlk);
             const int nblk = last_q_block(p.tok_end, p.T, k0) - i_lo + 1;
-            const int n_it = G * nblk;
+            const int n_it = SHARE ? share_begin(G * nblk, rank + 1, size) - share_begin(G * nblk, rank, size) : G * nblk;
             // ---- dS group: dS^T = P^T o (dP^T - D) ----
             for (int it = 0; it < n_it && ok; ++it, ++it_all) {
                 const uint32_t ds = it_all % DS;
@@ -432,7 +516,8 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             const int64_t k0 = (int64_t)(t / p.hkv) * kBlk;
             const int i_lo = (int)(k0 / kBlk);
             const int nblk = last_q_block(p.tok_end, p.T, k0) - i_lo + 1;
-            const int n_it = G * nblk;
+            const int it0 = SHARE ? share_begin(G * nblk, rank, size) : 0;
+            const int n_it = (SHARE ? share_begin(G * nblk, rank + 1, size) : G * nblk) - it0;
             const int64_t key = k0 + r;
             const bool key_ok = key < p.T;
             // ---- exp groups: P^T = exp2(S^T * c - LSE), zero where the query does not see the key ----
@@ -442,7 +527,7 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             const int min_kend = p.tok_end[k0];
             const bool partial = k0 + kBlk > p.T;
             for (int it = 0; it < n_it && ok; ++it, ++it_all) {
-                const int qb = (i_lo + it % nblk) * kBlk;
+                const int qb = (i_lo + (it0 + it) % nblk) * kBlk;
                 const uint32_t qs = it_all % QS;
                 const float* lse2 = reinterpret_cast<const float*>(smem + L::kLseOff + qs * 512) + c0;
                 const bool need_mask = (qb == k0) || (qb + kBlk - 1 >= min_kend) || partial;
@@ -497,9 +582,16 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             if (!ok) break;
             ++ucnt;
             // ---- unit epilogue: dK * scale and dV to global (each exp group stores half of the columns) ----
-            ok = warp_wait(bar_dkvfull, (ucnt - 1) & 1, abort_flag);
+            if (!SHARE || n_it > 0) ok = warp_wait(bar_dkvfull, (ucnt - 1) & 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
+            if constexpr (SHARE) {
+                __nv_bfloat16* gdst = (grp == 0 ? p.dk : p.dv) + ((size_t)key * p.hkv + kvh) * D;
+                const bool done = finish_shared<D>(smem, bar_spent, tmem_base + lane_addr + (grp == 0 ? kColDK : kColDV), G * nblk,
+                                                   grp == 0 ? p.scale : 1.0f, key_ok ? gdst : nullptr, abort_flag);
+                ok = __all_sync(0xffffffffu, done);
+                break;
+            }
             constexpr int kCols = D / 2;
             const uint32_t t_dk = tmem_base + lane_addr + kColDK + grp * kCols;
             const uint32_t t_dv = tmem_base + lane_addr + kColDV + grp * kCols;
@@ -534,6 +626,7 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     // ---------------- teardown ----------------
     tc_fence_before();
     __syncthreads();
+    if (SHARE) cluster_sync();   // nothing of the other CTAs is on its way here any more
     if (warp == kDkvMmaWarp) tmem_dealloc(tmem_base, 512);
     if (threadIdx.x == 0) {
         p.outcome[cta] = abort_flag[0] ? LIBRA_ERR_TIMEOUT : LIBRA_OK;
@@ -640,17 +733,26 @@ static int set_smem(Kernel k, int bytes) {
 template <int D>
 static int launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tdo,
                       const CUtensorMap& tdq,
-                      const DkvParams& pa, int Wa, const DqParams& pb, int Wb, libra_plan_t* mp, cudaStream_t s) {
+                      const DkvParams& pa, int Wa, int share, const DqParams& pb, int Wb, libra_plan_t* mp, cudaStream_t s) {
     constexpr int kSlot = D == 128 ? 2 : 3;
     if (!cfg_done(kSlot)) {   // per device
-        if (set_smem(k_attn_bwd_dkdv<D>, DkvSmem<D>::kBytes) != LIBRA_OK) return LIBRA_ERR_CUDA;
+        if (set_smem(k_attn_bwd_dkdv<D, false>, DkvSmem<D>::kBytes) != LIBRA_OK) return LIBRA_ERR_CUDA;
+        if (set_smem(k_attn_bwd_dkdv<D, true>, DkvSmem<D>::kBytes) != LIBRA_OK) return LIBRA_ERR_CUDA;
         if (set_smem(k_attn_bwd_dq<D>, DqSmem<D>::kBytes) != LIBRA_OK) return LIBRA_ERR_CUDA;
-        if (!regs_pool_ok(k_attn_bwd_dkdv<D>, 128, kDkvRegsDs, 128, kDkvRegsOther)) return LIBRA_ERR_UNSUPPORTED;
+        if (!regs_pool_ok(k_attn_bwd_dkdv<D, false>, 128, kDkvRegsDs, 128, kDkvRegsOther)) return LIBRA_ERR_UNSUPPORTED;
+        if (!regs_pool_ok(k_attn_bwd_dkdv<D, true>, 128, kDkvRegsDs, 128, kDkvRegsOther)) return LIBRA_ERR_UNSUPPORTED;
         if (!regs_pool_ok(k_attn_bwd_dq<D>, 128 * kDqGroups, kDqRegsCompute, 128, kDqRegsOther)) return LIBRA_ERR_UNSUPPORTED;
         cfg_mark(kSlot);
     }
     time_begin(mp, 1, s);
-    cudaError_t e = launch_dependent(k_attn_bwd_dkdv<D>, Wa, kBwdThreads, DkvSmem<D>::kBytes, s, tq, tk, tv, tdo, pa);
+    cudaError_t e;
+    constexpr size_t bytes = DkvSmem<D>::kBytes;
+    switch (share) {
+        case 8: e = launch_dependent<8>(k_attn_bwd_dkdv<D, true>, Wa / 8 * 8, kBwdThreads, bytes, s, tq, tk, tv, tdo, pa); break;
+        case 4: e = launch_dependent<4>(k_attn_bwd_dkdv<D, true>, Wa / 4 * 4, kBwdThreads, bytes, s, tq, tk, tv, tdo, pa); break;
+        case 2: e = launch_dependent<2>(k_attn_bwd_dkdv<D, true>, Wa / 2 * 2, kBwdThreads, bytes, s, tq, tk, tv, tdo, pa); break;
+        default: e = launch_dependent(k_attn_bwd_dkdv<D, false>, Wa, kBwdThreads, bytes, s, tq, tk, tv, tdo, pa);
+    }
     time_end(mp, 1, s);
     time_begin(mp, 2, s);
     if (e == cudaSuccess)
@@ -873,7 +975,13 @@ extern "C" int libra_attn_pool_bwd(const void* q_dev, const void* k_dev, const v
     pb.wait_limit_ns = plan->wait_limit_ns;
     pb.inject_stall = plan->inject_stall;
     pb.busy = dq_dir.d_busy2;
+    // Several CTAs a dK/dV tile when there are that many for each (the first NT workers then have one tile each) and a key
+    // block's samples give every one of them a few iterations on average.  Not with one query head per kv head: the dQ tiles
+    // are as long then (2000 tokens, 4 / 4 heads of 64: step 53.1 us without, 54.8 with two).
+    const int64_t its = (int64_t)(dims->hq / dims->hkv) * (T / plan->n) / kBlk;
+    int share = dims->hq > dims->hkv ? 8 : 1;
+    while (share > 1 && (share * dkv_dir.NT > dkv_dir.W || 2 * share > its)) share /= 2;
     libra_plan_t* mp = const_cast<libra_plan_t*>(plan);
-    return D == 128 ? launch_bwd<128>(tq, tk, tv, tdo, tdq, pa, dkv_dir.W, pb, dq_dir.W, mp, s)
-                    : launch_bwd<64>(tq, tk, tv, tdo, tdq, pa, dkv_dir.W, pb, dq_dir.W, mp, s);
+    return D == 128 ? launch_bwd<128>(tq, tk, tv, tdo, tdq, pa, dkv_dir.W, share, pb, dq_dir.W, mp, s)
+                    : launch_bwd<64>(tq, tk, tv, tdo, tdq, pa, dkv_dir.W, share, pb, dq_dir.W, mp, s);
 }

@@ -80,6 +80,18 @@ def test_boundary_lengths_and_three_samples_in_one_tile():
     _check(got, ref, cu)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("lengths,hq,hkv", [([1500], 2, 1), ([1301], 8, 1), ([900, 700, 30], 4, 1), ([3000], 4, 1), ([3001], 4, 2),
+                                            ([40, 2000, 1500], 8, 2)])
+def test_tiles_shared_by_a_cluster(lengths, hq, hkv, d):
+    """Few key tiles: 8, 4 or 2 CTAs share the iterations of one (the last tiles have fewer iterations than CTAs), and two
+    runs agree bit by bit."""
+    got, ref, cu = _run(lengths, hq, hkv, d, seed=hq + d)
+    _check(got, ref, cu)
+    for a, b in zip(got, _run(lengths, hq, hkv, d, seed=hq + d)[0]):
+        assert np.array_equal(a, b)
+
+
 def test_peaked_softmax():
     got, ref, cu = _run([700, 900], 2, 2, 64, seed=4, qscale=4.0)
     _check(got, ref, cu)
