@@ -172,7 +172,7 @@ int libra_plan_destroy(libra_plan_t* plan);
  *     out_i = sum_k softmax_k(scale * <q_i, k_k>) v_k,   lse_i = ln sum_k exp(scale * <q_i, k_k>)
  * bf16 inputs, fp32 accumulation and softmax, bf16 out (round to nearest even), fp32 lse
  * (natural log).  One persistent kernel walks the plan's query-major tile lists.  head_dim 256 (the
- * micro-benchmark head shape of Table 1) runs a kernel of its own: one 128-row slot at a time against
+ * micro-benchmark head shape of Table 1) runs a kernel of its own: 256 rows on a pair of CTAs against
  * 64-key blocks, the 256-column output accumulator taking half of the tensor memory.
  * Requires a plan with LIBRA_DIR_Q, tile_q == 256 and n_heads dividing hq.
  * Errors: INVALID_ARG, UNSUPPORTED, PLAN_MISMATCH (plan T != dims->total_tokens), CUDA.
