@@ -211,6 +211,7 @@ size_t libra_attn_pool_bwd_workspace_bytes(const libra_plan_t* plan, const libra
  *   pair-tile plan the dV and dK passes walk the pair tiles instead and add their partial sums to fp32 accumulators
  *   in the workspace (T * hkv * 256 floats each), rounded once at the end; like the fused form, those results agree
  *   to rounding from run to run, not bit for bit.
+ * dq_dev may be q_dev or dout_dev (dq then replaces it); the other outputs overlap no input that is still read.
  * `workspace_dev` must hold libra_attn_pool_bwd_workspace_bytes bytes, 256-byte aligned; every byte the call reads
  * is written (or cleared) inside the call.  Errors: INVALID_ARG, UNSUPPORTED, PLAN_MISMATCH, CUDA.
  */

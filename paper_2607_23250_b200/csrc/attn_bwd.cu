@@ -970,7 +970,7 @@ extern "C" int libra_attn_pool_bwd(const void* q_dev, const void* k_dev, const v
     pb.scale = scale;
     pb.scale_log2 = scale * 1.4426950408889634f;
     pb.outcome = plan->d_outcome[3];
-    pb.side_by_side = side_by_side(dkv_dir.NT, dkv_dir.W);
+    pb.side_by_side = side_by_side(dkv_dir.NT, dkv_dir.W) && !dq_in_place(dq_dev, q_dev, dout_dev, dims);
     pb.plan_status = plan->d_status;
     pb.wait_limit_ns = plan->wait_limit_ns;
     pb.inject_stall = plan->inject_stall;

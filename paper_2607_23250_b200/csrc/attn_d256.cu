@@ -802,6 +802,7 @@ int launch_bwd_d256(const void* q, const void* k, const void* v, const void* dou
     prm.cta_offsets = dq_dir.d_cta_offsets; prm.cta_tiles = dq_dir.d_cta_exec; prm.busy = dq_dir.d_busy2;
     prm.out = reinterpret_cast<__nv_bfloat16*>(dq);
     prm.outcome = plan->d_outcome[3];
+    if (dq_in_place(dq, q, dout, dims)) prm.side_by_side = 0;
     time_begin(mp, 2, s);
     rc = launch<DQ>(q128, do128, k32, v32, k64, prm, dq_dir.W, s);
     time_end(mp, 2, s);

@@ -146,6 +146,13 @@ static inline cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned gr
 // 21.9 -> 19.2, 130 -> 115 ms; 128 / 4 heads of 256 on 32768 tokens, pair tiles (11.6): 99.9 -> 103.4 ms.
 constexpr int64_t kOverlapTiles = 8;   // per worker
 inline bool side_by_side(int64_t tiles, int workers) { return tiles <= kOverlapTiles * workers; }
+// dq may be written over q or dout: a kernel that writes dq reads of either only the tile it is about to replace, once the
+// kernels ahead, which read all of both, are done.  Such a call's dQ kernel waits for them.
+inline bool dq_in_place(const void* dq, const void* q, const void* dout, const libra_dims* dims) {
+    const uintptr_t n = (uintptr_t)dims->total_tokens * dims->hq * dims->head_dim * 2, a = (uintptr_t)dq;
+    auto meets = [&](const void* p) { return a < (uintptr_t)p + n && (uintptr_t)p < a + n; };
+    return meets(q) || meets(dout);
+}
 
 // setmaxnreg moves registers inside the pool the CTA got at launch (registers per thread as compiled x
 // threads): what the shrinking warps release must cover what the growing warps ask for, or the last

@@ -48,3 +48,22 @@ def test_back_to_back_passes(d, hq, hkv, pairs, T):
             else:
                 assert torch.equal(a, b), k
     plan.destroy()
+
+
+@pytest.mark.parametrize("d,hq,hkv,T", [(64, 4, 4, 4096), (128, 8, 2, 9000), (128, 4, 1, 300), (256, 4, 1, 3000)])
+@pytest.mark.parametrize("name", ["q", "dout"])
+def test_dq_in_place(d, hq, hkv, T, name):
+    """dq written over q or over dout, with few enough tiles that the dQ kernel could run beside the kernel ahead of it, which
+    reads all of both.  Bit for bit the results of a call with buffers of its own (the two-kernel forms are reproducible)."""
+    from paper_2607_23250_b200 import binding as lb
+    cu = torch.from_numpy(pools.cu_seqlens([T])).cuda()
+    plan = lb.libra_plan_tiles(cu, hq, 256, tile_kv=128, n_heads_kv=hkv)
+    t = pools.make_tensors(T, hq, hkv, d, seed=5, device="cuda")
+    out, lse = lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
+    want = lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan)
+    for _ in range(3):
+        x = {n: v.clone() for n, v in t.items()}
+        got = lb.libra_attn_pool_bwd(x["q"], x["k"], x["v"], out, lse, x["dout"], plan, dq=x[name])
+        for a, b in zip(got, want):
+            assert torch.equal(a, b)
+    plan.destroy()
