@@ -340,7 +340,8 @@ int libra_tap_schedule(const int32_t* cu_seqlens_dev, int n_samples, const int32
 /* ---- instrumentation -------------------------------------------------------------------
  * Per-CTA busy time of the most recent launch of kernel `which` (LIBRA_KERNEL_*) that used this
  * plan: nanoseconds between the CTA starting and finishing its tile list, read with the GPU's
- * global timer.  Copies n_workers values to ns_host and synchronises the device.  Returns the
+ * global timer.  Copies n_workers values to ns_host (0 for workers that the launch had no CTA for) and
+ * synchronises the device.  Returns the
  * status of the most recent forward (LIBRA_KERNEL_FWD) or backward (the other two) launch:
  * LIBRA_OK, LIBRA_ERR_TIMEOUT if a bounded wait gave up, LIBRA_ERR_BAD_SEQLENS if the plan's
  * cu_seqlens was malformed and the kernels therefore did no work. */

@@ -747,11 +747,14 @@ static int launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtens
     time_begin(mp, 1, s);
     cudaError_t e;
     constexpr size_t bytes = DkvSmem<D>::kBytes;
+    const unsigned grid = Wa / share * share;
+    mp->n_outcome[1] = (int)grid;
+    mp->n_outcome[3] = Wb;
     switch (share) {
-        case 8: e = launch_dependent<8>(k_attn_bwd_dkdv<D, true>, Wa / 8 * 8, kBwdThreads, bytes, s, tq, tk, tv, tdo, pa); break;
-        case 4: e = launch_dependent<4>(k_attn_bwd_dkdv<D, true>, Wa / 4 * 4, kBwdThreads, bytes, s, tq, tk, tv, tdo, pa); break;
-        case 2: e = launch_dependent<2>(k_attn_bwd_dkdv<D, true>, Wa / 2 * 2, kBwdThreads, bytes, s, tq, tk, tv, tdo, pa); break;
-        default: e = launch_dependent(k_attn_bwd_dkdv<D, false>, Wa, kBwdThreads, bytes, s, tq, tk, tv, tdo, pa);
+        case 8: e = launch_dependent<8>(k_attn_bwd_dkdv<D, true>, grid, kBwdThreads, bytes, s, tq, tk, tv, tdo, pa); break;
+        case 4: e = launch_dependent<4>(k_attn_bwd_dkdv<D, true>, grid, kBwdThreads, bytes, s, tq, tk, tv, tdo, pa); break;
+        case 2: e = launch_dependent<2>(k_attn_bwd_dkdv<D, true>, grid, kBwdThreads, bytes, s, tq, tk, tv, tdo, pa); break;
+        default: e = launch_dependent(k_attn_bwd_dkdv<D, false>, grid, kBwdThreads, bytes, s, tq, tk, tv, tdo, pa);
     }
     time_end(mp, 1, s);
     time_begin(mp, 2, s);
@@ -834,6 +837,7 @@ static int launch_fused(const void* q_dev, const void* k_dev, const void* v_dev,
     fp.wait_limit_ns = plan->wait_limit_ns; fp.inject_stall = plan->inject_stall;
     fp.busy = d.d_busy;
     fp.tile_ns = d.d_tile_ns;
+    mp->n_outcome[1] = d.W;
     time_begin(mp, 4, s);
     cudaError_t e = launch_dependent(k_attn_bwd_fused, d.W, kFusedThreads, FusedSmem::kBytes, s, tq, tk, tv, tdo, tacc, tdkacc,
                                      tdvacc, fp);

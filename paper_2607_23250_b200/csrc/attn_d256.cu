@@ -48,7 +48,7 @@ constexpr int kD = 256;
 constexpr uint32_t kColAcc = 256;
 constexpr uint64_t kDrainNs = 2000000;
 constexpr int kSmemMax = 232448;
-enum Mode { FWD = 0, DV = 1, DK = 2, DQ = 3 };
+enum Mode { FWD = 0, DV = 1, DK = 2, DQ = 3 };   // (also the index of the pass's outcome words)
 
 template <int MODE>
 struct Cfg {
@@ -705,7 +705,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
 
 template <int MODE>
 static int launch(const CUtensorMap& sa, const CUtensorMap& sb, const CUtensorMap& t0, const CUtensorMap& t1, const CUtensorMap& t2,
-                  const Params& prm, int W, cudaStream_t s) {
+                  const Params& prm, int W, libra_plan* mp, cudaStream_t s) {
     using L = Cfg<MODE>;
     if (!cfg_done(8 + MODE)) {   // per device
         if (cudaFuncSetAttribute(k_attn_d256<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kBytes) != cudaSuccess)
@@ -714,6 +714,7 @@ static int launch(const CUtensorMap& sa, const CUtensorMap& sb, const CUtensorMa
     }
     count_launch();
     const unsigned grid = 2 * ((W + 1) / 2);   // a pair of CTAs for every two workers
+    mp->n_outcome[MODE] = (int)grid;
     return launch_dependent(k_attn_d256<MODE>, grid, kThreads, L::kBytes, s, sa, sb, t0, t1, t2, prm) == cudaSuccess ? LIBRA_OK
                                                                                                                 : LIBRA_ERR_CUDA;
 }
@@ -744,7 +745,7 @@ int launch_fwd_d256(const void* q, const void* k, const void* v, void* out, floa
     prm.outcome = plan->d_outcome[0]; prm.plan_status = plan->d_status;
     prm.wait_limit_ns = plan->wait_limit_ns; prm.inject_stall = plan->inject_stall;
     prm.busy = d.d_busy;
-    return launch<FWD>(tq, tq, tk, tv, to, prm, d.W, s);
+    return launch<FWD>(tq, tq, tk, tv, to, prm, d.W, const_cast<libra_plan*>(plan), s);
 }
 
 // Backward at head_dim 256: the dV and dK passes over the key-major lists, the dQ pass over the query-major lists.
@@ -788,13 +789,13 @@ int launch_bwd_d256(const void* q, const void* k, const void* v, const void* dou
     time_begin(mp, 1, s);
     prm.out = reinterpret_cast<__nv_bfloat16*>(dv);
     prm.acc32 = dv_acc;
-    rc = launch<DV>(k128, k128, q32, do64, do64, prm, plan->W, s);
+    rc = launch<DV>(k128, k128, q32, do64, do64, prm, plan->W, mp, s);
     prm.out = reinterpret_cast<__nv_bfloat16*>(dk);
     prm.acc32 = dk_acc;
     prm.outcome = plan->d_outcome[2];
     prm.side_by_side = side_by_side(kv_dir.NT, kv_dir.W);
     prm.busy = plan->dir[pairs ? 2 : 1].d_busy;
-    if (rc == LIBRA_OK) rc = launch<DK>(k128, v128, q32, do32, q64, prm, plan->W, s);
+    if (rc == LIBRA_OK) rc = launch<DK>(k128, v128, q32, do32, q64, prm, plan->W, mp, s);
     time_end(mp, 1, s);
     prm.acc32 = nullptr;
     if (rc != LIBRA_OK) return rc;
@@ -804,7 +805,7 @@ int launch_bwd_d256(const void* q, const void* k, const void* v, const void* dou
     prm.outcome = plan->d_outcome[3];
     if (dq_in_place(dq, q, dout, dims)) prm.side_by_side = 0;
     time_begin(mp, 2, s);
-    rc = launch<DQ>(q128, do128, k32, v32, k64, prm, dq_dir.W, s);
+    rc = launch<DQ>(q128, do128, k32, v32, k64, prm, dq_dir.W, mp, s);
     time_end(mp, 2, s);
     return rc;
 }

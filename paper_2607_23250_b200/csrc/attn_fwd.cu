@@ -670,7 +670,7 @@ int make_f32_3d_map(CUtensorMap* m, const void* base, int64_t T, int H, int d, i
 
 template <int D, bool PAIR>
 static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tout,
-                      const FwdParams& prm, int W, cudaStream_t s) {
+                      const FwdParams& prm, int W, libra_plan_t* mp, cudaStream_t s) {
     using L = FwdSmem<D>;
     constexpr int kSlot = (D == 128 ? 0 : 1) + (PAIR ? 5 : 0);
     if (!cfg_done(kSlot)) {   // per device: the attribute belongs to the device's copy of the kernel
@@ -680,7 +680,8 @@ static int launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtens
         cfg_mark(kSlot);
     }
     count_launch();
-    const cudaError_t e = launch_dependent<PAIR ? 2 : 1>(k_attn_fwd<D, PAIR>, PAIR ? W / 2 * 2 : W, kFwdThreads, L::kAlloc, s, tq, tk, tv,
+    mp->n_outcome[0] = PAIR ? W / 2 * 2 : W;
+    const cudaError_t e = launch_dependent<PAIR ? 2 : 1>(k_attn_fwd<D, PAIR>, mp->n_outcome[0], kFwdThreads, L::kAlloc, s, tq, tk, tv,
                                                          tout, prm);
     return e == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
@@ -744,9 +745,9 @@ extern "C" int libra_attn_pool_fwd(const void* q_dev, const void* k_dev, const v
     // up to 300 / 800 / 4000 tokens took 12.0 / 18.0 / 55.3 us with one CTA a tile and 14.0 / 18.4 / 38.1 with two.
     const bool pair = d.NT <= d.W / 2 && d.H == dims->hq && plan->T >= 4 * kBN * (int64_t)plan->n;
     if (dims->head_dim == 128)
-        rc = pair ? launch_fwd<128, true>(tq, tk, tv, tout, prm, d.W, s) : launch_fwd<128, false>(tq, tk, tv, tout, prm, d.W, s);
+        rc = pair ? launch_fwd<128, true>(tq, tk, tv, tout, prm, d.W, mp, s) : launch_fwd<128, false>(tq, tk, tv, tout, prm, d.W, mp, s);
     else
-        rc = pair ? launch_fwd<64, true>(tq, tk, tv, tout, prm, d.W, s) : launch_fwd<64, false>(tq, tk, tv, tout, prm, d.W, s);
+        rc = pair ? launch_fwd<64, true>(tq, tk, tv, tout, prm, d.W, mp, s) : launch_fwd<64, false>(tq, tk, tv, tout, prm, d.W, mp, s);
     time_end(mp, 0, s);
     return rc;
 }

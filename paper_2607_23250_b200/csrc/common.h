@@ -52,7 +52,8 @@ struct libra_plan {
     int* d_status = nullptr;         // the planner's verdict on cu_seqlens
     // Outcome of each CTA of the last launch of a kernel (0 or LIBRA_ERR_*), written by every CTA when it leaves, so
     // that nothing has to be cleared before a launch: forward; dK/dV, fused or dV pass; dK pass; dQ kernel or pass.
-    int* d_outcome[4] = {};          // [W] each
+    int* d_outcome[4] = {};          // [W + 1] each: kernels on pairs of CTAs round the workers up to even
+    int n_outcome[4] = {};           // CTAs of that launch: clusters leave the last workers out, pairs may add one
     int W = 0;                       // workers of every direction
     int bwd_mask = 0;                // which of d_outcome[1..3] the last backward wrote
     // 0 = query-major, 1 = key-major, 2 = pair tiles (key block x query chunk), 3 = the key-stationary tiles of kernels that

@@ -798,20 +798,24 @@ extern "C" int libra_busy_times(const libra_plan_t* plan, int which, uint64_t* n
                                                               : (which == LIBRA_KERNEL_BWD_DKDV ? LIBRA_DIR_KV : LIBRA_DIR_Q));
     if (!d) return LIBRA_ERR_PLAN_MISMATCH;
     if (cudaDeviceSynchronize() != cudaSuccess) return LIBRA_ERR_CUDA;
-    uint64_t* tmp = new (std::nothrow) uint64_t[3 * (size_t)d->W];   // the stamps, then one kernel's outcomes
+    const size_t most = (size_t)d->W + 1;
+    uint64_t* tmp = new (std::nothrow) uint64_t[3 * most];   // the stamps, then one kernel's outcomes
     if (!tmp) return LIBRA_ERR_CUDA;
-    int* outcome = reinterpret_cast<int*>(tmp + 2 * (size_t)d->W);
+    int* outcome = reinterpret_cast<int*>(tmp + 2 * most);
     int st = 0;
     const uint64_t* src = which == LIBRA_KERNEL_BWD_DQ ? d->d_busy2 : d->d_busy;
     cudaError_t e = cudaMemcpy(tmp, src, sizeof(uint64_t) * 2 * d->W, cudaMemcpyDeviceToHost);
     const int mask = which == LIBRA_KERNEL_FWD ? 1 : plan->bwd_mask;
     for (int k = 0; k < 4 && e == cudaSuccess; ++k) {
         if (!((mask >> k) & 1)) continue;
-        e = cudaMemcpy(outcome, plan->d_outcome[k], sizeof(int) * d->W, cudaMemcpyDeviceToHost);
-        for (int r = 0; r < d->W && e == cudaSuccess; ++r)
+        const int n = plan->n_outcome[k];   // words beyond are an earlier launch's
+        e = cudaMemcpy(outcome, plan->d_outcome[k], sizeof(int) * n, cudaMemcpyDeviceToHost);
+        for (int r = 0; r < n && e == cudaSuccess; ++r)
             if (outcome[r] != 0) st = outcome[r];
     }
-    for (int r = 0; r < d->W; ++r) ns_host[r] = tmp[2 * r + 1] >= tmp[2 * r] ? tmp[2 * r + 1] - tmp[2 * r] : 0;
+    const int ran = plan->n_outcome[which == LIBRA_KERNEL_FWD ? 0 : (which == LIBRA_KERNEL_BWD_DQ ? 3 : 1)];
+    for (int r = 0; r < d->W; ++r)
+        ns_host[r] = r < ran && tmp[2 * r + 1] >= tmp[2 * r] ? tmp[2 * r + 1] - tmp[2 * r] : 0;
     delete[] tmp;
     if (e != cudaSuccess) return LIBRA_ERR_CUDA;
     return st;

@@ -198,3 +198,58 @@ def test_tile_times_cover_every_tile_that_ran():
         plan.tile_times(lb.KERNEL_BWD_DQ)
     assert err.value.code == lb.ERR_INVALID_ARG
     plan.destroy()
+
+
+def _stalled(plan, call, kern):
+    """`call` with the producers stalled and a budget of 0.2 ms: reports TIMEOUT.  Leaves the plan's settings as they were."""
+    from paper_2607_23250_b200 import binding as lb
+    plan.set_wait_limit_ns(200_000)
+    plan.inject_stall(True)
+    call()
+    plan.inject_stall(False)
+    plan.set_wait_limit_ns(0)
+    with pytest.raises(lb.LibraError) as err:
+        plan.busy_times(kern)
+    assert err.value.code == lb.ERR_TIMEOUT
+
+
+def test_outcome_of_a_smaller_launch_after_a_stalled_one():
+    """A stalled launch on all 148 workers (the fused backward of 171 pair tiles), then on the same plan one in clusters of
+    eight, 144 CTAs: its outcome is its own, and workers it had no CTA for have no busy time."""
+    from paper_2607_23250_b200 import binding as lb
+    T, hq, hkv = 2300, 8, 1
+    cu = torch.tensor([0, T], dtype=torch.int32).cuda()
+    plan = lb.libra_plan_tiles(cu, hq, 256, n_workers=148, directions=lb.LIBRA_DIR_Q | lb.LIBRA_DIR_KV | lb.LIBRA_DIR_PAIR,
+                               tile_kv=128, n_heads_kv=hkv, pair_chunk=128)
+    for d, stall in ((128, True), (64, False)):
+        t = pools.make_tensors(T, hq, hkv, d, seed=1, device="cuda")
+        out, lse = lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
+
+        def bwd():
+            lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan)
+        if stall:
+            _stalled(plan, bwd, lb.KERNEL_BWD_FUSED)
+        else:
+            bwd()
+    busy = plan.busy_times(lb.KERNEL_BWD_DKDV)
+    assert (busy[:144] > 0).all() and (busy[144:] == 0).all()
+    plan.destroy()
+
+
+def test_outcome_of_an_odd_number_of_workers():
+    """One worker at head_dim 256 is a pair of CTAs: the outcome words of both are read, busy times are the worker's."""
+    from paper_2607_23250_b200 import binding as lb
+    T, hq, hkv, d = 700, 2, 1, 256
+    cu = torch.tensor([0, T], dtype=torch.int32).cuda()
+    plan = lb.libra_plan_tiles(cu, hq, 256, n_workers=1, tile_kv=128, n_heads_kv=hkv)
+    t = pools.make_tensors(T, hq, hkv, d, seed=1, device="cuda")
+
+    def fwd():
+        return lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
+    out, lse = fwd()
+    assert plan.busy_times(lb.KERNEL_FWD).shape == (1,)
+    _stalled(plan, fwd, lb.KERNEL_FWD)
+    _stalled(plan, lambda: lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan), lb.KERNEL_BWD_DKDV)
+    again, _ = fwd()
+    assert (plan.busy_times(lb.KERNEL_FWD) > 0).all() and torch.equal(again, out)
+    plan.destroy()
