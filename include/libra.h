@@ -118,11 +118,12 @@ typedef struct {
  * With opts->weight_model = LIBRA_WEIGHT_BLOCKS the weight is the block count described at
  * LIBRA_WEIGHT_BLOCKS above; everything else is unchanged.
  * Errors: INVALID_ARG (null, n_samples <= 0, n_heads <= 0, tile_q <= 0, a negative option,
- * an unknown weight model), OVERFLOW (n_heads * T^2 >= 9e15, the bound under which loads fit the
- * placement's packed keys, or NB * H >= 2^31), CUDA.  A malformed cu_seqlens is detected on the
- * device and reported by libra_plan_status as BAD_SEQLENS; the per-token sample bounds of such a
- * plan are clamped into [0, T], and the attention kernels given it do no work: they leave their
- * outputs untouched and report BAD_SEQLENS through libra_busy_times.
+ * an unknown weight model), OVERFLOW (n_heads * T^2 >= 9e15, the bound under which pair-count loads fit
+ * the placement's packed keys, or NB * H >= 2^31), CUDA.  Found on the device and reported by
+ * libra_plan_status: BAD_SEQLENS, a malformed cu_seqlens (the per-token sample bounds of such a plan are
+ * clamped into [0, T]), and OVERFLOW, a block-count load (LIBRA_WEIGHT_BLOCKS) beyond the packed keys' 54
+ * bits.  The attention kernels given such a plan do no work: they leave their outputs untouched and report
+ * the same code through libra_busy_times.
  */
 int libra_plan_tiles(const int32_t* cu_seqlens_dev, int n_samples, int n_heads, int tile_q,
                      const libra_plan_opts* opts /* nullable */, void* stream,
@@ -343,8 +344,8 @@ int libra_tap_schedule(const int32_t* cu_seqlens_dev, int n_samples, const int32
  * global timer.  Copies n_workers values to ns_host (0 for workers that the launch had no CTA for) and
  * synchronises the device.  Returns the
  * status of the most recent forward (LIBRA_KERNEL_FWD) or backward (the other two) launch:
- * LIBRA_OK, LIBRA_ERR_TIMEOUT if a bounded wait gave up, LIBRA_ERR_BAD_SEQLENS if the plan's
- * cu_seqlens was malformed and the kernels therefore did no work. */
+ * LIBRA_OK, LIBRA_ERR_TIMEOUT if a bounded wait gave up, or the plan's own status (libra_plan_status) when that is
+ * not OK and the kernels therefore did no work. */
 int libra_busy_times(const libra_plan_t* plan, int which, uint64_t* ns_host);
 
 /* Time each tile took in the most recent launch of the forward kernel (which = LIBRA_KERNEL_FWD, tiles of the

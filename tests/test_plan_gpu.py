@@ -83,6 +83,23 @@ def test_block_model_rejects_bad_options():
             lb.libra_plan_tiles(cu, 1, 4, n_workers=2, **kw)
 
 
+@pytest.mark.parametrize("unit,fits", [(2 ** 31 - 600_000, True), (2 ** 31 - 1, False)])
+def test_block_model_loads_beyond_the_packed_keys(unit, fits):
+    """2^17 tokens, 64 head shards, one worker, a chunk per token: the load is 64 (8 T (T + 1) / 2 + T unit), just under and just
+    over the 54 bits that the placement's keys have for it."""
+    from paper_2607_23250_b200 import binding as lb
+    T, H = 1 << 17, 64
+    load = H * (4 * T * (T + 1) + T * unit)
+    cu = torch.tensor([0, T], dtype=torch.int32).cuda()
+    plan = lb.libra_plan_tiles(cu, H, 256, n_workers=1, directions=lb.LIBRA_DIR_Q, weight_model=lb.LIBRA_WEIGHT_BLOCKS,
+                               cost_block=1, unit_cost_q=unit)
+    if fits:
+        assert load < 1 << 54 and plan.status() == 0 and plan.export()["loads"].tolist() == [load]
+    else:
+        assert load > 1 << 54 and plan.status() == lb.ERR_OVERFLOW
+    plan.destroy()
+
+
 def test_edge_cases():
     _compare(np.array([0, 1], dtype=np.int32), 1, 256, 148)                      # one token
     _compare(np.array([0, 0, 3, 3, 3, 700, 700], dtype=np.int32), 2, 256, 5)     # empty samples, ragged tail
