@@ -35,6 +35,7 @@
 #include <math.h>
 
 #include "common.h"
+#include "drain.cuh"
 #include "ptx.cuh"
 
 namespace libra {
@@ -78,7 +79,7 @@ struct Cfg {
     // acc_step[2], st_full[2], st_empty[2], l_full[3]
     static constexpr int kNumBars = 2 * kStreams * kStages + kStages + 19;
     static constexpr int kMiscOff = kBarOff + kNumBars * 8;
-    static constexpr int kBytes = kMiscOff + 16;
+    static constexpr int kBytes = kMiscOff + 32;
     static_assert(kBytes <= kSmemMax, "exceeds the shared memory of an sm_100 CTA");
     // TMEM columns of a block's X1, X2 and W (see above)
     static constexpr uint32_t kX1Bufs = kHasX2 ? 2 : 3;
@@ -206,6 +207,8 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
     uint64_t* bar_lfull = b2 + 16;     // [3] FWD: the row sums of a unit are there
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kMiscOff);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMiscOff + 4);
+    volatile uint32_t* peer_gave_up = reinterpret_cast<volatile uint32_t*>(smem + L::kMiscOff + 12);
+    volatile uint32_t* issued = peer_gave_up + 1;   // [2][2] leader: units and streamed tiles whose loads either CTA has issued
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -245,6 +248,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
         mbar_init(bar_drain, 1);
         abort_flag[0] = 0;
         abort_flag[1] = (int)p.wait_limit_ns;
+        *peer_gave_up = 0;
         fence_mbar_init();
         p.busy[2 * cta] = globaltimer_ns();
     }
@@ -270,8 +274,9 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
         if (elect_one()) {
             Units<MODE> u(p, cta);
             uint32_t n = 0, uc = 0;          // n: iterations so far (over all units)
+            uint32_t tiles = 0;
             bool ok = true;
-            while (ok && !p.inject_stall && u.next(rank)) {
+            while (ok && !(p.inject_stall && rank == 1) && u.next(rank)) {
                 const uint32_t sbuf = uc % L::kStBufs, a_off = L::kSaOff + sbuf * L::kBig;
                 ok = mbar_wait(&bar_stempty[sbuf], ((uc / L::kStBufs) & 1) ^ 1, abort_flag);
                 if (!ok) break;
@@ -307,13 +312,17 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                             if (L::kStatBytes == 512)
                                 bulk_load_1d(smem + L::kStatOff + s * 512 + 256, p.dvec + (size_t)sh * p.Tpad + row, 256, &bar_stat[s]);
                         }
+                        ++tiles;
                     }
                     if (++j == u.n_blk) { j = 0; ++sh; }
                 }
             }
-            if (!ok || abort_flag[0]) {   // give-up path: the copies already issued land before shared memory is released
-                const uint64_t t0 = globaltimer_ns();
-                while (globaltimer_ns() - t0 < kDrainNs) {}
+            issued[2 * rank] = uc;
+            issued[2 * rank + 1] = tiles;
+            if (rank == 1) {
+                const uint32_t there = map_to_rank(const_cast<const uint32_t*>(issued) + 2, 0);
+                st_cluster(there, uc);
+                st_cluster(there + 4, tiles);
             }
         }
         __syncwarp();
@@ -693,7 +702,32 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
     // ---------------- teardown ----------------
     tc_fence_before();
     __syncthreads();
-    cluster_sync();      // nothing of the other CTA is on its way here any more
+    if (threadIdx.x == 0 && abort_flag[0]) st_cluster(map_to_rank(const_cast<const uint32_t*>(peer_gave_up), rank ^ 1), 1u);
+    cluster_sync();      // no role of either CTA runs any more
+    if (abort_flag[0] | (int)*peer_gave_up) {   // give-up path: the copies already issued land before the CTAs leave
+        if (threadIdx.x == 0) {
+            if (rank == 0) {
+                // a half that never was issued is counted as arrived, one that the leader had not got to is expected now
+                auto land = [&](uint64_t* bar, uint32_t parity, bool mine, bool peers, uint32_t half) {
+                    if (!mine) mbar_arrive_expect_tx(bar, half);
+                    if (!peers) mbar_complete_tx(bar, half);
+                    mbar_wait_drain(bar, parity, kDrainNs);
+                };
+                open_loads(issued[0], issued[2], L::kStBufs, [](uint32_t m) { return m % L::kStBufs; },
+                           [&](uint32_t b, uint32_t parity, bool mine, bool peers) {
+                               land(&bar_stfull[b], parity, mine, peers, L::kStationary * L::kBig);
+                           });
+                open_loads(issued[1], issued[3], N * S, [](uint32_t m) { return stream_barrier(m, N, S); },
+                           [&](uint32_t b, uint32_t parity, bool mine, bool peers) {
+                               land(&bar_full[b], parity, mine, peers, L::kHalfTile);
+                           });
+            }
+            if (L::kStatBytes > 0)               // issued with the last of a block's tiles, counted by this CTA alone
+                open_loads(issued[2 * rank + 1] / N, 0, S, [](uint32_t m) { return m % S; },
+                           [&](uint32_t b, uint32_t parity, bool, bool) { mbar_wait_drain(&bar_stat[b], parity, kDrainNs); });
+        }
+        cluster_sync();  // the leader's wait is for the other CTA's copies, too
+    }
     tc_fence_after();
     if (warp == kMmaWarp) tmem_dealloc_pair(tmem_base, 512);
     if (threadIdx.x == 0) {

@@ -198,3 +198,42 @@ def test_give_up_path_of_the_256_wide_kernel():
     for g, r in zip((dq, dk, dv), ref):
         assert np.abs(g.float().cpu().numpy() - r).max() <= TOL_G * np.abs(r).max()
     plan.destroy()
+
+
+@pytest.mark.parametrize("pairs", [False, True])
+def test_give_up_path_with_copies_under_way(pairs):
+    """The stall leaves out the loads of one CTA of each pair only: the other's have been issued and half of what their
+    barriers count never comes.  Each pass gives up after its budget of 0.2 ms and counts the missing halves as arrived,
+    so that it is done well before one wait for copies in flight would have run out (2 ms)."""
+    from paper_2607_23250_b200 import binding as lb
+    T, hq, hkv = 3000, 4, 2
+    cu = torch.tensor([0, 1000, T], dtype=torch.int32).cuda()
+    directions = lb.LIBRA_DIR_Q | (lb.LIBRA_DIR_PAIR if pairs else lb.LIBRA_DIR_KV)
+    plan = lb.libra_plan_tiles(cu, hq, 256, directions=directions, tile_kv=128, n_heads_kv=hkv)
+    t = pools.make_tensors(T, hq, hkv, D, seed=12, device="cuda")
+    out, lse = lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
+    good = lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan)
+    torch.cuda.synchronize()
+    plan.set_timing(True)
+    plan.set_wait_limit_ns(200_000)
+    plan.inject_stall(True)
+    lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
+    lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan)
+    plan.inject_stall(False)
+    plan.set_wait_limit_ns(0)
+    for kern in (lb.KERNEL_FWD, lb.KERNEL_BWD_FUSED if pairs else lb.KERNEL_BWD_DKDV):
+        with pytest.raises(lb.LibraError) as err:
+            plan.busy_times(kern)
+        assert err.value.code == lb.ERR_TIMEOUT
+    for kern in (lb.KERNEL_FWD, lb.KERNEL_BWD_DKDV, lb.KERNEL_BWD_DQ):
+        assert 0.2 <= plan.kernel_time_ms(kern) < 2.0
+    plan.set_timing(False)
+    again, _ = lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
+    grads = lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan)
+    torch.cuda.synchronize()
+    plan.busy_times(lb.KERNEL_FWD)
+    plan.busy_times(lb.KERNEL_BWD_FUSED if pairs else lb.KERNEL_BWD_DKDV)
+    assert torch.equal(again, out)
+    for a, b in zip(grads, good):   # sums in another order with pair tiles: one rounding of bf16 results
+        assert (a.float() - b.float()).abs().max() <= (2.0 ** -7 * b.float().abs().max() if pairs else 0)
+    plan.destroy()
