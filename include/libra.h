@@ -365,8 +365,9 @@ int libra_tile_times(const libra_plan_t* plan, int which, uint32_t* ns_host);
 int libra_plan_set_wait_limit_ns(libra_plan_t* plan, uint64_t ns);
 
 /* Test aid (no counterpart in the paper): while enabled, the producer role of the attention kernels launched
- * with this plan issues no loads at all (where two CTAs load halves of the same tiles, at head_dim 256, that of
- * one of them does not), so every consumer's first wait runs out of its budget on an otherwise healthy GPU.  This is how the give-up path is exercised without a fault or an endless loop: set a
+ * with this plan issues no loads at all, so every consumer's first wait runs out of its budget on an otherwise
+ * healthy GPU.  Where CTAs of a cluster work on the same tile only every other one's producer stalls, so that the
+ * rest wait for them.  This is how the give-up path is exercised without a fault or an endless loop: set a
  * short budget with libra_plan_set_wait_limit_ns, launch, and libra_busy_times reports LIBRA_ERR_TIMEOUT; the
  * outputs of such a launch are undefined.  Off by default. */
 int libra_plan_inject_stall(libra_plan_t* plan, int enabled);

@@ -81,7 +81,7 @@ struct DkvParams {
     int* outcome;            // [gridDim.x] 0 or what kept this CTA from doing its work
     const int* plan_status;  // the planner's verdict on cu_seqlens: non-zero = do not run
     uint32_t wait_limit_ns;
-    int inject_stall;        // test aid: the producer issues no loads, so the consumers' waits run out
+    int inject_stall;        // test aid: the producer (SHARE: of odd ranks) issues no loads, so the consumers' waits run out
     uint64_t* busy;
 };
 
@@ -271,7 +271,7 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if (elect_one()) {  // one elected thread runs the whole role
             uint32_t ucnt = 0, it_all = 0;
             bool ok = true;
-            for (int idx = unit_begin; idx < unit_end && ok && !p.inject_stall; ++idx) {
+            for (int idx = unit_begin; idx < unit_end && ok && !(p.inject_stall && (!SHARE || rank % 2 == 1)); ++idx) {
                 const int t = p.cta_tiles[idx];
                 const int kvh = t % p.hkv;
                 const int64_t k0 = (int64_t)(t / p.hkv) * kBlk;

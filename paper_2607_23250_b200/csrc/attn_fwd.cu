@@ -71,7 +71,7 @@ struct FwdParams {
     int* outcome;      // [gridDim.x] 0 or what kept this CTA from doing its work
     const int* plan_status;  // the planner's verdict on cu_seqlens: non-zero = do not run
     uint32_t wait_limit_ns;  // budget of one device-side wait
-    int inject_stall;        // test aid: the producer issues no loads, so the consumers' waits run out
+    int inject_stall;        // test aid: the producer (PAIR: of rank 1) issues no loads, so the consumers' waits run out
     uint64_t* busy;    // [2 * gridDim.x]
     uint32_t* tile_ns; // [tiles] time spent on each tile (slot 0's first softmax thread), ns
 };
@@ -286,7 +286,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             bool ok = true;
             FwdTiles tiles(p, tile_begin, tile_end);
             FwdTile x;
-            while (ok && !p.inject_stall && tiles.next(x)) {
+            while (ok && !(p.inject_stall && (!PAIR || rank == 1)) && tiles.next(x)) {
                 if (PAIR && !x.take_half(cluster_rank())) continue;
                 const bool act1 = x.hi[1] >= 0;
                 const int top = act1 ? x.hi[1] : x.hi[0];

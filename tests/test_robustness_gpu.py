@@ -213,6 +213,36 @@ def _stalled(plan, call, kern):
     assert err.value.code == lb.ERR_TIMEOUT
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("lengths,hq,hkv", [([3000], 2, 1), ([1500], 2, 1), ([3000], 4, 1), ([3001], 4, 2)])
+def test_shared_tiles_give_up_cleanly_when_half_of_the_producers_stall(lengths, hq, hkv, d):
+    """Forward tiles shared by two CTAs, dK/dV tiles shared by 4, 8, 4 and 2: every other CTA's loads stay out, so the rest
+    finish their part and wait for partial results that never come.  Every kernel reports TIMEOUT, and the next
+    passes on the same plan give the same bits as the passes before."""
+    from paper_2607_23250_b200 import binding as lb
+    cu_np = pools.cu_seqlens(lengths)
+    t = pools.make_tensors(int(cu_np[-1]), hq, hkv, d, seed=6, device="cuda")
+    plan = lb.libra_plan_tiles(torch.from_numpy(cu_np).cuda(), hq, 256, tile_kv=128, n_heads_kv=hkv)
+
+    def fwd():
+        return lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
+
+    def bwd():
+        return lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan)
+    out, lse = fwd()
+    want = [out, lse, *bwd()]
+    torch.cuda.synchronize()
+    _stalled(plan, fwd, lb.KERNEL_FWD)
+    _stalled(plan, bwd, lb.KERNEL_BWD_DKDV)
+    got = [*fwd(), *bwd()]
+    torch.cuda.synchronize()
+    for kern in (lb.KERNEL_FWD, lb.KERNEL_BWD_DKDV, lb.KERNEL_BWD_DQ):
+        plan.busy_times(kern)
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+    plan.destroy()
+
+
 def test_outcome_of_a_smaller_launch_after_a_stalled_one():
     """A stalled launch on all 148 workers (the fused backward of 171 pair tiles), then on the same plan one in clusters of
     eight, 144 CTAs: its outcome is its own, and workers it had no CTA for have no busy time."""
