@@ -67,3 +67,41 @@ def test_dq_in_place(d, hq, hkv, T, name):
         for a, b in zip(got, want):
             assert torch.equal(a, b)
     plan.destroy()
+
+
+@pytest.mark.parametrize("side_stream", [False, True])
+@pytest.mark.parametrize("d", [64, 256])
+def test_plans_destroyed_behind_their_last_pass(d, side_stream):
+    """Plan, forward, backward, destroy, over and over with another layout each time and no wait on the host: on the
+    legacy stream the plan's memory is given back in the stream's order, and the next plan takes it; a plan whose passes ran
+    on another stream is waited for.  Bit for bit the results of passes that were waited for."""
+    from paper_2607_23250_b200 import binding as lb
+    T, hq, hkv = 6000, 4, 2
+    rng = np.random.default_rng(d)
+    cus = [torch.from_numpy(pools.cu_seqlens(pools.random_layout(rng, T, int(m)))).cuda() for m in (6000, 200, 2000, 700)]
+    t = pools.make_tensors(T, hq, hkv, d, seed=5, device="cuda")
+    other = torch.cuda.Stream() if side_stream else None
+    torch.cuda.synchronize()
+
+    def once(cu):
+        plan = lb.libra_plan_tiles(cu, hq, 256, tile_kv=128, n_heads_kv=hkv, total_tokens=T)
+        if other is None:
+            out, lse = lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
+            res = (out, lse, *lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan))
+        else:
+            other.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(other):
+                out, lse = lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
+                res = (out, lse, *lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan))
+        plan.destroy()
+        return res
+
+    want = []
+    for cu in cus:
+        want.append(once(cu))
+        torch.cuda.synchronize()
+    got = [(i % 4, once(cus[i % 4])) for i in range(16)]
+    torch.cuda.synchronize()
+    for i, res in got:
+        for a, b in zip(res, want[i]):
+            assert torch.equal(a, b)
