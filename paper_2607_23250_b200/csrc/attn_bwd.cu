@@ -560,10 +560,10 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                                          f2_mul(l4.x, neg1)), x0, x1);
                         f2_unpack(f2_fma(f2_pack(__uint_as_float(sv[jj + 2]), __uint_as_float(sv[jj + 3])), scale2,
                                          f2_mul(l4.y, neg1)), x2, x3);
-                        pf[j] = ex2_sel(x0, jj);
-                        pf[j + 1] = ex2_sel(x1, jj + 1);
-                        pf[j + 2] = ex2_sel(x2, jj + 2);
-                        pf[j + 3] = ex2_sel(x3, jj + 3);
+                        pf[j] = ex2_approx(x0);
+                        pf[j + 1] = ex2_approx(x1);
+                        pf[j + 2] = ex2_approx(x2);
+                        pf[j + 3] = ex2_approx(x3);
                     }
                     if (need_mask) {   // one uniform branch per half: the exponentials above stay one straight run
                         const uint32_t vis = range_bits(j_lo - half * 32, j_hi - half * 32);

@@ -18,9 +18,6 @@
 
 namespace libra {
 
-#ifndef LIBRA_DQ_PREFETCH
-#define LIBRA_DQ_PREFETCH 0
-#endif
 constexpr int kDqGroups = 4;                      // compute warpgroups: each owns 128 / kDqGroups key columns
 constexpr int kDqCW = 128 / kDqGroups;            // S / dP columns per compute thread
 // The producer / MMA warps sit in a warpgroup of their own (two of its warps idle) so that it can hand
@@ -242,15 +239,6 @@ k_attn_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             uint32_t ucnt = 0, kcnt = 0, vcnt = 0;
             uint32_t n_q = 0, n_do = 0;   // Q / dO loads armed so far (for the give-up path)
             bool ok = true;
-            // Tiles a unit will need are pulled into L2 this many key blocks ahead: the shared-memory rings
-            // hold one block of lead, which covers an L2 hit but not a first touch in DRAM.
-            constexpr int kAhead = LIBRA_DQ_PREFETCH;
-            auto prefetch_kv = [&](int kvh, int j) {
-                for (int half = 0; half < D / 64; ++half) {
-                    tma_prefetch_3d(&tm_k, half * 64, kvh, j * kBlk);
-                    tma_prefetch_3d(&tm_v, half * 64, kvh, j * kBlk);
-                }
-            };
             DqUnitIter units(p, tile_begin, tile_end, heads_per_shard);
             DqUnit u = units.next();
             // Q and dO of unit `un`, whose tiles go through phase `cnt` of their barriers.  The shared-memory
@@ -277,18 +265,7 @@ k_attn_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 const int h = u.h, kvh = h / G, lo = u.lo, hi = u.hi;
                 const int j_q = lo + 1 < hi ? lo + 1 : hi;  // after this block's K/V the next unit's Q / dO are requested
                 ++ucnt;
-                const int j_next = hi - kAhead > lo ? hi - kAhead : lo;  // where the next unit's first tiles are requested
                 for (int j = lo; j <= hi && ok; ++j) {
-                    if (kAhead > 0) {
-                        if (j + kAhead <= hi) prefetch_kv(kvh, j + kAhead);
-                        if (j == j_next && nx.valid) {
-                            for (int half = 0; half < D / 64; ++half) {
-                                tma_prefetch_3d(&tm_q, half * 64, nx.h, (int)nx.q0);
-                                tma_prefetch_3d(&tm_do, half * 64, nx.h, (int)nx.q0);
-                            }
-                            for (int jj = nx.lo; jj <= nx.hi && jj < nx.lo + kAhead; ++jj) prefetch_kv(nx.h / G, jj);
-                        }
-                    }
                     const uint32_t ks = kcnt % L::kKStages;
                     ok = mbar_wait(&bar_kempty[ks], ((kcnt / L::kKStages) & 1) ^ 1, abort_flag);
                     if (!ok) break;
@@ -312,8 +289,13 @@ k_attn_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     if (j == j_q && nx.valid) {
                         ok = load_q_do(nx, ucnt);
                         if (!ok) break;
-                        if (kAhead == 0)   // pull the next unit's first K / V blocks into L2 meanwhile
-                            for (int jj = nx.lo; jj <= nx.hi && jj < nx.lo + 2; ++jj) prefetch_kv(nx.h / G, jj);
+                        // pull the next unit's first K / V blocks into L2 meanwhile: the rings hold one block of lead, which
+                        // covers an L2 hit but not a first touch in DRAM
+                        for (int jj = nx.lo; jj <= nx.hi && jj < nx.lo + 2; ++jj)
+                            for (int half = 0; half < D / 64; ++half) {
+                                tma_prefetch_3d(&tm_k, half * 64, nx.h / G, jj * kBlk);
+                                tma_prefetch_3d(&tm_v, half * 64, nx.h / G, jj * kBlk);
+                            }
                     }
                 }
                 u = nx;
@@ -520,8 +502,8 @@ k_attn_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 float pf[CW];
 #pragma unroll
                 for (int i = 0; i < CW; i += 2) {
-                    pf[i] = ex2_sel(fmaf(__uint_as_float(sv[i]), p.scale_log2, -lse2), i);
-                    pf[i + 1] = ex2_sel(fmaf(__uint_as_float(sv[i + 1]), p.scale_log2, -lse2), i + 1);
+                    pf[i] = ex2_approx(fmaf(__uint_as_float(sv[i]), p.scale_log2, -lse2));
+                    pf[i + 1] = ex2_approx(fmaf(__uint_as_float(sv[i + 1]), p.scale_log2, -lse2));
                 }
                 if (need_mask) {
 #pragma unroll

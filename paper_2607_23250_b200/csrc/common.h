@@ -100,8 +100,6 @@ namespace libra {
 // bf16 [T, H, d] tensor viewed as (d, H, T); TMA box = 64 columns x 1 head x box_rows tokens,
 // 128-byte swizzle, out-of-range rows read as zero.  Defined in attn_fwd.cu.
 int make_thd_map(CUtensorMap* m, const void* base, int64_t T, int H, int d, int box_rows);
-// fp32 matrix [rows, cols] (cols contiguous); box = box_cols x box_rows, 128-byte swizzle.
-int make_f32_2d_map(CUtensorMap* m, const void* base, int64_t rows, int64_t cols, int box_cols, int box_rows);
 // fp32 tensor [T, H, d] viewed as (d, H, T); box = box_cols x 1 x box_rows, 128-byte swizzle.
 int make_f32_3d_map(CUtensorMap* m, const void* base, int64_t T, int H, int d, int box_cols, int box_rows);
 // head_dim 256 (attn_d256.cu): the forward over the plan's query-major lists; the three gradient passes over

@@ -65,10 +65,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // Wall-clock budget of one wait.  A healthy kernel never waits longer than microseconds to
 // milliseconds; the limit only ends a wait that can no longer be satisfied.  The kernels keep two
 // control words in shared memory: ctl[0] = abort flag, ctl[1] = the budget in nanoseconds (set by
-// the host per launch, LIBRA_WAIT_LIMIT_NS when the plan does not override it).
-#ifndef LIBRA_WAIT_LIMIT_NS
-#define LIBRA_WAIT_LIMIT_NS 2000000000u
-#endif
+// the host per launch).
 
 // ---- pairs of CTAs (clusters of two: the even rank leads) ----
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -205,10 +202,6 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* m, const void* s
 __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // Returns when the bulk stores committed so far have finished READING shared memory (the tile may be reused).
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// Barrier among `count` threads (a multiple of 32) on hardware barrier `id` (1..15; 0 is __syncthreads).
-__device__ __forceinline__ void named_barrier_sync(int id, int count) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
 // Make generic-proxy shared-memory writes visible to the async proxy (TMA, tcgen05.mma).
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -369,11 +362,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
         "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
         : "memory");
 }
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]),
-                 "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-                 : "memory");
-}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
@@ -382,32 +370,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
-}
-// 2^x without the special-function unit (the MUFU pipe does 16 exp2 per clock per SM, the FMA
-// pipes 128 flops): round x to the nearest integer n with the magic-number trick, evaluate 2^f on
-// f = x - n in [-0.5, 0.5] with a cubic (relative error < 1e-4, far below bf16 resolution),
-// then add n to the exponent field.  Valid for x in [-126, 126]; smaller x is clamped (result
-// 2^-126, which rounds to zero in every use here).
-__device__ __forceinline__ float ex2_emul(float x) {
-    x = fmaxf(x, -126.0f);
-    const float t = x + 12582912.0f;             // 1.5 * 2^23: low mantissa bits now hold n
-    const float f = x - (t - 12582912.0f);
-    float p = fmaf(f, 0.05550410866f, 0.2402265070f);
-    p = fmaf(p, f, 0.6931471806f);
-    p = fmaf(p, f, 1.0f);
-    return __int_as_float(__float_as_int(p) + (__float_as_int(t) << 23));
-}
-// Optionally move one exponential in every LIBRA_EX2_EMUL_MOD onto the FMA pipes (0 = never).  `idx`
-// must be a compile-time constant after unrolling so the choice folds away.
-#ifndef LIBRA_EX2_EMUL_MOD
-#define LIBRA_EX2_EMUL_MOD 0
-#endif
-__device__ __forceinline__ float ex2_sel(float x, int idx) {
-#if LIBRA_EX2_EMUL_MOD > 0
-    return (idx % LIBRA_EX2_EMUL_MOD) == (LIBRA_EX2_EMUL_MOD - 1) ? ex2_emul(x) : ex2_approx(x);
-#else
-    return ex2_approx(x);
-#endif
 }
 
 // Bits [lo, hi] of a 32-bit word (either may lie outside 0..31; empty when lo > hi).  A row's visible columns tested
