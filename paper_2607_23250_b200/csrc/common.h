@@ -140,9 +140,9 @@ static inline cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned gr
 
 // Whether two backward kernels over the same pool that do not depend on one another run side by side: while the first has
 // few tiles for the SMs (`tiles` on `workers`) the second takes the idle ones; beyond that they only push one another's
-// tiles out of L2.  Forward and backward, 4 heads of 64 on 4096 / 16384 / 65536 tokens (1, 3.5 and 14 tiles per worker): 67
-// -> 55, 471 -> 392, 3147 -> 3140 us; 32 / 1 heads of 256 on 1500 / 32768 / 65536 tokens (0.1, 1.7, 3.5): 1431 -> 774 us,
-// 21.9 -> 19.2, 130 -> 115 ms; 128 / 4 heads of 256 on 32768 tokens, pair tiles (11.6): 99.9 -> 103.4 ms.
+// tiles out of L2.  Backward of one sample, one after the other and side by side: 4 / 4 heads of 64 on 4096 / 16384 / 65536
+// tokens (0.9, 3.5 and 13.8 tiles per worker): 121 -> 74, 597 -> 570, 9060 -> 9155 us; 32 / 1 heads of 256 on 1500 / 65536
+// tokens (0.1, 3.5): 1.42 -> 0.88, 246 -> 240 ms; 32 / 8 heads of 256 on 32768 (13.8): 60.2 -> 61.4 ms.
 constexpr int64_t kOverlapTiles = 8;   // per worker
 inline bool side_by_side(int64_t tiles, int workers) { return tiles <= kOverlapTiles * workers; }
 // dq may be written over q or dout: a kernel that writes dq reads of either only the tile it is about to replace, once the
