@@ -384,7 +384,9 @@ int libra_selftest_wait_timeout(uint32_t limit_ns, int* status_host, int* waited
  * enabling it again starts a fresh record.  libra_kernel_time_ms synchronises on the closing event
  * of the most recent launch of kernel `which` and returns its duration in milliseconds;
  * libra_kernel_times_ms returns the durations of up to `capacity` most recent recorded launches,
- * oldest first, and their number in *n_out.  Off by default.
+ * oldest first, and their number in *n_out.  The events stand between the kernels, so that kernels which
+ * otherwise run side by side (dK/dV and dQ of a pool with few tiles) run one after the other while timing is on, and
+ * the sum can exceed what the call takes without it.  Off by default.
  * Errors: INVALID_ARG, PLAN_MISMATCH (nothing recorded yet), CUDA. */
 int libra_plan_set_timing(libra_plan_t* plan, int enabled);
 int libra_kernel_time_ms(const libra_plan_t* plan, int which, float* ms_host);

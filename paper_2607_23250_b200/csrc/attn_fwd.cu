@@ -728,8 +728,9 @@ extern "C" int libra_attn_pool_fwd(const void* q_dev, const void* k_dev, const v
     prm.tile_ns = d.d_tile_ns;
     time_begin(mp, 0, s);
     // Two CTAs a tile when there are two for each (the first NT workers then have one tile each), a tile is one head (the
-    // exchange goes through the spent ring) and samples average four key blocks: 4000 tokens, 4 heads of 128, in samples of
-    // up to 300 / 800 / 4000 tokens took 12.0 / 18.0 / 55.3 us with one CTA a tile and 14.0 / 18.4 / 38.1 with two.
+    // exchange goes through the spent ring) and samples, empty ones counted, average four key blocks (the longest, which
+    // bounds the launch, is not known here): 4000 tokens, 4 heads of 128, in samples of up to 300 / 800 / 4000 tokens took
+    // 12.0 / 18.0 / 55.3 us with one CTA a tile and 14.0 / 18.4 / 38.1 with two.
     const bool pair = d.NT <= d.W / 2 && d.H == dims->hq && plan->T >= 4 * kBN * (int64_t)plan->n;
     if (dims->head_dim == 128)
         rc = pair ? launch_fwd<128, true>(tq, tk, tv, tout, prm, d.W, mp, s) : launch_fwd<128, false>(tq, tk, tv, tout, prm, d.W, mp, s);

@@ -485,7 +485,7 @@ static void add_pair_cands(const libra_plan* p, PairCands& cands, int k, bool ha
 // at the end.  Fused backward, best of 4096 ... 128 rows (4096): one sequence of 1500 tokens, 32 / 8 heads: 128, 60 us
 // (120); 12000 tokens, 4 / 1 heads: 1024, 159 us (345); 10007 tokens in samples of up to 400, 8 / 2 heads: 128, 64 us (91);
 // 16000 tokens, 32 / 4 heads: 1024, 0.98 ms (1.28); 32768 tokens, 32 / 8 heads: 2048, 5.88 ms (5.93), 128: 7.31; one sample of
-// 32768: 4096, 23.4 ms, 2048: 23.6, 128: 29.8.  The rule's choice is within 4 % of the best on each of ten such pools.
+// 32768: 4096, 23.4 ms, 2048: 23.6, 128: 29.8.
 static const PairTables* choose_pair_chunk(const libra_plan* p, const PairCands& cands, const int64_t* totals, int k, double G) {
     const PairTables* best = nullptr;
     double least = 0;
