@@ -286,7 +286,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
             bool ok = true;
             FwdTiles tiles(p, tile_begin, tile_end);
             FwdTile x;
-            while (ok && !(p.inject_stall && (!PAIR || rank == 1)) && tiles.next(x)) {
+            while (ok && !(p.inject_stall && (!PAIR || cluster_rank() == 1)) && tiles.next(x)) {
                 if (PAIR && !x.take_half(cluster_rank())) continue;
                 const bool act1 = x.hi[1] >= 0;
                 const int top = act1 ? x.hi[1] : x.hi[0];
