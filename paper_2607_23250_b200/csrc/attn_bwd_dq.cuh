@@ -145,8 +145,8 @@ k_attn_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     }
     // The row statistics are complete: the dK/dV kernel ahead waited for them before it let this one start.  Nothing else
     // is needed from it, so the wait for its end may come last (a stream's later work waits for this kernel only).
-    if (p.side_by_side) grid_dep_see(); else grid_dep_wait();
-    if (const int ps = *p.plan_status; ps != 0) {  // malformed cu_seqlens: report and leave
+    if (!p.side_by_side) grid_dep_wait();
+    if (const int ps = ld_acquire(p.plan_status); ps != 0) {  // malformed cu_seqlens: report and leave
         if (threadIdx.x == 0) { p.outcome[cta] = ps; p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
         grid_dep_wait();
         return;

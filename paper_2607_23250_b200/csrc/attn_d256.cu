@@ -222,9 +222,9 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
     }
     // The dK and dQ passes need what the dV pass had waited for and nothing of the pass ahead: they take the SMs that
     // fall free and wait for the pass ahead before they end.
-    if (MODE == FWD || MODE == DV || !p.side_by_side) grid_dep_wait(); else grid_dep_see();
+    if (MODE == FWD || MODE == DV || !p.side_by_side) grid_dep_wait();
     if (MODE == DV || MODE == DK) grid_dep_launch();
-    if (const int ps = *p.plan_status; ps != 0) {  // malformed cu_seqlens: report and leave
+    if (const int ps = ld_acquire(p.plan_status); ps != 0) {  // malformed cu_seqlens: report and leave
         if (threadIdx.x == 0) { p.outcome[cta] = ps; p.busy[2 * cta] = p.busy[2 * cta + 1] = 0; }
         if (MODE == DK || MODE == DQ) grid_dep_wait();
         return;
