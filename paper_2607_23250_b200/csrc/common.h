@@ -46,6 +46,7 @@ struct libra_plan {
     static constexpr int kMaxBlocks = 2;
     void* blocks[kMaxBlocks] = {};   // the device memory all pointers below lead into
     int n_blocks = 0;
+    bool plain_memory = false;       // built while its stream was being captured: the blocks are not stream-ordered
     int other_stream = 0;            // built or used on a stream other than the legacy one
     int32_t* d_tok_start = nullptr;  // [T] first token of the sample that holds token t
     int32_t* d_tok_end = nullptr;    // [T] one past the last token of that sample

@@ -405,8 +405,14 @@ static inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + b
 // array cost 0.5 + 0.4 ms a plan, and now and then ten times that.)
 static int plan_block(libra_plan* p, size_t bytes, uint8_t** out) {
     if (p->n_blocks == libra_plan::kMaxBlocks) return LIBRA_ERR_CUDA;
+    // A stream-ordered allocation would become part of a graph that is being captured, and the plan's memory would only
+    // exist while the graph runs.  A plain one outlives it where the capture's mode allows it, and fails elsewhere.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     void* q = nullptr;
-    if (scratch_alloc(&q, bytes ? bytes : 1, p->stream) != cudaSuccess) return LIBRA_ERR_CUDA;
+    cudaError_t e = cudaStreamIsCapturing(p->stream, &capture);
+    p->plain_memory = capture != cudaStreamCaptureStatusNone;
+    if (e == cudaSuccess) e = p->plain_memory ? cudaMalloc(&q, bytes ? bytes : 1) : scratch_alloc(&q, bytes ? bytes : 1, p->stream);
+    if (e != cudaSuccess) return LIBRA_ERR_CUDA;
     p->blocks[p->n_blocks++] = q;
     *out = reinterpret_cast<uint8_t*>(q);
     return LIBRA_OK;
@@ -706,6 +712,7 @@ extern "C" int libra_plan_tiles(const int32_t* cu_seqlens_dev, int n_samples, in
     const int rc = build_plan(p, cu_seqlens_dev, o, want);
     if (rc != LIBRA_OK) {
         libra_plan_destroy(p);
+        cudaGetLastError();   // not the next call's
         return rc;
     }
     *plan_out = p;
@@ -800,8 +807,11 @@ extern "C" int libra_plan_destroy(libra_plan_t* plan) {
     if (dev != plan->device) cudaSetDevice(plan->device);
     // Used on the legacy stream only (which outlives every plan): its order keeps the memory until the last kernel that
     // reads it is done, and the caller's next launches need not wait for an idle GPU.
-    if (plan->other_stream) cudaDeviceSynchronize();
-    for (int k = 0; k < plan->n_blocks; ++k) scratch_free(plan->blocks[k], nullptr);
+    if (plan->other_stream && plan->n_blocks > 0) cudaDeviceSynchronize();
+    for (int k = 0; k < plan->n_blocks; ++k) {
+        if (plan->plain_memory) cudaFree(plan->blocks[k]);
+        else scratch_free(plan->blocks[k], nullptr);
+    }
     if (dev != plan->device) cudaSetDevice(dev);
     for (int a = 0; a < libra_plan::kTimedKernels; ++a)
         for (int r = 0; r < libra_plan::kTimeRing; ++r)

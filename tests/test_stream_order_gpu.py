@@ -105,3 +105,34 @@ def test_plans_destroyed_behind_their_last_pass(d, side_stream):
     for i, res in got:
         for a, b in zip(res, want[i]):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("mode", ["global", "thread_local", "relaxed"])
+def test_plan_built_while_a_stream_is_captured(mode):
+    """A plan outlives the call that builds it, so its memory may not belong to a graph: where the capture forbids an ordinary
+    allocation the plan is refused, in relaxed mode it is good from the graph's first replay on, and after the graph is gone."""
+    import oracle
+    from paper_2607_23250_b200 import binding as lb
+    cu_np = np.array([0, 300, 1000], np.int32)
+    cu = torch.from_numpy(cu_np).cuda()
+    lb.libra_plan_tiles(cu, 2, 256, total_tokens=1000).destroy()     # what a first call sets up is there
+    torch.cuda.synchronize()
+    graph, plans, refused = torch.cuda.CUDAGraph(), [], False
+    try:
+        with torch.cuda.graph(graph, capture_error_mode=mode):
+            try:
+                plans.append(lb.libra_plan_tiles(cu, 2, 256, total_tokens=1000))
+            except lb.LibraError as err:
+                refused = err.code == lb.ERR_CUDA
+    except RuntimeError:
+        assert refused          # the capture is void after a call that it forbids
+    if mode == "relaxed":
+        graph.replay()
+        torch.cuda.synchronize()
+        del graph
+        got, want = plans[0].export(), oracle.plan(cu_np, 2, 256, plans[0].info()["n_workers"], 0)
+        assert plans[0].status() == 0 and np.array_equal(got["loads"], want["loads"])
+        plans[0].destroy()
+    else:
+        assert refused and not plans
+    assert torch.ones(4, device="cuda").sum().item() == 4
