@@ -47,7 +47,11 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
     int dev = 0;
     if (const cudaError_t e = cudaGetDevice(&dev); e != cudaSuccess) return e;
     cudaMemPool_t pool = nullptr;
-    if (dev >= 0 && dev < kMaxDevices) {
+    // A stream under capture takes the driver's default pool: the first call could not make one of our own there, and the
+    // memory belongs to the graph anyway.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (const cudaError_t e = cudaStreamIsCapturing(s, &capture); e != cudaSuccess) return e;
+    if (capture == cudaStreamCaptureStatusNone && dev >= 0 && dev < kMaxDevices) {
         std::lock_guard<std::mutex> lock(pools.mu);
         if (!pools.pool[dev]) {
             cudaMemPoolProps props = {};

@@ -85,3 +85,24 @@ def test_bad_arguments():
         lb.libra_tap_plan(cu, [0, 9], 1, 4, 3, 4, 2, 8)    # 3 shards do not divide 4 heads
     with pytest.raises(Exception):
         lb.libra_tap_plan(cu, [0, 9], 0, 4, 2, 4, 2, 8)
+
+
+def test_planner_as_the_first_call_of_a_process_under_capture():
+    """The exchange planner allocates in stream order, which a capture allows, also before anything else of the library has
+    run on the device (a child process, since this one has long called it)."""
+    import os
+    import subprocess
+    import sys
+    code = """
+import torch
+from paper_2607_23250_b200 import binding as lb
+cu = torch.tensor([0, 3000, 8192], dtype=torch.int32).cuda()
+torch.cuda.synchronize()
+graph = torch.cuda.CUDAGraph()
+with torch.cuda.graph(graph):
+    lb.libra_tap_plan(cu, [0, 8192], 2, 1024, 2, 4, 2, 128)
+res = lb.libra_tap_plan(cu, [0, 8192], 2, 1024, 2, 4, 2, 128)
+torch.cuda.synchronize()
+assert int(res["status"].item()) == 0
+"""
+    subprocess.run([sys.executable, "-c", code], check=True, timeout=300, cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
