@@ -114,7 +114,9 @@ typedef struct {
  * All planning runs in device kernels on `stream`; results stay on the device inside the
  * plan and are reused by every forward and backward call on the same layout (the paper
  * builds one plan per pool and reuses it across layers and for the backward pass,
- * Sections 4.1 and 4.3.3).  cu_seqlens_dev is read during the call only.
+ * Sections 4.1 and 4.3.3).  cu_seqlens_dev is read by the work enqueued in this call only.  The plan allocates device
+ * memory that outlives the call: on a stream under capture it is refused (CUDA) unless the capture's mode is relaxed, and
+ * then holds what the last replay of the graph computed.
  * With opts->weight_model = LIBRA_WEIGHT_BLOCKS the weight is the block count described at
  * LIBRA_WEIGHT_BLOCKS above; everything else is unchanged.
  * Errors: INVALID_ARG (null, n_samples <= 0, n_heads <= 0, tile_q <= 0, a negative option,
