@@ -19,7 +19,8 @@
 // 21.5 / 54.1 / 22.7 ms, now 14.3 / 33.9 / 20.7; the clock is at 1.35 GHz then, the power limit's).  Of a streamed tile that is the B operand of an X GEMM (N = its 64 rows) a CTA holds 32 rows;
 // of one that the accumulating GEMM multiplies with (N = 256 head-dim columns) it holds 128 columns; the tile that is
 // both (Q in DK, K in DQ) is loaded in both halves.  The leader (even rank) issues all MMAs; its barriers count the
-// copies and the compute warps of both CTAs; commits arrive in both.
+// copies and the compute warps of both CTAs; commits arrive in both.  A block that no row of one of the two sees (past its
+// diagonal, before its first sample) leaves that one's lanes out of the accumulating GEMM.
 //
 // TMEM: X1, X2, W (32 columns a block: the bf16 result of the element-wise step, A operand of the last GEMM) in 256
 // columns, acc (256).  FWD, DV: X1 3 x 64 | W 2 x 32; X1 runs two blocks ahead.  DK, DQ: X1 2 x 64 | X2 2 x 64, one block
@@ -176,6 +177,17 @@ struct Units {
             r0 = q0 + rank * kRows;
         }
         return true;
+    }
+    // Streamed blocks of a head that some row of CTA c sees: [lo, hi], of the unit's 0 .. n_blk - 1 (lo > hi: none).
+    __device__ void seen_by(uint32_t c, int& lo, int& hi) const {
+        const int64_t a = r0 + ((int64_t)c - (int64_t)cluster_rank()) * kRows, z = a + kRows - 1 < p.T ? a + kRows - 1 : p.T - 1;
+        lo = 0;
+        hi = -1;
+        if (a >= p.T) return;
+        lo = Cfg<MODE>::kKeyStationary ? (int)(a / kBlk) : p.tok_start[a] / kBlk;
+        hi = Cfg<MODE>::kKeyStationary ? (p.tok_end[z] - 1) / kBlk : (int)(z / kBlk);
+        lo = lo > b_lo ? lo - b_lo : 0;
+        hi = hi - b_lo < n_blk ? hi - b_lo : n_blk - 1;
     }
     // First row of the streamed block j of a head; the iterations of a unit take its heads in turn, blocks ascending.
     __device__ int stream_row(int j) const { return (b_lo + j) * kBlk; }
@@ -369,6 +381,12 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
             while (ok && u.next(rank)) {
                 const uint32_t sbuf = uc % L::kStBufs;
                 a_off = L::kSaOff + sbuf * L::kBig;
+                // The accumulating GEMM leaves out a CTA none of whose rows see the block: W is zero there, but times an
+                // infinity or a NaN of the block that is NaN.
+                int lo[2], hi[2], j = 0;
+                u.seen_by(0, lo[0], hi[0]);
+                u.seen_by(1, lo[1], hi[1]);
+                uint32_t begun = 0;              // bit per CTA: its rows of the unit's accumulator have been written
                 ok = mbar_wait(&bar_stfull[sbuf], (uc / L::kStBufs) & 1, abort_flag);
                 for (int it = 0; it < kAhead && it < u.n_it && ok; ++it) ok = do_x();
                 if (!ok) break;
@@ -385,10 +403,23 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                     tc_fence_after();
                     {
                         const uint64_t db = sdesc_advance(mdesc0, L::tile_off(L::kAcc, s));
+                        const uint32_t see = (j >= lo[0] && j <= hi[0] ? 1u : 0u) | (j >= lo[1] && j <= hi[1] ? 2u : 0u);
+                        if (see == 3 && (begun == 0 || begun == 3)) {
 #pragma unroll
-                        for (int kk = 0; kk < kBlk / 16; ++kk)
-                            mma_ts_pair(tmem_base + kColAcc, tmem_base + L::col_w(b, kk), sdesc_advance(db, kk * 2048), idesc_acc,
-                                        (it > 0 || kk > 0) ? 1u : 0u);
+                            for (int kk = 0; kk < kBlk / 16; ++kk)
+                                mma_ts_pair(tmem_base + kColAcc, tmem_base + L::col_w(b, kk), sdesc_advance(db, kk * 2048), idesc_acc,
+                                            (begun || kk > 0) ? 1u : 0u);
+                        } else {
+                            for (uint32_t c = 0; c < 2; ++c) {
+                                if (!((see >> c) & 1)) continue;
+#pragma unroll
+                                for (int kk = 0; kk < kBlk / 16; ++kk)
+                                    mma_ts_pair_one(tmem_base + kColAcc, tmem_base + L::col_w(b, kk), sdesc_advance(db, kk * 2048),
+                                                    idesc_acc, ((begun >> c) & 1 || kk > 0) ? 1u : 0u, c);
+                            }
+                        }
+                        begun |= see;
+                        if (++j == u.n_blk) j = 0;
                     }
                     tc_commit_pair(&bar_accstep[b]);
                     tc_commit_pair(&bar_empty[L::kAcc * S + s]);
@@ -423,7 +454,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
         bool ok = true;
         while (ok && u.next(rank)) {
             const int64_t row = u.r0 + r;            // this thread's query row (FWD, DQ) or key (DV, DK)
-            const bool row_ok = row < p.T;
+            bool row_ok = row < p.T;
             // visible columns of streamed block starting at b0: [lo_abs - b0, hi_abs - b0]
             //   query-stationary: keys from the start of the row's sample to the row itself
             //   key-stationary:   queries from the key itself to the end of its sample
@@ -613,6 +644,11 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
             const int n_heads = L::kKeyStationary ? p.hkv : p.hq;
             const int head = L::kKeyStationary ? u.kvh : u.h;
             __nv_bfloat16* dst_row = p.out + ((size_t)row * n_heads + head) * kD + grp * (kD / L::kGroups);
+            if (L::kKeyStationary && p.acc32) {      // of a query chunk's blocks this CTA's keys may have seen none
+                int lo, hi;
+                u.seen_by(rank, lo, hi);
+                row_ok = row_ok && lo <= hi;
+            }
             float* acc_row = L::kKeyStationary && p.acc32
                                  ? p.acc32 + ((size_t)row * n_heads + head) * kD + grp * (kD / L::kGroups) : nullptr;
 #pragma unroll

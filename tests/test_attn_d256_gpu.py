@@ -161,6 +161,36 @@ def test_sampled_rows_of_a_long_sample(pairs):
     plan.destroy()
 
 
+@pytest.mark.parametrize("pairs", [False, True])
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_values_that_are_not_finite_stay_in_their_tile(pairs, value):
+    """Rows of the other CTA of a pair that do not see a block are left out of its products: an infinity or a NaN in a key or
+    value reaches no row of an earlier 128-row tile, one in a query or an output gradient no later 128-key tile, although the
+    pair streams that block (inside a tile zero weights times such a value are NaN)."""
+    from paper_2607_23250_b200 import binding as lb
+    T, hq, hkv, at = 1100, 2, 1, {"v": 700, "k": 200, "q": 300, "dout": 800}
+    cu = torch.tensor([0, T], dtype=torch.int32).cuda()
+    directions = lb.LIBRA_DIR_Q | (lb.LIBRA_DIR_PAIR if pairs else lb.LIBRA_DIR_KV)
+    plan = lb.libra_plan_tiles(cu, hq, 256, directions=directions, tile_kv=128, n_heads_kv=hkv, pair_chunk=256 if pairs else 0)
+    clean = pools.make_tensors(T, hq, hkv, D, seed=3, device="cuda")
+    out0, lse0 = lb.libra_attn_pool_fwd(clean["q"], clean["k"], clean["v"], plan)
+    for name, row in at.items():
+        t = {n: x.clone() for n, x in clean.items()}
+        t[name][row, 0, 5] = value
+        first, behind = row // 128 * 128, row // 128 * 128 + 128
+        if name in ("k", "v"):
+            out, lse = lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
+            assert torch.isfinite(out[:first].float()).all() and torch.isfinite(lse[:, :first]).all(), name
+            assert not torch.isfinite(out[row:behind].float()).all()
+        dq, dk, dv = lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out0, lse0, t["dout"], plan)
+        if name in ("k", "v"):
+            assert torch.isfinite(dq[:first].float()).all(), name
+        else:
+            assert torch.isfinite(dk[behind:].float()).all() and torch.isfinite(dv[behind:].float()).all(), name
+            assert not torch.isfinite(dk[first:row].float()).all()
+    plan.destroy()
+
+
 def test_give_up_path_of_the_256_wide_kernel():
     """Producer stall injected on a healthy GPU (no loads are issued, a flag nothing sets): every pass reports
     TIMEOUT through the status words and returns; with the injection off the same plan gives correct results."""
