@@ -131,13 +131,15 @@ struct Params {
 // r0 is the first of this CTA's 128 stationary rows.
 template <int MODE>
 struct Units {
+    static constexpr bool kKeys = Cfg<MODE>::kKeyStationary;
     const Params& p;
     int idx, end, hh, hps, G;
-    int64_t r0;
+    int64_t base, r0;       // first stationary row of the pair and of this CTA
     int h, kvh, b_lo, n_blk, n_it;
+    int bound0, bound1;     // of each CTA's rows: start of the first one's sample (queries), end of the last one's (keys)
     __device__ Units(const Params& p_, int cta) : p(p_) {
         const int c = cta >> 1;
-        if (Cfg<MODE>::kKeyStationary) {
+        if (kKeys) {
             idx = p.cta_offsets[c];
             end = p.cta_offsets[c + 1];
         } else {   // neighbouring lists are contiguous
@@ -145,19 +147,21 @@ struct Units {
             end = p.cta_offsets[2 * c + 2 < p.W ? 2 * c + 2 : p.W];
         }
         G = p.hq / p.hkv;
-        hps = Cfg<MODE>::kKeyStationary ? 1 : p.hq / p.H;
+        hps = kKeys ? 1 : p.hq / p.H;
         hh = hps - 1;
         --idx;
     }
     __device__ bool next(uint32_t rank) {
         if (++hh == hps) { hh = 0; if (++idx >= end) return false; }
         const int t = p.cta_tiles[idx];
-        if constexpr (Cfg<MODE>::kKeyStationary) {
+        if constexpr (kKeys) {
             const int j = p.acc32 ? p.u_blk[(int)(t % p.NU)] : t / p.hkv;
             kvh = p.acc32 ? (int)(t / p.NU) : t % p.hkv;
-            const int64_t k0 = (int64_t)j * (2 * kRows), last_key = k0 + 2 * kRows - 1 < p.T ? k0 + 2 * kRows - 1 : p.T - 1;
-            int last64 = (p.tok_end[last_key] - 1) / kBlk;
-            b_lo = (int)(k0 / kBlk);
+            base = (int64_t)j * (2 * kRows);
+            bound0 = p.tok_end[base + kRows - 1 < p.T ? base + kRows - 1 : p.T - 1];
+            bound1 = p.tok_end[base + 2 * kRows - 1 < p.T ? base + 2 * kRows - 1 : p.T - 1];
+            int last64 = (bound1 - 1) / kBlk;
+            b_lo = (int)(base / kBlk);
             if (p.acc32) {   // pair tile: the query blocks of one chunk only
                 const int c = p.u_chunk[(int)(t % p.NU)], lo64 = 2 * c * p.R, hi64 = 2 * (c * p.R + p.R) - 1;
                 b_lo = lo64 > b_lo ? lo64 : b_lo;
@@ -166,28 +170,27 @@ struct Units {
             n_blk = last64 - b_lo + 1;
             h = kvh * G;
             n_it = G * n_blk;
-            r0 = k0 + rank * kRows;
         } else {
-            const int64_t q0 = (int64_t)(t / p.H) * (2 * kRows), last_row = q0 + 2 * kRows - 1 < p.T ? q0 + 2 * kRows - 1 : p.T - 1;
+            base = (int64_t)(t / p.H) * (2 * kRows);
+            bound0 = p.tok_start[base];
+            const int64_t last_row = base + 2 * kRows - 1 < p.T ? base + 2 * kRows - 1 : p.T - 1;
             h = (t % p.H) * hps + hh;
             kvh = h / G;
-            b_lo = p.tok_start[q0] / kBlk;
+            b_lo = bound0 / kBlk;
             n_blk = (int)(last_row / kBlk) - b_lo + 1;
             n_it = n_blk;
-            r0 = q0 + rank * kRows;
         }
+        r0 = base + rank * kRows;
         return true;
     }
     // Streamed blocks of a head that some row of CTA c sees: [lo, hi], of the unit's 0 .. n_blk - 1 (lo > hi: none).
     __device__ void seen_by(uint32_t c, int& lo, int& hi) const {
-        const int64_t a = r0 + ((int64_t)c - (int64_t)cluster_rank()) * kRows, z = a + kRows - 1 < p.T ? a + kRows - 1 : p.T - 1;
-        lo = 0;
-        hi = -1;
-        if (a >= p.T) return;
-        lo = Cfg<MODE>::kKeyStationary ? (int)(a / kBlk) : p.tok_start[a] / kBlk;
-        hi = Cfg<MODE>::kKeyStationary ? (p.tok_end[z] - 1) / kBlk : (int)(z / kBlk);
+        const int64_t a = base + c * kRows, z = a + kRows - 1 < p.T ? a + kRows - 1 : p.T - 1;
+        const int bound = c == 0 ? bound0 : (kKeys ? bound1 : (a < p.T ? p.tok_start[a] : 0));   // (most roles do without the last)
+        lo = kKeys ? (int)(a / kBlk) : bound / kBlk;
+        hi = kKeys ? (bound - 1) / kBlk : (int)(z / kBlk);
         lo = lo > b_lo ? lo - b_lo : 0;
-        hi = hi - b_lo < n_blk ? hi - b_lo : n_blk - 1;
+        hi = a >= p.T ? -1 : (hi - b_lo < n_blk ? hi - b_lo : n_blk - 1);
     }
     // First row of the streamed block j of a head; the iterations of a unit take its heads in turn, blocks ascending.
     __device__ int stream_row(int j) const { return (b_lo + j) * kBlk; }
@@ -381,21 +384,24 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
             while (ok && u.next(rank)) {
                 const uint32_t sbuf = uc % L::kStBufs;
                 a_off = L::kSaOff + sbuf * L::kBig;
-                // The accumulating GEMM leaves out a CTA none of whose rows see the block: W is zero there, but times an
-                // infinity or a NaN of the block that is NaN.
-                int lo[2], hi[2], j = 0;
-                u.seen_by(0, lo[0], hi[0]);
-                u.seen_by(1, lo[1], hi[1]);
-                uint32_t begun = 0;              // bit per CTA: its rows of the unit's accumulator have been written
                 ok = mbar_wait(&bar_stfull[sbuf], (uc / L::kStBufs) & 1, abort_flag);
                 for (int it = 0; it < kAhead && it < u.n_it && ok; ++it) ok = do_x();
                 if (!ok) break;
+                // The accumulating GEMM leaves out a CTA none of whose rows see the block: W is zero there, but times an
+                // infinity or a NaN of the block that is NaN.
+                int lo0, hi0, lo1, hi1, j = 0;
+                u.seen_by(0, lo0, hi0);
+                u.seen_by(1, lo1, hi1);
+                uint32_t begun = 0;              // bit per CTA: its rows of the unit's accumulator have been written
                 for (int it = 0; it < u.n_it && ok; ++it, ++itc) {
                     const uint32_t s = itc % S, ph = (itc / S) & 1, b = itc & 1;
                     // The X GEMMs of a block ahead run under the element-wise step of this one.  Their buffers were read out
                     // before W of the previous block was ready, and its accumulating GEMM, which may read W there, is ahead
                     // of them in the pipe.
                     if (it + kAhead < u.n_it) ok = do_x();
+                    const uint32_t see = (j >= lo0 && j <= hi0 ? 1u : 0u) | (j >= lo1 && j <= hi1 ? 2u : 0u);
+                    const bool plain = see == 3 && (begun == 0 || begun == 3);
+                    if (++j == u.n_blk) j = 0;
                     if (ok) ok = mbar_wait(&bar_full[L::kAcc * S + s], ph, abort_flag);
                     if (ok) ok = mbar_wait(&bar_wready[b], (itc >> 1) & 1, abort_flag);
                     if (ok && it == 0 && uc > 0) ok = mbar_wait(bar_accfree, (uc - 1) & 1, abort_flag);
@@ -403,23 +409,25 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                     tc_fence_after();
                     {
                         const uint64_t db = sdesc_advance(mdesc0, L::tile_off(L::kAcc, s));
-                        const uint32_t see = (j >= lo[0] && j <= hi[0] ? 1u : 0u) | (j >= lo[1] && j <= hi[1] ? 2u : 0u);
-                        if (see == 3 && (begun == 0 || begun == 3)) {
+                        const uint32_t t_w = tmem_base + L::col_w(b, 0), adds = see & begun;
+                        if (plain) {
 #pragma unroll
                             for (int kk = 0; kk < kBlk / 16; ++kk)
                                 mma_ts_pair(tmem_base + kColAcc, tmem_base + L::col_w(b, kk), sdesc_advance(db, kk * 2048), idesc_acc,
                                             (begun || kk > 0) ? 1u : 0u);
-                        } else {
-                            for (uint32_t c = 0; c < 2; ++c) {
-                                if (!((see >> c) & 1)) continue;
+                        } else if (see == 3) {   // a CTA's first product overwrites; these two did not begin with the same block
+                            mma_ts_pair_one(tmem_base + kColAcc, t_w, db, idesc_acc, 1, adds - 1);
+                            mma_ts_pair_one(tmem_base + kColAcc, t_w, db, idesc_acc, 0, 2 - adds);
 #pragma unroll
-                                for (int kk = 0; kk < kBlk / 16; ++kk)
-                                    mma_ts_pair_one(tmem_base + kColAcc, tmem_base + L::col_w(b, kk), sdesc_advance(db, kk * 2048),
-                                                    idesc_acc, ((begun >> c) & 1 || kk > 0) ? 1u : 0u, c);
-                            }
+                            for (int kk = 1; kk < kBlk / 16; ++kk)
+                                mma_ts_pair(tmem_base + kColAcc, tmem_base + L::col_w(b, kk), sdesc_advance(db, kk * 2048), idesc_acc, 1);
+                        } else if (see) {
+#pragma unroll
+                            for (int kk = 0; kk < kBlk / 16; ++kk)
+                                mma_ts_pair_one(tmem_base + kColAcc, tmem_base + L::col_w(b, kk), sdesc_advance(db, kk * 2048), idesc_acc,
+                                                (adds || kk > 0) ? 1u : 0u, see - 1);
                         }
                         begun |= see;
-                        if (++j == u.n_blk) j = 0;
                     }
                     tc_commit_pair(&bar_accstep[b]);
                     tc_commit_pair(&bar_empty[L::kAcc * S + s]);
