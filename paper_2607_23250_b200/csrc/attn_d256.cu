@@ -218,7 +218,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
     uint64_t* bar_wready = b2 + 8;     // [2] leader: W is in both CTAs' TMEM
     uint64_t* bar_accstep = b2 + 10;   // [2] the accumulating GEMM has run: W may be rewritten, acc rescaled
     uint64_t* bar_stfull = b2 + 12;    // [2] leader
-    uint64_t* bar_stempty = b2 + 14;   // [2] FWD: the output tile has left the buffer; else the unit's MMAs have run
+    uint64_t* bar_stempty = b2 + 14;   // [2] FWD: the output tile has left the buffer; else the unit's X MMAs have run
     uint64_t* bar_lfull = b2 + 16;     // [3] FWD: the row sums of a unit are there
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kMiscOff);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMiscOff + 4);
@@ -362,7 +362,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
             bool ok = true;
             // X1 (and X2) of the next block; its streamed halves are free again as soon as they have run
             uint32_t a_off = 0;                 // stationary tile of the unit
-            auto do_x = [&]() -> bool {
+            auto do_x = [&](bool last) -> bool {
                 const uint32_t s = xi % S, ph = (xi / S) & 1;
                 if (!mbar_wait(&bar_full[s], ph, abort_flag)) return false;
                 tc_fence_after();
@@ -376,6 +376,8 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                     tc_commit_pair(&bar_x2full[xb]);
                     tc_commit_pair(&bar_empty[S + s]);
                 }
+                // (the unit's stationary tiles are not read again; FWD stages its output there)
+                if (MODE != FWD && last) tc_commit_pair(&bar_stempty[0]);
                 ++xi;
                 if (++xb == L::kX1Bufs) xb = 0;
                 return true;
@@ -385,7 +387,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                 const uint32_t sbuf = uc % L::kStBufs;
                 a_off = L::kSaOff + sbuf * L::kBig;
                 ok = mbar_wait(&bar_stfull[sbuf], (uc / L::kStBufs) & 1, abort_flag);
-                for (int it = 0; it < kAhead && it < u.n_it && ok; ++it) ok = do_x();
+                for (int it = 0; it < kAhead && it < u.n_it && ok; ++it) ok = do_x(it == u.n_it - 1);
                 if (!ok) break;
                 // The accumulating GEMM leaves out a CTA none of whose rows see the block: W is zero there, but times an
                 // infinity or a NaN of the block that is NaN.
@@ -398,7 +400,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                     // The X GEMMs of a block ahead run under the element-wise step of this one.  Their buffers were read out
                     // before W of the previous block was ready, and its accumulating GEMM, which may read W there, is ahead
                     // of them in the pipe.
-                    if (it + kAhead < u.n_it) ok = do_x();
+                    if (it + kAhead < u.n_it) ok = do_x(it + kAhead == u.n_it - 1);
                     const uint32_t see = (j >= lo0 && j <= hi0 ? 1u : 0u) | (j >= lo1 && j <= hi1 ? 2u : 0u);
                     const bool plain = see == 3 && (begun == 0 || begun == 3);
                     if (++j == u.n_blk) j = 0;
@@ -431,10 +433,7 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                     }
                     tc_commit_pair(&bar_accstep[b]);
                     tc_commit_pair(&bar_empty[L::kAcc * S + s]);
-                    if (it == u.n_it - 1) {
-                        tc_commit_pair(bar_accdone);
-                        if (MODE != FWD) tc_commit_pair(&bar_stempty[sbuf]);
-                    }
+                    if (it == u.n_it - 1) tc_commit_pair(bar_accdone);
                 }
                 ++uc;
             }
