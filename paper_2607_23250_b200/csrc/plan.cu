@@ -50,7 +50,8 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
     // A stream under capture takes the driver's default pool: the first call could not make one of our own there, and the
     // memory belongs to the graph anyway.
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (const cudaError_t e = cudaStreamIsCapturing(s, &capture); e != cudaSuccess) return e;
+    if (s)   // (the legacy stream cannot be captured)
+        if (const cudaError_t e = cudaStreamIsCapturing(s, &capture); e != cudaSuccess) return e;
     if (capture == cudaStreamCaptureStatusNone && dev >= 0 && dev < kMaxDevices) {
         std::lock_guard<std::mutex> lock(pools.mu);
         if (!pools.pool[dev]) {
@@ -413,7 +414,7 @@ static int plan_block(libra_plan* p, size_t bytes, uint8_t** out) {
     // exist while the graph runs.  A plain one outlives it where the capture's mode allows it, and fails elsewhere.
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     void* q = nullptr;
-    cudaError_t e = cudaStreamIsCapturing(p->stream, &capture);
+    cudaError_t e = p->stream ? cudaStreamIsCapturing(p->stream, &capture) : cudaSuccess;
     p->plain_memory = capture != cudaStreamCaptureStatusNone;
     if (e == cudaSuccess) e = p->plain_memory ? cudaMalloc(&q, bytes ? bytes : 1) : scratch_alloc(&q, bytes ? bytes : 1, p->stream);
     if (e != cudaSuccess) return LIBRA_ERR_CUDA;
