@@ -115,8 +115,6 @@ struct DirView {
 };
 struct DirViews {
     DirView v[4];
-    int check_loads;        // bit per view: block counts that might add up beyond the placement's keys
-    int* status;
 };
 
 // Weight of block b (Eq. 6): a token at position p of a sample of length len contributes
@@ -181,7 +179,7 @@ __global__ void __launch_bounds__(256) k_rank_blocks(const DirViews views) {
 
 // Placement (Algorithm 2's greedy rule: the next tile goes to the least-loaded worker, lowest index among equals) in
 // waves, one block per direction (waves.cuh).  There are at most 1024 workers, so a key has 54 bits for the load: enough for
-// pair counts by the host's bound on H T^2; block counts with a large unit cost can exceed them, which k_exec_order finds
+// pair counts by the host's bound on H T^2; block counts with a large unit cost can exceed them, which k_check_loads finds
 // in the lists (they hold every tile once all the same, in no particular balance).  Tiles come in batches held in shared
 // memory, the next batch in registers.  Both directions of 131072 tokens with 32 / 8 heads (16384 and 13464 tiles): 0.6 ms,
 // by a warp per direction 1.4 ms; of two 65536-token samples (69632 pair tiles): 1.5 and 5.3 ms.
@@ -273,20 +271,6 @@ __global__ void k_exec_order(const DirViews views) {
     const int r = blockIdx.x;
     if (!d.blk_order || r >= d.W) return;
     const int beg = d.cta_offsets[r], n = d.cta_offsets[r + 1] - beg;
-    if ((views.check_loads >> blockIdx.y) & 1) {   // did the worker's load fit its key?  (~0 stands for none)
-        __shared__ unsigned long long load;
-        if (threadIdx.x == 0) load = 0;
-        __syncthreads();
-        const unsigned long long full = (1ull << 54) - 1;
-        unsigned long long sum = 0;                       // at most `full`, so that the total fits 64 bits
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const unsigned long long w = (unsigned long long)d.weight_blk[d.cta_tiles[beg + i] / d.H];
-            sum = w < full - sum ? sum + w : full;
-        }
-        atomicAdd(&load, sum);
-        __syncthreads();
-        if (threadIdx.x == 0 && load >= full) atomicCAS(views.status, LIBRA_OK, LIBRA_ERR_OVERFLOW);
-    }
     if (n > 16384) {  // quadratic sort too slow: keep placement order
         for (int i = threadIdx.x; i < n; i += blockDim.x) d.cta_exec[beg + i] = d.cta_tiles[beg + i];
         return;
@@ -301,6 +285,24 @@ __global__ void k_exec_order(const DirViews views) {
         }
         d.cta_exec[beg + rank] = t;
     }
+}
+
+// Did the workers' loads of a direction fit their keys?  (~0 stands for none.)  Launched only where block counts might add
+// up that far.
+__global__ void k_check_loads(const DirView d, int* __restrict__ status) {
+    __shared__ unsigned long long load;
+    const int beg = d.cta_offsets[blockIdx.x], end = d.cta_offsets[blockIdx.x + 1];
+    if (threadIdx.x == 0) load = 0;
+    __syncthreads();
+    const unsigned long long full = (1ull << 54) - 1;
+    unsigned long long sum = 0;                       // at most `full`, so that the total fits 64 bits
+    for (int i = beg + threadIdx.x; i < end; i += blockDim.x) {
+        const unsigned long long w = (unsigned long long)d.weight_blk[d.cta_tiles[i] / d.H];
+        sum = w < full - sum ? sum + w : full;
+    }
+    atomicAdd(&load, sum);
+    __syncthreads();
+    if (threadIdx.x == 0 && load >= full) atomicCAS(status, LIBRA_OK, LIBRA_ERR_OVERFLOW);
 }
 
 // ---- pair tiles: key block x query chunk x head (the fused backward's units) ---------------------------------
@@ -620,16 +622,11 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
     }
     // ---- weights, order, placement and lists of all directions together
     DirViews views = {};
-    views.status = p->d_status;
     int n = 0, max_w = 0;
     int64_t max_nb = 0, max_nt = 0;
     for (int k = 0; k < 4; ++k)
         if (sorted[k]) {
-            const DirView& v = views.v[n] = view_of(p->dir[k], k != 0, o);
-            const double chunks = v.g > 0 ? (double)((T + v.g - 1) / v.g) : 0;   // at most each of them against all
-            // (not the internal direction, whose tiles are twice as heavy: only the balance of its lists would suffer)
-            if (k != 3 && v.H * chunks * (8 * chunks + v.unit_cost) >= 0x1p53) views.check_loads |= 1 << n;
-            ++n;
+            views.v[n++] = view_of(p->dir[k], k != 0, o);
             max_nb = p->dir[k].NB > max_nb ? p->dir[k].NB : max_nb;
         }
     if (n > 0) {
@@ -651,6 +648,14 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
     count_launch(2);
     if (n_sorted > 0) {
         k_exec_order<<<dim3(max_w, n_sorted), 256, 0, s>>>(views);
+        count_launch();
+    }
+    for (int k = 0; k < 2; ++k) {   // (not the internal direction, whose tiles are twice as heavy: only its balance would suffer)
+        if (!want[k] || o.weight_model != LIBRA_WEIGHT_BLOCKS) continue;
+        const DirView v = view_of(p->dir[k], k != 0, o);
+        const double chunks = (double)((T + v.g - 1) / v.g);   // at most each of them against all
+        if (v.H * chunks * (8 * chunks + v.unit_cost) < 0x1p53) continue;
+        k_check_loads<<<v.W, 256, 0, s>>>(v, p->d_status);
         count_launch();
     }
     for (int k = 0; k < 4; ++k) p->dir[k].enabled = want[k] ? 1 : 0;
