@@ -8,11 +8,10 @@
 // inside the range weigh nothing and change no decision.
 //
 // Placement is sequential by nature (every choice depends on the loads and residency left by the previous
-// ones), so the latency of one step bounds it.  Up to 128 workers: one warp, up to four workers per lane, sample
-// volumes and residency bit rows in shared memory, the blocks' records (gathered in placement order by the ranking
-// kernel) held in registers a batch ahead, the lexicographic arg-min by warp-wide integer reductions.  More
-// workers, or tables beyond shared memory: one CTA with a thread per worker, block-wide arg-min, tables in global
-// memory.  1024 tiles on 16 workers with their schedule: 0.65 ms, all in the second form 2.8 ms.
+// ones), so the latency of one step bounds it.  Up to 128 workers whose tables fit shared memory: one block whose
+// warps work on neighbouring steps (k_tap_place_team).  Otherwise: one CTA with a thread per worker, block-wide
+// arg-min, tables in global memory.  1024 tiles on 16 workers with their schedule: 0.30 ms, with one warp for all of a
+// step 0.65 ms, all in the second form 2.8 ms.
 #include <cstdint>
 #include <new>
 #include <cuda_runtime.h>
@@ -238,115 +237,254 @@ __global__ void __launch_bounds__(1024) k_tap_place(
 }
 
 // Smallest x among the lanes with `in`; `in` is left set on the lanes that hold it.  Values are not negative.
-__device__ __forceinline__ int64_t tap_warp_min(int64_t x, bool& in) {
-    const uint32_t hi = __reduce_min_sync(0xffffffffu, in ? (uint32_t)((uint64_t)x >> 32) : 0xffffffffu);
-    in = in && (uint32_t)((uint64_t)x >> 32) == hi;
+__device__ __forceinline__ uint64_t tap_warp_min(uint64_t x, bool& in) {
+    const uint32_t hi = __reduce_min_sync(0xffffffffu, in ? (uint32_t)(x >> 32) : 0xffffffffu);
+    in = in && (uint32_t)(x >> 32) == hi;
     const uint32_t lo = __reduce_min_sync(0xffffffffu, in ? (uint32_t)x : 0xffffffffu);
     in = in && (uint32_t)x == lo;
-    return (int64_t)((uint64_t)hi << 32 | lo);
+    return (uint64_t)hi << 32 | lo;
 }
 
-// Algorithm 2 by one warp (PER * 32 >= W): lane l is the workers l, l + 32, ...; a worker's bit row is read and written
-// by its own lane only.  Same choices as k_tap_place.  Dynamic shared memory: v_smp [n], then W rows of `pitch` words.
-template <int PER>
-__global__ void __launch_bounds__(32) k_tap_place_warp(
-    const TapRec* __restrict__ rec, const int64_t* __restrict__ v_smp_g, const int32_t* __restrict__ res_smp, int64_t NB, int H,
-    int W, int n, int tau_num, int tau_den, uint32_t* __restrict__ Cbits /*[W][words]*/, int words, int pitch,
-    int32_t* __restrict__ sigma, int64_t* __restrict__ loads, int64_t* __restrict__ comm_total, int* __restrict__ status) {
-    extern __shared__ __align__(16) uint8_t tap_smem[];
-    int64_t* v_smp = reinterpret_cast<int64_t*>(tap_smem);
-    uint32_t* bits = reinterpret_cast<uint32_t*>(v_smp + n);
-    const int lane = threadIdx.x;
-    for (int w = lane; w < W * pitch; w += 32) bits[w] = 0;
-    for (int j = lane; j < n; j += 32) v_smp[j] = v_smp_g[j];
-    __syncwarp();
-    for (int j = lane; j < n; j += 32) {   // the groups a worker holds in full
-        const int r = res_smp[j];
-        if (r >= 0 && r < W)
-            for (int h = 0; h < H; ++h) { const int g = j * H + h; atomicOr(&bits[r * pitch + (g >> 5)], 1u << (g & 31)); }
-    }
-    int64_t sum_f = 0;
-    for (int64_t b = lane; b < NB; b += 32) sum_f += rec[b].f * H;
+// Algorithm 2 by one block (PER * 32 >= W); same choices as k_tap_place.  Up to kTapTeam shards of a block are a step, and
+// three kinds of warps work on neighbouring steps, with a barrier between steps:
+//   placing     one warp; lane l is the workers l, l + 32, ..., whose loads it keeps.  Step s.
+//   walking     one per shard of a step: what every worker would have to fetch for its tile of step s + 1, once as things
+//               stand without step s and once as if it were given step s's tile of the shard, so that the placing warp
+//               only has to choose between the two.
+//   recording   one per shard: enters step s - 1's pick into the residency, per shard and sample a bit for each worker.  A
+//               walking warp may meet a word before or after that; it looks at the pick itself.
+// What is serial is the placing warp's minimum and the load it changes, 290 clk a tile (1024 tiles, 4 shards, 16 workers: 1165 a
+// step, of which the placing warp is busy 1100 and the others as long); one warp that did all of it took 1100 clk a tile.
+// Its loop over the shards is unrolled: rolled up, with the next shard's volumes fetched ahead, it took 1.3 times as long.
+// Volumes are multiples of 4 head_dim bytes and are kept in that unit, in 32 bits where a block's samples and its rows fit
+// them together (Delta).
+// Dynamic shared memory: sample volumes [n] (64 bits), then residency [H][n][PER].
+constexpr int kTapTeam = 8;
+constexpr int kTapThreads = 32 * (1 + 2 * kTapTeam);
+constexpr size_t kTapTeamStatic = 2 * kTapTeam * 32 * 16 + 1024;   // shared memory beside the tables, a PER
+constexpr size_t kTapTeamSmem = 227 * 1024 - 4 * kTapTeamStatic;
+template <typename Delta> struct __align__(2 * sizeof(Delta)) TapDelta { Delta as_is, if_given; };
+
+struct TapPlace {
+    const TapRec* rec;        // the blocks in placement order
+    const int64_t* v_smp;
+    const int32_t* res_smp;
+    int64_t NB, unit;         // unit: bytes a volume counts in
+    int H, W, n, tau_num, tau_den, words;
+    uint32_t* Cbits;          // [W][words]
+    int32_t* sigma;
+    int64_t* loads;
+    int64_t* comm_total;
+    int* status;
+};
+
+template <int PER, typename Mask, typename Delta>
+__device__ __forceinline__ void tap_place_steps(const TapPlace& p, int64_t cap, const uint64_t* v_smp, Mask* held, void* deltas,
+                                                int (*s_pick)[kTapTeam]) {
+    using Two = TapDelta<Delta>;
+    Two (*s_delta)[kTapTeam][32 * PER] = reinterpret_cast<Two (*)[kTapTeam][32 * PER]>(deltas);   // [2]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = p.n, H = p.H, W = p.W;
+    const int groups = (H + kTapTeam - 1) / kTapTeam;   // steps a block takes
+    const int64_t NB = p.NB, steps = NB * groups;
+    const TapRec* __restrict__ rec = p.rec;
+    if (warp == 0) {
+        int64_t L[PER];
+        uint64_t comm = 0;
+        int last[kTapTeam];   // picks of the step before
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) sum_f += __shfl_xor_sync(0xffffffffu, sum_f, off);
-    if (sum_f > (INT64_MAX / ((int64_t)(tau_den + tau_num) * 2)) / W) {  // the integer cap test would overflow
-        if (lane == 0) *status = LIBRA_ERR_OVERFLOW;   // the exchange kernels see the flag and add nothing
-        for (int64_t x = lane; x < NB; x += 32)
-            for (int h = 0; h < H; ++h) sigma[(int64_t)rec[x].blk * H + h] = rec[x].q_home;
-        return;
-    }
-    __syncwarp();
-    const int64_t cap_rhs = (int64_t)(tau_den + tau_num) * sum_f, cap_mul = (int64_t)tau_den * W;
-    int64_t L[PER], comm = 0;
+        for (int u = 0; u < PER; ++u) L[u] = 0;
 #pragma unroll
-    for (int u = 0; u < PER; ++u) L[u] = 0;
-    TapRec mine = rec[lane < NB ? lane : NB - 1];
-    for (int64_t x0 = 0; x0 < NB; x0 += 32) {
-        const int64_t xn = x0 + 32 + lane;
-        const TapRec coming = rec[xn < NB ? xn : NB - 1];   // the next batch lands while this one is placed
-        const int lim = (int)(NB - x0 < 32 ? NB - x0 : 32);
-        for (int i = 0; i < lim; ++i) {
-            const int64_t f = __shfl_sync(0xffffffffu, mine.f, i), vqo = __shfl_sync(0xffffffffu, mine.v_qo, i);
-            const int home = __shfl_sync(0xffffffffu, mine.q_home, i), blk = __shfl_sync(0xffffffffu, mine.blk, i);
-            const int j0 = __shfl_sync(0xffffffffu, mine.j0, i), j1 = __shfl_sync(0xffffffffu, mine.j1, i);
-            for (int h = 0; h < H; ++h) {
+        for (int k = 0; k < kTapTeam; ++k) last[k] = -1;
+        int64_t f_in = rec[lane < NB ? lane : NB - 1].f, f_next = f_in;
+        int64_t x = 0;
+        int grp = 0;
+        __syncthreads();
+        for (int64_t st = 0; st < steps; ++st) {
+            const int buf = (int)(st & 1), cnt = H - grp * kTapTeam < kTapTeam ? H - grp * kTapTeam : kTapTeam;
+            constexpr bool kAhead = PER * sizeof(Delta) <= 8;   // all at once while registers last
+            Two two[kTapTeam][PER];
+#pragma unroll
+            for (int k = 0; k < kTapTeam && kAhead; ++k)
+#pragma unroll
+                for (int u = 0; u < PER; ++u) two[k][u] = s_delta[buf][k][lane + 32 * u];
+            if (grp == 0 && (x & 31) == 0) {   // the next batch of blocks lands while this one is placed
+                if (x > 0) f_in = f_next;
+                const int64_t xn = x + 32 + lane;
+                f_next = rec[xn < NB ? xn : NB - 1].f;
+            }
+            const int64_t f = __shfl_sync(0xffffffffu, f_in, (int)(x & 31));
+            const int64_t room = cap - f;
+#pragma unroll
+            for (int k = 0; k < kTapTeam; ++k) {
+                if (k >= cnt) break;
                 // the lane's best worker under the soft cap, by (delta, load, index)
-                int64_t delta[PER], bd = 0, bl = 0;
-                int br = INT32_MAX;
+                Delta d[PER], bd = 0;
+                int64_t bl = 0;
+                int br = -1;
 #pragma unroll
                 for (int u = 0; u < PER; ++u) {
                     const int r = lane + 32 * u;
-                    int64_t d = r != home ? vqo : 0;
-                    if (r < W) {
-                        const uint32_t* row = bits + r * pitch;
-                        for (int j = j0; j <= j1; ++j) {
-                            const int g = j * H + h;
-                            if (!((row[g >> 5] >> (g & 31)) & 1u)) d += v_smp[j];
-                        }
-                        if (cap_mul * (L[u] + f) <= cap_rhs && (br == INT32_MAX || d < bd || (d == bd && L[u] < bl))) {
-                            bd = d; bl = L[u]; br = r;
-                        }
-                    }
-                    delta[u] = d;
+                    if (!kAhead) two[k][u] = s_delta[buf][k][r];
+                    d[u] = last[k] == r ? two[k][u].if_given : two[k][u].as_is;
+                    if (r < W && L[u] <= room && (br < 0 || d[u] < bd || (d[u] == bd && L[u] < bl))) { bd = d[u]; bl = L[u]; br = r; }
                 }
-                bool in = br != INT32_MAX;
+                bool in = br >= 0, some;
                 int pick;
-                int64_t pick_delta;
-                if (__any_sync(0xffffffffu, in)) {             // some worker stays under the soft cap
-                    pick_delta = tap_warp_min(bd, in);
-                    tap_warp_min(bl, in);
-                    pick = (int)__reduce_min_sync(0xffffffffu, in ? (uint32_t)br : 0xffffffffu);
+                Delta pick_delta;
+                if (sizeof(Delta) == 4) {
+                    pick_delta = (Delta)__reduce_min_sync(0xffffffffu, in ? (uint32_t)bd : 0xffffffffu);
+                    some = (uint32_t)pick_delta != 0xffffffffu;
+                    in = in && bd == pick_delta;
+                } else {
+                    some = __any_sync(0xffffffffu, in);
+                    pick_delta = (Delta)tap_warp_min(bd, in);
+                }
+                if (some) {                                    // some worker stays under the soft cap
+                    unsigned who = __ballot_sync(0xffffffffu, in);
+                    if (who & (who - 1)) {
+                        tap_warp_min((uint64_t)bl, in);
+                        who = __ballot_sync(0xffffffffu, in);
+                    }
+                    if (PER == 1) pick = __ffs(who) - 1;
+                    else pick = (int)__reduce_min_sync(0xffffffffu, in ? (uint32_t)br : 0xffffffffu);
                 } else {                                       // nobody does: by (load, delta, index)
-                    br = INT32_MAX;
 #pragma unroll
                     for (int u = 0; u < PER; ++u) {
                         const int r = lane + 32 * u;
-                        if (r < W && (br == INT32_MAX || L[u] < bl || (L[u] == bl && delta[u] < bd))) { bd = delta[u]; bl = L[u]; br = r; }
+                        if (r < W && (br < 0 || L[u] < bl || (L[u] == bl && d[u] < bd))) { bd = d[u]; bl = L[u]; br = r; }
                     }
-                    in = br != INT32_MAX;
-                    tap_warp_min(bl, in);
-                    pick_delta = tap_warp_min(bd, in);
+                    in = br >= 0;
+                    tap_warp_min((uint64_t)bl, in);
+                    pick_delta = (Delta)tap_warp_min(bd, in);
                     pick = (int)__reduce_min_sync(0xffffffffu, in ? (uint32_t)br : 0xffffffffu);
                 }
-                if ((pick & 31) == lane) {
 #pragma unroll
-                    for (int u = 0; u < PER; ++u)
-                        if (u == pick >> 5) L[u] += f;
-                    uint32_t* row = bits + pick * pitch;
-                    for (int j = j0; j <= j1; ++j) { const int g = j * H + h; row[g >> 5] |= 1u << (g & 31); }
-                    sigma[(int64_t)blk * H + h] = pick;
-                }
+                for (int u = 0; u < PER; ++u)
+                    if (pick == lane + 32 * u) L[u] += f;
+                if (lane == 0) s_pick[buf][k] = pick;
+                last[k] = groups == 1 ? pick : -1;   // with more than one step a block the next step has other shards
                 comm += pick_delta;
             }
+            if (++grp == groups) { grp = 0; ++x; }
+            __syncthreads();
         }
-        mine = coming;
-    }
 #pragma unroll
-    for (int u = 0; u < PER; ++u)
-        if (lane + 32 * u < W) loads[lane + 32 * u] = L[u];
-    if (lane == 0) *comm_total = comm;
-    __syncwarp();
-    for (int w = lane; w < W * words; w += 32) Cbits[w] = bits[w / words * pitch + w % words];
+        for (int u = 0; u < PER; ++u)
+            if (lane + 32 * u < W) p.loads[lane + 32 * u] = L[u];
+        if (lane == 0) *p.comm_total = (int64_t)(comm * (uint64_t)p.unit);
+        __syncthreads();
+        return;
+    }
+    const bool walks = warp <= kTapTeam;
+    const int k = (warp - 1) % kTapTeam;
+    // the blocks of steps s - 1, s and s + 1; h: the warp's shard, H or more: none
+    int j0_a = 0, j1_a = -1, h_a = H, blk_a = 0, j0_b = 0, j1_b = -1, h_b = H, blk_b = 0;
+    TapRec in = rec[lane < NB ? lane : NB - 1], next_in = in;
+    in.v_qo /= p.unit;
+    int64_t x = 0;             // the block of step s + 1
+    int grp = 0;
+    for (int64_t st = -1; st <= steps; ++st) {
+        int j0 = 0, j1 = -1, h = H, blk = 0, home = 0;
+        Delta vqo = 0;
+        if (st + 1 < steps) {
+            if (grp == 0 && (x & 31) == 0) {
+                if (x > 0) { in = next_in; in.v_qo /= p.unit; }
+                const int64_t xn = x + 32 + lane;
+                next_in = rec[xn < NB ? xn : NB - 1];
+            }
+            const int src = (int)(x & 31);
+            j0 = __shfl_sync(0xffffffffu, in.j0, src);
+            j1 = __shfl_sync(0xffffffffu, in.j1, src);
+            blk = __shfl_sync(0xffffffffu, in.blk, src);
+            home = __shfl_sync(0xffffffffu, in.q_home, src);
+            vqo = __shfl_sync(0xffffffffu, (Delta)in.v_qo, src);
+            h = grp * kTapTeam + k;
+            if (++grp == groups) { grp = 0; ++x; }
+        }
+        if (st >= 0) __syncthreads();   // step st - 1 is placed
+        const int pick = h_a < H ? s_pick[(st + 1) & 1][k] : -1;
+        if (walks) {
+            if (h < H) {
+                const Mask* row = held + (size_t)h * n * PER;
+                const bool same = h == h_a;   // (else that pick was of another shard)
+                Two d[PER];
+#pragma unroll
+                for (int u = 0; u < PER; ++u) d[u].as_is = d[u].if_given = lane + 32 * u != home ? vqo : 0;
+#pragma unroll 4
+                for (int j = j0; j <= j1; ++j) {
+                    const Delta v = (Delta)v_smp[j];
+                    const Delta v_other = j >= j0_b && j <= j1_b ? 0 : v;
+                    const bool just = same && j >= j0_a && j <= j1_a;
+#pragma unroll
+                    for (int u = 0; u < PER; ++u) {
+                        const bool has = (((uint32_t)row[j * PER + u] >> lane) & 1u) || (just && pick == lane + 32 * u);
+                        d[u].as_is += has ? 0 : v;
+                        d[u].if_given += has ? 0 : v_other;
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < PER; ++u) s_delta[(st + 1) & 1][k][lane + 32 * u] = d[u];
+            }
+        } else if (h_a < H) {
+            Mask* row = held + (size_t)h_a * n * PER + (PER > 1 ? pick >> 5 : 0);
+            for (int j = j0_a + lane; j <= j1_a; j += 32) row[j * PER] |= (Mask)(1u << (pick & 31));
+            if (lane == 0) p.sigma[(int64_t)blk_a * H + h_a] = pick;
+        }
+        j0_a = j0_b; j1_a = j1_b; h_a = h_b; blk_a = blk_b;
+        j0_b = j0; j1_b = j1; h_b = h; blk_b = blk;
+    }
+    __syncthreads();
+}
+
+template <int PER, typename Mask>
+__global__ void __launch_bounds__(kTapThreads) k_tap_place_team(const TapPlace p) {
+    static_assert(PER == 1 || sizeof(Mask) == 4, "a worker's bit is in word r / 32");
+    extern __shared__ __align__(16) uint8_t tap_smem[];
+    uint64_t* v_smp = reinterpret_cast<uint64_t*>(tap_smem);
+    Mask* held = reinterpret_cast<Mask*>(v_smp + p.n);
+    __shared__ TapDelta<uint64_t> s_delta[2][kTapTeam][32 * PER];
+    __shared__ int s_pick[2][kTapTeam];
+    __shared__ unsigned long long s_sum, s_vol;
+    const int n = p.n, H = p.H, W = p.W;
+    if (threadIdx.x == 0) s_sum = s_vol = 0;
+    __syncthreads();
+    unsigned long long part = 0, vol = 0, most = 0;
+    for (int j = threadIdx.x; j < n; j += kTapThreads) { v_smp[j] = (uint64_t)(p.v_smp[j] / p.unit); vol += v_smp[j]; }
+    for (int j = threadIdx.x; j < n; j += kTapThreads) {   // the groups a worker holds in full
+        const int r = p.res_smp[j];
+        for (int h = 0; h < H; ++h)
+#pragma unroll
+            for (int u = 0; u < PER; ++u)
+                held[((size_t)h * n + j) * PER + u] = r >= 0 && r < W && r >> 5 == u ? (Mask)(1u << (r & 31)) : (Mask)0;
+    }
+    for (int64_t b = threadIdx.x; b < p.NB; b += kTapThreads) {
+        part += (unsigned long long)p.rec[b].f * H;
+        const unsigned long long v = (unsigned long long)(p.rec[b].v_qo / p.unit);
+        most = v > most ? v : most;
+    }
+    atomicAdd(&s_sum, part);
+    atomicAdd(&s_vol, vol);
+    if (most >> 31) atomicAdd(&s_vol, 1ull << 32);
+    __syncthreads();
+    const int64_t sum_f = (int64_t)s_sum;
+    if (sum_f > (INT64_MAX / ((int64_t)(p.tau_den + p.tau_num) * 2)) / W) {  // the integer cap test would overflow
+        if (threadIdx.x == 0) *p.status = LIBRA_ERR_OVERFLOW;   // the exchange kernels see the flag and add nothing
+        for (int64_t x = threadIdx.x; x < p.NB * H; x += kTapThreads) p.sigma[(int64_t)p.rec[x / H].blk * H + x % H] = p.rec[x / H].q_home;
+        return;
+    }
+    // tau_den W (L + f) <= (tau_den + tau_num) sum f, as a bound on L + f
+    const int64_t cap = (int64_t)(p.tau_den + p.tau_num) * sum_f / ((int64_t)p.tau_den * W);
+    if (s_vol >> 31 == 0) tap_place_steps<PER, Mask, uint32_t>(p, cap, v_smp, held, s_delta, s_pick);
+    else tap_place_steps<PER, Mask, uint64_t>(p, cap, v_smp, held, s_delta, s_pick);
+    for (int64_t i = threadIdx.x; i < (int64_t)W * p.words; i += kTapThreads) {   // as bit rows per worker
+        const int r = (int)(i / p.words), g0 = (int)(i % p.words) * 32;
+        uint32_t bits = 0;
+        for (int b = 0; b < 32 && g0 + b < n * H; ++b) {
+            const int j = (g0 + b) / H, h = (g0 + b) % H;
+            bits |= ((uint32_t)held[((size_t)h * n + j) * PER + (r >> 5)] >> (r & 31) & 1u) << b;
+        }
+        p.Cbits[i] = bits;
+    }
 }
 
 // Forward / backward send-byte matrices [src][dst].
@@ -586,14 +724,19 @@ extern "C" int libra_tap_plan(const int32_t* cu_seqlens_dev, int n_samples, cons
         k_tap_blocks<<<(unsigned)((NB + 127) / 128), 128, 0, s>>>(g, NB, f_blk, q_home, v_qo, j0, j1, comm_total_dev);
         k_tap_samples<<<tap_sample_grid(n_samples, (int64_t)W * W), 128, 0, s>>>(g, v_smp, res_smp, clear);
         k_tap_rank<<<(unsigned)((NB + 255) / 256), 256, 0, s>>>(f_blk, NB, q_home, v_qo, j0, j1, ord, rec);
-        // one warp while its tables fit the shared memory a CTA has without opting in; an odd pitch keeps the lanes'
-        // rows on different banks
-        const int pitch = words | 1;
-        const size_t smem = sizeof(int64_t) * n_samples + sizeof(uint32_t) * (size_t)pitch * W;
-        if (W <= 128 && smem <= 48 * 1024) {
-            auto place = W <= 32 ? k_tap_place_warp<1> : (W <= 64 ? k_tap_place_warp<2> : k_tap_place_warp<4>);
-            place<<<1, 32, smem, s>>>(rec, v_smp, res_smp, NB, H, W, n_samples, o->tau_num, o->tau_den, cbits, words, pitch,
-                                      sigma_dev, loads_dev, comm_total_dev, status_dev);
+        // By one block while its tables fit shared memory.  (Bytes for up to eight workers: as few bits a group as the
+        // general kernel's bit rows, so that many shards of many samples fit as well.)
+        const int per = W <= 32 ? 1 : (W <= 64 ? 2 : 4);
+        const size_t smem = sizeof(int64_t) * n_samples + (W <= 8 ? sizeof(uint8_t) : sizeof(uint32_t)) * (size_t)per * H * n_samples;
+        if (W <= 128 && smem <= kTapTeamSmem) {
+            auto place = W <= 8 ? k_tap_place_team<1, uint8_t>
+                                : (W <= 32 ? k_tap_place_team<1, uint32_t> : (W <= 64 ? k_tap_place_team<2, uint32_t> : k_tap_place_team<4, uint32_t>));
+            if (smem > 48 * 1024 - kTapTeamStatic * per &&
+                cudaFuncSetAttribute(place, cudaFuncAttributeMaxDynamicSharedMemorySize, kTapTeamSmem) != cudaSuccess)
+                rc = LIBRA_ERR_CUDA;
+            const TapPlace tp = {rec, v_smp, res_smp, NB, (int64_t)4 * o->head_dim, H, W, n_samples, o->tau_num, o->tau_den, words, cbits,
+                                 sigma_dev, loads_dev, comm_total_dev, status_dev};
+            place<<<1, kTapThreads, smem, s>>>(tp);
         } else {
             k_tap_place<<<1, ((W + 31) / 32) * 32, 0, s>>>(f_blk, ord, q_home, v_qo, j0, j1, v_smp, res_smp, NB, H, W,
                                                             n_samples, o->tau_num, o->tau_den, cbits, words, sigma_dev,

@@ -73,6 +73,24 @@ def test_worker_counts_around_the_one_warp_placement(P, CP, max_len):
     _compare(cu, np.arange(P + 1, dtype=np.int32) * 1500, CP, 100, 2, 8, 4, 64)
 
 
+@pytest.mark.parametrize("P,CP,H,hq,hkv,max_len,total", [
+    (2, 4, 8, 8, 4, 400, 3000),            # a byte of residency per group; a full step of shards
+    (3, 3, 16, 16, 4, 60, 3000),           # two steps a block, nine workers
+    (2, 20, 24, 24, 8, 150, 2000),         # three steps a block, two workers a lane
+    (2, 4, 20, 20, 5, 100, 2000),          # the last step half full
+    (2, 2, 2, 1 << 17, 1 << 17, 900, 20000),   # volumes beyond 32 bits
+    (2, 40, 1, 1 << 18, 1 << 18, 900, 5000),   # the same with four workers a lane
+    (4, 2, 8, 8, 8, 3, 3000),              # tables beyond the shared memory a block has without opting in
+    (4, 4, 32, 32, 8, 2, 6000),            # tables beyond shared memory
+])
+def test_steps_of_the_one_block_placement(P, CP, H, hq, hkv, max_len, total):
+    rng = np.random.default_rng(P * CP + H)
+    seqs = [pools.random_layout(rng, total, max_len) for _ in range(P)]
+    cu = pools.cu_seqlens([x for s in seqs for x in s])
+    for tau in ((3, 100), (0, 1)):
+        _compare(cu, np.arange(P + 1, dtype=np.int32) * total, CP, 128, H, hq, hkv, 8, tau)
+
+
 def test_zero_length_samples_and_short_tail():
     _compare([0, 0, 3, 3, 3, 40, 40, 41], [0, 41], 2, 16, 2, 4, 2, 8)
     _compare([0, 7, 7, 30, 30], [0, 7, 30], 1, 4, 1, 2, 2, 8)
