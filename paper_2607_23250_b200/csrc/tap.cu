@@ -10,7 +10,7 @@
 // Placement is sequential by nature (every choice depends on the loads and residency left by the previous
 // ones), so the latency of one step bounds it.  Up to 128 workers whose tables fit shared memory: one block whose
 // warps work on neighbouring steps (k_tap_place_team).  Otherwise: one CTA with a thread per worker, block-wide
-// arg-min, tables in global memory.  1024 tiles on 16 workers with their schedule: 0.30 ms, with one warp for all of a
+// arg-min, tables in global memory.  1024 tiles on 16 workers with their schedule: 0.26 ms, with one warp for all of a
 // step 0.65 ms, all in the second form 2.8 ms.
 #include <cstdint>
 #include <new>
@@ -18,6 +18,7 @@
 
 #include "../../include/libra.h"
 #include "common.h"
+#include "ptx.cuh"
 
 namespace libra {
 
@@ -26,6 +27,13 @@ struct TapGeom {
     const int32_t* seq_off;   // [P+1] token offsets of the packed sequences
     const int32_t* blk_off;   // [P+1] first block of each sequence
     int n, P, CP, B, H, hq, hkv, d;
+};
+// The two tables of a pool of up to kTapParamSeqs sequences, as a kernel argument: the first kernel of a call reads them
+// there and leaves them in the call's scratch for the others.  (A copy from pageable memory instead took the host 10 us a
+// call and the stream 3.)
+constexpr int kTapParamSeqs = 255;
+struct TapTables {
+    int32_t seq_off[kTapParamSeqs + 1], blk_off[kTapParamSeqs + 1];
 };
 
 __device__ __forceinline__ int tap_seq_of_token(const TapGeom& g, int64_t tok) {
@@ -38,70 +46,94 @@ __device__ __forceinline__ int tap_owner(const TapGeom& g, int s, int64_t tok) {
     const int64_t run = (len + g.CP - 1) / g.CP;
     return s * g.CP + (int)((tok - g.seq_off[s]) / (run > 0 ? run : 1));
 }
-// index of the sample that holds token tok (the last j with cu[j] <= tok; it is never empty)
-__device__ __forceinline__ int tap_sample_of_token(const TapGeom& g, int64_t tok) {
-    int lo = 0, hi = g.n;  // invariant: cu[lo] <= tok < cu[hi]
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (g.cu[mid] <= tok) lo = mid; else hi = mid;
+// Index of the sample that holds token tok (the last j with cu[j] <= tok; it is never empty), by a warp, 32 probes at a time.
+__device__ __forceinline__ int tap_sample_of_token_warp(const TapGeom& g, int64_t tok) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0, len = g.n;   // the sample is one of [lo, lo + len)
+    while (len > 1) {
+        const int step = (len + 31) / 32, at = lo + lane * step;
+        const unsigned below = __ballot_sync(0xffffffffu, lane == 0 || (lane * step < len && g.cu[at] <= tok));
+        const int skip = (31 - __clz(below)) * step;
+        lo += skip;
+        len = len - skip < step ? len - skip : step;
     }
     return lo;
 }
 
-// Per block: work (Eq. 6 in closed form), Q-home, Q + output bytes, first and last sample.
-__global__ void k_tap_blocks(TapGeom g, int64_t NB, int64_t* __restrict__ f_blk, int32_t* __restrict__ q_home,
-                             int64_t* __restrict__ v_qo, int32_t* __restrict__ j_first, int32_t* __restrict__ j_last,
-                             int64_t* comm_total) {
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b == 0 && comm_total) *comm_total = 0;
-    if (b >= NB) return;
-    int s = 0;
-    while (s + 1 < g.P && g.blk_off[s + 1] <= b) ++s;
-    const int64_t q0 = g.seq_off[s] + (b - g.blk_off[s]) * g.B;
-    const int64_t q1 = q0 + g.B < g.seq_off[s + 1] ? q0 + g.B : g.seq_off[s + 1];
-    const int j0 = tap_sample_of_token(g, q0), j1 = tap_sample_of_token(g, q1 - 1);
-    int64_t w = 0;
-    for (int j = j0; j <= j1; ++j) {
-        const int64_t lo = q0 > g.cu[j] ? q0 : g.cu[j], hi = q1 < g.cu[j + 1] ? q1 : g.cu[j + 1];
-        if (lo < hi) {
-            const int64_t a = lo - g.cu[j], e = hi - g.cu[j];
-            w += (e * (e + 1) - a * (a + 1)) / 2;
-        }
-    }
-    f_blk[b] = w;
-    q_home[b] = tap_owner(g, s, q0);
-    v_qo[b] = 2 * ((q1 - q0) * (g.hq / g.H) * g.d * 2);
-    j_first[b] = j0;
-    j_last[b] = j1;
-}
-
-// Per sample: bytes of its K and V on one head shard, and the worker that holds all of it (or -1).
-// The grid also clears up to three arrays of 64-bit words (and the status) that later kernels add to.
-struct TapClear {
-    int64_t* p[3];
-    int64_t n[3];
+// What the first kernel of a call writes: per block its work (Eq. 6 in closed form), Q-home, Q + output bytes, first and
+// last sample; per sample the bytes of its K and V on one head shard and the worker that holds all of it (or -1).  The grid
+// also clears up to three arrays of 64-bit words, the status and the volume total, which later kernels add to.
+struct TapSetup {
+    int64_t NB;
+    int block_ctas;          // CTAs that go through blocks, a warp each; the rest through samples
+    int from_params;         // the tables come as an argument: write them to seq_off, blk_off
+    int32_t *seq_off, *blk_off;
+    int64_t* f_blk;
+    int32_t* q_home;
+    int64_t* v_qo;
+    int32_t *j_first, *j_last;
+    int64_t* v_smp;
+    int32_t* res_smp;
+    int64_t* clear[3];
+    int64_t n_clear[3];
     int* status;
+    int64_t* comm_total;
 };
-static unsigned tap_sample_grid(int n_samples, int64_t words) {   // a thread per sample, and enough of them to clear
-    const int64_t a = ((int64_t)n_samples + 127) / 128, b = (words + 1023) / 1024;
-    return (unsigned)(a > b ? a : (b < 148 ? b : (a > 148 ? a : 148)));
-}
-__global__ void k_tap_samples(TapGeom g, int64_t* __restrict__ v_smp, int32_t* __restrict__ res_smp, TapClear c) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(128) k_tap_setup(TapGeom g, const TapSetup p, const __grid_constant__ TapTables tables) {
+    grid_dep_wait();
+    grid_dep_launch();
+    if (p.from_params) {
+        if (blockIdx.x == 0)
+            for (int q = threadIdx.x; q <= g.P; q += 128) { p.seq_off[q] = tables.seq_off[q]; p.blk_off[q] = tables.blk_off[q]; }
+        g.seq_off = tables.seq_off;
+        g.blk_off = tables.blk_off;
+    }
+    const int64_t all = (int64_t)gridDim.x * 128, at = blockIdx.x * (int64_t)128 + threadIdx.x;
+#pragma unroll
     for (int k = 0; k < 3; ++k)
-        for (int64_t x = j; x < c.n[k]; x += (int64_t)gridDim.x * blockDim.x) c.p[k][x] = 0;
-    if (j == 0 && c.status) *c.status = 0;
+        for (int64_t x = at; x < p.n_clear[k]; x += all) p.clear[k][x] = 0;
+    if (at == 0 && p.status) *p.status = 0;
+    if (at == 0 && p.comm_total) *p.comm_total = 0;
+    if ((int)blockIdx.x < p.block_ctas) {
+        const int64_t b = at >> 5;
+        const int lane = threadIdx.x & 31;
+        if (b >= p.NB) return;
+        int s = 0;
+        while (s + 1 < g.P && g.blk_off[s + 1] <= b) ++s;
+        const int64_t q0 = g.seq_off[s] + (b - g.blk_off[s]) * g.B;
+        const int64_t q1 = q0 + g.B < g.seq_off[s + 1] ? q0 + g.B : g.seq_off[s + 1];
+        const int j0 = tap_sample_of_token_warp(g, q0), j1 = tap_sample_of_token_warp(g, q1 - 1);
+        int64_t w = 0;
+        for (int j = j0 + lane; j <= j1; j += 32) {
+            const int64_t lo = q0 > g.cu[j] ? q0 : g.cu[j], hi = q1 < g.cu[j + 1] ? q1 : g.cu[j + 1];
+            if (lo < hi) {
+                const int64_t a = lo - g.cu[j], e = hi - g.cu[j];
+                w += (e * (e + 1) - a * (a + 1)) / 2;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+        if (lane == 0) {
+            if (p.f_blk) p.f_blk[b] = w;
+            p.q_home[b] = tap_owner(g, s, q0);
+            if (p.v_qo) p.v_qo[b] = 2 * ((q1 - q0) * (g.hq / g.H) * g.d * 2);
+            p.j_first[b] = j0;
+            p.j_last[b] = j1;
+        }
+        return;
+    }
+    const int64_t j = at - (int64_t)p.block_ctas * 128;
     if (j >= g.n) return;
     const int64_t a = g.cu[j], e = g.cu[j + 1];
     const int kvps = g.H <= g.hkv ? g.hkv / g.H : 1;
-    v_smp[j] = 2 * (e - a) * kvps * g.d * 2;
+    if (p.v_smp) p.v_smp[j] = 2 * (e - a) * kvps * g.d * 2;
     int res = -1;
     if (e > a) {
         const int s = tap_seq_of_token(g, a);
         const int first = tap_owner(g, s, a), last = tap_owner(g, s, e - 1);
         res = first == last ? first : -1;
     }
-    res_smp[j] = res;
+    p.res_smp[j] = res;
 }
 
 // A block as the placement reads it.
@@ -110,22 +142,31 @@ struct __align__(16) TapRec {
     int32_t q_home, j0, j1, blk;
 };
 
-__global__ void k_tap_rank(const int64_t* __restrict__ f_blk, int64_t NB, const int32_t* __restrict__ q_home,
-                           const int64_t* __restrict__ v_qo, const int32_t* __restrict__ j_first,
-                           const int32_t* __restrict__ j_last, int32_t* __restrict__ blk_order, TapRec* __restrict__ rec) {
-    __shared__ int64_t sw[256];
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// Blocks by (work descending, index ascending); sixteen lanes share a block's comparisons, so that a few hundred blocks
+// fill more than one CTA (256 blocks: 9 us by a thread each, 4 so).
+__global__ void __launch_bounds__(256) k_tap_rank(const int64_t* __restrict__ f_blk, int64_t NB, const int32_t* __restrict__ q_home,
+                                                  const int64_t* __restrict__ v_qo, const int32_t* __restrict__ j_first,
+                                                  const int32_t* __restrict__ j_last, int32_t* __restrict__ blk_order, TapRec* __restrict__ rec) {
+    __shared__ int64_t sw[1024];
+    const int64_t b = blockIdx.x * (int64_t)16 + (threadIdx.x >> 4);
+    const int sub = threadIdx.x & 15;
+    grid_dep_wait();
+    grid_dep_launch();
     const int64_t wb = b < NB ? f_blk[b] : 0;
-    int64_t rank = 0;
-    for (int64_t base = 0; base < NB; base += 256) {
-        const int64_t o = base + threadIdx.x;
-        sw[threadIdx.x] = o < NB ? f_blk[o] : -1;
+    int rank = 0;
+    for (int64_t base = 0; base < NB; base += 1024) {
+        const int lim = (int)(NB - base < 1024 ? NB - base : 1024);
+        for (int o = threadIdx.x; o < lim; o += 256) sw[o] = f_blk[base + o];
         __syncthreads();
-        const int lim = (int)((NB - base < 256) ? NB - base : 256);
-        for (int i = 0; i < lim; ++i) rank += (sw[i] > wb) || (sw[i] == wb && base + i < b);
+        for (int k = sub; k < lim; k += 16) {
+            const int64_t w = sw[k];
+            rank += (w > wb) || (w == wb && base + k < b);
+        }
         __syncthreads();
     }
-    if (b < NB) {
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (b < NB && sub == 0) {
         blk_order[rank] = (int32_t)b;
         rec[rank] = TapRec{wb, v_qo[b], q_home[b], j_first[b], j_last[b], (int32_t)b};
     }
@@ -163,6 +204,7 @@ __global__ void __launch_bounds__(1024) k_tap_place(
     __shared__ int64_t s_pick_delta;
     const int r = threadIdx.x, lane = r & 31, warp = r >> 5, nwarps = blockDim.x >> 5;
     const bool live = r < W;
+    grid_dep_wait();
     // residency rows start with the groups the worker already holds in full
     if (live) {
         uint32_t* row = Cbits + (size_t)r * words;
@@ -446,6 +488,7 @@ __global__ void __launch_bounds__(kTapThreads) k_tap_place_team(const TapPlace p
     __shared__ int s_pick[2][kTapTeam];
     __shared__ unsigned long long s_sum, s_vol;
     const int n = p.n, H = p.H, W = p.W;
+    grid_dep_wait();
     if (threadIdx.x == 0) s_sum = s_vol = 0;
     __syncthreads();
     unsigned long long part = 0, vol = 0, most = 0;
@@ -476,6 +519,7 @@ __global__ void __launch_bounds__(kTapThreads) k_tap_place_team(const TapPlace p
     const int64_t cap = (int64_t)(p.tau_den + p.tau_num) * sum_f / ((int64_t)p.tau_den * W);
     if (s_vol >> 31 == 0) tap_place_steps<PER, Mask, uint32_t>(p, cap, v_smp, held, s_delta, s_pick);
     else tap_place_steps<PER, Mask, uint64_t>(p, cap, v_smp, held, s_delta, s_pick);
+    grid_dep_launch();   // (not before: the next kernel's blocks would sit on the other SMs all the while)
     for (int64_t i = threadIdx.x; i < (int64_t)W * p.words; i += kTapThreads) {   // as bit rows per worker
         const int r = (int)(i / p.words), g0 = (int)(i % p.words) * 32;
         uint32_t bits = 0;
@@ -487,27 +531,27 @@ __global__ void __launch_bounds__(kTapThreads) k_tap_place_team(const TapPlace p
     }
 }
 
-// Forward / backward send-byte matrices [src][dst].
-__global__ void k_tap_exchange_qo(const int32_t* __restrict__ sigma, const int32_t* __restrict__ q_home,
-                                  const int64_t* __restrict__ v_qo, int64_t NT, int H, int W,
-                                  const int* __restrict__ status, unsigned long long* __restrict__ fwd,
-                                  unsigned long long* __restrict__ bwd) {
+// Forward / backward send-byte matrices [src][dst]: a thread per tile (Q and output), then one per worker and KV group.
+__global__ void k_tap_exchange(TapGeom g, int64_t NT, const int32_t* __restrict__ sigma, const int32_t* __restrict__ q_home,
+                               const int64_t* __restrict__ v_qo, const uint32_t* __restrict__ Cbits, int words,
+                               const int32_t* __restrict__ res_smp, int W, const int* __restrict__ status,
+                               unsigned long long* __restrict__ fwd, unsigned long long* __restrict__ bwd) {
+    grid_dep_wait();
+    grid_dep_launch();
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= NT || *status != 0) return;   // a placement that gave up left sigma unwritten
-    const int q = q_home[t / H], r = sigma[t];
-    if (q == r || r < 0 || r >= W || q < 0 || q >= W) return;
-    const unsigned long long v = (unsigned long long)(v_qo[t / H] / 2);
-    atomicAdd(&fwd[(size_t)q * W + r], v);   // Q out
-    atomicAdd(&fwd[(size_t)r * W + q], v);   // output back
-    atomicAdd(&bwd[(size_t)q * W + r], v);   // dO along the Q path
-    atomicAdd(&bwd[(size_t)r * W + q], v);   // dQ along the output path
-}
-__global__ void k_tap_exchange_kv(TapGeom g, const uint32_t* __restrict__ Cbits, int words,
-                                  const int32_t* __restrict__ res_smp, int W, const int* __restrict__ status,
-                                  unsigned long long* __restrict__ fwd, unsigned long long* __restrict__ bwd) {
-    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t NG = (int64_t)g.n * g.H;
-    if (idx >= NG * W || *status != 0) return;
+    if (*status != 0) return;   // a placement that gave up left sigma unwritten
+    if (t < NT) {
+        const int q = q_home[t / g.H], r = sigma[t];
+        if (q == r || r < 0 || r >= W || q < 0 || q >= W) return;
+        const unsigned long long v = (unsigned long long)(v_qo[t / g.H] / 2);
+        atomicAdd(&fwd[(size_t)q * W + r], v);   // Q out
+        atomicAdd(&fwd[(size_t)r * W + q], v);   // output back
+        atomicAdd(&bwd[(size_t)q * W + r], v);   // dO along the Q path
+        atomicAdd(&bwd[(size_t)r * W + q], v);   // dQ along the output path
+        return;
+    }
+    const int64_t idx = t - NT, NG = (int64_t)g.n * g.H;
+    if (idx >= NG * W) return;
     const int r = (int)(idx / NG);
     const int grp = (int)(idx % NG), j = grp / g.H;
     if (!((Cbits[(size_t)r * words + (grp >> 5)] >> (grp & 31)) & 1u) || res_smp[j] == r) return;
@@ -537,6 +581,8 @@ __global__ void k_tap_exchange_kv(TapGeom g, const uint32_t* __restrict__ Cbits,
 __global__ void k_tap_mark(const int32_t* __restrict__ sigma, const int32_t* __restrict__ j_first,
                            const int32_t* __restrict__ j_last, int64_t NT, int H, int W, int words,
                            uint32_t* __restrict__ marks) {
+    grid_dep_wait();
+    grid_dep_launch();
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= NT) return;
     const int r = sigma[t], h = (int)(t % H);
@@ -568,23 +614,46 @@ __device__ __forceinline__ int tap_slot_count(const TapGeom& g, int64_t x, int64
     return c;
 }
 
-__global__ void k_tap_sched_count(TapGeom g, int64_t NT, int64_t NG, int W, const int32_t* __restrict__ sigma,
-                                  const int32_t* __restrict__ q_home, const uint32_t* __restrict__ marks, int words,
-                                  const int32_t* __restrict__ res_smp, int64_t* __restrict__ offs /*[slots]*/) {
-    const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (x < NT + NG * W) offs[x] = tap_slot_count(g, x, NT, NG, W, sigma, q_home, marks, words, res_smp);
+constexpr int kTapSlots = 256;         // slots per CTA
+constexpr int kTapInlineCtas = 2048;   // up to so many CTAs each adds up the totals of those before it; beyond, k_tap_sched_scan
+
+// Inclusive prefix sum over the CTA's kTapSlots threads.
+__device__ __forceinline__ int tap_scan(int c, int* part) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, c, o); if (lane >= o) c += v; }
+    if (lane == 31) part[warp] = c;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) c += part[w];
+    return c;
 }
 
-// One block: exclusive prefix sum of the slot counts in place, 4096 of them per pass, total to n_out.
-__global__ void __launch_bounds__(1024) k_tap_sched_scan(int64_t slots, int64_t* __restrict__ offs /*[slots]*/, int64_t* n_out) {
+// Records ahead of each slot among its CTA's, and the CTA's total.
+__global__ void __launch_bounds__(kTapSlots) k_tap_sched_count(TapGeom g, int64_t NT, int64_t NG, int W, const int32_t* __restrict__ sigma,
+                                  const int32_t* __restrict__ q_home, const uint32_t* __restrict__ marks, int words,
+                                  const int32_t* __restrict__ res_smp, int32_t* __restrict__ ahead /*[slots]*/, int64_t* __restrict__ total) {
+    __shared__ int part[kTapSlots / 32];
+    grid_dep_wait();
+    grid_dep_launch();
+    const int64_t x = blockIdx.x * (int64_t)kTapSlots + threadIdx.x;
+    const int c = x < NT + NG * W ? tap_slot_count(g, x, NT, NG, W, sigma, q_home, marks, words, res_smp) : 0;
+    const int incl = tap_scan(c, part);
+    if (x < NT + NG * W) ahead[x] = incl - c;
+    if (threadIdx.x == kTapSlots - 1) total[blockIdx.x] = incl;
+}
+
+// One block: exclusive prefix sum of n numbers in place, 4096 of them per pass, total to n_out.
+__global__ void __launch_bounds__(1024) k_tap_sched_scan(int64_t n, int64_t* __restrict__ sums, int64_t* n_out) {
     __shared__ int64_t part[32];
+    grid_dep_wait();
+    grid_dep_launch();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t run = 0;
-    for (int64_t base = 0; base < slots; base += 4096) {
+    for (int64_t base = 0; base < n; base += 4096) {
         const int64_t x0 = base + threadIdx.x * 4;
         int64_t c[4], sum = 0;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) { c[k] = x0 + k < slots ? offs[x0 + k] : 0; sum += c[k]; }
+        for (int k = 0; k < 4; ++k) { c[k] = x0 + k < n ? sums[x0 + k] : 0; sum += c[k]; }
         int64_t incl = sum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) { const int64_t v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
@@ -594,20 +663,34 @@ __global__ void __launch_bounds__(1024) k_tap_sched_scan(int64_t slots, int64_t*
         for (int w = 0; w < 32; ++w) { if (w < warp) before += part[w]; all += part[w]; }
         int64_t at = run + before + incl - sum;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) { if (x0 + k < slots) offs[x0 + k] = at; at += c[k]; }
+        for (int k = 0; k < 4; ++k) { if (x0 + k < n) sums[x0 + k] = at; at += c[k]; }
         run += all;
         __syncthreads();
     }
     if (threadIdx.x == 0) *n_out = run;
 }
 
-__global__ void k_tap_sched_fill(TapGeom g, int64_t NT, int64_t NG, int W, const int32_t* __restrict__ sigma,
+__global__ void __launch_bounds__(kTapSlots) k_tap_sched_fill(TapGeom g, int64_t NT, int64_t NG, int W, const int32_t* __restrict__ sigma,
                                  const int32_t* __restrict__ q_home, const uint32_t* __restrict__ marks, int words,
-                                 const int32_t* __restrict__ res_smp, const int64_t* __restrict__ offs,
-                                 int64_t capacity, int32_t* __restrict__ rec) {
-    const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+                                 const int32_t* __restrict__ res_smp, const int32_t* __restrict__ ahead, const int64_t* __restrict__ total,
+                                 int scanned, int64_t* __restrict__ n_out, int64_t capacity, int32_t* __restrict__ rec) {
+    __shared__ unsigned long long s_before;
+    if (threadIdx.x == 0) s_before = 0;
+    grid_dep_wait();
+    grid_dep_launch();
+    __syncthreads();
+    if (scanned) {
+        if (threadIdx.x == 0) s_before = (unsigned long long)total[blockIdx.x];
+    } else {
+        unsigned long long sum = 0;
+        for (unsigned c = threadIdx.x; c < blockIdx.x; c += kTapSlots) sum += (unsigned long long)total[c];
+        if (sum) atomicAdd(&s_before, sum);
+    }
+    __syncthreads();
+    if (!scanned && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *n_out = (int64_t)s_before + total[blockIdx.x];
+    const int64_t x = blockIdx.x * (int64_t)kTapSlots + threadIdx.x;
     if (x >= NT + NG * W) return;
-    int64_t at = offs[x];
+    int64_t at = (int64_t)s_before + ahead[x];
     if (x < NT) {
         const int r = sigma[x];
         const int64_t b = x / g.H;
@@ -654,6 +737,38 @@ extern "C" int64_t libra_tap_num_tiles(const int32_t* seq_offsets_host, int n_se
     return nb * n_shards;
 }
 
+// First kernel of a call.  The tables of the pool (`table`: 2 (P + 1) words of scratch) go with it as an argument, or, of more
+// sequences than an argument holds, ahead of it in a copy.
+static int launch_setup(TapGeom& g, TapSetup p, const int32_t* seq_offsets_host, int32_t* table, cudaStream_t s) {
+    static const TapTables none = {};
+    TapTables tables;
+    p.from_params = g.P <= kTapParamSeqs;
+    int32_t* h_tab = p.from_params ? nullptr : new (std::nothrow) int32_t[2 * (g.P + 1)];
+    if (!p.from_params && !h_tab) return LIBRA_ERR_CUDA;
+    int32_t* seq_off = p.from_params ? tables.seq_off : h_tab;
+    int32_t* blk_off = p.from_params ? tables.blk_off : h_tab + g.P + 1;
+    int64_t nb = 0;
+    for (int q = 0; q <= g.P; ++q) {
+        seq_off[q] = seq_offsets_host[q];
+        blk_off[q] = (int32_t)nb;
+        if (q < g.P) nb += ((int64_t)seq_offsets_host[q + 1] - seq_offsets_host[q] + g.B - 1) / g.B;
+    }
+    cudaError_t e = cudaSuccess;
+    if (h_tab) {   // from pageable memory, so the copy has left h_tab when the call returns
+        e = cudaMemcpyAsync(table, h_tab, sizeof(int32_t) * 2 * (g.P + 1), cudaMemcpyHostToDevice, s);
+        delete[] h_tab;
+    }
+    p.seq_off = table;
+    p.blk_off = table + g.P + 1;
+    g.seq_off = p.seq_off;
+    g.blk_off = p.blk_off;
+    p.block_ctas = (int)((p.NB + 3) / 4);
+    const unsigned sample_ctas = (unsigned)(((int64_t)g.n + 127) / 128);
+    if (e == cudaSuccess) e = launch_dependent(k_tap_setup, (unsigned)p.block_ctas + sample_ctas, 128u, 0, s, g, p, p.from_params ? tables : none);
+    count_launch();
+    return e == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
+}
+
 extern "C" int libra_tap_plan(const int32_t* cu_seqlens_dev, int n_samples, const int32_t* seq_offsets_host,
                               int n_sequences, const libra_tap_opts* o, int32_t* sigma_dev, int64_t* loads_dev,
                               int64_t* fwd_bytes_dev, int64_t* bwd_bytes_dev, int64_t* comm_total_dev,
@@ -679,15 +794,6 @@ extern "C" int libra_tap_plan(const int32_t* cu_seqlens_dev, int n_samples, cons
     cudaStream_t s = (cudaStream_t)stream;
     const int words = (int)(((int64_t)n_samples * H + 31) / 32);
 
-    // small host tables -> device (stream-ordered scratch; nothing outlives the call's work on `stream`)
-    int32_t* h_tab = new (std::nothrow) int32_t[2 * (P + 1)];
-    if (!h_tab) return LIBRA_ERR_CUDA;
-    int64_t nb = 0;
-    for (int q = 0; q <= P; ++q) {
-        h_tab[q] = seq_offsets_host[q];
-        h_tab[P + 1 + q] = (int32_t)nb;
-        if (q < P) nb += ((int64_t)seq_offsets_host[q + 1] - seq_offsets_host[q] + o->block - 1) / o->block;
-    }
     uint8_t* scratch = nullptr;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t at = off; off += (bytes + 255) & ~size_t(255); return at; };
@@ -697,17 +803,7 @@ extern "C" int libra_tap_plan(const int32_t* cu_seqlens_dev, int n_samples, cons
     const size_t o_ord = take(sizeof(int32_t) * NB), o_rec = take(sizeof(TapRec) * NB);
     const size_t o_vs = take(sizeof(int64_t) * n_samples), o_rs = take(sizeof(int32_t) * n_samples);
     const size_t o_c = take(sizeof(uint32_t) * (size_t)words * W);
-    if (scratch_alloc((void**)&scratch, off, s) != cudaSuccess) { delete[] h_tab; return LIBRA_ERR_CUDA; }
-    int rc = LIBRA_OK;
-    // the table is copied from pageable memory, so the copy has left h_tab when the call returns
-    if (cudaMemcpyAsync(scratch + o_tab, h_tab, sizeof(int32_t) * 2 * (P + 1), cudaMemcpyHostToDevice, s) != cudaSuccess)
-        rc = LIBRA_ERR_CUDA;
-    delete[] h_tab;
-    TapGeom g;
-    g.cu = cu_seqlens_dev;
-    g.seq_off = (const int32_t*)(scratch + o_tab);
-    g.blk_off = g.seq_off + (P + 1);
-    g.n = n_samples; g.P = P; g.CP = o->cp; g.B = o->block; g.H = H; g.hq = o->hq; g.hkv = o->hkv; g.d = o->head_dim;
+    if (scratch_alloc((void**)&scratch, off, s) != cudaSuccess) return LIBRA_ERR_CUDA;
     int64_t* f_blk = (int64_t*)(scratch + o_f);
     int64_t* v_qo = (int64_t*)(scratch + o_vqo);
     int32_t* q_home = (int32_t*)(scratch + o_q);
@@ -718,12 +814,16 @@ extern "C" int libra_tap_plan(const int32_t* cu_seqlens_dev, int n_samples, cons
     int64_t* v_smp = (int64_t*)(scratch + o_vs);
     int32_t* res_smp = (int32_t*)(scratch + o_rs);
     uint32_t* cbits = (uint32_t*)(scratch + o_c);
+    TapGeom g;
+    g.cu = cu_seqlens_dev;
+    g.n = n_samples; g.P = P; g.CP = o->cp; g.B = o->block; g.H = H; g.hq = o->hq; g.hkv = o->hkv; g.d = o->head_dim;
+    // W * W byte matrices, loads, the volume total and the status start from zero
+    const TapSetup setup = {NB, 0, 0, nullptr, nullptr, f_blk, q_home, v_qo, j0, j1, v_smp, res_smp,
+                            {fwd_bytes_dev, bwd_bytes_dev, loads_dev}, {(int64_t)W * W, (int64_t)W * W, W}, status_dev, comm_total_dev};
+    int rc = launch_setup(g, setup, seq_offsets_host, (int32_t*)(scratch + o_tab), s);
+    auto launched = [&](cudaError_t e) { if (e != cudaSuccess) rc = LIBRA_ERR_CUDA; };
     if (rc == LIBRA_OK) {
-        // W * W byte matrices, loads and the volume total start from zero
-        const TapClear clear = {{fwd_bytes_dev, bwd_bytes_dev, loads_dev}, {(int64_t)W * W, (int64_t)W * W, W}, status_dev};
-        k_tap_blocks<<<(unsigned)((NB + 127) / 128), 128, 0, s>>>(g, NB, f_blk, q_home, v_qo, j0, j1, comm_total_dev);
-        k_tap_samples<<<tap_sample_grid(n_samples, (int64_t)W * W), 128, 0, s>>>(g, v_smp, res_smp, clear);
-        k_tap_rank<<<(unsigned)((NB + 255) / 256), 256, 0, s>>>(f_blk, NB, q_home, v_qo, j0, j1, ord, rec);
+        launched(launch_dependent(k_tap_rank, (unsigned)((NB + 15) / 16), 256u, 0, s, f_blk, NB, q_home, v_qo, j0, j1, ord, rec));
         // By one block while its tables fit shared memory.  (Bytes for up to eight workers: as few bits a group as the
         // general kernel's bit rows, so that many shards of many samples fit as well.)
         const int per = W <= 32 ? 1 : (W <= 64 ? 2 : 4);
@@ -736,21 +836,16 @@ extern "C" int libra_tap_plan(const int32_t* cu_seqlens_dev, int n_samples, cons
                 rc = LIBRA_ERR_CUDA;
             const TapPlace tp = {rec, v_smp, res_smp, NB, (int64_t)4 * o->head_dim, H, W, n_samples, o->tau_num, o->tau_den, words, cbits,
                                  sigma_dev, loads_dev, comm_total_dev, status_dev};
-            place<<<1, kTapThreads, smem, s>>>(tp);
+            launched(launch_dependent(place, 1u, kTapThreads, smem, s, tp));
         } else {
-            k_tap_place<<<1, ((W + 31) / 32) * 32, 0, s>>>(f_blk, ord, q_home, v_qo, j0, j1, v_smp, res_smp, NB, H, W,
-                                                            n_samples, o->tau_num, o->tau_den, cbits, words, sigma_dev,
-                                                            loads_dev, comm_total_dev, status_dev);
+            launched(launch_dependent(k_tap_place, 1u, (unsigned)((W + 31) / 32 * 32), 0, s, f_blk, ord, q_home, v_qo, j0, j1, v_smp, res_smp,
+                                      NB, H, W, n_samples, o->tau_num, o->tau_den, cbits, words, sigma_dev, loads_dev, comm_total_dev,
+                                      status_dev));
         }
-        k_tap_exchange_qo<<<(unsigned)((NT + 255) / 256), 256, 0, s>>>(sigma_dev, q_home, v_qo, NT, H, W, status_dev,
-                                                                       (unsigned long long*)fwd_bytes_dev,
-                                                                       (unsigned long long*)bwd_bytes_dev);
-        const int64_t pairs = (int64_t)n_samples * H * W;
-        k_tap_exchange_kv<<<(unsigned)((pairs + 255) / 256), 256, 0, s>>>(g, cbits, words, res_smp, W, status_dev,
-                                                                          (unsigned long long*)fwd_bytes_dev,
-                                                                          (unsigned long long*)bwd_bytes_dev);
-        count_launch(6);
-        if (cudaGetLastError() != cudaSuccess) rc = LIBRA_ERR_CUDA;
+        const int64_t threads = NT + (int64_t)n_samples * H * W;
+        launched(launch_dependent(k_tap_exchange, (unsigned)((threads + 255) / 256), 256u, 0, s, g, NT, sigma_dev, q_home, v_qo, cbits, words,
+                                  res_smp, W, status_dev, (unsigned long long*)fwd_bytes_dev, (unsigned long long*)bwd_bytes_dev));
+        count_launch(3);
     }
     scratch_free(scratch, s);
     return rc;
@@ -772,54 +867,40 @@ extern "C" int libra_tap_schedule(const int32_t* cu_seqlens_dev, int n_samples, 
     if (NT >= INT32_MAX || NG * W >= INT32_MAX) return LIBRA_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;
     const int words = (int)((NG + 31) / 32);
-    int32_t* h_tab = new (std::nothrow) int32_t[2 * (P + 1)];
-    if (!h_tab) return LIBRA_ERR_CUDA;
-    int64_t nb = 0;
-    for (int q = 0; q <= P; ++q) {
-        h_tab[q] = seq_offsets_host[q];
-        h_tab[P + 1 + q] = (int32_t)nb;
-        if (q < P) nb += ((int64_t)seq_offsets_host[q + 1] - seq_offsets_host[q] + o->block - 1) / o->block;
-    }
+    const int64_t slots = NT + NG * W, ctas = (slots + kTapSlots - 1) / kTapSlots;
     uint8_t* scratch = nullptr;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t at = off; off += (bytes + 255) & ~size_t(255); return at; };
     const size_t o_tab = take(sizeof(int32_t) * 2 * (P + 1));
-    const size_t o_f = take(sizeof(int64_t) * NB), o_vqo = take(sizeof(int64_t) * NB);
     const size_t o_q = take(sizeof(int32_t) * NB), o_j0 = take(sizeof(int32_t) * NB), o_j1 = take(sizeof(int32_t) * NB);
-    const size_t o_vs = take(sizeof(int64_t) * n_samples), o_rs = take(sizeof(int32_t) * n_samples);
+    const size_t o_rs = take(sizeof(int32_t) * n_samples);
     const size_t o_m = take(sizeof(uint32_t) * ((size_t)words * W + 1));
-    const size_t o_offs = take(sizeof(int64_t) * (size_t)(NT + NG * W));
-    if (scratch_alloc((void**)&scratch, off, s) != cudaSuccess) { delete[] h_tab; return LIBRA_ERR_CUDA; }
-    int rc = LIBRA_OK;
-    if (cudaMemcpyAsync(scratch + o_tab, h_tab, sizeof(int32_t) * 2 * (P + 1), cudaMemcpyHostToDevice, s) != cudaSuccess)
-        rc = LIBRA_ERR_CUDA;
-    delete[] h_tab;
+    const size_t o_ahead = take(sizeof(int32_t) * (size_t)slots), o_total = take(sizeof(int64_t) * (size_t)ctas);
+    if (scratch_alloc((void**)&scratch, off, s) != cudaSuccess) return LIBRA_ERR_CUDA;
     TapGeom g;
     g.cu = cu_seqlens_dev;
-    g.seq_off = (const int32_t*)(scratch + o_tab);
-    g.blk_off = g.seq_off + (P + 1);
     g.n = n_samples; g.P = P; g.CP = o->cp; g.B = o->block; g.H = H; g.hq = o->hq; g.hkv = o->hkv; g.d = o->head_dim;
     int32_t* q_home = (int32_t*)(scratch + o_q);
     int32_t* j0 = (int32_t*)(scratch + o_j0);
     int32_t* j1 = (int32_t*)(scratch + o_j1);
     int32_t* res_smp = (int32_t*)(scratch + o_rs);
     uint32_t* marks = (uint32_t*)(scratch + o_m);
-    int64_t* offs = (int64_t*)(scratch + o_offs);
+    int32_t* ahead = (int32_t*)(scratch + o_ahead);
+    int64_t* total = (int64_t*)(scratch + o_total);
+    // the marks start from zero (rows rounded up to whole 64-bit words)
+    const TapSetup setup = {NB, 0, 0, nullptr, nullptr, nullptr, q_home, nullptr, j0, j1, nullptr, res_smp,
+                            {(int64_t*)marks, nullptr, nullptr}, {((int64_t)words * W + 1) / 2, 0, 0}, nullptr, nullptr};
+    int rc = launch_setup(g, setup, seq_offsets_host, (int32_t*)(scratch + o_tab), s);
+    auto launched = [&](cudaError_t e) { if (e != cudaSuccess) rc = LIBRA_ERR_CUDA; };
     if (rc == LIBRA_OK) {
-        // the marks are cleared by the sample kernel (rows rounded up to whole 64-bit words)
-        const TapClear clear = {{(int64_t*)marks, nullptr, nullptr}, {((int64_t)words * W + 1) / 2, 0, 0}, nullptr};
-        k_tap_blocks<<<(unsigned)((NB + 127) / 128), 128, 0, s>>>(g, NB, (int64_t*)(scratch + o_f), q_home,
-                                                                  (int64_t*)(scratch + o_vqo), j0, j1, nullptr);
-        k_tap_samples<<<tap_sample_grid(n_samples, clear.n[0]), 128, 0, s>>>(g, (int64_t*)(scratch + o_vs), res_smp, clear);
-        k_tap_mark<<<(unsigned)((NT + 255) / 256), 256, 0, s>>>(sigma_dev, j0, j1, NT, H, W, words, marks);
-        const int64_t slots = NT + NG * W;
-        k_tap_sched_count<<<(unsigned)((slots + 255) / 256), 256, 0, s>>>(g, NT, NG, W, sigma_dev, q_home, marks, words,
-                                                                         res_smp, offs);
-        k_tap_sched_scan<<<1, 1024, 0, s>>>(slots, offs, n_records_dev);
-        k_tap_sched_fill<<<(unsigned)((slots + 255) / 256), 256, 0, s>>>(g, NT, NG, W, sigma_dev, q_home, marks, words,
-                                                                        res_smp, offs, capacity, records_dev);
-        count_launch(6);
-        if (cudaGetLastError() != cudaSuccess) rc = LIBRA_ERR_CUDA;
+        launched(launch_dependent(k_tap_mark, (unsigned)((NT + 255) / 256), 256u, 0, s, sigma_dev, j0, j1, NT, H, W, words, marks));
+        launched(launch_dependent(k_tap_sched_count, (unsigned)ctas, kTapSlots, 0, s, g, NT, NG, W, sigma_dev, q_home, marks, words, res_smp,
+                                  ahead, total));
+        const bool scan = ctas > kTapInlineCtas;
+        if (scan) launched(launch_dependent(k_tap_sched_scan, 1u, 1024u, 0, s, ctas, total, n_records_dev));
+        launched(launch_dependent(k_tap_sched_fill, (unsigned)ctas, kTapSlots, 0, s, g, NT, NG, W, sigma_dev, q_home, marks, words, res_smp,
+                                  ahead, total, scan ? 1 : 0, n_records_dev, capacity, records_dev));
+        count_launch(scan ? 4 : 3);
     }
     scratch_free(scratch, s);
     return rc;
