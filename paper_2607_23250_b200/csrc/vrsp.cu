@@ -11,6 +11,7 @@
 
 #include "../../include/libra.h"
 #include "common.h"
+#include "ptx.cuh"
 #include "waves.cuh"
 
 namespace libra {
@@ -20,6 +21,8 @@ namespace libra {
 __global__ void k_vrsp_work(const int32_t* __restrict__ sample_offsets, const int32_t* __restrict__ seq_first_sample,
                             int D, int64_t* __restrict__ work) {
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    grid_dep_wait();
+    grid_dep_launch();
     if (i >= D) return;
     int64_t f = 0;
     const int end = seq_first_sample[i + 1];
@@ -36,6 +39,8 @@ __global__ void k_vrsp_work(const int32_t* __restrict__ sample_offsets, const in
 // so that a window of a few hundred sequences fills more than a block or two.
 __global__ void __launch_bounds__(256) k_vrsp_rank(const int64_t* __restrict__ work, int D, int32_t* __restrict__ sorted) {
     __shared__ int64_t sw[1024];
+    grid_dep_wait();
+    grid_dep_launch();
     const int i = blockIdx.x * 16 + (threadIdx.x >> 4), sub = threadIdx.x & 15;
     const int64_t wi = i < D ? work[i] : 0;
     int rank = 0;
@@ -122,6 +127,7 @@ __global__ void __launch_bounds__(1024) k_vrsp_place(const int64_t* __restrict__
                                                    int D, int P, int K, int32_t* __restrict__ order,
                                                    int32_t* __restrict__ pool_of_seq, int64_t* __restrict__ pool_load) {
     const int lane = threadIdx.x;
+    grid_dep_wait();
     {   // sorted descending: the first work bounds every load, the last one tells whether any is negative
         const int64_t most = work[sorted[0]], least = work[sorted[D - 1]];
         if (least >= 0 && most < (int64_t(1) << 52) / P) {
@@ -187,9 +193,10 @@ extern "C" int libra_vrsp_work(const int32_t* sample_offsets_dev, const int32_t*
                                int64_t* work_dev, void* stream) {
     if (!sample_offsets_dev || !seq_first_sample_dev || !work_dev || n_sequences <= 0) return LIBRA_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    k_vrsp_work<<<(n_sequences + 7) / 8, 256, 0, s>>>(sample_offsets_dev, seq_first_sample_dev, n_sequences, work_dev);
     count_launch(1);
-    return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
+    const cudaError_t e = launch_dependent(k_vrsp_work, (unsigned)((n_sequences + 7LL) / 8), 256u, 0, s, sample_offsets_dev, seq_first_sample_dev,
+                                           n_sequences, work_dev);
+    return e == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
 
 extern "C" int libra_vrsp_place(const int64_t* work_dev, int n_sequences, int pool_size, int32_t* order_dev,
@@ -200,13 +207,11 @@ extern "C" int libra_vrsp_place(const int64_t* work_dev, int n_sequences, int po
     if (K > 1024 || D > (1 << 20)) return LIBRA_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;
     const int threads = (K + 31) / 32 * 32;
-    k_vrsp_rank<<<(D + 15) / 16, 256, 0, s>>>(work_dev, D, scratch_dev);
-    if (K <= 32)
-        k_vrsp_place<1><<<1, threads, 0, s>>>(work_dev, scratch_dev, D, P, K, order_dev, pool_of_seq_dev, pool_load_dev);
-    else if (K <= 128)
-        k_vrsp_place<4><<<1, threads, 0, s>>>(work_dev, scratch_dev, D, P, K, order_dev, pool_of_seq_dev, pool_load_dev);
-    else
-        k_vrsp_place<32><<<1, threads, 0, s>>>(work_dev, scratch_dev, D, P, K, order_dev, pool_of_seq_dev, pool_load_dev);
+    cudaError_t e = launch_dependent(k_vrsp_rank, (unsigned)((D + 15) / 16), 256u, 0, s, work_dev, D, scratch_dev);
+    if (e == cudaSuccess) {
+        auto place = K <= 32 ? k_vrsp_place<1> : (K <= 128 ? k_vrsp_place<4> : k_vrsp_place<32>);
+        e = launch_dependent(place, 1u, (unsigned)threads, 0, s, work_dev, scratch_dev, D, P, K, order_dev, pool_of_seq_dev, pool_load_dev);
+    }
     count_launch(2);
-    return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
+    return e == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
