@@ -638,6 +638,7 @@ k_attn_bwd_dkdv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 
 #include "attn_bwd_dq.cuh"
 #include "attn_bwd_fused.cuh"
+#include "attn_bwd_pair.cuh"
 
 namespace libra {
 
@@ -824,33 +825,66 @@ static int launch_fused(const void* q_dev, const void* k_dev, const void* v_dev,
     if (rc == LIBRA_OK) rc = make_f32_thd_map(&tdkacc, dk_acc, T, dims->hkv);
     if (rc == LIBRA_OK) rc = make_f32_thd_map(&tdvacc, dv_acc, T, dims->hkv);
     if (rc != LIBRA_OK) return rc;
-    if (!cfg_done(4)) {
-        if (set_smem(k_attn_bwd_fused, FusedSmem::kBytes) != LIBRA_OK) return LIBRA_ERR_CUDA;
-        {   // the register pool: what warps 12-15 release must cover what the exp and dS groups ask for
-            cudaFuncAttributes a;
-            if (cudaFuncGetAttributes(&a, k_attn_bwd_fused) != cudaSuccess) return LIBRA_ERR_CUDA;
-            const long long wanted = 256LL * (kFuRegsExp - a.numRegs) + 128LL * (kFuRegsDs - a.numRegs);
-            if (a.numRegs < kFuRegsOther || wanted > 128LL * (a.numRegs - kFuRegsOther)) return LIBRA_ERR_UNSUPPORTED;
-        }
-        cfg_mark(4);
-    }
     libra_plan_t* mp = const_cast<libra_plan_t*>(plan);
-    FusedParams fp;
-    fp.dq_acc = dq_acc; fp.dk_acc = dk_acc; fp.dv_acc = dv_acc;
-    fp.lse2 = lse2; fp.dvec = dvec;
-    fp.cta_offsets = d.d_cta_offsets; fp.cta_tiles = d.d_cta_exec;
-    fp.u_blk = d.d_u_blk; fp.u_chunk = d.d_u_chunk; fp.tok_end = plan->d_tok_end;
-    fp.T = T; fp.Tpad = ws.Tpad; fp.NU = d.NB;
-    fp.hq = dims->hq; fp.hkv = dims->hkv; fp.R = d.chunk / d.tile;
-    fp.scale_log2 = scale * 1.4426950408889634f;
-    fp.outcome = plan->d_outcome[1]; fp.plan_status = plan->d_status;
-    fp.wait_limit_ns = plan->wait_limit_ns; fp.inject_stall = plan->inject_stall;
-    fp.busy = d.d_busy;
-    fp.tile_ns = d.d_tile_ns;
-    mp->n_outcome[1] = d.W;
-    time_begin(mp, 4, s);
-    cudaError_t e = launch_dependent(k_attn_bwd_fused, d.W, kFusedThreads, FusedSmem::kBytes, s, tq, tk, tv, tdo, tacc, tdkacc,
-                                     tdvacc, fp);
+    cudaError_t e;
+    const PlanDir& wide = plan->dir[4];
+    if (wide.enabled) {   // 256 keys a tile, on pairs of CTAs
+        CUtensorMap tq64, tdo64;
+        rc = make_thd_map(&tq64, q_dev, T, dims->hq, 128, 64);
+        if (rc == LIBRA_OK) rc = make_thd_map(&tdo64, dout_dev, T, dims->hq, 128, 64);
+        if (rc != LIBRA_OK) return rc;
+        if (!cfg_done(7)) {
+            if (set_smem(k_attn_bwd_pair, PairSmem::kBytes) != LIBRA_OK) return LIBRA_ERR_CUDA;
+            cudaFuncAttributes a;   // the register pool: what the dQ group and the last warps release must cover the rest
+            if (cudaFuncGetAttributes(&a, k_attn_bwd_pair) != cudaSuccess) return LIBRA_ERR_CUDA;
+            const long long wanted = 2LL * (kPrRegsExp - a.numRegs) + (kPrRegsDs - a.numRegs);
+            if (a.numRegs < kPrRegsDq || a.numRegs < kPrRegsOther || wanted > 2LL * a.numRegs - kPrRegsDq - kPrRegsOther)
+                return LIBRA_ERR_UNSUPPORTED;
+            cfg_mark(7);
+        }
+        PairParams pp;
+        pp.lse2 = lse2; pp.dvec = dvec;
+        pp.cta_offsets = wide.d_cta_offsets; pp.cta_tiles = wide.d_cta_exec;
+        pp.u_blk = wide.d_u_blk; pp.u_chunk = wide.d_u_chunk; pp.tok_end = plan->d_tok_end;
+        pp.T = T; pp.Tpad = ws.Tpad; pp.NU = (int)wide.NB;
+        pp.hq = dims->hq; pp.hkv = dims->hkv; pp.R = wide.chunk / kBlk;
+        pp.scale_log2 = scale * 1.4426950408889634f;
+        pp.outcome = plan->d_outcome[1]; pp.plan_status = plan->d_status;
+        pp.wait_limit_ns = plan->wait_limit_ns; pp.inject_stall = plan->inject_stall;
+        pp.busy = d.d_busy;
+        pp.tile_ns = d.d_tile_ns; pp.first_j = d.d_first_j; pp.base = d.d_base; pp.NU128 = d.NB;
+        mp->n_outcome[1] = 2 * wide.W;
+        time_begin(mp, 4, s);
+        e = launch_dependent(k_attn_bwd_pair, 2 * wide.W, kPairThreads, PairSmem::kBytes, s, tq, tk, tv, tdo, tq64, tdo64, tacc, tdkacc,
+                             tdvacc, pp);
+    } else {
+        if (!cfg_done(4)) {
+            if (set_smem(k_attn_bwd_fused, FusedSmem::kBytes) != LIBRA_OK) return LIBRA_ERR_CUDA;
+            {   // the register pool: what warps 12-15 release must cover what the exp and dS groups ask for
+                cudaFuncAttributes a;
+                if (cudaFuncGetAttributes(&a, k_attn_bwd_fused) != cudaSuccess) return LIBRA_ERR_CUDA;
+                const long long wanted = 256LL * (kFuRegsExp - a.numRegs) + 128LL * (kFuRegsDs - a.numRegs);
+                if (a.numRegs < kFuRegsOther || wanted > 128LL * (a.numRegs - kFuRegsOther)) return LIBRA_ERR_UNSUPPORTED;
+            }
+            cfg_mark(4);
+        }
+        FusedParams fp;
+        fp.dq_acc = dq_acc; fp.dk_acc = dk_acc; fp.dv_acc = dv_acc;
+        fp.lse2 = lse2; fp.dvec = dvec;
+        fp.cta_offsets = d.d_cta_offsets; fp.cta_tiles = d.d_cta_exec;
+        fp.u_blk = d.d_u_blk; fp.u_chunk = d.d_u_chunk; fp.tok_end = plan->d_tok_end;
+        fp.T = T; fp.Tpad = ws.Tpad; fp.NU = d.NB;
+        fp.hq = dims->hq; fp.hkv = dims->hkv; fp.R = d.chunk / d.tile;
+        fp.scale_log2 = scale * 1.4426950408889634f;
+        fp.outcome = plan->d_outcome[1]; fp.plan_status = plan->d_status;
+        fp.wait_limit_ns = plan->wait_limit_ns; fp.inject_stall = plan->inject_stall;
+        fp.busy = d.d_busy;
+        fp.tile_ns = d.d_tile_ns;
+        mp->n_outcome[1] = d.W;
+        time_begin(mp, 4, s);
+        e = launch_dependent(k_attn_bwd_fused, d.W, kFusedThreads, FusedSmem::kBytes, s, tq, tk, tv, tdo, tacc, tdkacc,
+                                         tdvacc, fp);
+    }
     time_end(mp, 4, s);
     time_begin(mp, 5, s);
     if (e == cudaSuccess) {

@@ -33,6 +33,8 @@ struct PlanDir {
     int chunk = 0;                     // tokens per query chunk
     int32_t* d_u_blk = nullptr;        // [NB] key block of pair-block u
     int32_t* d_u_chunk = nullptr;      // [NB] query chunk of pair-block u
+    int32_t* d_first_j = nullptr;      // [chunks] first key block of a query chunk
+    int64_t* d_base = nullptr;         // [chunks + 1] its pair-block
 };
 
 }  // namespace libra
@@ -58,8 +60,10 @@ struct libra_plan {
     int W = 0;                       // workers of every direction
     int bwd_mask = 0;                // which of d_outcome[1..3] the last backward wrote
     // 0 = query-major, 1 = key-major, 2 = pair tiles (key block x query chunk), 3 = the key-stationary tiles of kernels that
-    // run on pairs of CTAs: as 2 when that is there, else as 1, with 256 keys a tile and a worker for every two
-    libra::PlanDir dir[4];
+    // run on pairs of CTAs: as 2 when that is there, else as 1, with 256 keys a tile and a worker for every two; 4 = the pair
+    // tiles of the fused kernel on pairs of CTAs, 256 keys a tile and the query chunks of 2
+    static constexpr int kDirs = 5;
+    libra::PlanDir dir[kDirs];
     uint32_t wait_limit_ns = 2000000000u;  // budget of one device-side wait (libra_plan_set_wait_limit_ns)
     int inject_stall = 0;            // test aid: the producer role issues no loads (libra_plan_inject_stall)
     int timing = 0;                  // record events around the main kernels

@@ -114,7 +114,7 @@ struct DirView {
     int64_t* loads;
 };
 struct DirViews {
-    DirView v[4];
+    DirView v[libra_plan::kDirs];
 };
 
 // Weight of block b (Eq. 6): a token at position p of a sample of length len contributes
@@ -320,8 +320,8 @@ __device__ __forceinline__ int64_t pair_last_row_block(const int32_t* tok_end, i
 // every query chunk, the exclusive prefix sum of the counts and their total (base[NC] and totals[block]); one more block
 // for either finds the most live cells of a key block (totals[kPairCands + k]).
 struct PairTables { int dir = 0, kt = 0, R = 0; int32_t* first_j = nullptr; int32_t* count = nullptr; int64_t* base = nullptr; int64_t NC = 0; };
-constexpr int kPairCands = 12;
-struct PairCands { PairTables c[kPairCands]; int n = 0; int rt = 0; int kt[2] = {}; };
+constexpr int kChunkSizes = 6, kPairCands = 3 * kChunkSizes;
+struct PairCands { PairTables c[kPairCands]; int n = 0; int rt = 0; int kt[2] = {}; int n_longest = 0; };
 __global__ void __launch_bounds__(1024) k_pair_chunks(const int32_t* __restrict__ tok_end, int64_t T, const __grid_constant__ PairCands cands,
                                                       int64_t* __restrict__ totals) {
     const int rt = cands.rt;
@@ -485,7 +485,7 @@ static int64_t pair_chunks_of(int64_t T, int rt, int R) { return ((T + rt - 1) /
 static void add_pair_cands(const libra_plan* p, PairCands& cands, int k, bool halves) {
     const PlanDir& d = p->dir[k];
     int R = d.chunk / cands.rt;
-    for (int x = 0; x < (halves ? kPairCands / 2 : 1) && R > 0; ++x, R /= 2) {
+    for (int x = 0; x < (halves ? kChunkSizes : 1) && R > 0; ++x, R /= 2) {
         PairTables& t = cands.c[cands.n++];
         t.dir = k;
         t.kt = d.tile;
@@ -511,10 +511,13 @@ static const PairTables* choose_pair_chunk(const libra_plan* p, const PairCands&
     }
     return best;
 }
+// Whether the fused backward runs on pairs of CTAs with 256 keys a tile.
+constexpr int64_t kPairsSample = 1024;   // tokens per sample, empty ones counted, from which on it does
+static bool fused_on_pairs(int64_t T, int n_samples) { return T >= kPairsSample * (int64_t)n_samples; }
 static double heads_per_kv(const libra_plan* p) { return p->dir[0].H > p->dir[2].H ? (double)p->dir[0].H / p->dir[2].H : 1.0; }
 // Counts, choice and, while every size has more than 262144 pair-blocks, twice the largest.
-static int count_pair_blocks(libra_plan* p, PairCands& cands, int64_t* d_totals, PairTables (&chosen)[4], double G) {
-    const int dirs = cands.c[cands.n - 1].dir == 3 ? 2 : 1;
+static int count_pair_blocks(libra_plan* p, PairCands& cands, int64_t* d_totals, PairTables (&chosen)[libra_plan::kDirs], double G) {
+    const int dirs = cands.n_longest;
     for (;;) {
         int64_t totals[kPairCands + 2];
         k_pair_chunks<<<cands.n + dirs, 1024, 0, p->stream>>>(p->d_tok_end, p->T, cands, d_totals);
@@ -534,35 +537,46 @@ static int count_pair_blocks(libra_plan* p, PairCands& cands, int64_t* d_totals,
             all = false;
             for (int x = 0; x < cands.n; ++x) {
                 PairTables& c = cands.c[x];
-                if (c.dir != k) continue;
+                if (c.dir != k && !(k == 2 && c.dir == 4)) continue;
                 if ((int64_t)c.R * 2 * cands.rt > (int64_t)1 << 30) return LIBRA_ERR_UNSUPPORTED;
                 c.R *= 2;
                 c.NC = pair_chunks_of(p->T, cands.rt, c.R);   // never more than the tables were carved for
             }
         }
-        if (all) return LIBRA_OK;
+        if (!all) continue;
+        for (int x = 0; x < cands.n; ++x)   // the fused kernel's wide tiles have the chunks of the others
+            if (cands.c[x].dir == 4 && cands.c[x].R == chosen[2].R) {
+                p->dir[4].NB = totals[x];
+                p->dir[4].chunk = p->dir[2].chunk;
+                chosen[4] = cands.c[x];
+            }
+        return LIBRA_OK;
     }
 }
 
 // Builds the directions asked for; p->dir[k].tile / H / W / chunk are set.
-static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o, const bool (&want)[4]) {
+static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o, const bool (&want)[libra_plan::kDirs]) {
+    constexpr int kDirs = libra_plan::kDirs;
     const int64_t T = p->T;
     cudaStream_t s = p->stream;
     const bool wide_pairs = want[3] && want[2];                   // the wide tiles are pair tiles
-    const bool sorted[4] = {want[0], want[1], false, want[3] && !want[2]};   // sizes known, placed heaviest first
-    for (int k = 0; k < 4; ++k) {
+    const bool sorted[kDirs] = {want[0], want[1], false, want[3] && !want[2], false};   // sizes known, placed heaviest first
+    const bool pairs[kDirs] = {false, false, want[2], wide_pairs, want[4]};
+    for (int k = 0; k < kDirs; ++k) {
         if (!sorted[k]) continue;
         p->dir[k].NB = (T + p->dir[k].tile - 1) / p->dir[k].tile;
         if (const int rc = check_dir(p, p->dir[k], false); rc != LIBRA_OK) return rc;
     }
     PairCands cands;
-    PairTables chosen[4];
+    PairTables chosen[kDirs];
     int64_t* d_totals = nullptr;
     if (want[2]) {
         if (p->dir[2].chunk % p->dir[2].tile) return LIBRA_ERR_INVALID_ARG;
         cands.rt = p->dir[2].tile;
-        for (int k = 2; k < (wide_pairs ? 4 : 3); ++k) {
-            cands.kt[k - 2] = p->dir[k].tile;
+        cands.n_longest = wide_pairs ? 2 : 1;
+        for (int k = 2; k < kDirs; ++k) {
+            if (!pairs[k]) continue;
+            if (k < 4) cands.kt[k - 2] = p->dir[k].tile;
             add_pair_cands(p, cands, k, o.pair_chunk == 0);
         }
     }
@@ -571,12 +585,12 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
     auto carve = [&](Carver& c) {
         c.take(&p->d_status, 1);
         for (int k = 0; k < 4; ++k) c.take(&p->d_outcome[k], p->W + 1);
-        for (int k = 0; k < 4; ++k)
+        for (int k = 0; k < kDirs; ++k)
             if (sorted[k]) carve_dir(p->dir[k], c, true, false);
         zero_bytes = c.used;
         c.take(&p->d_tok_start, T);
         c.take(&p->d_tok_end, T);
-        for (int k = 0; k < 4; ++k)
+        for (int k = 0; k < kDirs; ++k)
             if (sorted[k]) carve_dir(p->dir[k], c, false, false);
         if (want[2]) {
             c.take(&d_totals, kPairCands + 2);
@@ -601,18 +615,25 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
         if (const int rc = count_pair_blocks(p, cands, d_totals, chosen, heads_per_kv(p)); rc != LIBRA_OK) return rc;
         Carver ps, pm;
         size_t pair_zero = 0;
-        for (int k = 2; k < (wide_pairs ? 4 : 3); ++k)
+        for (int k = 2; k < kDirs; ++k) {
+            if (!pairs[k]) continue;
             if (const int rc = check_dir(p, p->dir[k], true); rc != LIBRA_OK) return rc;
+            p->dir[k].d_first_j = chosen[k].first_j;
+            p->dir[k].d_base = chosen[k].base;
+        }
         auto carve_pairs = [&](Carver& c) {
-            for (int k = 2; k < (wide_pairs ? 4 : 3); ++k) carve_dir(p->dir[k], c, true, true);
+            for (int k = 2; k < kDirs; ++k)
+                if (pairs[k]) carve_dir(p->dir[k], c, true, true);
             pair_zero = c.used;
-            for (int k = 2; k < (wide_pairs ? 4 : 3); ++k) carve_dir(p->dir[k], c, false, true);
+            for (int k = 2; k < kDirs; ++k)
+                if (pairs[k]) carve_dir(p->dir[k], c, false, true);
         };
         carve_pairs(ps);
         if (const int rc = plan_block(p, ps.used, &pm.at); rc != LIBRA_OK) return rc;
         carve_pairs(pm);
         cudaMemsetAsync(pm.at, 0, pair_zero, s);
-        for (int k = 2; k < (wide_pairs ? 4 : 3); ++k) {
+        for (int k = 2; k < kDirs; ++k) {
+            if (!pairs[k]) continue;
             PlanDir& d = p->dir[k];
             const PairTables& t = chosen[k];
             k_pair_fill<<<(unsigned)t.NC, 128, 0, s>>>(p->d_tok_end, T, t.kt, cands.rt, t.R, t.NC, t.first_j, t.count, t.base, d.d_u_blk,
@@ -624,7 +645,7 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
     DirViews views = {};
     int n = 0, max_w = 0;
     int64_t max_nb = 0, max_nt = 0;
-    for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < kDirs; ++k)
         if (sorted[k]) {
             views.v[n++] = view_of(p->dir[k], k != 0, o);
             max_nb = p->dir[k].NB > max_nb ? p->dir[k].NB : max_nb;
@@ -635,10 +656,10 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
         count_launch(2);
     }
     const int n_sorted = n;
-    for (int k = 2; k < 4; ++k)
+    for (int k = 2; k < kDirs; ++k)
         if (want[k] && !sorted[k]) views.v[n++] = view_of(p->dir[k], 1, o);
     if (n == 0) return LIBRA_OK;
-    for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < kDirs; ++k)
         if (want[k]) {
             max_nt = p->dir[k].NT > max_nt ? p->dir[k].NT : max_nt;
             max_w = p->dir[k].W > max_w ? p->dir[k].W : max_w;
@@ -658,7 +679,7 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
         k_check_loads<<<v.W, 256, 0, s>>>(v, p->d_status);
         count_launch();
     }
-    for (int k = 0; k < 4; ++k) p->dir[k].enabled = want[k] ? 1 : 0;
+    for (int k = 0; k < kDirs; ++k) p->dir[k].enabled = want[k] ? 1 : 0;
     return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
 
@@ -701,13 +722,14 @@ extern "C" int libra_plan_tiles(const int32_t* cu_seqlens_dev, int n_samples, in
     const int dirs = o.directions ? o.directions : (LIBRA_DIR_Q | LIBRA_DIR_KV);
     const int tile_kv = o.tile_kv ? o.tile_kv : 128;
     const bool keys = (dirs & (LIBRA_DIR_KV | LIBRA_DIR_PAIR)) != 0;
-    const bool want[4] = {(dirs & LIBRA_DIR_Q) != 0, (dirs & LIBRA_DIR_KV) != 0, (dirs & LIBRA_DIR_PAIR) != 0,
-                          keys && tile_kv == 128};
-    for (int k = 0; k < 4; ++k) {
+    const bool want[libra_plan::kDirs] = {(dirs & LIBRA_DIR_Q) != 0, (dirs & LIBRA_DIR_KV) != 0, (dirs & LIBRA_DIR_PAIR) != 0,
+                                          keys && tile_kv == 128,
+                                          (dirs & LIBRA_DIR_PAIR) != 0 && tile_kv == 128 && p->W >= 2 && fused_on_pairs(T, n_samples)};
+    for (int k = 0; k < libra_plan::kDirs; ++k) {
         PlanDir& d = p->dir[k];
-        d.tile = k == 0 ? tile_q : (k == 3 ? 256 : tile_kv);
+        d.tile = k == 0 ? tile_q : (k >= 3 ? 256 : tile_kv);
         d.H = k == 0 ? n_heads : (o.n_heads_kv ? o.n_heads_kv : n_heads);
-        d.W = k == 3 ? (p->W + 1) / 2 : p->W;
+        d.W = k == 3 ? (p->W + 1) / 2 : (k == 4 ? p->W / 2 : p->W);
         d.chunk = k >= 2 ? (o.pair_chunk ? o.pair_chunk : 4096) : 0;
         if (k == 3) {
             // The 256-wide kernels go through a tile's heads one after the other and their workers are out of step, so what

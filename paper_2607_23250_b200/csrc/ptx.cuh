@@ -306,6 +306,18 @@ __device__ __forceinline__ void mma_ts_pair_one(uint32_t d_tmem, uint32_t a_tmem
         : "memory");
 }
 
+// The same for the rows of either or both (bit 0: the leader's, bit 1: the other's).
+__device__ __forceinline__ void mma_ts_pair_of(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate,
+                                               uint32_t ctas) {
+    const uint32_t off0 = ctas & 1 ? 0u : 0xffffffffu, off1 = ctas & 2 ? 0u : 0xffffffffu;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, {%5, %5, %5, %5, %6, %6, %6, %6}, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(off0), "r"(off1)
+        : "memory");
+}
+
 // Instruction descriptor for kind::f16 with bf16 inputs and fp32 accumulation.
 //   bits 4-5 D format (1 = f32), 7-9 A format (1 = bf16), 10-12 B format (1 = bf16),
 //   bit 15 A major (0 = K, 1 = MN), bit 16 B major, bits 17-22 N >> 3, bits 24-28 M >> 4.

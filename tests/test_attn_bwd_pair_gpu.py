@@ -1,0 +1,113 @@
+"""Fused backward on pairs of CTAs (256-key tiles; pools whose samples average 1024 tokens) against the CPU oracle's
+gradient.  The call and the plan are the fused backward's."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2607_23250_b200 import pools
+from test_attn_bwd_fused_gpu import _check, _run
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("lengths", [
+    [1024],                      # whole key blocks, an even number
+    [1100],                      # nine key blocks: the last pair lacks its upper half; a ragged end
+    [1025, 1153],                # a sample that starts inside a key block
+    [128 * 9 + 1, 128 * 7 - 1],  # samples that end just past and just before a block's edge
+    [2300, 1, 1900, 40],         # short ones between long ones
+])
+@pytest.mark.parametrize("hq,hkv", [(4, 2), (2, 2), (8, 1)])
+def test_edges_of_the_key_blocks(lengths, hq, hkv):
+    got, ref, cu, _ = _run(lengths, hq, hkv, seed=hq)
+    _check(got, ref, cu)
+
+
+@pytest.mark.parametrize("chunk", [128, 384, 512, 4096])
+def test_query_chunk_sizes(chunk):
+    """One row block a chunk makes tiles of which a half sees nothing; an odd number of them lets a chunk begin at the upper
+    key block."""
+    got, ref, cu, _ = _run([1500, 1700], 4, 2, seed=1, chunk=chunk)
+    _check(got, ref, cu)
+
+
+@pytest.mark.parametrize("W", [2, 3, 5, 148])
+def test_worker_counts(W):
+    """A pair of CTAs for every two workers; an odd one stays idle."""
+    got, ref, cu, _ = _run([1300, 1200], 4, 1, seed=W, W=W)
+    _check(got, ref, cu)
+
+
+def test_repeat_agrees_to_rounding():
+    got, ref, cu, again = _run([2500, 1800], 8, 2, seed=9, repeat=True)
+    _check(got, ref, cu)
+    for g, a in zip(got, again):
+        assert np.abs(g - a).max() <= 2.0 ** -7 * np.abs(g).max()     # one bf16 step of the largest values
+
+
+def test_tile_times_cover_every_tile():
+    from paper_2607_23250_b200 import binding as lb
+    lengths, hq, hkv = [2000, 1200], 4, 2
+    cu_np = pools.cu_seqlens(lengths)
+    t = pools.make_tensors(int(cu_np[-1]), hq, hkv, 128, seed=5, device="cuda")
+    plan = lb.libra_plan_tiles(torch.from_numpy(cu_np).cuda(), hq, 256, directions=lb.LIBRA_DIR_Q | lb.LIBRA_DIR_PAIR,
+                               tile_kv=128, n_heads_kv=hkv, pair_chunk=512)
+    out, lse = lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
+    lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan)
+    ns, busy = plan.tile_times(lb.KERNEL_BWD_FUSED), plan.busy_times(lb.KERNEL_BWD_FUSED)
+    assert len(ns) == plan.info(lb.LIBRA_DIR_PAIR)["n_tiles"] and (ns > 0).all()
+    assert int(ns.max()) <= int(busy.max()) and int(ns.astype(np.int64).sum()) <= int(busy.astype(np.int64).sum())
+    plan.destroy()
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_values_that_are_not_finite_stay_in_their_block(value):
+    """The pair streams row blocks that only one of its key blocks sees: what is not finite there reaches no key of the other,
+    and a key or value that is not finite no row that does not see its block."""
+    from paper_2607_23250_b200 import binding as lb
+    T, hq, hkv, at = 1100, 2, 1, {"v": 700, "k": 200, "q": 300, "dout": 800}
+    cu = torch.tensor([0, T], dtype=torch.int32).cuda()
+    plan = lb.libra_plan_tiles(cu, hq, 256, directions=lb.LIBRA_DIR_Q | lb.LIBRA_DIR_PAIR, tile_kv=128, n_heads_kv=hkv, pair_chunk=256)
+    clean = pools.make_tensors(T, hq, hkv, 128, seed=3, device="cuda")
+    out0, lse0 = lb.libra_attn_pool_fwd(clean["q"], clean["k"], clean["v"], plan)
+    for name, row in at.items():
+        t = {n: x.clone() for n, x in clean.items()}
+        t[name][row, 0, 5] = value
+        first, behind = row // 128 * 128, row // 128 * 128 + 128
+        dq, dk, dv = lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out0, lse0, t["dout"], plan)
+        if name in ("k", "v"):
+            assert torch.isfinite(dq[:first].float()).all(), name
+            assert not torch.isfinite(dq[row:].float()).all()
+        else:
+            assert torch.isfinite(dk[behind:].float()).all() and torch.isfinite(dv[behind:].float()).all(), name
+            assert not torch.isfinite(dk[first:row].float()).all()
+    plan.destroy()
+
+
+@pytest.mark.parametrize("lengths,W", [([1200], 0), ([1500, 1100], 4)])
+def test_gives_up_cleanly_when_one_producer_stalls(lengths, W):
+    """The odd CTAs' producers issue no loads (a flag that nothing sets): TIMEOUT is reported, the context stays usable, and
+    the next launch with the injection off is correct."""
+    from paper_2607_23250_b200 import binding as lb
+    hq, hkv = 4, 2
+    cu_np = pools.cu_seqlens(lengths)
+    t = pools.make_tensors(int(cu_np[-1]), hq, hkv, 128, seed=4)
+    q, k, v, dout = (t[n].cuda() for n in ("q", "k", "v", "dout"))
+    plan = lb.libra_plan_tiles(torch.from_numpy(cu_np).cuda(), hq, 256, n_workers=W, directions=lb.LIBRA_DIR_Q | lb.LIBRA_DIR_PAIR,
+                               tile_kv=128, n_heads_kv=hkv)
+    out, lse = lb.libra_attn_pool_fwd(q, k, v, plan)
+    plan.set_wait_limit_ns(200_000)
+    plan.inject_stall(True)
+    lb.libra_attn_pool_bwd(q, k, v, out, lse, dout, plan)
+    with pytest.raises(lb.LibraError) as err:
+        plan.busy_times(lb.KERNEL_BWD_FUSED)
+    assert err.value.code == lb.ERR_TIMEOUT
+    plan.inject_stall(False)
+    plan.set_wait_limit_ns(0)
+    got = [x.float().cpu().numpy() for x in lb.libra_attn_pool_bwd(q, k, v, out, lse, dout, plan)]
+    plan.busy_times(lb.KERNEL_BWD_FUSED)
+    f = {n: t[n].float().numpy() for n in t}
+    o_ref, l_ref = oracle.attn_fwd(f["q"], f["k"], f["v"], cu_np)
+    _check(got, oracle.attn_bwd(f["q"], f["k"], f["v"], o_ref, l_ref, f["dout"], cu_np), cu_np)
+    plan.destroy()
