@@ -10,7 +10,7 @@
 // Placement is sequential by nature (every choice depends on the loads and residency left by the previous
 // ones), so the latency of one step bounds it.  Up to 128 workers whose tables fit shared memory: one block whose
 // warps work on neighbouring steps (k_tap_place_team).  Otherwise: one CTA with a thread per worker, block-wide
-// arg-min, tables in global memory.  1024 tiles on 16 workers with their schedule: 0.26 ms, with one warp for all of a
+// arg-min, tables in global memory.  1024 tiles on 16 workers with their schedule: 0.25 ms, with one warp for all of a
 // step 0.65 ms, all in the second form 2.8 ms.
 #include <cstdint>
 #include <new>
@@ -505,9 +505,16 @@ __global__ void __launch_bounds__(kTapThreads) k_tap_place_team(const TapPlace p
         const unsigned long long v = (unsigned long long)(p.rec[b].v_qo / p.unit);
         most = v > most ? v : most;
     }
-    atomicAdd(&s_sum, part);
-    atomicAdd(&s_vol, vol);
-    if (most >> 31) atomicAdd(&s_vol, 1ull << 32);
+    if (most >> 31) vol += 1ull << 32;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {   // (an atomic a thread took 10 us)
+        part += __shfl_xor_sync(0xffffffffu, part, o);
+        vol += __shfl_xor_sync(0xffffffffu, vol, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&s_sum, part);
+        atomicAdd(&s_vol, vol);
+    }
     __syncthreads();
     const int64_t sum_f = (int64_t)s_sum;
     if (sum_f > (INT64_MAX / ((int64_t)(p.tau_den + p.tau_num) * 2)) / W) {  // the integer cap test would overflow
