@@ -860,11 +860,12 @@ static int launch_fused(const void* q_dev, const void* k_dev, const void* v_dev,
     } else {
         if (!cfg_done(4)) {
             if (set_smem(k_attn_bwd_fused, FusedSmem::kBytes) != LIBRA_OK) return LIBRA_ERR_CUDA;
-            {   // the register pool: what warps 12-15 release must cover what the exp and dS groups ask for
+            {   // the register pool: what the dQ group and the last warps release must cover the rest
                 cudaFuncAttributes a;
                 if (cudaFuncGetAttributes(&a, k_attn_bwd_fused) != cudaSuccess) return LIBRA_ERR_CUDA;
-                const long long wanted = 256LL * (kFuRegsExp - a.numRegs) + 128LL * (kFuRegsDs - a.numRegs);
-                if (a.numRegs < kFuRegsOther || wanted > 128LL * (a.numRegs - kFuRegsOther)) return LIBRA_ERR_UNSUPPORTED;
+                const long long wanted = 2LL * (kFuRegsExp - a.numRegs) + (kFuRegsDs - a.numRegs);
+                if (a.numRegs < kFuRegsDq || a.numRegs < kFuRegsOther || wanted > 2LL * a.numRegs - kFuRegsDq - kFuRegsOther)
+                    return LIBRA_ERR_UNSUPPORTED;
             }
             cfg_mark(4);
         }

@@ -22,15 +22,18 @@
 // been read out.
 // Roles (512 threads): warps 0-3 and 4-7 exp groups (64 query columns of S^T each; 64 head-dim columns of dQ
 // each), 8-11 dS group, 12 TMA thread, 13 MMA thread, 14-15 only hand their registers over.
+// Roles (640 threads): two exp groups, a dS group, a dQ group, the TMA thread, the MMA thread, the thread that watches the
+// clock for all of them; a warp only hands its registers over.  The exp groups moved dQ between their exponentials before
+// (512 threads); with that, the waits' code in one place and one copy of the exponentials' the kernel is 50 KB instead of
+// 63: backward of 10 samples of 1000 tokens, 8 / 2 heads, 137.0 -> 133.4 us, of one of 1500 42.8 -> 40.2.
 #pragma once
 
 namespace libra {
 
-constexpr int kFusedThreads = 512;
-constexpr int kFuTmaWarp = 12, kFuMmaWarp = 13;
-// setmaxnreg budgets: 512 threads x 128 compiled registers = 256 x 144 (exp groups: P^T(it) and dQ(it-1) held
-// together) + 128 x 144 (dS group) + 128 x 80
-constexpr int kFuRegsExp = 144, kFuRegsDs = 144, kFuRegsOther = 80;
+constexpr int kFusedThreads = 640;
+constexpr int kFuDqWarp = 12, kFuTmaWarp = 16, kFuMmaWarp = 17, kFuWatchWarp = 19;   // (warp 18 only donates registers)
+// setmaxnreg budgets: 640 threads x 96 compiled registers = 256 x 112 + 128 x (128 + 48 + 80)
+constexpr int kFuRegsExp = 112, kFuRegsDs = 128, kFuRegsDq = 48, kFuRegsOther = 80;
 
 struct FusedSmem {
     static constexpr int kTile = 32768;        // 128 x 128 bf16
@@ -46,10 +49,10 @@ struct FusedSmem {
     static constexpr int kDvecOff = kLseOff + kQStages * 512;   // two buffers: dvec(it+1) lands while dvec(it) is read
     static constexpr int kBarOff = kDvecOff + 2 * 512;
     // kv_full, kv_empty, q_full[2], q_empty[2], do_full, do_empty, s_full, x_free1, dp_full, x_free2, dq_full,
-    // y_free, p_half, p_ready, ds_ready, dkv_full, dkv_empty, drain
-    static constexpr int kNumBars = 2 + 2 * kQStages + 16;
+    // y_free[2], p_ready, ds_ready, dkv_full, dkv_empty, drain
+    static constexpr int kNumBars = 2 + 2 * kQStages + 15;
     static constexpr int kMiscOff = kBarOff + kNumBars * 8;
-    static constexpr int kBytes = kMiscOff + 16;
+    static constexpr int kBytes = kMiscOff + 24;
     static_assert(kBytes <= kSmemMax, "exceeds the shared memory of an sm_100 CTA");
 };
 
@@ -102,25 +105,40 @@ __device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap* m, const vo
                  : "memory");
 }
 
-// dQ of one iteration: out of Y (query rows in lanes; this thread's 64 head-dim columns at `taddr`) into registers,
-// after which Y is released.
-__device__ __forceinline__ bool fused_read_dq(uint64_t* bar_dqfull, uint64_t* bar_yfree, uint32_t i, volatile int* ctl,
-                                              uint32_t taddr, uint32_t (&dqv)[64]) {
-    if (!warp_wait(bar_dqfull, i & 1, ctl)) return false;
-    tc_fence_after();
-    tmem_ld32(taddr, dqv);
-    tmem_ld32(taddr + 32, dqv + 32);
-    tmem_ld_wait();
-    tc_fence_before();
-    mbar_arrive(bar_yfree);
+// Waits of kernels that have one warp look at the clock for all of them (a wait of mbar_wait's kind has that code at every
+// place).  They end when the phase has completed or the CTA has given up.
+__device__ __forceinline__ bool watched_wait(uint64_t* bar, uint32_t parity, volatile int* ctl) {
+    while (!mbar_try_wait(bar, parity))
+        if (ctl[0]) return false;
     return true;
 }
-// ... and from the registers through the warp's staging tile (32 rows of 128 bytes, 128-byte swizzle) into the fp32
+__device__ __forceinline__ bool watched_warp_wait(uint64_t* bar, uint32_t parity, volatile int* ctl) {
+    return __all_sync(0xffffffffu, watched_wait(bar, parity, ctl));
+}
+// That warp's thread: the CTA gives up when *progress has not moved for the budget of a wait.  Ends with the other warps.
+__device__ __forceinline__ void watch_progress(const volatile uint32_t* progress, const volatile uint32_t* finished, uint32_t warps,
+                                               uint32_t limit_ns, volatile int* ctl) {
+    uint64_t t0 = globaltimer_ns();
+    uint32_t seen = 0;
+    while (*finished < warps && !ctl[0]) {
+        asm volatile("nanosleep.u32 100;");
+        const uint64_t t = globaltimer_ns();
+        const uint32_t now = *progress;
+        if (now != seen) {
+            seen = now;
+            t0 = t;
+        } else if (t - t0 > (uint64_t)limit_ns) {
+            ctl[0] = 1;
+        }
+    }
+}
+// 32 columns of a row per thread, through the warp's staging tile (32 rows of 128 bytes, 128-byte swizzle) into the fp32
 // accumulator: one bulk tensor reduce-add of 32 head-dim columns (from column col0), rows row0 .. row0 + 31 of head h.
-// The reduce that last used the tile must have finished reading it.
+// The reduce that last used the tile must have finished reading it: all but the last PENDING of this thread's have.
+template <int PENDING = 0>
 __device__ __forceinline__ void fused_stage_dq(const CUtensorMap* tm, uint8_t* stage, const uint32_t* dq, int lane,
                                                int col0, int h, int row0) {
-    if (lane == 0) tma_store_wait_read();
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(PENDING) : "memory");
     __syncwarp();
 #pragma unroll
     for (int ch = 0; ch < 8; ++ch) {
@@ -156,8 +174,8 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     uint64_t* bar_dpfull = b2 + 4;
     uint64_t* bar_xfree2 = b2 + 5;     // dP^T(it) has been read out: S^T(it+1) may overwrite it
     uint64_t* bar_dqfull = b2 + 6;     // dQ(it) is in Y (so dV(it), dK(it) and dQ(it) have all run)
-    uint64_t* bar_yfree = b2 + 7;      // dQ(it) has been read out of Y: P^T(it+1), then dS^T(it+1), may be written
-    uint64_t* bar_phalf = b2 + 8;
+    uint64_t* bar_yfree = b2 + 7;      // [2] dQ(it) has been read out of Y's first 64 columns: P^T(it+1) may be written; of the
+                                       // other 64: dS^T(it+1) may (and dQ(it) has run, so that the shared-memory dS^T is spent)
     uint64_t* bar_pready = b2 + 9;
     uint64_t* bar_dsready = b2 + 10;   // dS^T(it) is in TMEM and in shared memory
     uint64_t* bar_dkvfull = b2 + 11;
@@ -165,6 +183,8 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     uint64_t* bar_drain = b2 + 13;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kMiscOff);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMiscOff + 4);
+    volatile uint32_t* progress = reinterpret_cast<volatile uint32_t*>(smem + L::kMiscOff + 12);   // iterations begun by the first exp warp
+    uint32_t* finished = reinterpret_cast<uint32_t*>(smem + L::kMiscOff + 16);                     // warps whose role is over
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -185,15 +205,16 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         mbar_init(bar_dpfull, 1);
         mbar_init(bar_xfree2, 128);
         mbar_init(bar_dqfull, 1);
-        mbar_init(bar_yfree, 256);
-        mbar_init(bar_phalf, 256);
+        mbar_init(&bar_yfree[0], 128);
+        mbar_init(&bar_yfree[1], 128);
         mbar_init(bar_pready, 256);
         mbar_init(bar_dsready, 128);
         mbar_init(bar_dkvfull, 1);
         mbar_init(bar_dkvempty, 256);
         mbar_init(bar_drain, 1);
         abort_flag[0] = 0;
-        abort_flag[1] = (int)p.wait_limit_ns;
+        *progress = 0;
+        *finished = 0;
         fence_mbar_init();
     }
     if (warp == kFuTmaWarp && lane == 0) {
@@ -227,6 +248,10 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 
     if (warp > kFuMmaWarp) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFuRegsOther));
+        if (warp == kFuWatchWarp) {
+            if (elect_one()) watch_progress(progress, finished, kFusedThreads / 32 - 1, p.wait_limit_ns, abort_flag);
+            __syncwarp();
+        }
     } else if (warp == kFuTmaWarp) {
         // ---------------- TMA producer ----------------
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFuRegsOther));
@@ -235,7 +260,7 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             bool ok = true;
             for (int idx = unit_begin; idx < unit_end && ok && !p.inject_stall; ++idx) {
                 const FusedUnit u = fused_unit(p, p.cta_tiles[idx]);
-                ok = mbar_wait(bar_kvempty, (ucnt & 1) ^ 1, abort_flag);
+                ok = watched_wait(bar_kvempty, (ucnt & 1) ^ 1, abort_flag);
                 if (!ok) break;
                 mbar_arrive_expect_tx(bar_kvfull, 2 * L::kTile);
                 for (int half = 0; half < 2; ++half) {
@@ -244,23 +269,23 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                 }
                 ++ucnt;
                 const int n_it = G * u.n_blk;
-                for (int it = 0; it < n_it && ok; ++it, ++it_all) {
-                    const int h = u.kvh * G + it / u.n_blk;
-                    const int qb = (u.i0 + it % u.n_blk) * kBlk;
+                for (int it = 0, i = 0, h = u.kvh * G; it < n_it && ok; ++it, ++it_all) {
+                    const int qb = (u.i0 + i) * kBlk;
                     const uint32_t qs = it_all % QS;
-                    ok = mbar_wait(&bar_qempty[qs], ((it_all / QS) & 1) ^ 1, abort_flag);
+                    ok = watched_wait(&bar_qempty[qs], ((it_all / QS) & 1) ^ 1, abort_flag);
                     if (!ok) break;
                     mbar_arrive_expect_tx(&bar_qfull[qs], L::kTile + 512);
                     for (int half = 0; half < 2; ++half)
                         tma_load_3d(smem + L::kQOff + qs * L::kTile + half * L::kHalf, &tm_q, &bar_qfull[qs], half * 64, h, qb);
                     bulk_load_1d(smem + L::kLseOff + qs * 512, p.lse2 + (size_t)h * p.Tpad + qb, 512, &bar_qfull[qs]);
-                    ok = mbar_wait(bar_doempty, (it_all & 1) ^ 1, abort_flag);
+                    ok = watched_wait(bar_doempty, (it_all & 1) ^ 1, abort_flag);
                     if (!ok) { mbar_wait_drain(&bar_qfull[qs], (it_all / QS) & 1, kDrainNs); break; }
                     mbar_arrive_expect_tx(bar_dofull, L::kTile + 512);
                     ++n_do;
                     for (int half = 0; half < 2; ++half)
                         tma_load_3d(smem + L::kDoOff + half * L::kHalf, &tm_do, bar_dofull, half * 64, h, qb);
                     bulk_load_1d(smem + L::kDvecOff + (it_all & 1) * 512, p.dvec + (size_t)h * p.Tpad + qb, 512, bar_dofull);
+                    if (++i == u.n_blk) { i = 0; ++h; }
                 }
             }
             if (!ok || abort_flag[0]) {   // give-up path: the copies already issued land before shared memory is released
@@ -301,11 +326,11 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             for (int idx = unit_begin; idx < unit_end && ok; ++idx) {
                 const FusedUnit u = fused_unit(p, p.cta_tiles[idx]);
                 const int n_it = G * u.n_blk;
-                ok = mbar_wait(bar_kvfull, ucnt & 1, abort_flag);
+                ok = watched_wait(bar_kvfull, ucnt & 1, abort_flag);
                 if (!ok) break;
                 // S(0): X is free once dP of the previous unit's last iteration has been read
-                ok = mbar_wait(&bar_qfull[it_all % QS], (it_all / QS) & 1, abort_flag);
-                if (ok && it_all > 0) ok = mbar_wait(bar_xfree2, (it_all - 1) & 1, abort_flag);
+                ok = watched_wait(&bar_qfull[it_all % QS], (it_all / QS) & 1, abort_flag);
+                if (ok && it_all > 0) ok = watched_wait(bar_xfree2, (it_all - 1) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
                 issue_kmajor(L::kKOff, L::kQOff + (it_all % QS) * L::kTile);
@@ -314,31 +339,31 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                     const uint32_t nx = it_all + 1;
                     const bool more = it + 1 < n_it;
                     // dP(it) over S(it), as soon as the exp groups hold S(it) in registers
-                    ok = mbar_wait(bar_dofull, it_all & 1, abort_flag);
-                    if (ok) ok = mbar_wait(bar_xfree1, it_all & 1, abort_flag);
+                    ok = watched_wait(bar_dofull, it_all & 1, abort_flag);
+                    if (ok) ok = watched_wait(bar_xfree1, it_all & 1, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                     issue_kmajor(L::kVOff, L::kDoOff);
                     tc_commit(bar_dpfull);
                     // S(it+1) over dP(it), as soon as the dS group holds dP(it) in registers
                     if (more) {
-                        ok = mbar_wait(&bar_qfull[nx % QS], (nx / QS) & 1, abort_flag);
-                        if (ok) ok = mbar_wait(bar_xfree2, it_all & 1, abort_flag);
+                        ok = watched_wait(&bar_qfull[nx % QS], (nx / QS) & 1, abort_flag);
+                        if (ok) ok = watched_wait(bar_xfree2, it_all & 1, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
                         issue_kmajor(L::kKOff, L::kQOff + (nx % QS) * L::kTile);
                         tc_commit(bar_sfull);
                     }
                     // dV(it) += P^T dO
-                    ok = mbar_wait(bar_pready, it_all & 1, abort_flag);
-                    if (ok && it == 0 && ucnt > 0) ok = mbar_wait(bar_dkvempty, (ucnt - 1) & 1, abort_flag);
+                    ok = watched_wait(bar_pready, it_all & 1, abort_flag);
+                    if (ok && it == 0 && ucnt > 0) ok = watched_wait(bar_dkvempty, (ucnt - 1) & 1, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                     issue_acc(kColDV, kColP, L::kDoOff, it > 0);
                     tc_commit(bar_doempty);
                     // dK(it) += dS^T Q from the TMEM copy of dS^T, then dQ(it) = dS K from the shared-memory copy,
                     // into Y over P^T and dS^T: dV(it) and dK(it) precede it in issue order
-                    ok = mbar_wait(bar_dsready, it_all & 1, abort_flag);
+                    ok = watched_wait(bar_dsready, it_all & 1, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                     issue_acc(kColDK, kColDS, L::kQOff + (it_all % QS) * L::kTile, it > 0);
@@ -360,7 +385,7 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             }
         }
         __syncwarp();
-    } else if (warp >= 8) {
+    } else if (warp >= 8 && warp < kFuDqWarp) {
         // ---------------- dS group ----------------
         // Thread r owns key row r: it turns dP^T and P^T (read back as bf16) into dS^T, which goes to TMEM (the A
         // operand of dK) and to shared memory (the A operand of dQ).
@@ -371,47 +396,48 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         const uint32_t t_p = tmem_base + lane_addr + kColP;
         const uint32_t t_ds = tmem_base + lane_addr + kColDS;
         uint8_t* ds_row = smem + L::kDsOff + r * 128;
-        uint32_t it_all = 0;
+        uint32_t ucnt = 0, it_all = 0;
         bool ok = true;
         for (int idx = unit_begin; idx < unit_end && ok; ++idx) {
             const FusedUnit u = fused_unit(p, p.cta_tiles[idx]);
             const int n_it = G * u.n_blk;
             for (int it = 0; it < n_it && ok; ++it, ++it_all) {
                 const float* dvec = reinterpret_cast<const float*>(smem + L::kDvecOff + (it_all & 1) * 512);
-                ok = warp_wait(bar_dofull, it_all & 1, abort_flag) && warp_wait(bar_dpfull, it_all & 1, abort_flag);
+                ok = watched_warp_wait(bar_dofull, it_all & 1, abort_flag) && watched_warp_wait(bar_dpfull, it_all & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
                 uint32_t xs[64];   // (dP^T - D) as packed bf16 pairs
                 {
                     const uint64_t neg1 = f2_pack(-1.f, -1.f);
 #pragma unroll
-                    for (int part = 0; part < 2; ++part) {   // 64 columns at a time keeps the live registers down
-                        uint32_t dpv[64];
-                        tmem_ld32(t_x + part * 64, dpv);
-                        tmem_ld32(t_x + part * 64 + 32, dpv + 32);
+                    for (int part = 0; part < 4; ++part) {   // 32 columns at a time keeps the live registers down
+                        uint32_t dpv[32];
+                        tmem_ld32(t_x + part * 32, dpv);
                         tmem_ld_wait();
-                        if (part == 1) {
+                        if (part == 3) {
                             tc_fence_before();
                             mbar_arrive(bar_xfree2);   // dP^T(it) is in registers: S^T(it+1) may take the columns
                         }
 #pragma unroll
-                        for (int j = 0; j < 64; j += 4) {
-                            const ulonglong2 d4 = *reinterpret_cast<const ulonglong2*>(dvec + part * 64 + j);
+                        for (int j = 0; j < 32; j += 4) {
+                            const ulonglong2 d4 = *reinterpret_cast<const ulonglong2*>(dvec + part * 32 + j);
                             float a0, a1, b0, b1;
                             f2_unpack(f2_fma(d4.x, neg1, f2_pack(__uint_as_float(dpv[j]), __uint_as_float(dpv[j + 1]))), a0, a1);
                             f2_unpack(f2_fma(d4.y, neg1, f2_pack(__uint_as_float(dpv[j + 2]), __uint_as_float(dpv[j + 3]))), b0, b1);
-                            xs[part * 32 + (j >> 1)] = pack_bf16x2(a0, a1);
-                            xs[part * 32 + (j >> 1) + 1] = pack_bf16x2(b0, b1);
+                            xs[part * 16 + (j >> 1)] = pack_bf16x2(a0, a1);
+                            xs[part * 16 + (j >> 1) + 1] = pack_bf16x2(b0, b1);
                         }
                     }
                 }
-                // P^T(it) only appears in Y after dQ(it-1) has been read out of it, and dQ(it-1) ran behind dK(it-1): by
-                // the time P^T(it) is seen, both copies of dS^T(it-1) have been consumed
+                // dQ(it-1) has been read out of Y's dS^T columns, so both copies of dS^T(it-1) have been consumed; the last
+                // unit's dK and dV have left through the shared-memory tile
+                if (it_all > 0) ok = watched_warp_wait(&bar_yfree[1], (it_all - 1) & 1, abort_flag);
+                if (ok && it == 0 && ucnt > 0) ok = watched_warp_wait(bar_dkvempty, (ucnt - 1) & 1, abort_flag);
+                if (ok) ok = watched_warp_wait(bar_pready, it_all & 1, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
-                    ok = warp_wait(half == 0 ? bar_phalf : bar_pready, it_all & 1, abort_flag);
-                    if (!ok) break;
-                    tc_fence_after();
                     uint32_t pa[16], pb[16];   // queries 32 half .. and 64 + 32 half ..
                     tmem_ld16(t_p + half * 16, pa);
                     tmem_ld16(t_p + 32 + half * 16, pb);
@@ -434,27 +460,58 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
                             make_uint4(pb[4 * ch], pb[4 * ch + 1], pb[4 * ch + 2], pb[4 * ch + 3]);
                     }
                 }
-                if (!ok) break;
                 tmem_st_wait();
                 fence_proxy_async_smem();     // the MMA reads the shared-memory tile through the async proxy
                 tc_fence_before();
                 mbar_arrive(bar_dsready);
             }
+            ++ucnt;
         }
+    } else if (warp >= kFuDqWarp) {
+        // ---------------- dQ group ----------------
+        // Thread r owns query row r of dQ.  (The exp groups moved it between their exponentials before: with a group of its own
+        // 3320 -> 3170 ns a cell and CTA on 8192 tokens, 8 / 2 heads.)
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFuRegsDq));
+        const uint32_t t_y = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + kColY;
+        uint8_t* stage = smem + L::kStageOff + (warp & 3) * 8192;   // two tiles of 32 rows x 32 floats
+        uint32_t it_all = 0;
+        bool ok = true;
+        for (int idx = unit_begin; idx < unit_end && ok; ++idx) {
+            const FusedUnit u = fused_unit(p, p.cta_tiles[idx]);
+            const int n_it = G * u.n_blk;
+            for (int it = 0, i = 0, h = u.kvh * G; it < n_it; ++it, ++it_all) {
+                const int row = (u.i0 + i) * kBlk + (warp & 3) * 32, head = h;
+                if (++i == u.n_blk) { i = 0; ++h; }
+                ok = watched_warp_wait(bar_dqfull, it_all & 1, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+#pragma unroll 1
+                for (int half = 0; half < 2; ++half) {
+                    uint32_t v[32];
+                    tmem_ld32(t_y + 64 * half, v);
+                    tmem_ld_wait();
+                    fused_stage_dq<1>(&tm_dqacc, stage, v, lane, 64 * half, head, row);
+                    tmem_ld32(t_y + 64 * half + 32, v);
+                    tmem_ld_wait();
+                    tc_fence_before();
+                    mbar_arrive(&bar_yfree[half]);
+                    fused_stage_dq<1>(&tm_dqacc, stage + 4096, v, lane, 64 * half + 32, head, row);
+                }
+            }
+        }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     } else {
         // ---------------- exp groups ----------------
-        // Thread r of group grp owns key row r and the query columns [64 grp, 64 grp + 64) of S^T; when dQ comes
-        // back in Y (query rows in lanes) it owns query row r and the head-dim columns [64 grp, 64 grp + 64).
+        // Thread r of group grp owns key row r and the query columns [64 grp, 64 grp + 64) of S^T.
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kFuRegsExp));
         const int grp = warp >> 2;
         const int r = (warp & 3) * 32 + lane;
         const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t t_x = tmem_base + lane_addr + kColX;
         const uint32_t t_p = tmem_base + lane_addr + kColP;
-        const uint32_t t_y = tmem_base + lane_addr + kColY;
         const int c0 = 64 * grp;
-        const uint64_t scale2 = f2_pack(p.scale_log2, p.scale_log2), neg1 = f2_pack(-1.f, -1.f);
-        uint8_t* stage = smem + L::kStageOff + warp * 4096;   // this warp's staging tile: 32 rows x 32 floats
+        const uint64_t neg_scale2 = f2_pack(-p.scale_log2, -p.scale_log2);
+        uint8_t* stage = smem + L::kDsOff + warp * 4096;      // between units: this warp's staging tile for dK and dV
         uint32_t ucnt = 0, it_all = 0;
         bool ok = true;
         for (int idx = unit_begin; idx < unit_end && ok; ++idx) {
@@ -466,106 +523,82 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             const int kend = key_ok ? p.tok_end[key] : 0;
             const int min_kend = p.tok_end[u.k0];
             const bool partial = u.k0 + kBlk > p.T;
-            int prev_h = 0, prev_qb = 0;
-            for (int it = 0; it < n_it && ok; ++it, ++it_all) {
-                const int h = u.kvh * G + it / u.n_blk;
-                const int qb = (u.i0 + it % u.n_blk) * kBlk;
+            for (int it = 0, i = 0; it < n_it && ok; ++it, ++it_all) {
+                const int qb = (u.i0 + i) * kBlk;
+                if (++i == u.n_blk) i = 0;
+                if (threadIdx.x == 0) *progress = it_all + 1;
                 const uint32_t qs = it_all % QS;
                 const float* lse2 = reinterpret_cast<const float*>(smem + L::kLseOff + qs * 512) + c0;
                 const bool need_mask = (qb == u.k0) || (qb + kBlk - 1 >= min_kend) || partial;
                 const int j_lo = (int)(key - qb) - c0;
                 const int j_hi = kend - 1 - qb - c0;
-                ok = warp_wait(&bar_qfull[qs], (it_all / QS) & 1, abort_flag) && warp_wait(bar_sfull, it_all & 1, abort_flag);
+                ok = watched_warp_wait(&bar_qfull[qs], (it_all / QS) & 1, abort_flag) && watched_warp_wait(bar_sfull, it_all & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
-                uint32_t pk[32];   // P^T(it) of this thread's 64 queries, packed, kept until Y is free
-                {
-                    uint32_t sv[64];
-                    tmem_ld32(t_x + c0, sv);
-                    tmem_ld32(t_x + c0 + 32, sv + 32);
-                    tmem_ld_wait();
-                    tc_fence_before();
-                    mbar_arrive(bar_xfree1);
+                uint32_t sv[32], sv2[32];   // S^T of the 32 queries at hand and of the other 32
+                tmem_ld32(t_x + c0, sv);
+                tmem_ld32(t_x + c0 + 32, sv2);
+                tmem_ld_wait();
+                tc_fence_before();
+                mbar_arrive(bar_xfree1);
+                // (one copy of the code for both halves)
+#pragma unroll 1
+                for (int half = 0; half < 2; ++half) {
+                    const float* l2 = lse2 + 32 * half;
+                    float pf[32];
 #pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        float pf[32];
-#pragma unroll
-                        for (int j = 0; j < 32; j += 4) {
-                            const int jj = half * 32 + j;
-                            const ulonglong2 l4 = *reinterpret_cast<const ulonglong2*>(lse2 + jj);
-                            float x0, x1, x2, x3;
-                            f2_unpack(f2_fma(f2_pack(__uint_as_float(sv[jj]), __uint_as_float(sv[jj + 1])), scale2,
-                                             f2_mul(l4.x, neg1)), x0, x1);
-                            f2_unpack(f2_fma(f2_pack(__uint_as_float(sv[jj + 2]), __uint_as_float(sv[jj + 3])), scale2,
-                                             f2_mul(l4.y, neg1)), x2, x3);
-                            pf[j] = ex2_approx(x0);
-                            pf[j + 1] = ex2_approx(x1);
-                            pf[j + 2] = ex2_approx(x2);
-                            pf[j + 3] = ex2_approx(x3);
-                        }
-                        if (need_mask) {   // as bits: compares per element became branches (10007 tokens in samples of up to
-                            // 400, 8 heads: this kernel 112.9 us with them, 102.6 without)
-                            const uint32_t vis = range_bits(j_lo - half * 32, j_hi - half * 32);
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) pf[j] = (vis >> j) & 1u ? pf[j] : 0.f;
-                        }
-#pragma unroll
-                        for (int j = 0; j < 32; j += 2) pk[half * 16 + (j >> 1)] = pack_bf16x2(pf[j], pf[j + 1]);
+                    for (int j = 0; j < 32; j += 4) {
+                        const ulonglong2 l4 = *reinterpret_cast<const ulonglong2*>(l2 + j);
+                        float x0, x1, x2, x3;   // LSE - S c
+                        f2_unpack(f2_fma(f2_pack(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1])), neg_scale2, l4.x), x0, x1);
+                        f2_unpack(f2_fma(f2_pack(__uint_as_float(sv[j + 2]), __uint_as_float(sv[j + 3])), neg_scale2, l4.y), x2, x3);
+                        pf[j] = ex2_approx(-x0);
+                        pf[j + 1] = ex2_approx(-x1);
+                        pf[j + 2] = ex2_approx(-x2);
+                        pf[j + 3] = ex2_approx(-x3);
                     }
+                    if (need_mask) {   // as bits: compares per element became branches (10007 tokens in samples of up to
+                        // 400, 8 heads: this kernel 112.9 us with them, 102.6 without)
+                        const uint32_t vis = range_bits(j_lo - half * 32, j_hi - half * 32);
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) pf[j] = (vis >> j) & 1u ? pf[j] : 0.f;
+                    }
+                    uint32_t pk[16];
+#pragma unroll
+                    for (int j = 0; j < 32; j += 2) pk[j >> 1] = pack_bf16x2(pf[j], pf[j + 1]);
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) sv[j] = sv2[j];
+                    // dQ(it-1) has left Y's P^T columns (its MMA ran behind dV(it-1), so P^T(it-1) is spent)
+                    if (half == 0 && it_all > 0) {
+                        ok = watched_warp_wait(&bar_yfree[0], (it_all - 1) & 1, abort_flag);
+                        if (!ok) break;
+                        tc_fence_after();
+                    }
+                    tmem_st16(t_p + c0 / 2 + half * 16, pk);
                 }
-                // dQ(it-1) leaves Y (its MMA ran behind dV(it-1) and dK(it-1), so P^T(it-1) and dS^T(it-1) are spent)
-                uint32_t dqv[64];   // this thread's share of dQ(it-1): head-dim columns c0 .. c0 + 63 of query row r
-                if (it > 0) {
-                    ok = fused_read_dq(bar_dqfull, bar_yfree, it_all - 1, abort_flag, t_y + c0, dqv);
-                    if (!ok) break;
-                }
-                if (it_all > 0) {   // every exp thread has read its part of the last dQ: Y is free
-                    ok = warp_wait(bar_yfree, (it_all - 1) & 1, abort_flag);
-                    if (!ok) break;
-                }
-                tc_fence_after();
-                tmem_st16(t_p + c0 / 2, pk);
-                tmem_st16(t_p + c0 / 2 + 16, pk + 16);
+                if (!ok) break;
                 tmem_st_wait();
                 tc_fence_before();
-                mbar_arrive(bar_phalf);
                 mbar_arrive(bar_pready);
-                if (it > 0) {
-                    fused_stage_dq(&tm_dqacc, stage, dqv, lane, c0, prev_h, prev_qb + (warp & 3) * 32);
-                    fused_stage_dq(&tm_dqacc, stage, dqv + 32, lane, c0 + 32, prev_h, prev_qb + (warp & 3) * 32);
-                }
-                prev_h = h;
-                prev_qb = qb;
             }
             if (!ok) break;
-            // the unit's last dQ, then its dK and dV
-            {
-                uint32_t dqv[64];
-                ok = fused_read_dq(bar_dqfull, bar_yfree, it_all - 1, abort_flag, t_y + c0, dqv);
-                if (!ok) break;
-                fused_stage_dq(&tm_dqacc, stage, dqv, lane, c0, prev_h, prev_qb + (warp & 3) * 32);
-                fused_stage_dq(&tm_dqacc, stage, dqv + 32, lane, c0 + 32, prev_h, prev_qb + (warp & 3) * 32);
-            }
             ++ucnt;
             // ---- unit epilogue: dK and dV of the pair tile are added to the fp32 accumulators ----
-            ok = warp_wait(bar_dkvfull, (ucnt - 1) & 1, abort_flag);
+            ok = watched_warp_wait(bar_dkvfull, (ucnt - 1) & 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t t_dk = tmem_base + lane_addr + kColDK + c0;
-            const uint32_t t_dv = tmem_base + lane_addr + kColDV + c0;
-            // through the warp's staging tile, like dQ: bulk reduce-adds of 32 key rows x 32 head-dim columns (rows
-            // past the end of the pool are dropped by the hardware)
-#pragma unroll
-            for (int which = 0; which < 2; ++which) {
-#pragma unroll
-                for (int cc = 0; cc < 64; cc += 32) {
-                    uint32_t v[32];
-                    tmem_ld32((which == 0 ? t_dk : t_dv) + cc, v);
-                    tmem_ld_wait();
-                    fused_stage_dq(which == 0 ? &tm_dkacc : &tm_dvacc, stage, v, lane, c0 + cc, u.kvh,
-                                   (int)u.k0 + (warp & 3) * 32);
-                }
+            // through the shared-memory dS^T tile, which dQ has read, like dQ: bulk reduce-adds of 32 key rows x 32 head-dim
+            // columns (rows past the end of the pool are dropped by the hardware)
+#pragma unroll 1
+            for (int c = 0; c < 4; ++c) {
+                uint32_t v[32];
+                const int col = c0 + (c & 1) * 32;
+                tmem_ld32(tmem_base + lane_addr + (c < 2 ? kColDK : kColDV) + col, v);
+                tmem_ld_wait();
+                fused_stage_dq(c < 2 ? &tm_dkacc : &tm_dvacc, stage, v, lane, col, u.kvh, (int)u.k0 + (warp & 3) * 32);
             }
+            if (lane == 0) tma_store_wait_read();
+            __syncwarp();
             tc_fence_before();
             mbar_arrive(bar_dkvempty);
             if (threadIdx.x == 0) p.tile_ns[p.cta_tiles[idx]] = (uint32_t)(globaltimer_ns() - tile_t0);
@@ -575,6 +608,7 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     }
 
     // ---------------- teardown ----------------
+    if (warp != kFuWatchWarp && lane == 0) atomicAdd(finished, 1u);
     tc_fence_before();
     __syncthreads();
     if (warp == kFuMmaWarp) tmem_dealloc(tmem_base, 512);

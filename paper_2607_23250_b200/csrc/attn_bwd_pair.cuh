@@ -147,16 +147,6 @@ __device__ __forceinline__ void warp_arrive_cluster(uint32_t bar, int lane) {
     __syncwarp();
     if (lane == 0) mbar_arrive_cluster(bar);
 }
-// A wait that ends when the phase has completed or the CTA has given up; the clock is the watching warp's business.
-__device__ __forceinline__ bool pair_wait(uint64_t* bar, uint32_t parity, volatile int* ctl) {
-    while (!mbar_try_wait(bar, parity))
-        if (ctl[0]) return false;
-    return true;
-}
-__device__ __forceinline__ bool pair_warp_wait(uint64_t* bar, uint32_t parity, volatile int* ctl) {
-    return __all_sync(0xffffffffu, pair_wait(bar, parity, ctl));
-}
-
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
@@ -237,21 +227,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (warp == kPrWatchWarp) {
         // ---------------- the clock of all waits: no iteration has begun for the budget of one, so the CTA gives up ----------------
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPrRegsOther));
-        if (elect_one()) {
-            uint64_t t0 = globaltimer_ns();
-            uint32_t seen = 0;
-            while (*const_cast<volatile uint32_t*>(finished) < kPairThreads / 32 - 1 && !abort_flag[0]) {
-                asm volatile("nanosleep.u32 100;");
-                const uint64_t t = globaltimer_ns();
-                const uint32_t now = *progress;
-                if (now != seen) {
-                    seen = now;
-                    t0 = t;
-                } else if (t - t0 > (uint64_t)p.wait_limit_ns) {
-                    abort_flag[0] = 1;
-                }
-            }
-        }
+        if (elect_one()) watch_progress(progress, finished, kPairThreads / 32 - 1, p.wait_limit_ns, abort_flag);
         __syncwarp();
     } else if (warp == kPrInWarp) {
         // ---------------- the other CTA's half of dS: its copies count on a barrier here, the leader is told ----------------
@@ -266,7 +242,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 for (int it = 0; it < n_it; ++it) {
                     mbar_arrive_expect_tx(&bars[L::kDsIn], L::kHalf);
                     armed = 1;
-                    ok = pair_wait(&bars[L::kDsIn], n & 1, abort_flag);
+                    ok = watched_wait(&bars[L::kDsIn], n & 1, abort_flag);
                     if (!ok) break;
                     armed = 0;
                     ++n;
@@ -308,7 +284,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 for (int k = 0; k < kPairLoads; ++k) {
                     const bool rows = k == kLoadQr || k == kLoadDor, prev = k == kLoadDoc || k == kLoadQc;
                     if (prev ? prev_qb >= 0 : more && (rows || unit)) {   // (K and V behind the last loads of the unit before)
-                        ok = pair_wait(&bars[L::kSFull + k], ((phase >> k) & 1) ^ 1, abort_flag);
+                        ok = watched_wait(&bars[L::kSFull + k], ((phase >> k) & 1) ^ 1, abort_flag);
                         if (!ok) break;
                         phase ^= 1u << k;
                         issued[rank * kPairLoads + k] = issued[rank * kPairLoads + k] + 1;
@@ -361,7 +337,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             const uint64_t mdesc0 = make_sdesc(sb, L::kHalf, 1024);      // MN-major view (64 columns: one atom)
             uint32_t ucnt = 0, n = 0;
             bool ok = true;
-            auto wait = [&](int bar, uint32_t parity) { ok = pair_wait(&bars[bar], parity & 1, abort_flag); return ok; };
+            auto wait = [&](int bar, uint32_t parity) { ok = watched_wait(&bars[bar], parity & 1, abort_flag); return ok; };
             auto issue_x = [&](uint32_t a_off, uint32_t b_off) {
                 const uint64_t da = sdesc_advance(kdesc0, a_off), db = sdesc_advance(kdesc0, b_off);
 #pragma unroll
@@ -471,7 +447,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             for (int it = 0, i = 0, h = u.kvh * G; it < n_it; ++it, ++n) {
                 const int row = (u.i0 + i) * kBlk + 64 * (int)rank + 32 * (w & 1), head = h;
                 if (++i == u.n_blk) { i = 0; ++h; }
-                ok = pair_warp_wait(&bars[L::kDqFull], n & 1, abort_flag);
+                ok = watched_warp_wait(&bars[L::kDqFull], n & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
                 uint32_t v[64];
@@ -507,7 +483,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             const int n_it = G * u.n_blk;
             for (int it = 0; it < n_it && ok; ++it, ++n) {
                 const float* dvec = reinterpret_cast<const float*>(smem + L::kDvecOff + (n & 1) * 512);
-                ok = pair_warp_wait(&bars[L::kDvecFull + (n & 1)], (n >> 1) & 1, abort_flag) && pair_warp_wait(&bars[L::kDpFull], n & 1, abort_flag);
+                ok = watched_warp_wait(&bars[L::kDvecFull + (n & 1)], (n >> 1) & 1, abort_flag) && watched_warp_wait(&bars[L::kDpFull], n & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
                 uint32_t xs[64];   // (dP^T - D) as packed bf16 pairs
@@ -532,12 +508,12 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 }
                 // dQ(it-1) has been read out of dS^T's columns (so its MMA, which read dS of both CTAs, has run); the last unit's
                 // dK and dV have left both CTAs through the dS tiles
-                if (n > 0) ok = pair_warp_wait(&bars[L::kZFree], (n - 1) & 1, abort_flag);
-                if (ok && it == 0 && ucnt > 0) ok = pair_warp_wait(&bars[L::kDkvEmpty], (ucnt - 1) & 1, abort_flag);
+                if (n > 0) ok = watched_warp_wait(&bars[L::kZFree], (n - 1) & 1, abort_flag);
+                if (ok && it == 0 && ucnt > 0) ok = watched_warp_wait(&bars[L::kDkvEmpty], (ucnt - 1) & 1, abort_flag);
                 if (!ok) break;
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
-                    ok = pair_warp_wait(&bars[half == 0 ? L::kPHalf : L::kPLocal], n & 1, abort_flag);
+                    ok = watched_warp_wait(&bars[half == 0 ? L::kPHalf : L::kPLocal], n & 1, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                     uint32_t pa[16], pb[16];   // queries 32 half .. and 64 + 32 half ..
@@ -603,7 +579,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 const bool need_mask = (qb <= k0) || (qb + kBlk - 1 >= min_kend) || partial;
                 const int j_lo = (int)(key - qb) - c0;
                 const int j_hi = kend - 1 - qb - c0;
-                ok = pair_warp_wait(&bars[L::kLseFull + (n & 1)], (n >> 1) & 1, abort_flag) && pair_warp_wait(&bars[L::kSFull], n & 1, abort_flag);
+                ok = watched_warp_wait(&bars[L::kLseFull + (n & 1)], (n >> 1) & 1, abort_flag) && watched_warp_wait(&bars[L::kSFull], n & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
                 uint32_t sv[32], sv2[32];   // S^T of the 32 queries at hand and of the other 32
@@ -638,7 +614,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 #pragma unroll
                     for (int j = 0; j < 32; ++j) sv[j] = sv2[j];
                     if (half == 0 && n > 0) {   // P^T(it-1) has been read by the dS group and consumed by dV(it-1)
-                        ok = pair_warp_wait(&bars[L::kPRead], (n - 1) & 1, abort_flag) && pair_warp_wait(&bars[L::kDocEmpty], (n - 1) & 1, abort_flag);
+                        ok = watched_warp_wait(&bars[L::kPRead], (n - 1) & 1, abort_flag) && watched_warp_wait(&bars[L::kDocEmpty], (n - 1) & 1, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
                     }
@@ -652,7 +628,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             ++ucnt;
             // ---- unit epilogue: dK and dV of the CTA's key block are added to the fp32 accumulators, through the dS tile (dQ has
             // read it) and bulk reduce-adds of 32 key rows x 32 head-dim columns ----
-            ok = pair_warp_wait(&bars[L::kDkvFull], (ucnt - 1) & 1, abort_flag);
+            ok = watched_warp_wait(&bars[L::kDkvFull], (ucnt - 1) & 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
             // of a query chunk's row blocks this CTA's keys may have seen none

@@ -512,7 +512,11 @@ static const PairTables* choose_pair_chunk(const libra_plan* p, const PairCands&
     return best;
 }
 // Whether the fused backward runs on pairs of CTAs with 256 keys a tile.
-constexpr int64_t kPairsSample = 1024;   // tokens per sample, empty ones counted, from which on it does
+// From 1024 tokens per sample on, empty ones counted: a pair's cells are 256 keys wide, and where only one of its key blocks sees a
+// row block the other CTA's work is lost.  Fused kernel, 33000 tokens, 32 / 8 heads, on single CTAs and on pairs (us): samples
+// of up to 400 627 and 729, of 512 584 and 581, of 750 902 and 916, of 1024 944 and 927; one sequence of the usual mix of
+// lengths (mean 1200), 8 / 2 heads: 3114 and 2857.
+constexpr int64_t kPairsSample = 1024;
 static bool fused_on_pairs(int64_t T, int n_samples) { return T >= kPairsSample * (int64_t)n_samples; }
 static double heads_per_kv(const libra_plan* p) { return p->dir[0].H > p->dir[2].H ? (double)p->dir[0].H / p->dir[2].H : 1.0; }
 // Counts, choice and, while every size has more than 262144 pair-blocks, twice the largest.
@@ -561,7 +565,7 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
     cudaStream_t s = p->stream;
     const bool wide_pairs = want[3] && want[2];                   // the wide tiles are pair tiles
     const bool sorted[kDirs] = {want[0], want[1], false, want[3] && !want[2], false};   // sizes known, placed heaviest first
-    const bool pairs[kDirs] = {false, false, want[2], wide_pairs, want[4]};
+    bool pairs[kDirs] = {false, false, want[2], wide_pairs, want[4]};
     for (int k = 0; k < kDirs; ++k) {
         if (!sorted[k]) continue;
         p->dir[k].NB = (T + p->dir[k].tile - 1) / p->dir[k].tile;
@@ -613,6 +617,9 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
     // ---- pair tiles: their number comes back, then their arrays
     if (want[2]) {
         if (const int rc = count_pair_blocks(p, cands, d_totals, chosen, heads_per_kv(p)); rc != LIBRA_OK) return rc;
+        // (Of a pool so small that a chunk is one row block the launch counts, and pairs of CTAs take longer to get going: backward
+        // of 1500 tokens, 8 / 2 heads, 40.2 us on single ones and 42.8 on pairs; of 4000, chunks of two row blocks, 133 and 114.)
+        if (o.pair_chunk == 0 && chosen[2].R == 1) pairs[4] = false;
         Carver ps, pm;
         size_t pair_zero = 0;
         for (int k = 2; k < kDirs; ++k) {
@@ -657,10 +664,10 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
     }
     const int n_sorted = n;
     for (int k = 2; k < kDirs; ++k)
-        if (want[k] && !sorted[k]) views.v[n++] = view_of(p->dir[k], 1, o);
+        if (pairs[k]) views.v[n++] = view_of(p->dir[k], 1, o);
     if (n == 0) return LIBRA_OK;
     for (int k = 0; k < kDirs; ++k)
-        if (want[k]) {
+        if (sorted[k] || pairs[k]) {
             max_nt = p->dir[k].NT > max_nt ? p->dir[k].NT : max_nt;
             max_w = p->dir[k].W > max_w ? p->dir[k].W : max_w;
         }
@@ -679,7 +686,7 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
         k_check_loads<<<v.W, 256, 0, s>>>(v, p->d_status);
         count_launch();
     }
-    for (int k = 0; k < kDirs; ++k) p->dir[k].enabled = want[k] ? 1 : 0;
+    for (int k = 0; k < kDirs; ++k) p->dir[k].enabled = sorted[k] || pairs[k] ? 1 : 0;
     return cudaGetLastError() == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
 
