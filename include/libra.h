@@ -205,6 +205,9 @@ size_t libra_attn_pool_bwd_workspace_bytes(const libra_plan_t* plan, const libra
  *   kernel that walks the pair-tile lists and computes S, dP, dV, dK and dQ of a cell together (five GEMMs per
  *   cell), and a conversion pass.  dK and dV of a pair tile accumulate on chip and are added to fp32 accumulators
  *   in the workspace when the tile ends; dQ of every cell is added to its fp32 accumulator; all by bulk reduce-adds.
+ *   Where samples average 1024 tokens or more (and pair_chunk was given or the chunk chosen is more than one row block) the
+ *   kernel runs on pairs of CTAs: a pair takes 256 keys, two neighbouring pair tiles at once, from lists of its own that
+ *   Algorithm 2's rule makes from the same cells.
  *   The accumulators are rounded to bf16 once, at the end, so the result is at least as accurate as the two-kernel
  *   form's, but the order of the floating-point additions varies from run to run: results agree to rounding, not
  *   bit for bit.  The other directions of the plan are not used by this form.
@@ -351,7 +354,8 @@ int libra_tap_schedule(const int32_t* cu_seqlens_dev, int n_samples, const int32
 int libra_busy_times(const libra_plan_t* plan, int which, uint64_t* ns_host);
 
 /* Time each tile took in the most recent launch of the forward kernel (which = LIBRA_KERNEL_FWD, tiles of the
- * query-major direction) or of the fused backward kernel (LIBRA_KERNEL_BWD_FUSED, pair tiles): nanoseconds of the
+ * query-major direction) or of the fused backward kernel (LIBRA_KERNEL_BWD_FUSED, pair tiles; of two that a pair of CTAs
+ * takes together, each gets the time of both): nanoseconds of the
  * global timer from the moment a compute thread of the CTA turns to the tile until it has finished the tile's
  * last output, indexed by tile id; 0 for a tile that was not run.  With the plan's weights (libra_plan_export)
  * this shows how well the tile weight predicts time: the paper notes that a FLOPs-balanced assignment need not
@@ -363,7 +367,8 @@ int libra_tile_times(const libra_plan_t* plan, int which, uint32_t* ns_host);
  * (0 restores the default of 2 s, the maximum is 4 s).  Every wait on a barrier inside the kernels
  * is bounded: a wait that outlives the budget makes its CTA stop issuing work, let the copies and
  * MMAs it has in flight finish, free its tensor memory and return, and the launch reports
- * LIBRA_ERR_TIMEOUT through libra_busy_times.  A healthy run never comes near the default. */
+ * LIBRA_ERR_TIMEOUT through libra_busy_times.  (In the fused backward one warp watches the clock for all waits of a CTA: the
+ * budget is for the time without a new 128-row query block.)  A healthy run never comes near the default. */
 int libra_plan_set_wait_limit_ns(libra_plan_t* plan, uint64_t ns);
 
 /* Test aid (no counterpart in the paper): while enabled, the producer role of the attention kernels launched

@@ -1,7 +1,8 @@
 // Backward pool attention for sm_100a.
 //
 // Two forms of the same computation; the plan decides (see libra_attn_pool_bwd in the public header).
-// Fused form (attn_bwd_fused.cuh, plans with pair tiles, head_dim 128): row statistics, ONE kernel that computes
+// Fused form (attn_bwd_fused.cuh, on pairs of CTAs attn_bwd_pair.cuh; plans with pair tiles, head_dim 128): row
+// statistics, ONE kernel that computes
 // S, dP, dV, dK and dQ of every 128 x 128 cell together (five GEMMs) with fp32 accumulators in global memory,
 // and a conversion pass.
 // Two-kernel form (this file and attn_bwd_dq.cuh): (1) prep: D_i = <dO_i, O_i> and LSE in log2 units, padded

@@ -1,5 +1,6 @@
 // Fused backward kernel (included by attn_bwd.cu): dQ, dK and dV of a pair tile in one pass, five GEMMs per
-// 128 x 128 cell instead of the seven of the two-kernel form (S and dP are computed once).
+// 128 x 128 cell instead of the seven of the two-kernel form (S and dP are computed once).  On single CTAs: for pools of
+// short samples and pools cut into single row blocks; the others run on pairs of CTAs (attn_bwd_pair.cuh).
 //
 // A unit is a pair tile: 128 keys of one kv head against the query row blocks of one query chunk, for every
 // query head of the kv head's group.  K and V stay in shared memory, dK and dV accumulate in TMEM over the
@@ -20,9 +21,7 @@
 // once dV(it) and dK(it) have consumed them, receives dQ(it) (fp32, 128 columns: the MMAs run in issue order, so
 // the overwrite needs no extra barrier); P^T(it+1), already computed in registers, is written as soon as dQ(it) has
 // been read out.
-// Roles (512 threads): warps 0-3 and 4-7 exp groups (64 query columns of S^T each; 64 head-dim columns of dQ
-// each), 8-11 dS group, 12 TMA thread, 13 MMA thread, 14-15 only hand their registers over.
-// Roles (640 threads): two exp groups, a dS group, a dQ group, the TMA thread, the MMA thread, the thread that watches the
+// Roles (640 threads): two exp groups (64 query columns of S^T each), a dS group, a dQ group, the TMA thread, the MMA thread, the thread that watches the
 // clock for all of them; a warp only hands its registers over.  The exp groups moved dQ between their exponentials before
 // (512 threads); with that, the waits' code in one place and one copy of the exponentials' the kernel is 50 KB instead of
 // 63: backward of 10 samples of 1000 tokens, 8 / 2 heads, 137.0 -> 133.4 us, of one of 1500 42.8 -> 40.2.
@@ -44,7 +43,7 @@ struct FusedSmem {
     static constexpr int kQOff = 2 * kTile;
     static constexpr int kDoOff = kQOff + kQStages * kTile;
     static constexpr int kDsOff = kDoOff + kTile;          // dS^T tile (bf16, the operand layout of K / V tiles)
-    static constexpr int kStageOff = kDsOff + kTile;       // dQ staging: per exp warp a tile of 32 rows x 32 floats, swizzled
+    static constexpr int kStageOff = kDsOff + kTile;       // dQ staging: tiles of 32 rows x 32 floats, swizzled
     static constexpr int kLseOff = kStageOff + 2 * kHalf;  // per Q stage: lse2[128]
     static constexpr int kDvecOff = kLseOff + kQStages * 512;   // two buffers: dvec(it+1) lands while dvec(it) is read
     static constexpr int kBarOff = kDvecOff + 2 * 512;

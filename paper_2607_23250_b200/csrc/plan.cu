@@ -495,10 +495,10 @@ static void add_pair_cands(const libra_plan* p, PairCands& cands, int k, bool ha
 }
 // The chunk size of direction k.  In units of one cell of one query head (3.1 us), a worker's time over its mean is about
 // the tiles it starts, 3 each (operands in, accumulators out), and up to the length of one tile, R cells of G heads: idle
-// at the end.  Fused backward, best of 4096 ... 128 rows (4096): one sequence of 1500 tokens, 32 / 8 heads: 128, 60 us
-// (120); 12000 tokens, 4 / 1 heads: 1024, 159 us (345); 10007 tokens in samples of up to 400, 8 / 2 heads: 128, 64 us (91);
-// 16000 tokens, 32 / 4 heads: 1024, 0.98 ms (1.28); 32768 tokens, 32 / 8 heads: 2048, 5.88 ms (5.93), 128: 7.31; one sample of
-// 32768: 4096, 23.4 ms, 2048: 23.6, 128: 29.8.
+// at the end.  Backward (us) with the best of 4096 ... 128 rows and with 4096: one sequence of 1500 tokens, 32 / 8 heads: 256, 97
+// (133); 10007 tokens in samples of up to 400, 8 / 2 heads: 128, 86 (109); one of 4000, 8 / 2 heads: 512, 114 (289); 12000 tokens,
+// 4 / 1 heads: 1024, 407 (426); 16000, 32 / 4 heads: 1024, 5190 (5230); 8 samples of 4096, 32 / 8 heads: 4096, 3320, with 128: 4350;
+// one sample of 32768: 4096, 21.0 ms, 2048: 21.3, 128: 29.9.  On 13 further pools the choice was within 4 % of the best.
 static const PairTables* choose_pair_chunk(const libra_plan* p, const PairCands& cands, const int64_t* totals, int k, double G) {
     const PairTables* best = nullptr;
     double least = 0;

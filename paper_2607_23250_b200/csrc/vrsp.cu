@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(256) k_vrsp_rank(const int64_t* __restrict__ w
 }
 
 // Placement in waves by one block (waves.cuh): the bins are the pools with room; a full pool leaves the array.  Needs
-// 0 <= work and loads below 2^53 (the caller checks).  1024 sequences into 128 pools, all three kernels: 31 us; 502 us
+// 0 <= work and loads below 2^53 (the caller checks).  1024 sequences into 128 pools, all three kernels: 29 us; 502 us
 // with an arg-min over all pools per sequence, 75 us in waves of up to 32 by one warp.
 __device__ void vrsp_place_waves(const int64_t* __restrict__ work, const int32_t* __restrict__ sorted, int D, int P, int K,
                                  int32_t* __restrict__ order, int32_t* __restrict__ pool_of_seq,
