@@ -646,69 +646,80 @@ namespace libra {
 // ---- prep kernel ------------------------------------------------------------------------------
 
 // D = <dO, O> per (token, head) and LSE in log2 units; rows in [T, Tpad) get zeros.
-// One warp per head and run of kPrepRows consecutive tokens: D / 8 lanes read a row with 16-byte loads, eight steps of them cover
-// the run and are all issued before the first is used; lane i ends up with the sum of row i.  clear_ctas of the CTAs,
-// spread evenly over the grid, only zero the accumulators that the coming kernels add to, so that these stores and the
-// others' loads are under way together.  (With 32 tokens a warp for every D it went through two or four rounds of steps, and
-// clearing ran ahead of the loads in every thread.)
+// A warp takes `rounds` runs of kPrepRows consecutive tokens of a head: D / 8 lanes read a row with 16-byte loads, eight steps of
+// them cover the run and are all issued before the first is used; lane i ends up with the sum of row i.  Some CTAs, spread
+// evenly over the grid, only zero the accumulators that the coming kernels add to, so that these stores and the others'
+// loads are under way together.  Bound by memory; where few bytes are under way the instructions in front of the loads count: the
+// indices are 32-bit.  us with 64-bit ones and a round, with a round, two and four (GB/s): 524288 tokens, 32 / 8 heads of 128,
+// accumulators cleared, 4322, 3677, 3518 and 3499 (6200); 131072 of them 941, 857, 846, 841 (6450); 32768: 237, 214, 216, 221; 10007, 8
+// / 2 heads: 25.7, 25.8, 25.4, 29.8; 65536 tokens, 32 heads, nothing to clear: 247, 225, 208, 193 (5700).  Hence four where
+// there are seven waves of the warps that fit all the same.
 constexpr int kClearPerThread = 16;
 template <int D>
 constexpr int kPrepRows = 8 * 256 / D;
+// Readers and clearers: of the first `spread` CTAs every period-th is of the rarer kind.
+struct PrepMix { uint32_t period, spread, clear_is_rare; };
+constexpr int64_t kPrepManyWarps = 24576;
 template <int D>
 __global__ void k_bwd_prep(const __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ dout,
                            const float* __restrict__ lse, int64_t T, int64_t Tpad, int hq, float* __restrict__ dvec,
-                           float* __restrict__ lse2, float4* __restrict__ clear, int64_t n_clear, int64_t clear_ctas) {
+                           float* __restrict__ lse2, float4* __restrict__ clear, int64_t n_clear, PrepMix mix, int rounds) {
     grid_dep_wait();
     grid_dep_launch();
-    const int64_t before = blockIdx.x * clear_ctas / gridDim.x;   // clearing CTAs with a lower index
-    if ((blockIdx.x + 1) * clear_ctas / gridDim.x != before) {
-        int64_t i = before * (256 * kClearPerThread) + threadIdx.x;
+    const uint32_t turn = blockIdx.x / mix.period, odd = blockIdx.x < mix.spread && blockIdx.x % mix.period == 0;
+    const uint32_t rare = blockIdx.x < mix.spread ? turn : mix.spread / mix.period, usual = blockIdx.x - rare - (blockIdx.x < mix.spread);
+    if (odd == mix.clear_is_rare) {
+        int64_t i = (int64_t)(odd ? rare : usual) * (256 * kClearPerThread) + threadIdx.x;
 #pragma unroll
         for (int k = 0; k < kClearPerThread; ++k, i += 256)
             if (i < n_clear) clear[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         return;
     }
-    const int64_t w = ((blockIdx.x - before) * (int64_t)256 + threadIdx.x) >> 5;
+    const uint32_t w = (odd ? rare : usual) * 8u + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     constexpr int LPR = D / 8, RPS = 32 / LPR, STEPS = 8, ROWS = kPrepRows<D>;
     static_assert(ROWS == STEPS * RPS && 128 % ROWS == 0, "steps of a warp");
-    const int64_t groups = Tpad / ROWS;  // Tpad is a multiple of 128
+    const uint32_t groups = (uint32_t)(Tpad / ROWS) / rounds;  // Tpad is a multiple of 128
     if (w >= groups * hq) return;
     const int h = (int)(w / groups);
-    const int64_t t0 = (w % groups) * ROWS;
     const int sub = lane / LPR, part = lane % LPR;
-    float mine = 0.f;
-    uint4 a[STEPS], b[STEPS];
+#pragma unroll 1
+    for (int round = 0; round < rounds; ++round) {
+        const int64_t t0 = ((int64_t)(w % groups) * rounds + round) * ROWS;
+        float mine = 0.f;
+        uint4 a[STEPS], b[STEPS];
 #pragma unroll
-    for (int u = 0; u < STEPS; ++u) {
-        const int64_t t = t0 + u * RPS + sub;
-        a[u] = b[u] = make_uint4(0, 0, 0, 0);
-        if (t < T) {
-            a[u] = __ldg(reinterpret_cast<const uint4*>(out + ((size_t)t * hq + h) * D) + part);
-            b[u] = __ldg(reinterpret_cast<const uint4*>(dout + ((size_t)t * hq + h) * D) + part);
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < STEPS; ++u) {
-        const uint32_t* x = reinterpret_cast<const uint32_t*>(&a[u]);
-        const uint32_t* y = reinterpret_cast<const uint32_t*>(&b[u]);
-        float acc = 0.f;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 fa = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&x[i]));
-            const float2 fb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&y[i]));
-            acc += fa.x * fb.x + fa.y * fb.y;
+        for (int u = 0; u < STEPS; ++u) {
+            const int64_t t = t0 + u * RPS + sub;
+            a[u] = b[u] = make_uint4(0, 0, 0, 0);
+            if (t < T) {
+                a[u] = __ldg(reinterpret_cast<const uint4*>(out + ((size_t)t * hq + h) * D) + part);
+                b[u] = __ldg(reinterpret_cast<const uint4*>(dout + ((size_t)t * hq + h) * D) + part);
+            }
         }
 #pragma unroll
-        for (int off = LPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        // row u * RPS + sub of the warp's goes to the lane of that number
-        const float got = __shfl_sync(0xffffffffu, acc, (lane % RPS) * LPR);
-        if (lane / RPS == u) mine = got;
+        for (int u = 0; u < STEPS; ++u) {
+            const uint32_t* x = reinterpret_cast<const uint32_t*>(&a[u]);
+            const uint32_t* y = reinterpret_cast<const uint32_t*>(&b[u]);
+            float acc = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 fa = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&x[i]));
+                const float2 fb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&y[i]));
+                acc += fa.x * fb.x + fa.y * fb.y;
+            }
+#pragma unroll
+            for (int off = LPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+            // row u * RPS + sub of the warp's goes to the lane of that number
+            const float got = __shfl_sync(0xffffffffu, acc, (lane % RPS) * LPR);
+            if (lane / RPS == u) mine = got;
+        }
+        if (lane < ROWS) {
+            const int64_t t = t0 + lane;
+            dvec[(size_t)h * Tpad + t] = mine;
+            lse2[(size_t)h * Tpad + t] = t < T ? lse[(size_t)h * T + t] * 1.4426950408889634f : 0.f;
+        }
     }
-    if (lane >= ROWS) return;
-    const int64_t t = t0 + lane;
-    dvec[(size_t)h * Tpad + t] = mine;
-    lse2[(size_t)h * Tpad + t] = t < T ? lse[(size_t)h * T + t] * 1.4426950408889634f : 0.f;
 }
 
 struct BwdWorkspace {
@@ -780,11 +791,18 @@ static int launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtens
 template <int D>
 static cudaError_t launch_prep(const void* out, const void* dout, const float* lse, int64_t T, int64_t Tpad, int hq, float* dvec,
                                float* lse2, float* clear, size_t clear_bytes, cudaStream_t s) {
-    const int64_t warps = Tpad / kPrepRows<D> * hq, n_clear = (int64_t)(clear_bytes / 16);
-    const int64_t clear_ctas = (n_clear + 256 * kClearPerThread - 1) / (256 * kClearPerThread);
+    const int64_t n_clear = (int64_t)(clear_bytes / 16);
+    const int rounds = Tpad / kPrepRows<D> * hq >= 4 * kPrepManyWarps ? 4 : 2;
+    static_assert(128 % (4 * kPrepRows<D>) == 0, "rounds of a warp");
+    const int64_t readers = (Tpad / kPrepRows<D> / rounds * hq + 7) / 8, clearers = (n_clear + 256 * kClearPerThread - 1) / (256 * kClearPerThread);
+    const int64_t rare = clearers < readers ? clearers : readers, usual = clearers + readers - rare;
+    PrepMix mix;
+    mix.clear_is_rare = clearers < readers;
+    mix.period = (uint32_t)(rare ? usual / rare + 1 : 1);
+    mix.spread = (uint32_t)(rare * mix.period);
     count_launch();
-    return launch_dependent(k_bwd_prep<D>, (unsigned)((warps * 32 + 255) / 256 + clear_ctas), 256u, 0, s, (const __nv_bfloat16*)out,
-                            (const __nv_bfloat16*)dout, lse, T, Tpad, hq, dvec, lse2, (float4*)clear, n_clear, clear_ctas);
+    return launch_dependent(k_bwd_prep<D>, (unsigned)(readers + clearers), 256u, 0, s, (const __nv_bfloat16*)out,
+                            (const __nv_bfloat16*)dout, lse, T, Tpad, hq, dvec, lse2, (float4*)clear, n_clear, mix, rounds);
 }
 
 }  // namespace libra
