@@ -13,7 +13,6 @@
 // arg-min, tables in global memory.  1024 tiles on 16 workers with their schedule: 0.25 ms, with one warp for all of a
 // step 0.65 ms, all in the second form 2.8 ms.
 #include <cstdint>
-#include <new>
 #include <cuda_runtime.h>
 
 #include "../../include/libra.h"
@@ -28,12 +27,14 @@ struct TapGeom {
     const int32_t* blk_off;   // [P+1] first block of each sequence
     int n, P, CP, B, H, hq, hkv, d;
 };
-// The two tables of a pool of up to kTapParamSeqs sequences, as a kernel argument: the first kernel of a call reads them
-// there and leaves them in the call's scratch for the others.  (A copy from pageable memory instead took the host 10 us a
-// call and the stream 3.)
-constexpr int kTapParamSeqs = 255;
+// The two tables of a pool of up to SEQS sequences, as a kernel argument: the first kernel of a call reads them there and
+// leaves them in the call's scratch for the others.  (A copy from pageable memory instead took the host 10 us a call and
+// the stream 3; and a graph that is captured around the call would read that memory at every replay.)  2 KB for the usual
+// pools, 8 KB for as many sequences as there can be workers.
+constexpr int kTapFewSeqs = 255, kTapMaxWorkers = 1024;
+template <int SEQS>
 struct TapTables {
-    int32_t seq_off[kTapParamSeqs + 1], blk_off[kTapParamSeqs + 1];
+    int32_t seq_off[SEQS + 1], blk_off[SEQS + 1];
 };
 
 __device__ __forceinline__ int tap_seq_of_token(const TapGeom& g, int64_t tok) {
@@ -66,8 +67,7 @@ __device__ __forceinline__ int tap_sample_of_token_warp(const TapGeom& g, int64_
 struct TapSetup {
     int64_t NB;
     int block_ctas;          // CTAs that go through blocks, a warp each; the rest through samples
-    int from_params;         // the tables come as an argument: write them to seq_off, blk_off
-    int32_t *seq_off, *blk_off;
+    int32_t *seq_off, *blk_off;   // where the tables go
     int64_t* f_blk;
     int32_t* q_home;
     int64_t* v_qo;
@@ -79,15 +79,14 @@ struct TapSetup {
     int* status;
     int64_t* comm_total;
 };
-__global__ void __launch_bounds__(128) k_tap_setup(TapGeom g, const TapSetup p, const __grid_constant__ TapTables tables) {
+template <int SEQS>
+__global__ void __launch_bounds__(128) k_tap_setup(TapGeom g, const TapSetup p, const __grid_constant__ TapTables<SEQS> tables) {
     grid_dep_wait();
     grid_dep_launch();
-    if (p.from_params) {
-        if (blockIdx.x == 0)
-            for (int q = threadIdx.x; q <= g.P; q += 128) { p.seq_off[q] = tables.seq_off[q]; p.blk_off[q] = tables.blk_off[q]; }
-        g.seq_off = tables.seq_off;
-        g.blk_off = tables.blk_off;
-    }
+    if (blockIdx.x == 0)
+        for (int q = threadIdx.x; q <= g.P; q += 128) { p.seq_off[q] = tables.seq_off[q]; p.blk_off[q] = tables.blk_off[q]; }
+    g.seq_off = tables.seq_off;
+    g.blk_off = tables.blk_off;
     const int64_t all = (int64_t)gridDim.x * 128, at = blockIdx.x * (int64_t)128 + threadIdx.x;
 #pragma unroll
     for (int k = 0; k < 3; ++k)
@@ -546,7 +545,7 @@ __global__ void k_tap_exchange(TapGeom g, int64_t NT, const int32_t* __restrict_
     grid_dep_wait();
     grid_dep_launch();
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (*status != 0) return;   // a placement that gave up left sigma unwritten
+    if (*status != 0) return;   // a placement that gave up left the bit rows unwritten
     if (t < NT) {
         const int q = q_home[t / g.H], r = sigma[t];
         if (q == r || r < 0 || r >= W || q < 0 || q >= W) return;
@@ -744,26 +743,15 @@ extern "C" int64_t libra_tap_num_tiles(const int32_t* seq_offsets_host, int n_se
     return nb * n_shards;
 }
 
-// First kernel of a call.  The tables of the pool (`table`: 2 (P + 1) words of scratch) go with it as an argument, or, of more
-// sequences than an argument holds, ahead of it in a copy.
-static int launch_setup(TapGeom& g, TapSetup p, const int32_t* seq_offsets_host, int32_t* table, cudaStream_t s) {
-    static const TapTables none = {};
-    TapTables tables;
-    p.from_params = g.P <= kTapParamSeqs;
-    int32_t* h_tab = p.from_params ? nullptr : new (std::nothrow) int32_t[2 * (g.P + 1)];
-    if (!p.from_params && !h_tab) return LIBRA_ERR_CUDA;
-    int32_t* seq_off = p.from_params ? tables.seq_off : h_tab;
-    int32_t* blk_off = p.from_params ? tables.blk_off : h_tab + g.P + 1;
+// First kernel of a call.  The tables of the pool go with it as an argument and stay in `table` (2 (P + 1) words of scratch).
+template <int SEQS>
+static cudaError_t launch_setup_of(TapGeom& g, TapSetup p, const int32_t* seq_offsets_host, int32_t* table, cudaStream_t s) {
+    TapTables<SEQS> tables;
     int64_t nb = 0;
     for (int q = 0; q <= g.P; ++q) {
-        seq_off[q] = seq_offsets_host[q];
-        blk_off[q] = (int32_t)nb;
+        tables.seq_off[q] = seq_offsets_host[q];
+        tables.blk_off[q] = (int32_t)nb;
         if (q < g.P) nb += ((int64_t)seq_offsets_host[q + 1] - seq_offsets_host[q] + g.B - 1) / g.B;
-    }
-    cudaError_t e = cudaSuccess;
-    if (h_tab) {   // from pageable memory, so the copy has left h_tab when the call returns
-        e = cudaMemcpyAsync(table, h_tab, sizeof(int32_t) * 2 * (g.P + 1), cudaMemcpyHostToDevice, s);
-        delete[] h_tab;
     }
     p.seq_off = table;
     p.blk_off = table + g.P + 1;
@@ -771,8 +759,12 @@ static int launch_setup(TapGeom& g, TapSetup p, const int32_t* seq_offsets_host,
     g.blk_off = p.blk_off;
     p.block_ctas = (int)((p.NB + 3) / 4);
     const unsigned sample_ctas = (unsigned)(((int64_t)g.n + 127) / 128);
-    if (e == cudaSuccess) e = launch_dependent(k_tap_setup, (unsigned)p.block_ctas + sample_ctas, 128u, 0, s, g, p, p.from_params ? tables : none);
     count_launch();
+    return launch_dependent(k_tap_setup<SEQS>, (unsigned)p.block_ctas + sample_ctas, 128u, 0, s, g, p, tables);
+}
+static int launch_setup(TapGeom& g, const TapSetup& p, const int32_t* seq_offsets_host, int32_t* table, cudaStream_t s) {
+    const cudaError_t e = g.P <= kTapFewSeqs ? launch_setup_of<kTapFewSeqs>(g, p, seq_offsets_host, table, s)
+                                             : launch_setup_of<kTapMaxWorkers>(g, p, seq_offsets_host, table, s);
     return e == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
 
@@ -789,7 +781,7 @@ extern "C" int libra_tap_plan(const int32_t* cu_seqlens_dev, int n_samples, cons
     if (!((o->n_shards <= o->hkv && o->hkv % o->n_shards == 0) || (o->n_shards > o->hkv && o->n_shards % o->hkv == 0)))
         return LIBRA_ERR_INVALID_ARG;
     const int P = n_sequences, W = P * o->cp, H = o->n_shards;
-    if (W > 1024 || P > 4096) return LIBRA_ERR_UNSUPPORTED;
+    if (W > kTapMaxWorkers || P > kTapMaxWorkers) return LIBRA_ERR_UNSUPPORTED;
     const int64_t NT = libra_tap_num_tiles(seq_offsets_host, P, o->block, H);
     if (NT <= 0) return LIBRA_ERR_INVALID_ARG;
     const int64_t NB = NT / H;
@@ -825,7 +817,7 @@ extern "C" int libra_tap_plan(const int32_t* cu_seqlens_dev, int n_samples, cons
     g.cu = cu_seqlens_dev;
     g.n = n_samples; g.P = P; g.CP = o->cp; g.B = o->block; g.H = H; g.hq = o->hq; g.hkv = o->hkv; g.d = o->head_dim;
     // W * W byte matrices, loads, the volume total and the status start from zero
-    const TapSetup setup = {NB, 0, 0, nullptr, nullptr, f_blk, q_home, v_qo, j0, j1, v_smp, res_smp,
+    const TapSetup setup = {NB, 0, nullptr, nullptr, f_blk, q_home, v_qo, j0, j1, v_smp, res_smp,
                             {fwd_bytes_dev, bwd_bytes_dev, loads_dev}, {(int64_t)W * W, (int64_t)W * W, W}, status_dev, comm_total_dev};
     int rc = launch_setup(g, setup, seq_offsets_host, (int32_t*)(scratch + o_tab), s);
     auto launched = [&](cudaError_t e) { if (e != cudaSuccess) rc = LIBRA_ERR_CUDA; };
@@ -867,7 +859,7 @@ extern "C" int libra_tap_schedule(const int32_t* cu_seqlens_dev, int n_samples, 
         o->hkv <= 0 || o->head_dim <= 0 || o->hq % o->n_shards != 0)
         return LIBRA_ERR_INVALID_ARG;
     const int P = n_sequences, W = P * o->cp, H = o->n_shards;
-    if (W > 1024 || P > 4096) return LIBRA_ERR_UNSUPPORTED;
+    if (W > kTapMaxWorkers || P > kTapMaxWorkers) return LIBRA_ERR_UNSUPPORTED;
     const int64_t NT = libra_tap_num_tiles(seq_offsets_host, P, o->block, H);
     if (NT <= 0) return LIBRA_ERR_INVALID_ARG;
     const int64_t NB = NT / H, NG = (int64_t)n_samples * H;
@@ -895,7 +887,7 @@ extern "C" int libra_tap_schedule(const int32_t* cu_seqlens_dev, int n_samples, 
     int32_t* ahead = (int32_t*)(scratch + o_ahead);
     int64_t* total = (int64_t*)(scratch + o_total);
     // the marks start from zero (rows rounded up to whole 64-bit words)
-    const TapSetup setup = {NB, 0, 0, nullptr, nullptr, nullptr, q_home, nullptr, j0, j1, nullptr, res_smp,
+    const TapSetup setup = {NB, 0, nullptr, nullptr, nullptr, q_home, nullptr, j0, j1, nullptr, res_smp,
                             {(int64_t*)marks, nullptr, nullptr}, {((int64_t)words * W + 1) / 2, 0, 0}, nullptr, nullptr};
     int rc = launch_setup(g, setup, seq_offsets_host, (int32_t*)(scratch + o_tab), s);
     auto launched = [&](cudaError_t e) { if (e != cudaSuccess) rc = LIBRA_ERR_CUDA; };

@@ -91,6 +91,39 @@ def test_steps_of_the_one_block_placement(P, CP, H, hq, hkv, max_len, total):
         _compare(cu, np.arange(P + 1, dtype=np.int32) * total, CP, 128, H, hq, hkv, 8, tau)
 
 
+@pytest.mark.parametrize("P", [255, 256, 300, 1024])
+def test_many_sequences(P):
+    """As many sequences as the smaller tables hold, more, and as many as there can be workers."""
+    rng = np.random.default_rng(P)
+    seqs = [pools.random_layout(rng, int(rng.integers(3, 20)), 9) for _ in range(P)]
+    cu = pools.cu_seqlens([x for s in seqs for x in s])
+    seq_off = np.concatenate([[0], np.cumsum([sum(s) for s in seqs])]).astype(np.int32)
+    _compare(cu, seq_off, 1, 16, 1, 2, 1, 8)
+
+
+@pytest.mark.parametrize("P", [3, 300])
+def test_replays_of_a_captured_call_need_nothing_of_the_host(P):
+    """A graph captured around the planner gives the eager call's results after the host memory of that time has been used
+    for something else."""
+    from paper_2607_23250_b200 import binding as lb
+    rng = np.random.default_rng(P)
+    seqs = [pools.random_layout(rng, 24, 9) for _ in range(P)]
+    cu = torch.from_numpy(pools.cu_seqlens([x for s in seqs for x in s])).cuda()
+    seq_off = [24 * i for i in range(P + 1)]
+    want = lb.libra_tap_plan(cu, seq_off, 1, 16, 1, 2, 1, 8)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = lb.libra_tap_plan(cu, seq_off, 1, 16, 1, 2, 1, 8)
+    junk = [np.full(2 * (P + 1), -1, np.int32) for _ in range(4096)]
+    for _ in range(3):
+        graph.replay()
+        torch.cuda.synchronize()
+        for name in want:
+            assert torch.equal(got[name], want[name]), name
+    assert int(want["status"].item()) == 0 and len(junk) == 4096
+
+
 def test_zero_length_samples_and_short_tail():
     _compare([0, 0, 3, 3, 3, 40, 40, 41], [0, 41], 2, 16, 2, 4, 2, 8)
     _compare([0, 7, 7, 30, 30], [0, 7, 30], 1, 4, 1, 2, 2, 8)
