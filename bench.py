@@ -467,8 +467,7 @@ def headline(args, world, spec, pool, value, ms_per_step, ms_local, kern, busy, 
     # dK/dV kernel of the two-kernel form: the four GEMMs it owns (8 d).  It is timed inside the timed region; that
     # region's length decides which measured peak applies (burst under a second, else sustained).
     if pool.fused and d == 128:
-        # (the fused backward runs on pairs of CTAs from 1024 tokens per sample on)
-        dom = "k_attn_bwd_pair" if T >= 1024 * len(pool.lengths) else "k_attn_bwd_fused"
+        dom = "k_attn_bwd_pair" if pool.plan.fused_ctas() == 2 else "k_attn_bwd_fused"
         dom_ms, fa = kern["bwd_fused"], fb
         executed = {"fused (10 d per pair)": round(fb / kern["bwd_fused"] / 1e9, 1)}
         ratio = "14 d / 14 d per causal pair (every GEMM of the gradient is computed once)"

@@ -165,6 +165,11 @@ int libra_plan_export(const libra_plan_t* plan, int direction, int64_t* weight_h
 int libra_plan_export_pairs(const libra_plan_t* plan, int32_t* key_block_host, int32_t* query_chunk_host,
                             int* chunk_tokens_host);
 
+/* CTAs that take a pair tile together in this plan's fused backward (head_dim 128): 1, or 2 where it runs on pairs of CTAs
+ * (see libra_attn_pool_bwd).  Host value, no synchronisation.  Errors (negative): INVALID_ARG, PLAN_MISMATCH (no pair
+ * tiles). */
+int libra_plan_fused_ctas(const libra_plan_t* plan);
+
 /* Frees the plan's device and host memory.  Synchronises the device first, unless the plan was built and used on the
  * legacy default stream only: the memory is then released in that stream's order. NULL is OK. */
 int libra_plan_destroy(libra_plan_t* plan);

@@ -27,7 +27,7 @@ ERR_OVERFLOW, ERR_TIMEOUT, ERR_BAD_SEQLENS, ERR_NO_DEVICE = -5, -6, -7, -8
 ERR_SCRATCH_TOO_SMALL = -9
 
 EXPORTS = ["libra_plan_tiles", "libra_plan_info", "libra_plan_status", "libra_plan_export",
-           "libra_plan_export_pairs", "libra_plan_destroy", "libra_attn_pool_fwd", "libra_attn_pool_bwd_workspace_bytes",
+           "libra_plan_export_pairs", "libra_plan_fused_ctas", "libra_plan_destroy", "libra_attn_pool_fwd", "libra_attn_pool_bwd_workspace_bytes",
            "libra_attn_pool_bwd", "libra_attn_pool_bwd_noalloc_max_bytes", "libra_attn_pool_bwd_noalloc",
            "libra_tap_schedule", "libra_busy_times", "libra_tile_times", "libra_plan_set_wait_limit_ns", "libra_plan_inject_stall", "libra_plan_set_timing", "libra_kernel_time_ms", "libra_kernel_times_ms", "libra_selftest_wait_timeout", "libra_launch_count",
            "libra_strerror"]
@@ -123,6 +123,12 @@ class Plan:
         kb, qc, chunk = np.empty(nb, np.int32), np.empty(nb, np.int32), ctypes.c_int()
         _check(_lib.libra_plan_export_pairs(self._h, _np(kb), _np(qc), ctypes.byref(chunk)), "libra_plan_export_pairs")
         return kb, qc, chunk.value
+
+    def fused_ctas(self) -> int:
+        """CTAs that take a pair tile together in the fused backward: 1, or 2 where it runs on pairs of CTAs."""
+        n = int(_lib.libra_plan_fused_ctas(self._h))
+        _check(min(n, 0), "libra_plan_fused_ctas")
+        return n
 
     def busy_times(self, which=KERNEL_FWD):
         w = self.info(LIBRA_DIR_PAIR if which == KERNEL_BWD_FUSED else

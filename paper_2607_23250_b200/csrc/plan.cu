@@ -839,6 +839,12 @@ extern "C" int libra_plan_export_pairs(const libra_plan_t* plan, int32_t* key_bl
     return e == cudaSuccess ? LIBRA_OK : LIBRA_ERR_CUDA;
 }
 
+extern "C" int libra_plan_fused_ctas(const libra_plan_t* plan) {
+    if (!plan) return LIBRA_ERR_INVALID_ARG;
+    if (!plan->dir[2].enabled) return LIBRA_ERR_PLAN_MISMATCH;
+    return plan->dir[4].enabled ? 2 : 1;
+}
+
 extern "C" int libra_plan_destroy(libra_plan_t* plan) {
     if (!plan) return LIBRA_OK;
     int dev = 0;

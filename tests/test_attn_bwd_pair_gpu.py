@@ -1,5 +1,6 @@
 """Fused backward on pairs of CTAs (256-key tiles; pools whose samples average 1024 tokens) against the CPU oracle's
-gradient.  The call and the plan are the fused backward's."""
+gradient.  The call and the plan are the fused backward's; a chunk of more than one row block is asked for where the planner
+would choose a single one for so small a pool, and with it single CTAs."""
 import numpy as np
 import pytest
 import torch
@@ -11,6 +12,48 @@ from test_attn_bwd_fused_gpu import _check, _run
 pytestmark = pytest.mark.gpu
 
 
+def _plan(lengths, hq, hkv, W=0, chunk=0):
+    from paper_2607_23250_b200 import binding as lb
+    return lb.libra_plan_tiles(torch.from_numpy(pools.cu_seqlens(lengths)).cuda(), hq, 256, n_workers=W,
+                               directions=lb.LIBRA_DIR_Q | lb.LIBRA_DIR_PAIR, tile_kv=128, n_heads_kv=hkv, pair_chunk=chunk)
+
+
+def _ctas(lengths, hq, hkv, W=0, chunk=0):
+    plan = _plan(lengths, hq, hkv, W, chunk)
+    n = plan.fused_ctas()
+    plan.destroy()
+    return n
+
+
+def _run_on_pairs(lengths, hq, hkv, W=0, chunk=0, **kw):
+    assert _ctas(lengths, hq, hkv, W, chunk) == 2
+    return _run(lengths, hq, hkv, W=W, chunk=chunk, **kw)
+
+
+@pytest.mark.parametrize("lengths,W,chunk,ctas", [
+    ([1024, 1024], 0, 512, 2), ([1024, 1023], 0, 512, 1),        # the mean length
+    ([1024, 1024, 0], 0, 512, 1),                                # empty samples count
+    ([4000], 0, 0, 2), ([600], 0, 0, 1), ([1100], 0, 0, 1),      # a chunk of one row block, unless it was asked for
+    ([1100], 0, 128, 2),
+    ([4000], 2, 0, 2), ([4000], 1, 0, 1),                        # two workers at least
+])
+def test_which_pools_run_on_pairs(lengths, W, chunk, ctas):
+    plan = _plan(lengths, 8, 2, W, chunk)
+    assert plan.fused_ctas() == ctas
+    if chunk == 0 and len(lengths) == 1 and lengths[0] >= 1024 and W == 0:
+        assert (plan.export_pairs()[2] > 128) == (ctas == 2)
+    plan.destroy()
+
+
+def test_no_form_without_pair_tiles():
+    from paper_2607_23250_b200 import binding as lb
+    plan = lb.libra_plan_tiles(torch.tensor([0, 3000], dtype=torch.int32).cuda(), 2, 256)
+    with pytest.raises(lb.LibraError) as err:
+        plan.fused_ctas()
+    assert err.value.code == lb.ERR_PLAN_MISMATCH
+    plan.destroy()
+
+
 @pytest.mark.parametrize("lengths", [
     [1024],                      # whole key blocks, an even number
     [1100],                      # nine key blocks: the last pair lacks its upper half; a ragged end
@@ -18,9 +61,9 @@ pytestmark = pytest.mark.gpu
     [128 * 9 + 1, 128 * 7 - 1],  # samples that end just past and just before a block's edge
     [2300, 1, 1900, 40],         # short ones between long ones
 ])
-@pytest.mark.parametrize("hq,hkv", [(4, 2), (2, 2), (8, 1)])
-def test_edges_of_the_key_blocks(lengths, hq, hkv):
-    got, ref, cu, _ = _run(lengths, hq, hkv, seed=hq)
+@pytest.mark.parametrize("hq,hkv,chunk", [(4, 2, 256), (2, 2, 512), (8, 1, 512)])
+def test_edges_of_the_key_blocks(lengths, hq, hkv, chunk):
+    got, ref, cu, _ = _run_on_pairs(lengths, hq, hkv, seed=hq, chunk=chunk)
     _check(got, ref, cu)
 
 
@@ -28,19 +71,19 @@ def test_edges_of_the_key_blocks(lengths, hq, hkv):
 def test_query_chunk_sizes(chunk):
     """One row block a chunk makes tiles of which a half sees nothing; an odd number of them lets a chunk begin at the upper
     key block."""
-    got, ref, cu, _ = _run([1500, 1700], 4, 2, seed=1, chunk=chunk)
+    got, ref, cu, _ = _run_on_pairs([1500, 1700], 4, 2, seed=1, chunk=chunk)
     _check(got, ref, cu)
 
 
 @pytest.mark.parametrize("W", [2, 3, 5, 148])
 def test_worker_counts(W):
     """A pair of CTAs for every two workers; an odd one stays idle."""
-    got, ref, cu, _ = _run([1300, 1200], 4, 1, seed=W, W=W)
+    got, ref, cu, _ = _run_on_pairs([1300, 1200], 4, 1, seed=W, W=W, chunk=512)
     _check(got, ref, cu)
 
 
 def test_repeat_agrees_to_rounding():
-    got, ref, cu, again = _run([2500, 1800], 8, 2, seed=9, repeat=True)
+    got, ref, cu, again = _run_on_pairs([2500, 1800], 8, 2, seed=9, repeat=True, chunk=512)
     _check(got, ref, cu)
     for g, a in zip(got, again):
         assert np.abs(g - a).max() <= 2.0 ** -7 * np.abs(g).max()     # one bf16 step of the largest values
@@ -51,8 +94,8 @@ def test_tile_times_cover_every_tile():
     lengths, hq, hkv = [2000, 1200], 4, 2
     cu_np = pools.cu_seqlens(lengths)
     t = pools.make_tensors(int(cu_np[-1]), hq, hkv, 128, seed=5, device="cuda")
-    plan = lb.libra_plan_tiles(torch.from_numpy(cu_np).cuda(), hq, 256, directions=lb.LIBRA_DIR_Q | lb.LIBRA_DIR_PAIR,
-                               tile_kv=128, n_heads_kv=hkv, pair_chunk=512)
+    plan = _plan(lengths, hq, hkv, chunk=512)
+    assert plan.fused_ctas() == 2
     out, lse = lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
     lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan)
     ns, busy = plan.tile_times(lb.KERNEL_BWD_FUSED), plan.busy_times(lb.KERNEL_BWD_FUSED)
@@ -67,8 +110,8 @@ def test_values_that_are_not_finite_stay_in_their_block(value):
     and a key or value that is not finite no row that does not see its block."""
     from paper_2607_23250_b200 import binding as lb
     T, hq, hkv, at = 1100, 2, 1, {"v": 700, "k": 200, "q": 300, "dout": 800}
-    cu = torch.tensor([0, T], dtype=torch.int32).cuda()
-    plan = lb.libra_plan_tiles(cu, hq, 256, directions=lb.LIBRA_DIR_Q | lb.LIBRA_DIR_PAIR, tile_kv=128, n_heads_kv=hkv, pair_chunk=256)
+    plan = _plan([T], hq, hkv, chunk=256)
+    assert plan.fused_ctas() == 2
     clean = pools.make_tensors(T, hq, hkv, 128, seed=3, device="cuda")
     out0, lse0 = lb.libra_attn_pool_fwd(clean["q"], clean["k"], clean["v"], plan)
     for name, row in at.items():
@@ -94,8 +137,8 @@ def test_gives_up_cleanly_when_one_producer_stalls(lengths, W):
     cu_np = pools.cu_seqlens(lengths)
     t = pools.make_tensors(int(cu_np[-1]), hq, hkv, 128, seed=4)
     q, k, v, dout = (t[n].cuda() for n in ("q", "k", "v", "dout"))
-    plan = lb.libra_plan_tiles(torch.from_numpy(cu_np).cuda(), hq, 256, n_workers=W, directions=lb.LIBRA_DIR_Q | lb.LIBRA_DIR_PAIR,
-                               tile_kv=128, n_heads_kv=hkv)
+    plan = _plan(lengths, hq, hkv, W, chunk=512)
+    assert plan.fused_ctas() == 2
     out, lse = lb.libra_attn_pool_fwd(q, k, v, plan)
     plan.set_wait_limit_ns(200_000)
     plan.inject_stall(True)
