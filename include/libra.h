@@ -210,9 +210,10 @@ size_t libra_attn_pool_bwd_workspace_bytes(const libra_plan_t* plan, const libra
  *   kernel that walks the pair-tile lists and computes S, dP, dV, dK and dQ of a cell together (five GEMMs per
  *   cell), and a conversion pass.  dK and dV of a pair tile accumulate on chip and are added to fp32 accumulators
  *   in the workspace when the tile ends; dQ of every cell is added to its fp32 accumulator; all by bulk reduce-adds.
- *   Where samples average 1024 tokens or more (and pair_chunk was given or the chunk chosen is more than one row block) the
- *   kernel runs on pairs of CTAs: a pair takes 256 keys, two neighbouring pair tiles at once, from lists of its own that
- *   Algorithm 2's rule makes from the same cells.
+ *   Where few of the cells of two neighbouring key blocks are live for one of them only (long samples, or short ones beside
+ *   them) the kernel runs on pairs of CTAs: a pair takes 256 keys, two neighbouring pair tiles at once, from lists of its own
+ *   that Algorithm 2's rule makes from the same cells.  Not where an odd worker would cost more than that gains, nor, unless
+ *   pair_chunk was given, on pools of few tiles a worker.  libra_plan_fused_ctas tells.
  *   The accumulators are rounded to bf16 once, at the end, so the result is at least as accurate as the two-kernel
  *   form's, but the order of the floating-point additions varies from run to run: results agree to rounding, not
  *   bit for bit.  The other directions of the plan are not used by this form.

@@ -318,26 +318,31 @@ __device__ __forceinline__ int64_t pair_last_row_block(const int32_t* tok_end, i
 }
 // Chunk sizes under consideration, for the tiles proper and the wide ones: one block each finds the key-block range of
 // every query chunk, the exclusive prefix sum of the counts and their total (base[NC] and totals[block]); one more block
-// for either finds the most live cells of a key block (totals[kPairCands + k]).
+// for either finds the most live cells of a key block (totals[kPairCands + k]) and the sum over all of them
+// (totals[kPairCands + 2 + k]).
 struct PairTables { int dir = 0, kt = 0, R = 0; int32_t* first_j = nullptr; int32_t* count = nullptr; int64_t* base = nullptr; int64_t NC = 0; };
-constexpr int kChunkSizes = 6, kPairCands = 3 * kChunkSizes;
+constexpr int kChunkSizes = 6, kPairCands = 3 * kChunkSizes, kPairTotals = kPairCands + 4;
 struct PairCands { PairTables c[kPairCands]; int n = 0; int rt = 0; int kt[2] = {}; int n_longest = 0; };
 __global__ void __launch_bounds__(1024) k_pair_chunks(const int32_t* __restrict__ tok_end, int64_t T, const __grid_constant__ PairCands cands,
                                                       int64_t* __restrict__ totals) {
     const int rt = cands.rt;
     if ((int)blockIdx.x >= cands.n) {
         __shared__ int longest;
+        __shared__ unsigned long long cells;
         const int k = blockIdx.x - cands.n, kt = cands.kt[k];
-        if (threadIdx.x == 0) longest = 0;
+        if (threadIdx.x == 0) { longest = 0; cells = 0; }
         __syncthreads();
         int most = 0;
+        unsigned long long sum = 0;
         for (int64_t j = threadIdx.x; j * kt < T; j += 1024) {
             const int64_t n = pair_last_row_block(tok_end, T, kt, rt, j) - j * kt / rt + 1;
             most = n > most ? (int)n : most;
+            sum += n;
         }
         atomicMax(&longest, most);
+        atomicAdd(&cells, sum);
         __syncthreads();
-        if (threadIdx.x == 0) totals[kPairCands + k] = longest;
+        if (threadIdx.x == 0) { totals[kPairCands + k] = longest; totals[kPairCands + 2 + k] = (int64_t)cells; }
         return;
     }
     const PairTables& t = cands.c[blockIdx.x];
@@ -511,19 +516,36 @@ static const PairTables* choose_pair_chunk(const libra_plan* p, const PairCands&
     }
     return best;
 }
-// Whether the fused backward runs on pairs of CTAs with 256 keys a tile.
-// From 1024 tokens per sample on, empty ones counted: a pair's cells are 256 keys wide, and where only one of its key blocks sees a
-// row block the other CTA's work is lost.  Fused kernel, 33000 tokens, 32 / 8 heads, on single CTAs and on pairs (us): samples
-// of up to 400 627 and 729, of 512 584 and 581, of 750 902 and 916, of 1024 944 and 927; one sequence of the usual mix of
-// lengths (mean 1200), 8 / 2 heads: 3114 and 2857.
-constexpr int64_t kPairsSample = 1024;
-static bool fused_on_pairs(int64_t T, int n_samples) { return T >= kPairsSample * (int64_t)n_samples; }
+// Whether the fused backward runs on pairs of CTAs with 256 keys a tile, from the live 128 x 128 cells and the 256 x 128 ones.
+// A pair's cell costs it as much where only one of its key blocks sees the row block.  That is so at the diagonal, once a
+// wide key block, and in the row blocks past the end of the lower key block's samples.  Backward on pairs over the same on single
+// CTAs, fitted to 44 pools of 30000 to 131072 tokens (log-normal and equal samples of 300 to 5000, 148 workers): 0.96 + 0.12
+// diagonal + 0.65 past ends, as shares of the live cells; to 44 of 8200 to 33000 on 16 workers 0.93 + 0.66 + 0.83.  The line lies
+// between the two.  Some of the pools, single / pairs in us with 148 workers, 32 / 8 or 8 / 2 heads: 20 samples of the usual
+// log-normal mix in 33000 tokens 6192 / 5732 at past ends + 0.4 diagonal = 0.009, 32 of 1024 1319 / 1263 (0.044), 43 of 3000 2764 /
+// 2738 (0.050), log-normal of median 500 2760 / 2755 (0.059); and beyond the line 62 of 2100 2187 / 2223 (0.071), 119 of 1100
+// 1489 / 1564 (0.121), 204 of 640 1051 / 1124 (0.233).
+// An odd worker has no CTA to pair with, and with it goes the balance of longer lists: 4096 tokens, 8 / 2 heads, on 7, 9, 13, 37, 63 and
+// 147 workers: single / pairs 0.92, 0.94, 0.95, 0.98, 1.01, 1.04; 16384 tokens on 9, 37, 147: 0.98, 1.05, 1.06.
+// Of a pool with few tiles a worker the launch counts and the coarser tiles leave more of the last round idle, as far as the
+// chunk was the planner's to choose: 1500 tokens, 8 / 2 heads, a chunk of one row block: 40.2 us on single CTAs and 42.8 on pairs; 1500,
+// 32 / 8 heads, 2.3 tiles a worker: 91.7 and 100.0; 3000, 8 / 2 heads, 2.1: 91.0 and 102.8; 9 samples of 1024, 2.4: 115.6 and 109.0; 4096, 3.7:
+// 115.1 and 110.8.
+static bool fused_on_pairs(const libra_plan* p, int64_t cells, int64_t wide_cells, int64_t wide_tiles, int R, bool own_choice) {
+    const int64_t wide_blocks = (p->T + 255) / 256;
+    const double past_ends = (double)(2 * wide_cells - cells - wide_blocks) / cells, diagonal = (double)wide_blocks / cells;
+    const double cost = 0.94 + past_ends + 0.4 * diagonal + (p->W % 2 ? 2.0 / p->W : 0.0);
+    if (cost >= 1.0) return false;
+    return !own_choice || (R > 1 && wide_tiles * p->dir[4].H >= 2.4 * p->dir[4].W);
+}
 static double heads_per_kv(const libra_plan* p) { return p->dir[0].H > p->dir[2].H ? (double)p->dir[0].H / p->dir[2].H : 1.0; }
-// Counts, choice and, while every size has more than 262144 pair-blocks, twice the largest.
-static int count_pair_blocks(libra_plan* p, PairCands& cands, int64_t* d_totals, PairTables (&chosen)[libra_plan::kDirs], double G) {
+// Counts, choice and, while every size has more than 262144 pair-blocks, twice the largest.  `pairs`: whether the fused kernel's
+// wide tiles are under consideration, and whether they were taken.
+static int count_pair_blocks(libra_plan* p, PairCands& cands, int64_t* d_totals, PairTables (&chosen)[libra_plan::kDirs], double G,
+                             bool own_choice, bool& pairs) {
     const int dirs = cands.n_longest;
     for (;;) {
-        int64_t totals[kPairCands + 2];
+        int64_t totals[kPairTotals];
         k_pair_chunks<<<cands.n + dirs, 1024, 0, p->stream>>>(p->d_tok_end, p->T, cands, d_totals);
         count_launch();
         if (cudaMemcpyAsync(totals, d_totals, sizeof(totals), cudaMemcpyDeviceToHost, p->stream) != cudaSuccess ||
@@ -548,12 +570,13 @@ static int count_pair_blocks(libra_plan* p, PairCands& cands, int64_t* d_totals,
             }
         }
         if (!all) continue;
-        for (int x = 0; x < cands.n; ++x)   // the fused kernel's wide tiles have the chunks of the others
+        for (int x = 0; x < cands.n && pairs; ++x)   // the fused kernel's wide tiles have the chunks of the others
             if (cands.c[x].dir == 4 && cands.c[x].R == chosen[2].R) {
                 p->dir[4].NB = totals[x];
                 p->dir[4].chunk = p->dir[2].chunk;
                 chosen[4] = cands.c[x];
             }
+        if (pairs) pairs = fused_on_pairs(p, totals[kPairCands + 2], totals[kPairCands + 3], p->dir[4].NB, chosen[2].R, own_choice);
         return LIBRA_OK;
     }
 }
@@ -597,7 +620,7 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
         for (int k = 0; k < kDirs; ++k)
             if (sorted[k]) carve_dir(p->dir[k], c, false, false);
         if (want[2]) {
-            c.take(&d_totals, kPairCands + 2);
+            c.take(&d_totals, kPairTotals);
             for (int x = 0; x < cands.n; ++x) {
                 PairTables& t = cands.c[x];
                 c.take(&t.first_j, t.NC);
@@ -616,10 +639,8 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
     count_launch();
     // ---- pair tiles: their number comes back, then their arrays
     if (want[2]) {
-        if (const int rc = count_pair_blocks(p, cands, d_totals, chosen, heads_per_kv(p)); rc != LIBRA_OK) return rc;
-        // (Of a pool so small that a chunk is one row block the launch counts, and pairs of CTAs take longer to get going: backward
-        // of 1500 tokens, 8 / 2 heads, 40.2 us on single ones and 42.8 on pairs; of 4000, chunks of two row blocks, 133 and 114.)
-        if (o.pair_chunk == 0 && chosen[2].R == 1) pairs[4] = false;
+        if (const int rc = count_pair_blocks(p, cands, d_totals, chosen, heads_per_kv(p), o.pair_chunk == 0, pairs[4]); rc != LIBRA_OK)
+            return rc;
         Carver ps, pm;
         size_t pair_zero = 0;
         for (int k = 2; k < kDirs; ++k) {
@@ -731,7 +752,7 @@ extern "C" int libra_plan_tiles(const int32_t* cu_seqlens_dev, int n_samples, in
     const bool keys = (dirs & (LIBRA_DIR_KV | LIBRA_DIR_PAIR)) != 0;
     const bool want[libra_plan::kDirs] = {(dirs & LIBRA_DIR_Q) != 0, (dirs & LIBRA_DIR_KV) != 0, (dirs & LIBRA_DIR_PAIR) != 0,
                                           keys && tile_kv == 128,
-                                          (dirs & LIBRA_DIR_PAIR) != 0 && tile_kv == 128 && p->W >= 2 && fused_on_pairs(T, n_samples)};
+                                          (dirs & LIBRA_DIR_PAIR) != 0 && tile_kv == 128 && p->W >= 2};
     for (int k = 0; k < libra_plan::kDirs; ++k) {
         PlanDir& d = p->dir[k];
         d.tile = k == 0 ? tile_q : (k >= 3 ? 256 : tile_kv);
