@@ -780,8 +780,8 @@ extern "C" int libra_tap_plan(const int32_t* cu_seqlens_dev, int n_samples, cons
         return LIBRA_ERR_INVALID_ARG;
     if (!((o->n_shards <= o->hkv && o->hkv % o->n_shards == 0) || (o->n_shards > o->hkv && o->n_shards % o->hkv == 0)))
         return LIBRA_ERR_INVALID_ARG;
+    if ((int64_t)n_sequences * o->cp > kTapMaxWorkers) return LIBRA_ERR_UNSUPPORTED;
     const int P = n_sequences, W = P * o->cp, H = o->n_shards;
-    if (W > kTapMaxWorkers || P > kTapMaxWorkers) return LIBRA_ERR_UNSUPPORTED;
     const int64_t NT = libra_tap_num_tiles(seq_offsets_host, P, o->block, H);
     if (NT <= 0) return LIBRA_ERR_INVALID_ARG;
     const int64_t NB = NT / H;
@@ -858,8 +858,8 @@ extern "C" int libra_tap_schedule(const int32_t* cu_seqlens_dev, int n_samples, 
     if (n_samples <= 0 || n_sequences <= 0 || o->cp <= 0 || o->block <= 0 || o->n_shards <= 0 || o->hq <= 0 ||
         o->hkv <= 0 || o->head_dim <= 0 || o->hq % o->n_shards != 0)
         return LIBRA_ERR_INVALID_ARG;
+    if ((int64_t)n_sequences * o->cp > kTapMaxWorkers) return LIBRA_ERR_UNSUPPORTED;
     const int P = n_sequences, W = P * o->cp, H = o->n_shards;
-    if (W > kTapMaxWorkers || P > kTapMaxWorkers) return LIBRA_ERR_UNSUPPORTED;
     const int64_t NT = libra_tap_num_tiles(seq_offsets_host, P, o->block, H);
     if (NT <= 0) return LIBRA_ERR_INVALID_ARG;
     const int64_t NB = NT / H, NG = (int64_t)n_samples * H;

@@ -42,6 +42,18 @@ def test_strerror_and_argument_checks_without_a_device():
     assert lib.libra_launch_count() >= 0
 
 
+def test_pool_planner_refuses_worker_counts_beyond_32_bits():
+    """4 x 2^30 workers wrap to 0 in 32 bits; refused before any CUDA call, like every count above 1024."""
+    from paper_2607_23250_b200 import build
+    lib = ctypes.CDLL(build.build())
+    seq = (ctypes.c_int32 * 5)(0, 8, 16, 24, 32)
+    some = ctypes.c_void_p(256)            # never dereferenced
+    for cp in (1 << 30, 1 << 29, 257):
+        opts = (ctypes.c_int * 8)(cp, 16, 1, 2, 1, 8, 3, 100)
+        assert lib.libra_tap_plan(some, 4, seq, 4, opts, *[some] * 6, None) == -2, cp
+        assert lib.libra_tap_schedule(some, 4, seq, 4, opts, some, some, ctypes.c_int64(1), some, None) == -2, cp
+
+
 def test_binding_names_match_header():
     src = open(os.path.join(ROOT, "paper_2607_23250_b200", "binding.py")).read()
     for name in _declared():
