@@ -653,7 +653,10 @@ namespace libra {
 // indices are 32-bit.  us with 64-bit ones and a round, with a round, two and four (GB/s): 524288 tokens, 32 / 8 heads of 128,
 // accumulators cleared, 4322, 3677, 3518 and 3499 (6200); 131072 of them 941, 857, 846, 841 (6450); 32768: 237, 214, 216, 221; 10007, 8
 // / 2 heads: 25.7, 25.8, 25.4, 29.8; 65536 tokens, 32 heads, nothing to clear: 247, 225, 208, 193 (5700).  Hence four where
-// there are seven waves of the warps that fit all the same.
+// there are seven waves of the warps that fit all the same.  Whole backward with a round and with two where two leave SMs without a
+// reading CTA: 1500 tokens, 4 heads of 64: 34.1 and 35.2 us (12 CTAs with two); 4096: 72.0 and 73.8 (32); 8 heads: 114.9 and 115.8
+// (64); 16384 tokens, 4 heads: 161.7 and 163.0 (128).  And where they do not: 4096 tokens, 32 heads of 128: 451 and 450; 16384, 8 heads
+// of 64: the statistics 14.7 and 12.7.
 constexpr int kClearPerThread = 16;
 template <int D>
 constexpr int kPrepRows = 8 * 256 / D;
@@ -790,9 +793,9 @@ static int launch_bwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtens
 // Row statistics; `clear` (16-byte words) is zeroed on the way: one pass over memory less to launch.
 template <int D>
 static cudaError_t launch_prep(const void* out, const void* dout, const float* lse, int64_t T, int64_t Tpad, int hq, float* dvec,
-                               float* lse2, float* clear, size_t clear_bytes, cudaStream_t s) {
-    const int64_t n_clear = (int64_t)(clear_bytes / 16);
-    const int rounds = Tpad / kPrepRows<D> * hq >= 4 * kPrepManyWarps ? 4 : 2;
+                               float* lse2, float* clear, size_t clear_bytes, int sms, cudaStream_t s) {
+    const int64_t n_clear = (int64_t)(clear_bytes / 16), runs = Tpad / kPrepRows<D> * hq;
+    const int rounds = runs >= 4 * kPrepManyWarps ? 4 : (runs > 2 * 8 * ((int64_t)sms - 1) ? 2 : 1);
     static_assert(128 % (4 * kPrepRows<D>) == 0, "rounds of a warp");
     const int64_t readers = (Tpad / kPrepRows<D> / rounds * hq + 7) / 8, clearers = (n_clear + 256 * kClearPerThread - 1) / (256 * kClearPerThread);
     const int64_t rare = clearers < readers ? clearers : readers, usual = clearers + readers - rare;
@@ -967,7 +970,7 @@ extern "C" int libra_attn_pool_bwd(const void* q_dev, const void* k_dev, const v
             dv_acc = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace_dev) + 2 * ws.stat_bytes + ws.dkv_acc_bytes);
         }
         const cudaError_t e256 = launch_prep<256>(out_dev, dout_dev, lse_dev, T, ws.Tpad, dims->hq, dvec, lse2, dk_acc,
-                                                  fused ? 2 * ws.dkv_acc_bytes : 0, s);
+                                                  fused ? 2 * ws.dkv_acc_bytes : 0, plan->sm_count, s);
         time_end(mp256, 3, s);
         if (e256 != cudaSuccess) return LIBRA_ERR_CUDA;
         mp256->bwd_mask = 2 | 4 | 8;
@@ -995,8 +998,8 @@ extern "C" int libra_attn_pool_bwd(const void* q_dev, const void* k_dev, const v
     {
         float* acc = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace_dev) + 2 * ws.stat_bytes);
         const size_t acc_bytes = fused ? ws.dq_acc_bytes + 2 * ws.dkv_acc_bytes : 0;   // the three accumulators are contiguous
-        const cudaError_t e = D == 128 ? launch_prep<128>(out_dev, dout_dev, lse_dev, T, ws.Tpad, dims->hq, dvec, lse2, acc, acc_bytes, s)
-                                       : launch_prep<64>(out_dev, dout_dev, lse_dev, T, ws.Tpad, dims->hq, dvec, lse2, acc, acc_bytes, s);
+        const cudaError_t e = D == 128 ? launch_prep<128>(out_dev, dout_dev, lse_dev, T, ws.Tpad, dims->hq, dvec, lse2, acc, acc_bytes, plan->sm_count, s)
+                                       : launch_prep<64>(out_dev, dout_dev, lse_dev, T, ws.Tpad, dims->hq, dvec, lse2, acc, acc_bytes, plan->sm_count, s);
         if (e != cudaSuccess) return LIBRA_ERR_CUDA;
     }
     time_end(mp0, 3, s);

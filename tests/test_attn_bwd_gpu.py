@@ -92,6 +92,14 @@ def test_tiles_shared_by_a_cluster(lengths, hq, hkv, d):
         assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("d,hq,hkv", [(64, 8, 2), (128, 4, 1)])
+@pytest.mark.parametrize("T", [9400, 9409])
+def test_rounds_of_the_row_statistics(T, d, hq, hkv):
+    """The last pool whose warps take one run of rows each on 148 SMs, and the first whose take two."""
+    got, ref, cu = _run(pools.random_layout(np.random.default_rng(T), T, 70), hq, hkv, d, seed=T)
+    _check(got, ref, cu)
+
+
 def test_peaked_softmax():
     got, ref, cu = _run([700, 900], 2, 2, 64, seed=4, qscale=4.0)
     _check(got, ref, cu)
