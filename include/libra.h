@@ -142,7 +142,9 @@ int libra_plan_status(const libra_plan_t* plan);
 /* Copies one direction of the plan to caller-allocated HOST arrays (any may be NULL):
  * weight int64[n_tiles], order int32[n_tiles], cta_of_tile int32[n_tiles],
  * cta_offsets int32[n_workers+1], cta_tiles int32[n_tiles], loads int64[n_workers].
- * Synchronises the plan's stream. */
+ * Synchronises the plan's stream.  LIBRA_DIR_PAIR: of a plan whose fused backward runs on pairs of CTAs
+ * (libra_plan_fused_ctas) this is the placement of the 128-key tiles on single workers, which that kernel does not follow:
+ * it walks lists of 256-key tiles of its own.  Nor do the kernels at head_dim 256. */
 int libra_plan_export(const libra_plan_t* plan, int direction, int64_t* weight_host,
                       int32_t* order_host, int32_t* cta_of_tile_host, int32_t* cta_offsets_host,
                       int32_t* cta_tiles_host, int64_t* loads_host);
@@ -353,7 +355,8 @@ int libra_tap_schedule(const int32_t* cu_seqlens_dev, int n_samples, const int32
  * Per-CTA busy time of the most recent launch of kernel `which` (LIBRA_KERNEL_*) that used this
  * plan: nanoseconds between the CTA starting and finishing its tile list, read with the GPU's
  * global timer.  Copies n_workers values to ns_host (0 for workers that the launch had no CTA for) and
- * synchronises the device.  Returns the
+ * synchronises the device.  Entry r is the CTA that walks list r of libra_plan_export; of a fused backward on pairs of CTAs,
+ * pair p, with list p of its own, is entries p and p + n_workers / 2.  Returns the
  * status of the most recent forward (LIBRA_KERNEL_FWD) or backward (the other two) launch:
  * LIBRA_OK, LIBRA_ERR_TIMEOUT if a bounded wait gave up, or the plan's own status (libra_plan_status) when that is
  * not OK and the kernels therefore did no work. */

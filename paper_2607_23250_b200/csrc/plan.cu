@@ -581,6 +581,13 @@ static int count_pair_blocks(libra_plan* p, PairCands& cands, int64_t* d_totals,
     }
 }
 
+// Placement and lists of n directions, side by side.
+static void place_lists(const DirViews& views, int n, int max_w, int64_t max_nt, cudaStream_t s) {
+    k_place<<<n, (max_w + 31) / 32 * 32, 0, s>>>(views);
+    k_scatter_lists<<<dim3(grid_for(max_nt > 0 ? max_nt : 1, 256), n), 256, 0, s>>>(views);
+    count_launch(2);
+}
+
 // Builds the directions asked for; p->dir[k].tile / H / W / chunk are set.
 static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o, const bool (&want)[libra_plan::kDirs]) {
     constexpr int kDirs = libra_plan::kDirs;
@@ -684,17 +691,18 @@ static int build_plan(libra_plan* p, const int32_t* cu, const libra_plan_opts& o
         count_launch(2);
     }
     const int n_sorted = n;
+    // No kernel walks the lists of the 128-key pair tiles where the fused backward has its wide ones: they are made when they
+    // are exported.
+    const bool listed[kDirs] = {sorted[0], sorted[1], pairs[2] && !pairs[4], sorted[3] || pairs[3], pairs[4]};
     for (int k = 2; k < kDirs; ++k)
-        if (pairs[k]) views.v[n++] = view_of(p->dir[k], 1, o);
+        if (listed[k] && !sorted[k]) views.v[n++] = view_of(p->dir[k], 1, o);
     if (n == 0) return LIBRA_OK;
     for (int k = 0; k < kDirs; ++k)
-        if (sorted[k] || pairs[k]) {
+        if (listed[k]) {
             max_nt = p->dir[k].NT > max_nt ? p->dir[k].NT : max_nt;
             max_w = p->dir[k].W > max_w ? p->dir[k].W : max_w;
         }
-    k_place<<<n, (max_w + 31) / 32 * 32, 0, s>>>(views);   // the directions' placements side by side
-    k_scatter_lists<<<dim3(grid_for(max_nt > 0 ? max_nt : 1, 256), n), 256, 0, s>>>(views);
-    count_launch(2);
+    place_lists(views, n, max_w, max_nt, s);
     if (n_sorted > 0) {
         k_exec_order<<<dim3(max_w, n_sorted), 256, 0, s>>>(views);
         count_launch();
@@ -820,6 +828,13 @@ extern "C" int libra_plan_export(const libra_plan_t* plan, int direction, int64_
     void* tmp = nullptr;
     if (weight_host || order_host) ok(cudaMalloc(&tmp, sizeof(int64_t) * (d->NT ? d->NT : 1)));
     if (e != cudaSuccess) return LIBRA_ERR_CUDA;
+    // Pair tiles whose lists no kernel walks: made here, the same ones at every call.
+    if (d == &plan->dir[2] && plan->dir[4].enabled && (cta_of_tile_host || cta_offsets_host || cta_tiles_host || loads_host)) {
+        DirViews views = {};
+        views.v[0] = view_of(*d, 1, libra_plan_opts{});
+        place_lists(views, 1, d->W, d->NT, s);
+        ok(cudaGetLastError());
+    }
     if (weight_host) {
         k_expand_weight<<<grid_for(d->NT, 256), 256, 0, s>>>(d->d_weight_blk, d->NT, d->H, d->d_u_blk ? d->NB : 0,
                                                              (int64_t*)tmp);

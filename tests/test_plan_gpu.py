@@ -137,6 +137,33 @@ def _compare_pairs(cu_np, H_kv, tile_kv, chunk, W):
     return chunk_used
 
 
+@pytest.mark.parametrize("chunk", [0, 512])
+def test_pair_lists_that_no_kernel_walks(chunk):
+    """Where the fused backward runs on pairs of CTAs the placement of the 128-key tiles is made by the export: the same at
+    every call, with any of the arrays left out, and of no effect on the passes."""
+    import ctypes
+    from paper_2607_23250_b200 import binding as lb
+    cu_np = np.array([0, 3100, 6900], np.int32)
+    t = pools.make_tensors(6900, 4, 2, 128, seed=1, device="cuda")
+    plan = lb.libra_plan_tiles(torch.from_numpy(cu_np).cuda(), 4, 256, directions=lb.LIBRA_DIR_Q | lb.LIBRA_DIR_PAIR, tile_kv=128,
+                               n_heads_kv=2, pair_chunk=chunk)
+    assert plan.fused_ctas() == 2
+    out, lse = lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
+    before = lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan)
+    want = oracle.plan_pairs(cu_np, 2, 128, plan.export_pairs()[2], 148)
+    loads = np.zeros(148, np.int64)
+    assert lb._lib.libra_plan_export(plan._h, lb.LIBRA_DIR_PAIR, None, None, None, None, None, ctypes.c_void_p(loads.ctypes.data)) == 0
+    assert np.array_equal(loads, want["loads"])
+    for _ in range(2):
+        got = plan.export(lb.LIBRA_DIR_PAIR)
+        for k in KEYS:
+            assert np.array_equal(got[k], want[k]), k
+    after = lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan)
+    for a, b in zip(after, before):
+        assert float((a.float() - b.float()).abs().max()) <= 2.0 ** -7 * float(b.float().abs().max())
+    plan.destroy()
+
+
 def test_pair_tiles_hand_example():
     _compare_pairs(np.array([0, 5, 6, 16], dtype=np.int32), 1, 4, 8, 2)
 
