@@ -363,10 +363,10 @@ int libra_tap_schedule(const int32_t* cu_seqlens_dev, int n_samples, const int32
 int libra_busy_times(const libra_plan_t* plan, int which, uint64_t* ns_host);
 
 /* Time each tile took in the most recent launch of the forward kernel (which = LIBRA_KERNEL_FWD, tiles of the
- * query-major direction) or of the fused backward kernel (LIBRA_KERNEL_BWD_FUSED, pair tiles; of two that a pair of CTAs
- * takes together, each gets the time of both): nanoseconds of the
+ * query-major direction) or of the fused backward kernel (LIBRA_KERNEL_BWD_FUSED, pair tiles): nanoseconds of the
  * global timer from the moment a compute thread of the CTA turns to the tile until it has finished the tile's
- * last output, indexed by tile id; 0 for a tile that was not run.  With the plan's weights (libra_plan_export)
+ * last output, indexed by tile id; 0 for a tile that was not run.  Of two pair tiles that a pair of CTAs takes together, each
+ * gets the share of that time that its live cells are of the row blocks the pair goes through.  With the plan's weights (libra_plan_export)
  * this shows how well the tile weight predicts time: the paper notes that a FLOPs-balanced assignment need not
  * be time-balanced (Section 3.2).  Copies n_tiles values to ns_host (HOST) and synchronises the device.
  * Errors: INVALID_ARG (another kernel id), PLAN_MISMATCH (the plan lacks the direction), CUDA. */

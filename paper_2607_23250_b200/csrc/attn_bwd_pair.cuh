@@ -110,6 +110,12 @@ struct PairUnit {
     int kvh, c, j0, i0, n_blk;
     int last0;                // last row block that sees the lower key block
     bool two;                 // the upper key block exists
+    // row blocks of it that see key block j0 + r
+    __device__ __forceinline__ int seen(uint32_t r) const {
+        const int end = i0 + n_blk;
+        if (r == 0) return (last0 < end ? last0 + 1 : end) - i0;
+        return two ? end - (i0 > j0 ? i0 : j0 + 1) : 0;
+    }
     // bit r: row block i sees key block j0 + r
     __device__ __forceinline__ uint32_t see(int i) const { return (i <= last0 ? 1u : 0u) | (two && i > j0 ? 2u : 0u); }
 };
@@ -632,8 +638,8 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             if (!ok) break;
             tc_fence_after();
             // of a query chunk's row blocks this CTA's keys may have seen none
-            const bool any = rank == 0 ? u.i0 <= u.last0 : u.two && u.i0 + u.n_blk - 1 > u.j0;
-            if (any) {
+            const int seen = u.seen(rank);
+            if (seen > 0) {
 #pragma unroll 1
                 for (int c = 0; c < 4; ++c) {
                     uint32_t v[32];
@@ -647,8 +653,8 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             tc_fence_before();
             __syncwarp();
             if (lane < 2) mbar_arrive_cluster(map_to_rank(&bars[L::kDkvEmpty], (uint32_t)lane));
-            if (threadIdx.x == 0 && any)
-                p.tile_ns[u.kvh * p.NU128 + p.base[u.c] + u.j0 + rank - p.first_j[u.c]] = (uint32_t)(globaltimer_ns() - tile_t0);
+            if (threadIdx.x == 0 && seen > 0)   // of the time of both halves the part in which this one had work
+                p.tile_ns[u.kvh * p.NU128 + p.base[u.c] + u.j0 + rank - p.first_j[u.c]] = (uint32_t)((globaltimer_ns() - tile_t0) * seen / u.n_blk);
         }
         // every bulk reduce this warp issued has completed before the CTA leaves
         if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");

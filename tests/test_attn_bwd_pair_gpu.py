@@ -103,6 +103,15 @@ def test_tile_times_cover_every_tile():
     ns, busy = plan.tile_times(lb.KERNEL_BWD_FUSED), plan.busy_times(lb.KERNEL_BWD_FUSED)
     assert len(ns) == plan.info(lb.LIBRA_DIR_PAIR)["n_tiles"] and (ns > 0).all()
     assert int(ns.max()) <= int(busy.max()) and int(ns.astype(np.int64).sum()) <= int(busy.astype(np.int64).sum())
+    # two neighbouring key blocks of a chunk share the pair's time by their live cells
+    kb, qc, _ = plan.export_pairs()
+    cells, compared = plan.export(lb.LIBRA_DIR_PAIR)["weight"], 0
+    for u in range(len(kb) - 1):
+        if kb[u] % 2 == 0 and kb[u + 1] == kb[u] + 1 and qc[u + 1] == qc[u] and cells[u] != cells[u + 1]:
+            a, b = ns[u] / cells[u], ns[u + 1] / cells[u + 1]
+            assert abs(a - b) <= 0.15 * max(a, b), (u, ns[u], ns[u + 1], cells[u], cells[u + 1])   # (each CTA reads its own clock)
+            compared += 1
+    assert compared >= 8
     plan.destroy()
 
 
