@@ -377,7 +377,7 @@ int libra_tile_times(const libra_plan_t* plan, int which, uint32_t* ns_host);
  * is bounded: a wait that outlives the budget makes its CTA stop issuing work, let the copies and
  * MMAs it has in flight finish, free its tensor memory and return, and the launch reports
  * LIBRA_ERR_TIMEOUT through libra_busy_times.  (In the fused backward one warp watches the clock for all waits of a CTA: the
- * budget is for the time without a new 128-row query block.)  A healthy run never comes near the default. */
+ * budget is for the time in which neither a new 128-row query block is begun nor the last products of a tile end.)  A healthy run never comes near the default. */
 int libra_plan_set_wait_limit_ns(libra_plan_t* plan, uint64_t ns);
 
 /* Test aid (no counterpart in the paper): while enabled, the producer role of the attention kernels launched

@@ -182,7 +182,7 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     uint64_t* bar_drain = b2 + 13;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kMiscOff);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::kMiscOff + 4);
-    volatile uint32_t* progress = reinterpret_cast<volatile uint32_t*>(smem + L::kMiscOff + 12);   // iterations begun by the first exp warp
+    volatile uint32_t* progress = reinterpret_cast<volatile uint32_t*>(smem + L::kMiscOff + 12);   // iterations begun and units finished by the first exp warp
     uint32_t* finished = reinterpret_cast<uint32_t*>(smem + L::kMiscOff + 16);                     // warps whose role is over
 
     const int warp = threadIdx.x >> 5;
@@ -525,7 +525,7 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             for (int it = 0, i = 0; it < n_it && ok; ++it, ++it_all) {
                 const int qb = (u.i0 + i) * kBlk;
                 if (++i == u.n_blk) i = 0;
-                if (threadIdx.x == 0) *progress = it_all + 1;
+                if (threadIdx.x == 0) *progress = it_all + ucnt + 1;
                 const uint32_t qs = it_all % QS;
                 const float* lse2 = reinterpret_cast<const float*>(smem + L::kLseOff + qs * 512) + c0;
                 const bool need_mask = (qb == u.k0) || (qb + kBlk - 1 >= min_kend) || partial;
@@ -585,6 +585,7 @@ k_attn_bwd_fused(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             // ---- unit epilogue: dK and dV of the pair tile are added to the fp32 accumulators ----
             ok = watched_warp_wait(bar_dkvfull, (ucnt - 1) & 1, abort_flag);
             if (!ok) break;
+            if (threadIdx.x == 0) *progress = it_all + ucnt;
             tc_fence_after();
             // through the shared-memory dS^T tile, which dQ has read, like dQ: bulk reduce-adds of 32 key rows x 32 head-dim
             // columns (rows past the end of the pool are dropped by the hardware)

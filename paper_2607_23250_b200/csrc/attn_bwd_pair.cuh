@@ -168,7 +168,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     volatile uint32_t* issued = peer_gave_up + 1;   // [2][kPairLoads] leader: loads of each kind that either CTA has issued
     volatile uint32_t* sent = issued + 2 * kPairLoads;   // [4] copies of dS that each dS warp of the other CTA has issued
     volatile uint32_t* taken = sent + 4;            // iterations whose copies have arrived; [1] whether the next was expected
-    volatile uint32_t* progress = taken + 2;        // iterations begun by the first exp warp
+    volatile uint32_t* progress = taken + 2;        // iterations begun and units finished by the first exp warp
     uint32_t* finished = const_cast<uint32_t*>(progress) + 1;   // warps whose role is over
 
     const int warp = threadIdx.x >> 5;
@@ -231,7 +231,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const int G = p.hq / p.hkv;
 
     if (warp == kPrWatchWarp) {
-        // ---------------- the clock of all waits: no iteration has begun for the budget of one, so the CTA gives up ----------------
+        // ------- the clock of all waits: no iteration has begun and no unit's products have ended for the budget of one -------
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPrRegsOther));
         if (elect_one()) watch_progress(progress, finished, kPairThreads / 32 - 1, p.wait_limit_ns, abort_flag);
         __syncwarp();
@@ -580,7 +580,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             for (int it = 0, i = 0; it < n_it && ok; ++it, ++n) {
                 const int qb = (u.i0 + i) * kBlk;
                 if (++i == u.n_blk) i = 0;
-                if (threadIdx.x == 0) *progress = n + 1;
+                if (threadIdx.x == 0) *progress = n + ucnt + 1;
                 const float* lse2 = reinterpret_cast<const float*>(smem + L::kLseOff + (n & 1) * 512) + c0;
                 const bool need_mask = (qb <= k0) || (qb + kBlk - 1 >= min_kend) || partial;
                 const int j_lo = (int)(key - qb) - c0;
@@ -636,6 +636,7 @@ k_attn_bwd_pair(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             // read it) and bulk reduce-adds of 32 key rows x 32 head-dim columns ----
             ok = watched_warp_wait(&bars[L::kDkvFull], (ucnt - 1) & 1, abort_flag);
             if (!ok) break;
+            if (threadIdx.x == 0) *progress = n + ucnt;
             tc_fence_after();
             // of a query chunk's row blocks this CTA's keys may have seen none
             const int seen = u.seen(rank);
