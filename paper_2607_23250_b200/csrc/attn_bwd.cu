@@ -21,7 +21,8 @@
 // region X: it is free again as soon as the compute groups have READ it, not when the MMA that consumes the
 // bf16 result has run, so dP^T(it) is issued right after S^T(it) has been read and S^T(it+1) right after
 // dP^T(it) has been read, while dV(it) and dK(it) read P^T / dS^T from their own columns.
-// P^T is handed to the dV MMA in two halves, so half of dV(it) runs under the second half's exponentials.
+// P^T is handed to the dS group in two halves, so it works on the first under the second half's exponentials; dV(it) waits
+// for both.
 // dQ kernel (attn_bwd_dq.cuh): a unit is 128 query rows x one head; Q and dO are copied once per unit from
 // shared memory into TMEM, dQ accumulates in TMEM, the CTA streams the key blocks the rows see (as the
 // forward does).  Queries sit in TMEM lanes:
@@ -892,7 +893,6 @@ static int launch_fused(const void* q_dev, const void* k_dev, const void* v_dev,
             cfg_mark(4);
         }
         FusedParams fp;
-        fp.dq_acc = dq_acc; fp.dk_acc = dk_acc; fp.dv_acc = dv_acc;
         fp.lse2 = lse2; fp.dvec = dvec;
         fp.cta_offsets = d.d_cta_offsets; fp.cta_tiles = d.d_cta_exec;
         fp.u_blk = d.d_u_blk; fp.u_chunk = d.d_u_chunk; fp.tok_end = plan->d_tok_end;

@@ -56,9 +56,6 @@ struct FusedSmem {
 };
 
 struct FusedParams {
-    float* dq_acc;      // [T, Hq, 128]   fp32, zero on entry
-    float* dk_acc;      // [T, Hkv, 128]  fp32, zero on entry
-    float* dv_acc;
     const float* lse2;  // [Hq, Tpad]  LSE * log2(e)
     const float* dvec;  // [Hq, Tpad]  D_i
     const int32_t* cta_offsets;

@@ -3,8 +3,9 @@
 //
 // What bounds the kernel of one CTA is the bandwidth of shared memory: of a 128 x 128 cell its MMAs read 256 KB (S and dP
 // 64 each, dQ 64, dV and dK 32), the copies of Q and dO write 64, dS^T 32, and dQ goes in and out of its staging tile,
-// 128 KB: 480 KB or 3750 clk for 2560 of MMA, and 5350 in all.  A pair halves every B operand and adds the two key blocks'
-// dQ up before it leaves: 384 KB a cell, 4140 clk in all, and half the reduce-adds in L2, which cost the most power.
+// 128 KB: 480 KB, 3840 clk at 128 bytes a clk, for 2560 of MMA, and 5350 in all.  A pair halves every B operand and adds the
+// two key blocks' dQ up before it leaves: 384 KB or 3072 clk a cell, 4140 in all, which is at neither limit, and half the
+// reduce-adds in L2, which cost the most power.
 //
 // CTA c of a pair has key block 2 J + c in its TMEM lanes and owns K and V of it.  Of what the GEMMs multiply with it holds
 //   Qr, dOr  rows 64 c .. 64 c + 63 of the query block, all columns    (B of S^T and dP^T, N = queries)

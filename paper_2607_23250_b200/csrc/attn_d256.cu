@@ -418,16 +418,16 @@ k_attn_d256(const __grid_constant__ CUtensorMap tm_sa, const __grid_constant__ C
                                 mma_ts_pair(tmem_base + kColAcc, tmem_base + L::col_w(b, kk), sdesc_advance(db, kk * 2048), idesc_acc,
                                             (begun || kk > 0) ? 1u : 0u);
                         } else if (see == 3) {   // a CTA's first product overwrites; these two did not begin with the same block
-                            mma_ts_pair_one(tmem_base + kColAcc, t_w, db, idesc_acc, 1, adds - 1);
-                            mma_ts_pair_one(tmem_base + kColAcc, t_w, db, idesc_acc, 0, 2 - adds);
+                            mma_ts_pair_of(tmem_base + kColAcc, t_w, db, idesc_acc, 1, adds);
+                            mma_ts_pair_of(tmem_base + kColAcc, t_w, db, idesc_acc, 0, 3 - adds);
 #pragma unroll
                             for (int kk = 1; kk < kBlk / 16; ++kk)
                                 mma_ts_pair(tmem_base + kColAcc, tmem_base + L::col_w(b, kk), sdesc_advance(db, kk * 2048), idesc_acc, 1);
                         } else if (see) {
 #pragma unroll
                             for (int kk = 0; kk < kBlk / 16; ++kk)
-                                mma_ts_pair_one(tmem_base + kColAcc, tmem_base + L::col_w(b, kk), sdesc_advance(db, kk * 2048), idesc_acc,
-                                                (adds || kk > 0) ? 1u : 0u, see - 1);
+                                mma_ts_pair_of(tmem_base + kColAcc, tmem_base + L::col_w(b, kk), sdesc_advance(db, kk * 2048), idesc_acc,
+                                               (adds || kk > 0) ? 1u : 0u, see);
                         }
                         begun |= see;
                     }
