@@ -1,7 +1,8 @@
 """Full-size parity: the Qwen3-8B-shaped pool in the launch configuration the benchmark times, the 30B-shaped
 pool with Pareto-tailed samples, the 1M-token pool with one 262144-token sample (Hq 64 / Hkv 4: sixteen query
 heads per kv head, tensors beyond 2^32 bytes) and the skew sweep of 65536-token sequences at every skew.  The
-"fused" cases run the same pools with a pair-tile plan, which makes the backward call take its fused form; config 6 is
+"fused" cases run the same pools with a pair-tile plan, which makes the backward call take its fused form, on pairs of CTAs;
+"short" is the 8B-shaped pool with samples of up to 1000 tokens, whose fused backward runs on single CTAs; config 6 is
 the micro-benchmark head shape (Hq 128 / Hkv 4 / d 256) on two packed 32768-token sequences.
 
 The whole oracle would take minutes here, so outputs are sampled: rows of O / LSE / dQ and
@@ -30,15 +31,17 @@ def _rel(got, want, floor=1e-3):
 @pytest.fixture(scope="module",
                 params=[(2, 0.0, False), (2, 0.0, True), (3, 0.0, False), (3, 0.0, True), (4, 0.0, False), (4, 0.0, True),
                         (5, 0.0, False), (5, 0.25, False), (5, 0.5, False), (5, 1.0, False), (5, 1.0, True),
-                        (6, 0.0, False), (6, 0.0, True)],
+                        (6, 0.0, False), (6, 0.0, True), (2, 0.0, True, 1000)],
                 ids=["config2", "config2_fused", "config3", "config3_fused", "config4", "config4_fused",
                      "config5_skew0", "config5_skew0.25", "config5_skew0.5", "config5_skew1", "config5_skew1_fused",
-                     "config6_d256", "config6_d256_pairs"])
+                     "config6_d256", "config6_d256_pairs", "short_fused"])
 def run(request):
     from paper_2607_23250_b200 import binding as lb
     fused = request.param[2]
     spec = pools.config(*request.param[:2])
     lengths = pools.pool_lengths(spec)
+    if len(request.param) > 3:
+        lengths = pools.random_layout(np.random.default_rng(7), spec.total_tokens, request.param[3])
     cu_np = pools.cu_seqlens(lengths)
     T, hq, hkv, d = spec.total_tokens, spec.hq, spec.hkv, spec.head_dim
     t = pools.make_tensors(T, hq, hkv, d, seed=0, device="cuda")
@@ -47,6 +50,8 @@ def run(request):
     plan = lb.libra_plan_tiles(cu, hq, 256, directions=directions, tile_kv=128, n_heads_kv=hkv,
                                total_tokens=T)                                             # as bench.py
     assert plan.status() == 0
+    if fused and d == 128:
+        assert plan.fused_ctas() == (1 if len(request.param) > 3 else 2)
     out, lse = lb.libra_attn_pool_fwd(t["q"], t["k"], t["v"], plan)
     dq, dk, dv = lb.libra_attn_pool_bwd(t["q"], t["k"], t["v"], out, lse, t["dout"], plan)
     torch.cuda.synchronize()

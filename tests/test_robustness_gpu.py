@@ -56,18 +56,20 @@ def test_token_bounds_of_a_malformed_plan_stay_inside_the_pool():
     plan.destroy()
 
 
-def test_pool_planner_overflow_leaves_defined_outputs():
+@pytest.mark.parametrize("cp,L", [(1024, 1_200_000), (128, 3_500_000), (7, 15_000_000)])
+def test_pool_planner_overflow_leaves_defined_outputs(cp, L):
     """One sample so long that the integer soft-cap test could overflow: the planner reports OVERFLOW, every tile
-    stays at its Q-home and the byte matrices stay zero.  Needs offsets only, no tensors."""
+    stays at its Q-home and the byte matrices stay zero.  Needs offsets only, no tensors.  64 shards x L (L + 1) / 2 pairs
+    are 4.6e13, 3.9e14 and 7.2e15; the bound, 2^63 / 206 / workers, is 4.4e13, 3.5e14 and 6.4e15.  1024 workers have a
+    thread each, the others are placed by one block."""
     from paper_2607_23250_b200 import binding as lb
-    L = 1_200_000          # 64 shards x L (L + 1) / 2 pairs = 4.6e13 > the bound of about 4.4e13 at 1024 workers
     cu = torch.tensor([0, L], dtype=torch.int32).cuda()
-    res = lb.libra_tap_plan(cu, [0, L], cp=1024, block=32768, n_shards=64, hq=64, hkv=4, head_dim=128)
+    res = lb.libra_tap_plan(cu, [0, L], cp=cp, block=32768, n_shards=64, hq=64, hkv=4, head_dim=128)
     torch.cuda.synchronize()
     assert int(res["status"].item()) == lb.ERR_OVERFLOW
     assert int(res["fwd_bytes"].abs().sum().item()) == 0 and int(res["bwd_bytes"].abs().sum().item()) == 0
-    sigma = res["sigma"].cpu().numpy()
-    assert sigma.min() >= 0 and sigma.max() < 1024
+    sigma, run = res["sigma"].cpu().numpy(), -(-L // cp)
+    assert np.array_equal(sigma, np.repeat(np.arange(0, L, 32768) // run, 64))
 
 
 def test_plan_of_another_device_or_shape_is_refused():

@@ -91,6 +91,14 @@ def test_steps_of_the_one_block_placement(P, CP, H, hq, hkv, max_len, total):
         _compare(cu, np.arange(P + 1, dtype=np.int32) * total, CP, 128, H, hq, hkv, 8, tau)
 
 
+@pytest.mark.parametrize("blocks", [1024, 1025, 2500])
+def test_blocks_beyond_a_batch_of_the_rank_sort(blocks):
+    rng = np.random.default_rng(blocks)
+    total = blocks * 4 - 1
+    cu = pools.cu_seqlens(pools.random_layout(rng, 2 * total, 300))
+    _compare(cu, [0, total, 2 * total], 4, 8, 1, 2, 1, 8)
+
+
 @pytest.mark.parametrize("P", [255, 256, 300, 1024])
 def test_many_sequences(P):
     """As many sequences as the smaller tables hold, more, and as many as there can be workers."""
